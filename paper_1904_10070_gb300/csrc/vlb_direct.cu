@@ -1,0 +1,368 @@
+// Direct Runge-Kutta stage for UW3 grids without the packed FP32 layout: FP64, and FP32 grids with a
+// ragged n_phi or too small for a staged box.  Same stage as stage_kernel (vlb_stage.cu); the populations
+// are read straight from global memory through L1 instead of being staged, so a tile can be small.
+//
+// FP64 is bound by the FP64 units (1.25 TFLOP/s nominal, pipe 99% active on the busiest SM): what counts is
+// the number of FP64 operations (780 a node and stage in the staged kernel, 500-550 here: parity basis
+// and row table of vlb_node.cuh, folded centre taps) and their spread over all SMs (16 x 32 tiles left 56 of 152
+// SMs idle on 128 x 384, and 148 on 32 x 64).  Per step: 32 x 64 304 -> 35 us, 128 x 384 305 -> 175 us.  FP64 CTAs
+// of one thread per node do not trigger the next stage early: its CTAs would fill the free slots of
+// lightly loaded SMs and unbalance it (85 us a stage against 66 on 128 x 384).
+// FP32 grids off the packed layout are bound by latency (one wave); no staging with a modulo and a
+// 4-byte copy per element: 250 x 501 diffusive 57.6 -> 40 us per step.
+#include "vlb_node.cuh"
+
+namespace vlb {
+
+namespace {
+
+__device__ const RowRules<float> g_rules32 = make_row_rules<float>();
+__device__ const RowRules<double> g_rules64 = make_row_rules<double>();
+template <typename T>
+__device__ __forceinline__ const RowRule<T>& row_rules(int e) {
+  if constexpr (sizeof(T) == 8)
+    return g_rules64.e[e];
+  else
+    return g_rules32.e[e];
+}
+
+template <typename T>
+struct DirectConst {
+  NodeConst<T> nc;
+  T v[4], K[4][4], ww[4][4];
+};
+
+// Element at byte offset `off` of an array whose base is uniform over the CTA.
+template <typename T>
+__device__ __forceinline__ T at(const T* base, uint32_t off) {
+  return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
+}
+template <typename T>
+__device__ __forceinline__ void put(T* base, uint32_t off, T v) {
+  *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off) = v;
+}
+
+__device__ __forceinline__ int wrap_near(int x, int n) {  // -n <= x
+  if (x < 0) return x + n;
+  while (x >= n) x -= n;
+  return x;
+}
+
+// Moment-box slots of a TQ x TSW tile: the tile's nodes, then one halo row on each side, then one halo
+// column on each side (no corners).
+template <int TQ, int TSW>
+__device__ __forceinline__ void slot_node(int it, int& mr, int& mc) {
+  if (it < TQ * TSW) {
+    mr = 1 + it / TSW;
+    mc = 1 + it % TSW;
+  } else if (it < TQ * TSW + 2 * TSW) {
+    const int j = it - TQ * TSW;
+    mr = j < TSW ? 0 : TQ + 1;
+    mc = 1 + j % TSW;
+  } else {
+    const int j = it - TQ * TSW - 2 * TSW;
+    mr = 1 + j % TQ;
+    mc = j < TQ ? 0 : TSW + 1;
+  }
+}
+
+// One CTA per TQ x TSW tile.  Step 1 puts the moments and mu of the tile and a halo of 1 into shared memory
+// (dn, 1/n, u^theta, u^phi, mu); step 2 evaluates the right-hand side and the update.
+template <typename T, int CH, bool F0, int TQ, int TSW, bool SPLIT>
+__global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
+    direct_kernel(StageArgs<T> a, const __grid_constant__ DirectConst<T> dc) {
+  constexpr bool DF = sizeof(T) == 4;
+  constexpr int MS = TSW + 2, MN = (TQ + 2) * MS, NTH = TQ * TSW * (SPLIT ? 4 : 1);
+  constexpr int ITEMS = TQ * TSW + 2 * TSW + 2 * TQ;
+  constexpr bool HOLD = sizeof(T) == 8;  // hold U^n in registers over step 1
+  constexpr bool TAB = !SPLIT && sizeof(T) == 8;  // row table in shared memory (FP64-bound), else per thread
+  constexpr int NE = row_entries<T>(), RP = NE | 1;  // odd row pitch: two rows of a warp on different banks
+  __shared__ T s_dn[MN], s_in[MN], s_ut[MN], s_up[MN], s_mu[MN], s_rt[TAB ? TQ * RP : 1];
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  const int nt = a.nt, ns = a.ns, tid = threadIdx.x;
+  const int tiles_s = (ns + TSW - 1) / TSW;  // 1-D grid: a column grid has more tile rows than gridDim.y may hold
+  const int q0 = (int)(blockIdx.x / tiles_s) * TQ, s0 = (int)(blockIdx.x % tiles_s) * TSW;
+  const int64_t st = a.stride;
+  constexpr uint32_t B = sizeof(T);
+  const NodeConst<T>& nc = dc.nc;
+  const T* phi = a.fin + NPOP * st;
+  T P[SPLIT ? 1 : 16], U0[SPLIT ? 4 : 16];
+  if (F0) {  // U^n of this thread's populations, in flight over step 1
+    const int node = SPLIT ? tid >> 2 : tid, q = q0 + node / TSW, s = s0 + node % TSW;
+    if (HOLD && q < nt && s < ns)
+#pragma unroll
+      for (int k = 0; k < (SPLIT ? 4 : 16); ++k)
+        U0[k] = SPLIT ? a.f0[(k + 4 * (tid & 3)) * st + (int64_t)q * ns + s]
+                      : at(a.f0 + k * st, (uint32_t)sizeof(T) * (uint32_t)(q * ns + s));
+  }
+  if constexpr (TAB) {
+    for (int e = tid; e < TQ * NE; e += NTH)
+      if (q0 + e / NE < nt) s_rt[(e / NE) * RP + e % NE] = row_entry(row_rules<T>(e % NE), a, q0 + e / NE, e % NE >= E_CC);
+  }
+
+  auto moments = [&](int it, bool keep) {
+    int mr, mc;
+    slot_node<TQ, TSW>(it, mr, mc);
+    if (q0 + mr - 1 > nt || s0 + mc - 1 > ns) return;  // beyond the halo of the last node
+    const int q = wrap_near(q0 + mr - 1, nt), s = wrap_near(s0 + mc - 1, ns);
+    const uint32_t id = B * (uint32_t)(q * ns + s);
+    T g[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) g[k] = at(a.fin + k * st, id);
+    const uint32_t in_ = B * (uint32_t)((q + 1 < nt ? q + 1 : 0) * ns + s);
+    const uint32_t is = B * (uint32_t)((q > 0 ? q - 1 : nt - 1) * ns + s);
+    const uint32_t ie = B * (uint32_t)(q * ns + (s + 1 < ns ? s + 1 : 0));
+    const uint32_t iw = B * (uint32_t)(q * ns + (s > 0 ? s - 1 : ns - 1));
+    const T ph = at(phi, id);
+    T dN = vsub(at(phi, in_), ph), dS = vsub(ph, at(phi, is)), lo = T(0);
+    T dE = vsub(at(phi, ie), ph), dW = vsub(ph, at(phi, iw));
+    if constexpr (DF) {
+      const T* pl = phi + st;
+      lo = at(pl, id);
+      dN = vadd(dN, vsub(at(pl, in_), lo));
+      dS = vadd(dS, vsub(lo, at(pl, is)));
+      dE = vadd(dE, vsub(at(pl, ie), lo));
+      dW = vadd(dW, vsub(lo, at(pl, iw)));
+    }
+    const T lt = a.coef[C_LT * nt + q], lp = a.coef[C_LP * nt + q];
+    const T jp = a.coef[C_JP * nt + q], jm = a.coef[C_JM * nt + q];
+    to_parity16(g);
+    T dn, mt, mp;
+    parity_moments(g, nc, dn, mt, mp);
+    const T inv_n = node_recip(vadd(a.n0, dn));
+    const int mi = mr * MS + mc;
+    s_dn[mi] = dn;
+    s_in[mi] = inv_n;
+    s_ut[mi] = vmul(mt, inv_n);
+    s_up[mi] = vmul(mp, inv_n);
+    const T lap = vfma(lp, vsub(dE, dW), vmul(lt, vsub(vmul(jp, dN), vmul(jm, dS))));
+    const T ph2 = vmul(ph, ph);
+    T cubic = vmul(ph, vsub(T(1), ph2));
+    if constexpr (DF) cubic = vfma(vsub(T(1), vmul(T(3), ph2)), lo, cubic);  // at hi + lo, to first order in lo
+    s_mu[mi] = vsub(vmul(-a.A, cubic), vmul(a.kappa, lap));
+    if constexpr (!SPLIT) {
+      if (keep)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) P[k] = g[k];
+    }
+  };
+  if constexpr (!SPLIT) {
+    moments(tid, true);
+    for (int it = NTH + tid; it < ITEMS; it += NTH) moments(it, false);
+  } else {
+    for (int it = tid; it < ITEMS; it += NTH) moments(it, false);
+  }
+  __syncthreads();
+  if (SPLIT || sizeof(T) == 4) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+
+  const int node = SPLIT ? tid >> 2 : tid;
+  const int lr = node / TSW, lc = node % TSW;
+  const int q = q0 + lr, s = s0 + lc;
+  if (q >= nt || s >= ns) return;
+  const int mi = (lr + 1) * MS + lc + 1;
+  T rl[TAB ? 1 : NE];
+  if constexpr (!TAB) row_all<T>(rl, a, q);
+  const T* rt = TAB ? s_rt + lr * RP : rl;
+  const uint32_t id = B * (uint32_t)(q * ns + s);  // byte offsets within one array (launch_direct checks the range)
+  const int qn = q + 1 < nt ? q + 1 : 0, qs = q > 0 ? q - 1 : nt - 1;
+  const int qnn = wrap_near(q + 2, nt), qss = wrap_near(q - 2, nt);
+  const int se = s + 1 < ns ? s + 1 : 0, sw = s > 0 ? s - 1 : ns - 1;
+  const int see = wrap_near(s + 2, ns), sww = s >= 2 ? s - 2 : (s - 2 + 2 * ns) % ns;
+  const T dt = a.dt, itau = a.inv_tau * dt;
+  const T dn = s_dn[mi], ut = s_ut[mi], up = s_up[mi], ph = at(phi, id);
+  const T mu_c = s_mu[mi], mu_n = s_mu[mi + MS], mu_s = s_mu[mi - MS], mu_e = s_mu[mi + 1], mu_w = s_mu[mi - 1];
+  T Ft = T(0), Fp = T(0);  // times dt
+  if (CH == VLB_HYDRO) {   // n F = -phi grad mu (Eq. pbin), central differences
+    const T pn = vmul(ph, s_in[mi]);
+    Ft = vmul(vmul(pn, vsub(mu_s, mu_n)), a.gt * dt);
+    Fp = vmul(vmul(pn, vsub(mu_w, mu_e)), rt[E_GP]);
+  }
+  const uint32_t on = B * (uint32_t)(qn * ns + s), os = B * (uint32_t)(qs * ns + s);
+  const uint32_t onn = B * (uint32_t)(qnn * ns + s), oss = B * (uint32_t)(qss * ns + s);
+  const uint32_t oe = B * (uint32_t)(q * ns + se), ow = B * (uint32_t)(q * ns + sw);
+  const uint32_t oee = B * (uint32_t)(q * ns + see), oww = B * (uint32_t)(q * ns + sww);
+  const int i_split = SPLIT ? tid & 3 : 0;
+  if (!SPLIT || i_split == 0) {
+    // Cahn-Hilliard: M Delta mu - div(u phi) (Eq. CH), flux form with mean face values, times dt
+    T L = vmul(rt[E_LP], vadd(vsub(mu_e, mu_c), vsub(mu_w, mu_c)));
+    L = vfma(rt[E_LN], vsub(mu_n, mu_c), L);
+    L = vfma(rt[E_LS], vsub(mu_s, mu_c), L);
+    if (CH == VLB_HYDRO) {
+      L = vfma(-rt[E_XN], vmul(s_ut[mi + MS], at(phi, on)), L);
+      L = vfma(rt[E_XS], vmul(s_ut[mi - MS], at(phi, os)), L);
+      L = vfma(-rt[E_YP], vsub(vmul(s_up[mi + 1], at(phi, oe)), vmul(s_up[mi - 1], at(phi, ow))), L);
+    }
+    if (a.dphi) {
+      put(a.dphi, id, L);  // the stabilised Cahn-Hilliard solve forms phi
+    } else {
+      const T lo = DF ? at(phi + st, id) : T(0);
+      T base = ph, base_lo = lo, inc = L;
+      if (F0) {
+        base = at(a.f0 + NPOP * st, id);
+        base_lo = DF ? at(a.f0 + (NPOP + 1) * st, id) : T(0);
+        inc = vmul(a.b, vadd(vadd(vsub(ph, base), vsub(lo, base_lo)), L));
+      }
+      if constexpr (DF) {  // (hi, lo) <- (base, base_lo) + inc, an error-free sum, renormalised
+        const T s1 = vadd(base, inc), bb = vsub(s1, base);
+        const T lo2 = vadd(base_lo, vadd(vsub(base, vsub(s1, bb)), vsub(inc, bb)));
+        const T hi = vadd(s1, lo2);
+        put(a.fout + NPOP * st, id, hi);
+        put(a.fout + (NPOP + 1) * st, id, vsub(lo2, vsub(hi, s1)));
+      } else {
+        put(a.fout + NPOP * st, id, vadd(base, inc));
+      }
+    }
+  }
+
+  // population k: acc (dt times the other terms) -> stored update.  UW3 seen from the upwind side has the
+  // weights 1, -6, 3, 2 on the far, near, centre and downwind nodes (tf .. td: theta, on J g; pv: varphi).
+  // FP64 folds the three centre taps into one coefficient, whose rounding is far below the scheme's;
+  // FP32 keeps the varphi difference on whole-number weights, which cancel on a uniform field.
+  auto update = [&](int k, T acc, T g0, T tf, T tn, T tm, T td, uint32_t rf, uint32_t rn, uint32_t rd, int y, T cc,
+                    uint32_t cf, uint32_t cn, uint32_t cd) {
+    const T* f = a.fin + k * st;
+    const T g = at(f, id), pv = rt[E_PVB + y];
+    if (F0 && !HOLD) g0 = at(a.f0 + k * st, id);
+    if (F0) acc = vadd(acc, vsub(g, g0));
+    acc = vfma(tf, at(f, rf), acc);
+    acc = vfma(tn, at(f, rn), acc);
+    acc = vfma(td, at(f, rd), acc);
+    if constexpr (DF) {
+      acc = vfma(tm, g, acc);
+      const T D = vfma(T(2), at(f, cd), vfma(T(3), g, vfma(T(-6), at(f, cn), at(f, cf))));
+      acc = vfma(-pv, D, acc);
+      acc = vfma(-itau, g, acc);
+    } else {
+      acc = vfma(-pv, at(f, cf), acc);
+      acc = vfma(rt[E_PV6 + y], at(f, cn), acc);
+      acc = vfma(rt[E_PV2 + y], at(f, cd), acc);
+      acc = vfma(cc, g, acc);
+    }
+    put(a.fout + k * st, id, F0 ? vfma(a.b, acc, g0) : vadd(acc, g));
+  };
+
+  if constexpr (!SPLIT) {
+    T R[16];
+    velocity_space(P, R, nc, rt, Ft, Fp, itau, a.n0, dn, ut, up);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int x = (i == 0 || i == 3) ? 0 : 1;
+      const T* t = rt + E_TH + 7 * x;
+      const T tf = t[i >= 2 ? TAP_FARP : TAP_FARN], tn = t[i >= 2 ? TAP_NEARP : TAP_NEARN], tm = t[TAP_MID];
+      const T td = t[i >= 2 ? TAP_DOWNP : TAP_DOWNN];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int y = (j == 0 || j == 3) ? 0 : 1;
+        update(4 * i + j, R[4 * i + j], U0[4 * i + j], tf, tn, tm, td, i >= 2 ? oss : onn, i >= 2 ? os : on,
+               i >= 2 ? on : os, y, DF ? T(0) : rt[E_CC + 2 * x + y], j >= 2 ? oww : oee, j >= 2 ? ow : oe,
+               j >= 2 ? oe : ow);
+      }
+    }
+  } else {
+    // four threads per node, thread i the populations of theta velocity v_i
+    const int i = i_split, x = (i == 0 || i == 3) ? 0 : 1;
+    const bool pos = i >= 2;
+    const T vi = dc.v[i], Ki[4] = {dc.K[i][0], dc.K[i][1], dc.K[i][2], dc.K[i][3]};
+    T dvt[4], h[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dvt[j] = vmul(Ki[0], at(a.fin + j * st, id));
+#pragma unroll
+    for (int m = 1; m < 4; ++m)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) dvt[j] = vfma(Ki[m], at(a.fin + (4 * m + j) * st, id), dvt[j]);
+    // Gamma v_i v_m from the row's products of magnitudes
+    T gb = x == 0 ? rt[E_GBB] : rt[E_GBA], ga = x == 0 ? rt[E_GBA] : rt[E_GAA];
+    gb = pos ? gb : -gb;
+    ga = pos ? ga : -ga;
+    h[0] = vmul(vsub(gb, Fp), at(a.fin + (4 * i) * st, id));
+    h[1] = vmul(vsub(ga, Fp), at(a.fin + (4 * i + 1) * st, id));
+    h[2] = vmul(vsub(-ga, Fp), at(a.fin + (4 * i + 2) * st, id));
+    h[3] = vmul(vsub(-gb, Fp), at(a.fin + (4 * i + 3) * st, id));
+    const T cyb = vsub(rt[E_GBB], Ft), cya = vsub(rt[E_GAA], Ft);
+    const T hu = vmul(T(-0.5), vfma(ut, ut, vmul(up, up))), c0 = vadd(T(1), hu);
+    const T dntau = vmul(dn, itau), ntau = vfma(itau, a.n0, dntau), ai = vmul(vi, ut);
+    // n0 v_i (E(sign v_i) + F^theta): the odd part changes sign with v_i, the even part does not
+    const T ci = vadd(dntau, vadd(x == 0 ? rt[E_NEB] : rt[E_NEA], vmul(a.n0 * vi, vadd(rt[E_EM], Ft)))), pF = vmul(a.n0, Fp);
+    const T vc = vmul(pos ? vi : -vi, vmul(a.coef[(int64_t)C_CT * nt + q], dt * T(1.0 / 6.0)));
+    const T* J = a.coef + (int64_t)C_J * nt;
+    const T tf = -vmul(vc, J[pos ? qss : qnn]), tn = vmul(T(6) * vc, J[pos ? qs : qn]);
+    const T td = vmul(T(-2) * vc, J[pos ? qn : qs]), tm = vmul(T(-3) * vc, J[q]);
+    const T ccx = vsub(tm, itau);
+    const uint32_t rf = pos ? oss : onn, rn = pos ? os : on, rd = pos ? on : os;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int y = (j == 0 || j == 3) ? 0 : 1;
+      T acc = vmul(dc.K[j][0], h[0]);
+#pragma unroll
+      for (int m = 1; m < 4; ++m) acc = vfma(dc.K[j][m], h[m], acc);
+      acc = vfma(y == 0 ? cyb : cya, dvt[j], acc);
+      const T xi = vfma(dc.v[j], up, ai);
+      const T pm1 = vfma(xi, vfma(xi, vfma(xi, T(1.0 / 6.0), T(0.5)), c0), hu);
+      acc = vfma(dc.ww[i][j], vfma(ntau, pm1, vfma(dc.v[j], pF, ci)), acc);
+      update(4 * i + j, acc, U0[j], tf, tn, tm, td, rf, rn, rd, y, DF ? T(0) : vfma(T(-3), rt[E_PVB + y], ccx),
+             j >= 2 ? oww : oee, j >= 2 ? ow : oe, j >= 2 ? oe : ow);
+    }
+  }
+}
+
+template <typename T>
+DirectConst<T> make_direct_const() {
+  const VelocityConsts d = velocity_consts();
+  DirectConst<T> c;
+  c.nc = make_node_const<T>();
+  for (int i = 0; i < 4; ++i) {
+    c.v[i] = (T)d.v[i];
+    for (int m = 0; m < 4; ++m) {
+      c.K[i][m] = (T)d.K[i][m];
+      c.ww[i][m] = (T)(d.w[i] * d.w[m]);
+    }
+  }
+  return c;
+}
+
+template <typename T, int CH, bool F0, int TQ, int TSW, bool SPLIT>
+cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
+  static const DirectConst<T> dc = make_direct_const<T>();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((a.ns + TSW - 1) / TSW) * (unsigned)((a.nt + TQ - 1) / TQ));
+  cfg.blockDim = dim3(TQ * TSW * (SPLIT ? 4 : 1));
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, direct_kernel<T, CH, F0, TQ, TSW, SPLIT>, a, dc);
+}
+
+// FP32: 4 x 32 tiles, one thread per node (8 x 32 tiles with 64 registers: 316 us against 304-320 on eight
+// steps of 250 x 501, within the spread).  FP64: 8 x 16 tiles, one thread per node, four warps a CTA: an SM
+// retires one FP64 warp instruction in 19 cycles, but a lone warp only one in 64 (measured), so four
+// warps saturate it and below about 32 nodes per SM the time is one warp's chain; there four
+// threads share a node (2 x 8 nodes a CTA).  Per step, one / four threads a node: 32 x 64 72 / 34 us, 64 x 128
+// 72 / 93 us, 128 x 384 175 / 330 us.
+constexpr int64_t kSplitNodes = 32 * 152;
+
+template <typename T, int CH, bool F0>
+cudaError_t launch_direct_v(const StageArgs<T>& a, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) return launch_direct_t<T, CH, F0, 4, 32, false>(a, st);
+  if ((int64_t)a.nt * a.ns <= kSplitNodes) return launch_direct_t<T, CH, F0, 2, 8, true>(a, st);
+  return launch_direct_t<T, CH, F0, 8, 16, false>(a, st);
+}
+
+}  // namespace
+
+template <typename T>
+cudaError_t launch_direct(const StageArgs<T>& a, int ch_mode, cudaStream_t st) {
+  // 32-bit byte offsets within an array: 2^32 bytes per array would need over 200 GB for the three
+  // states and as much again for the FP64 staging area, more than the device has
+  if ((uint64_t)a.nt * a.ns * sizeof(T) >= ((uint64_t)1 << 32)) return cudaErrorInvalidValue;
+  if (ch_mode == VLB_HYDRO)
+    return a.f0 ? launch_direct_v<T, VLB_HYDRO, true>(a, st) : launch_direct_v<T, VLB_HYDRO, false>(a, st);
+  return a.f0 ? launch_direct_v<T, VLB_DIFFUSIVE, true>(a, st) : launch_direct_v<T, VLB_DIFFUSIVE, false>(a, st);
+}
+
+template cudaError_t launch_direct<float>(const StageArgs<float>&, int, cudaStream_t);
+template cudaError_t launch_direct<double>(const StageArgs<double>&, int, cudaStream_t);
+
+}  // namespace vlb

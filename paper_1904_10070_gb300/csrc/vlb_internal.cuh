@@ -136,6 +136,9 @@ cudaError_t launch_wave(const StageArgs<float>& a, int ch_mode, float* U0, float
 template <typename T>
 cudaError_t launch_stage(const StageArgs<T>& a, int advection, int ch_mode, cudaStream_t s,
                          const StageMaps* maps = nullptr);
+// One UW3 stage without staging (vlb_direct.cu): FP64, and FP32 grids outside the packed layout.
+template <typename T>
+cudaError_t launch_direct(const StageArgs<T>& a, int ch_mode, cudaStream_t s);
 // Axisymmetric grids (n_phi = 1, n_theta <= kAxiMaxRows): `steps` whole SSP-RK3 steps of the
 // column in one single-CTA launch, on the buffers U0 (U^n, updated in place), U1, U2.  a.fin, a.f0,
 // a.fout and a.b are set per stage inside the kernel.

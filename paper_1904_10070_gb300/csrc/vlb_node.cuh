@@ -1,0 +1,289 @@
+// Per-node arithmetic shared by the step kernels: the velocity-space part of the right-hand side
+// (force, inertial and BGK terms of Eq. boltz_tor) in the parity basis of the velocity set.
+//
+// The Q = 4 velocities come in pairs +-b, +-a (b = v_4, a = v_3), so each velocity direction splits
+// into even and odd combinations c = 0..3: E_b = g_+b + g_-b, E_a, O_b = g_+b - g_-b, O_a.  The
+// derivative kernel K^H changes the sign of the velocity under reflection, so it maps even to odd and
+// odd to even: 8 multiplications instead of 16 per vector.  The Hermite equilibrium splits likewise
+// into even-even, odd-even, even-odd and odd-odd parts of a few operations each.  One node costs 32 (to the
+// basis) + 32 (back) additions and about 180 multiply-adds, against about 330 on the populations
+// themselves; the step kernels are bound by the floating-point units, so this is their main saving.
+// Moments are sums of the same combinations.
+//
+// V is the lane type: double, float, or float2 (two nodes in packed FP32x2 arithmetic).  All
+// operations are explicitly rounded (no contraction), so that every kernel and every column of a
+// grid evaluates the same sequence of roundings.
+#pragma once
+
+#include "vlb_internal.cuh"
+
+namespace vlb {
+
+template <typename V> struct LaneOf { using S = V; };
+template <> struct LaneOf<float2> { using S = float; };
+
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double vsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+template <typename V>
+__device__ __forceinline__ V bc(typename LaneOf<V>::S x) {
+  if constexpr (sizeof(V) == 8 && sizeof(typename LaneOf<V>::S) == 4)
+    return make_float2(x, x);
+  else
+    return x;
+}
+
+__device__ __forceinline__ float node_recip(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double node_recip(double x) { return __drcp_rn(x); }
+
+// Velocity constants in the parity basis (index 0: b, 1: a): kap maps even to odd, lam odd to even
+// (both with the basis's normalisation 1/4 folded in), ww = w_x w_y.
+template <typename T>
+struct NodeConst {
+  T v[2], v2[2], kap[2][2], lam[2][2], ww[2][2];
+};
+
+template <typename T>
+NodeConst<T> make_node_const() {
+  const VelocityConsts d = velocity_consts();
+  const int pos[2] = {3, 2}, neg[2] = {0, 1};
+  NodeConst<T> c;
+  for (int x = 0; x < 2; ++x) {
+    c.v[x] = (T)d.v[pos[x]];
+    c.v2[x] = (T)(d.v[pos[x]] * d.v[pos[x]]);
+    for (int y = 0; y < 2; ++y) {
+      c.kap[x][y] = (T)(0.25 * (d.K[pos[x]][pos[y]] + d.K[pos[x]][neg[y]]));
+      c.lam[x][y] = (T)(0.25 * (d.K[pos[x]][pos[y]] - d.K[pos[x]][neg[y]]));
+      c.ww[x][y] = (T)(d.w[pos[x]] * d.w[pos[y]]);
+    }
+  }
+  return c;
+}
+
+// Row table: everything of the right-hand side that depends on the theta row alone, times dt, formed once
+// per CTA and row in shared memory (about 70 operations that every node would otherwise repeat).  Entry e of
+// row q is  S (c1 X1(q) Y + c2 X2(q))  -  [e >= E_CC] dt / tau,  with X1, X2 coefficient arrays, S one
+// of dt, n0 dt, M dt and Y one of 1, J(q - 2 .. q + 2), J(q +- 1/2).
+enum RowEntry : int {
+  E_GBB = 0,  // Gamma v_b^2, Gamma v_b v_a, Gamma v_a^2
+  E_GBA,
+  E_GAA,
+  E_EM,   // (E_pos + E_neg) / 2 of the rest-state residual
+  E_NEB,  // n0 v_x (E_pos - E_neg) / 2, x = b, a
+  E_NEA,
+  E_GP,   // 1 / (2 R J dvarphi)
+  E_PVB,  // v_x / (6 R J dvarphi), x = b, a
+  E_PVA,
+  E_LP,   // M times the Laplace-Beltrami coefficients: varphi, north, south
+  E_LN,
+  E_LS,
+  E_XN,   // Cahn-Hilliard advection: J(q + 1), J(q - 1) over 2 r J dtheta; 1 / (2 R J dvarphi)
+  E_XS,
+  E_YP,
+  E_TH,   // theta taps of -v (flux difference), per x: far+, near+, down-, centre, near-, down+, far-
+  E_PV6 = E_TH + 14,  // FP64: 6 and -2 times E_PVx, then the sum of the three centre taps per (x, y)
+  E_PV2 = E_PV6 + 2,
+  E_CC = E_PV2 + 2,
+  NROW32 = E_PV6,
+  NROW64 = E_CC + 4
+};
+enum RowTap : int { TAP_FARP = 0, TAP_NEARP, TAP_DOWNN, TAP_MID, TAP_NEARN, TAP_DOWNP, TAP_FARN };
+template <typename T>
+constexpr int row_entries() { return sizeof(T) == 8 ? NROW64 : NROW32; }
+
+// One entry's rule; y: 0 none, 1 .. 5 J(q - 2) .. J(q + 2), 6 J(q + 1/2), 7 J(q - 1/2); s: 0 dt, 1 n0 dt, 2 M dt.
+// Compile-time tables in global memory: lanes of a warp read different entries, which a constant bank serialises.
+template <typename T>
+struct RowRule {
+  T c1, c2;
+  unsigned char s, x1, y, x2;
+};
+template <typename T>
+struct RowRules {
+  RowRule<T> e[NROW64];
+};
+constexpr double csqrt(double x) {
+  double r = x;
+  for (int i = 0; i < 60; ++i) r = 0.5 * (r + x / r);
+  return r;
+}
+constexpr double kVelA = csqrt(3.0 - csqrt(6.0)), kVelB = csqrt(3.0 + csqrt(6.0));  // Eq. vmatrix
+
+template <typename T>
+constexpr RowRules<T> make_row_rules() {
+  RowRules<T> r{};
+  auto set = [&](int e, double c1, int s, int x1, int y, double c2 = 0.0, int x2 = 0) {
+    r.e[e] = RowRule<T>{(T)c1, (T)c2, (unsigned char)s, (unsigned char)x1, (unsigned char)y, (unsigned char)x2};
+  };
+  const double v[2] = {kVelB, kVelA};
+  set(E_GBB, v[0] * v[0], 0, C_GAM, 0);
+  set(E_GBA, v[0] * v[1], 0, C_GAM, 0);
+  set(E_GAA, v[1] * v[1], 0, C_GAM, 0);
+  set(E_EM, 0.5, 0, C_EP, 0, 0.5, C_EN);
+  set(E_GP, 1.0, 0, C_GP, 0);
+  set(E_LP, 1.0, 2, C_LP, 0);
+  set(E_LN, 1.0, 2, C_LT, 6);
+  set(E_LS, 1.0, 2, C_LT, 7);
+  set(E_XN, 0.5, 0, C_CT, 4);
+  set(E_XS, 0.5, 0, C_CT, 2);
+  set(E_YP, 0.5, 0, C_CP, 0);
+  for (int x = 0; x < 2; ++x) {
+    set(E_NEB + x, 0.5 * v[x], 1, C_EP, 0, -0.5 * v[x], C_EN);
+    set(E_PVB + x, v[x] / 6.0, 0, C_CP, 0);
+    const int t = E_TH + 7 * x;
+    set(t + TAP_FARP, -v[x] / 6.0, 0, C_CT, 1);
+    set(t + TAP_NEARP, v[x], 0, C_CT, 2);
+    set(t + TAP_DOWNN, -v[x] / 3.0, 0, C_CT, 2);
+    set(t + TAP_MID, -v[x] / 2.0, 0, C_CT, 3);
+    set(t + TAP_NEARN, v[x], 0, C_CT, 4);
+    set(t + TAP_DOWNP, -v[x] / 3.0, 0, C_CT, 4);
+    set(t + TAP_FARN, -v[x] / 6.0, 0, C_CT, 5);
+    set(E_PV6 + x, v[x], 0, C_CP, 0);
+    set(E_PV2 + x, -v[x] / 3.0, 0, C_CP, 0);
+    for (int y = 0; y < 2; ++y) set(E_CC + 2 * x + y, -v[x] / 2.0, 0, C_CT, 3, -v[y] / 2.0, C_CP);
+  }
+  return r;
+}
+
+// Entry of row q by rule r (a lane each), or (row_entry<e>) for an entry known at compile time.
+template <typename T>
+__device__ __forceinline__ T row_entry(const RowRule<T>& r, const StageArgs<T>& a, int q, bool centre) {
+  const int nt = a.nt, y = r.y, s = r.s;
+  const T sc = vmul(a.dt, s == 0 ? T(1) : (s == 1 ? a.n0 : a.M));
+  T v = vmul(vmul(r.c1, sc), a.coef[(int64_t)r.x1 * nt + q]);
+  if (y) {
+    int row = q, arr = C_J;
+    if (y <= 5) {
+      row += y - 3;
+      row += row < 0 ? nt : (row >= nt ? -nt : 0);
+    } else {
+      arr = y == 6 ? C_JP : C_JM;
+    }
+    v = vmul(v, a.coef[(int64_t)arr * nt + row]);
+  }
+  if (r.c2 != T(0)) v = vfma(vmul(r.c2, sc), a.coef[(int64_t)r.x2 * nt + q], v);
+  if (centre) v = vfma(-a.dt, a.inv_tau, v);
+  return v;
+}
+template <typename T>
+__device__ __forceinline__ void row_all(T (&rt)[row_entries<T>()], const StageArgs<T>& a, int q) {
+  constexpr RowRules<T> R = make_row_rules<T>();
+#pragma unroll
+  for (int e = 0; e < row_entries<T>(); ++e) rt[e] = row_entry(R.e[e], a, q, e >= E_CC);
+}
+
+// (x_0 .. x_3) at velocities (-b, -a, a, b) <-> (E_b, E_a, O_b, O_a)
+template <typename V>
+__device__ __forceinline__ void to_parity(V& x0, V& x1, V& x2, V& x3) {
+  const V eb = vadd(x3, x0), ea = vadd(x2, x1), ob = vsub(x3, x0), oa = vsub(x2, x1);
+  x0 = eb;
+  x1 = ea;
+  x2 = ob;
+  x3 = oa;
+}
+template <typename V>
+__device__ __forceinline__ void from_parity(V& x0, V& x1, V& x2, V& x3) {
+  const V pb = vadd(x0, x2), mb = vsub(x0, x2), pa = vadd(x1, x3), ma = vsub(x1, x3);
+  x0 = mb;
+  x1 = ma;
+  x2 = pa;
+  x3 = pb;
+}
+
+// g[4 i + j] (i: theta velocity, j: varphi velocity) -> P[4 ci + cj]
+template <typename V>
+__device__ __forceinline__ void to_parity16(V (&g)[16]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) to_parity(g[4 * i], g[4 * i + 1], g[4 * i + 2], g[4 * i + 3]);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) to_parity(g[j], g[4 + j], g[8 + j], g[12 + j]);
+}
+template <typename V>
+__device__ __forceinline__ void from_parity16(V (&r)[16]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) from_parity(r[j], r[4 + j], r[8 + j], r[12 + j]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) from_parity(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+}
+
+// Deviation of the density and the momentum density (Sec. 2.3) from the parity combinations.
+template <typename V, typename T>
+__device__ __forceinline__ void parity_moments(const V (&P)[16], const NodeConst<T>& nc, V& dn, V& mt, V& mp) {
+  dn = vadd(vadd(P[0], P[1]), vadd(P[4], P[5]));
+  mt = vfma(bc<V>(nc.v[0]), vadd(P[8], P[9]), vmul(bc<V>(nc.v[1]), vadd(P[12], P[13])));
+  mp = vfma(bc<V>(nc.v[0]), vadd(P[2], P[6]), vmul(bc<V>(nc.v[1]), vadd(P[3], P[7])));
+}
+
+// Velocity-space terms of the right-hand side times dt, from the combinations P:
+//   dt { (Gamma v_j^2 - F^theta) K g  +  K~-term (-F^phi - Gamma v_i v_j)  +  w_i w_j X },
+//   X = (dn + n (poly - 1)) / tau + n0 v_i (E(sign v_i) + F^theta) + n0 v_j F^phi
+// (poly the third-order Hermite polynomial of Eq. feq; the -g/tau part is left to the caller), turned
+// back to populations in R.  Ft, Fp and itau arrive multiplied by dt; rt is the node's row of the table.
+template <typename V, typename T>
+__device__ __forceinline__ void velocity_space(const V (&P)[16], V (&R)[16], const NodeConst<T>& nc, const T* rt, V Ft,
+                                               V Fp, T itau, T n0, V dn, V ut, V up) {
+  const V g[2][2] = {{bc<V>(rt[E_GBB]), bc<V>(rt[E_GBA])}, {bc<V>(rt[E_GBA]), bc<V>(rt[E_GAA])}};
+#pragma unroll
+  for (int cj = 0; cj < 4; ++cj) {  // (Gamma v_j^2 - F^theta) K along theta velocities
+    const V c = vsub(g[cj & 1][cj & 1], Ft);
+    const V q0 = vmul(c, P[cj]), q1 = vmul(c, P[4 + cj]), q2 = vmul(c, P[8 + cj]), q3 = vmul(c, P[12 + cj]);
+    R[8 + cj] = vfma(bc<V>(nc.kap[0][1]), q1, vmul(bc<V>(nc.kap[0][0]), q0));
+    R[12 + cj] = vfma(bc<V>(nc.kap[1][1]), q1, vmul(bc<V>(nc.kap[1][0]), q0));
+    R[cj] = vfma(bc<V>(nc.lam[0][1]), q3, vmul(bc<V>(nc.lam[0][0]), q2));
+    R[4 + cj] = vfma(bc<V>(nc.lam[1][1]), q3, vmul(bc<V>(nc.lam[1][0]), q2));
+  }
+#pragma unroll
+  for (int ci = 0; ci < 4; ++ci) {
+    // minus K along varphi velocities of (F^phi + Gamma v_i v_m) g: v_i v_m flips both parities
+    const int x = ci & 1, cb = 4 * (ci ^ 2), c0 = 4 * ci;
+    const V h0 = vfma(g[x][0], P[cb + 2], vmul(Fp, P[c0])), h1 = vfma(g[x][1], P[cb + 3], vmul(Fp, P[c0 + 1]));
+    const V h2 = vfma(g[x][0], P[cb], vmul(Fp, P[c0 + 2])), h3 = vfma(g[x][1], P[cb + 1], vmul(Fp, P[c0 + 3]));
+    R[c0 + 2] = vfma(bc<V>(-nc.kap[0][0]), h0, vfma(bc<V>(-nc.kap[0][1]), h1, R[c0 + 2]));
+    R[c0 + 3] = vfma(bc<V>(-nc.kap[1][0]), h0, vfma(bc<V>(-nc.kap[1][1]), h1, R[c0 + 3]));
+    R[c0] = vfma(bc<V>(-nc.lam[0][0]), h2, vfma(bc<V>(-nc.lam[0][1]), h3, R[c0]));
+    R[c0 + 1] = vfma(bc<V>(-nc.lam[1][0]), h2, vfma(bc<V>(-nc.lam[1][1]), h3, R[c0 + 1]));
+  }
+  // equilibrium and reference part, with A = v_x u^theta, B = v_y u^phi per velocity magnitude
+  const V dntau = vmul(dn, bc<V>(itau)), ntau = vfma(bc<V>(itau), bc<V>(n0), dntau);
+  const V hut = vmul(vmul(bc<V>(T(0.5)), ut), ut), hup = vmul(vmul(bc<V>(T(0.5)), up), up);
+  const V us = vadd(hut, hup), one = vsub(bc<V>(T(1)), us);
+  const V tF = vmul(bc<V>(n0), vadd(Ft, bc<V>(rt[E_EM]))), pF = vmul(bc<V>(n0), Fp);
+  const V nut = vmul(ntau, ut), nup = vmul(ntau, up);
+  const V third = bc<V>(T(1) / T(3));
+  V hB[2], B[2], nhB[2], nB[2], pB[2];
+#pragma unroll
+  for (int y = 0; y < 2; ++y) {
+    hB[y] = vmul(bc<V>(nc.v2[y]), hup);
+    B[y] = vmul(bc<V>(nc.v[y]), up);
+    nhB[y] = vmul(ntau, hB[y]);
+    nB[y] = vmul(bc<V>(nc.v[y]), nup);
+    pB[y] = vmul(bc<V>(nc.v[y]), pF);
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const V hA = vmul(bc<V>(nc.v2[x]), hut), nA = vmul(bc<V>(nc.v[x]), nut);
+    const V pre = vfma(ntau, vsub(hA, us), vadd(dntau, bc<V>(rt[E_NEB + x])));
+    const V cx = vfma(third, hA, one), dx = vmul(bc<V>(nc.v[x]), tF), ox = vadd(hA, one);
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const V w = bc<V>(nc.ww[x][y]);
+      R[4 * x + y] = vfma(w, vadd(pre, nhB[y]), R[4 * x + y]);
+      R[4 * x + 8 + y] = vfma(w, vfma(nA, vadd(cx, hB[y]), dx), R[4 * x + 8 + y]);
+      R[4 * x + y + 2] = vfma(w, vfma(nB[y], vfma(third, hB[y], ox), pB[y]), R[4 * x + y + 2]);
+      R[4 * x + 8 + y + 2] = vfma(w, vmul(nA, B[y]), R[4 * x + 8 + y + 2]);
+    }
+  }
+  from_parity16(R);
+}
+
+}  // namespace vlb

@@ -20,7 +20,8 @@
 // arithmetic, two nodes per thread.  A persistent double-buffered variant (next tile copied in
 // while the current one computes, one 384-thread CTA per SM) measured 1.6x slower on GB300: with
 // 12 warps per SM and all warps issuing copies and shared loads in the same phase, the memory-
-// input queue throttled issue to 30%.
+// input queue throttled issue to 30%.  FP64 UW3 grids and FP32 UW3 grids off the packed layout are stepped by
+// direct_kernel (vlb_direct.cu).
 // Periodic wrap-around is resolved on the copy addresses, so ragged tiles need no special case.
 #include <vector>
 
@@ -1648,8 +1649,11 @@ cudaError_t launch_one(const StageArgs<T>& a, cudaStream_t st, const StageMaps* 
                   : launch_generic<T, ADV, CH, false, true, false>(a, st, nullptr);
     }
   }
-  return a.f0 ? launch_generic<T, ADV, CH, true, false, false>(a, st, nullptr)
-              : launch_generic<T, ADV, CH, false, false, false>(a, st, nullptr);
+  if constexpr (ADV == VLB_UW3)
+    return launch_direct<T>(a, CH, st);  // FP64, and FP32 off the packed layout (vlb_direct.cu)
+  else
+    return a.f0 ? launch_generic<T, ADV, CH, true, false, false>(a, st, nullptr)
+                : launch_generic<T, ADV, CH, false, false, false>(a, st, nullptr);
 }
 
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
