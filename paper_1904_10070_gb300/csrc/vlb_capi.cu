@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "vlb_handle.cuh"
+#include "vlb_node.cuh"
 
 // Raises the handle's device flag when a diagnostic vector shows an unstable state.
 cudaError_t vlb_internal_flag(const double* diag, int* flag, cudaStream_t s);
@@ -79,7 +80,7 @@ bool params_ok(const vlb_params* p, char* why, size_t n) {
 struct Layout {
   int64_t N, stride;
   size_t esize;
-  size_t off_coefT, off_coefD, off_U[3], off_staging, off_partials, off_totals, off_diag, off_flag, off_dphi, off_fft,
+  size_t off_coefT, off_coefD, off_rows, off_U[3], off_staging, off_partials, off_totals, off_diag, off_flag, off_dphi, off_fft,
       off_wave, total;
 };
 
@@ -93,6 +94,9 @@ Layout layout(const vlb_params* p) {
   off = align_up(off + (size_t)vlb::NCOEF * p->n_theta * L.esize, 256);
   L.off_coefD = off;
   off = align_up(off + (size_t)vlb::NCOEF * p->n_theta * 8, 256);
+  L.off_rows = off;
+  if (L.esize == 4 && p->advection == VLB_UW3)
+    off = align_up(off + sizeof(float) * vlb::kRowTable * p->n_theta, 256);
   for (int k = 0; k < 3; ++k) {
     L.off_U[k] = off;
     off = align_up(off + (size_t)vlb::state_arrays(L.esize) * L.stride * L.esize, 256);
@@ -161,6 +165,20 @@ void row_tables(const vlb_params* p, double* out) {
   }
 }
 
+// Row table of the FP32 pair kernels (RowEntry in vlb_node.cuh) from the FP64 coefficient tables.
+void pair_rows(const vlb_params* p, const double* tab, float* out) {
+  constexpr vlb::RowRules<double> rules = vlb::make_row_rules<double>();
+  const int nt = p->n_theta;
+  for (int q = 0; q < nt; ++q)
+    for (int e = 0; e < vlb::kRowTable; ++e) {
+      const vlb::RowRule<double>& r = rules.e[e];
+      double y = 1.0;
+      if (r.y) y = tab[vlb::C_J * nt + (q + r.y - 3 + nt) % nt];
+      const double s = r.s == 3 ? 1.0 : r.s == 2 ? p->kappa : (r.s == 1 ? p->dt * p->M : p->dt);
+      out[(size_t)q * vlb::kRowTable + e] = (float)(s * (r.c1 * tab[r.x1 * nt + q] * y + r.c2 * tab[r.x2 * nt + q]));
+    }
+}
+
 // The reference density n0 of the stored deviations from the row sums of n: the area-weighted mean
 // sum_q J_q row_q / sum_q J_q N_phi (J_q = 1 + (r/R) cos theta_q), rounded to 20 significant bits so
 // that it is exact in FP32.  False if it is not finite and positive.
@@ -218,9 +236,15 @@ vlb_status upload_tables(vlb_handle* h) {
     else
       ((float*)tabT)[i] = (float)tab[i];
   }
+  std::vector<float> rows;
   cudaError_t e = cudaMemcpyAsync(h->coefD, tab, sizeof(double) * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->coefT, tabT, h->esize * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess && h->rows) {
+    rows.resize((size_t)nt * vlb::kRowTable);
+    pair_rows(p, tab, rows.data());
+    e = cudaMemcpyAsync(h->rows, rows.data(), sizeof(float) * rows.size(), cudaMemcpyHostToDevice, h->stream);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   free(tab);
   free(tabT);
@@ -252,6 +276,7 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
   const vlb_params& p = h->p;
   vlb::StageArgs<T> a;
   a.coef = (const T*)h->coefT;
+  if constexpr (sizeof(T) == 4) a.rows = h->rows;
   a.nt = p.n_theta;
   a.ns = p.n_phi;
   a.stride = h->stride;
@@ -556,6 +581,7 @@ vlb_status vlb_create(const vlb_params* p, void* d_workspace, size_t bytes, void
   h->ws_bytes = bytes;
   h->coefT = h->ws + L.off_coefT;
   h->coefD = (double*)(h->ws + L.off_coefD);
+  if (L.off_rows < L.off_U[0]) h->rows = (float*)(h->ws + L.off_rows);
   for (int k = 0; k < 3; ++k) h->U[k] = h->ws + L.off_U[k];
   h->staging = (double*)(h->ws + L.off_staging);
   h->partials = (double*)(h->ws + L.off_partials);
@@ -593,6 +619,12 @@ vlb_status vlb_create(const vlb_params* p, void* d_workspace, size_t bytes, void
   e = cudaMemcpyAsync(h->coefD, tab, sizeof(double) * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->coefT, tabT, L.esize * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
+  std::vector<float> rows;
+  if (e == cudaSuccess && h->rows) {
+    rows.resize((size_t)nt * vlb::kRowTable);
+    pair_rows(p, tab, rows.data());
+    e = cudaMemcpyAsync(h->rows, rows.data(), sizeof(float) * rows.size(), cudaMemcpyHostToDevice, h->stream);
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.off_U[0], 0, L.off_staging - L.off_U[0], h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream);
   std::vector<double> lam;
@@ -1214,6 +1246,7 @@ vlb_status vlb_ensemble_create(const vlb_params* p, int32_t count, void* d_works
     v->ws_bytes = bytes;
     v->coefT = base + L.off_coefT;
     v->coefD = (double*)(base + L.off_coefD);
+    v->rows = (float*)(base + L.off_rows);
     for (int k = 0; k < 3; ++k) v->U[k] = base + L.off_U[k];
     v->staging = h->staging;
     v->partials = h->partials;
@@ -1236,6 +1269,7 @@ vlb_status vlb_ensemble_create(const vlb_params* p, int32_t count, void* d_works
     vlb::EnsembleMember& d = desc[m];
     for (int k = 0; k < 3; ++k) d.U[k] = (float*)v->U[k];
     d.coef = (const float*)v->coefT;
+    d.rows = v->rows;
     d.nt = p[m].n_theta;
     d.ns = p[m].n_phi;
     d.stride = L.stride;

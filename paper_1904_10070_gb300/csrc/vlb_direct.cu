@@ -185,8 +185,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
   if (!SPLIT || i_split == 0) {
     // Cahn-Hilliard: M Delta mu - div(u phi) (Eq. CH), flux form with mean face values, times dt
     T L = vmul(rt[E_LP], vadd(vsub(mu_e, mu_c), vsub(mu_w, mu_c)));
-    L = vfma(rt[E_LN], vsub(mu_n, mu_c), L);
-    L = vfma(rt[E_LS], vsub(mu_s, mu_c), L);
+    L = vfma(rt[E_LT], vfma(rt[E_JP], vsub(mu_n, mu_c), vmul(rt[E_JM], vsub(mu_s, mu_c))), L);
     if (CH == VLB_HYDRO) {
       L = vfma(-rt[E_XN], vmul(s_ut[mi + MS], at(phi, on)), L);
       L = vfma(rt[E_XS], vmul(s_ut[mi - MS], at(phi, os)), L);
@@ -221,7 +220,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
   auto update = [&](int k, T acc, T g0, T tf, T tn, T tm, T td, uint32_t rf, uint32_t rn, uint32_t rd, int y, T cc,
                     uint32_t cf, uint32_t cn, uint32_t cd) {
     const T* f = a.fin + k * st;
-    const T g = at(f, id), pv = rt[E_PVB + y];
+    const T g = at(f, id), pv = rt[E_TH + 8 * y + TAP_PV];
     if (F0 && !HOLD) g0 = at(a.f0 + k * st, id);
     if (F0) acc = vadd(acc, vsub(g, g0));
     acc = vfma(tf, at(f, rf), acc);
@@ -247,7 +246,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int x = (i == 0 || i == 3) ? 0 : 1;
-      const T* t = rt + E_TH + 7 * x;
+      const T* t = rt + E_TH + 8 * x;
       const T tf = t[i >= 2 ? TAP_FARP : TAP_FARN], tn = t[i >= 2 ? TAP_NEARP : TAP_NEARN], tm = t[TAP_MID];
       const T td = t[i >= 2 ? TAP_DOWNP : TAP_DOWNN];
 #pragma unroll
@@ -282,7 +281,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
     const T hu = vmul(T(-0.5), vfma(ut, ut, vmul(up, up))), c0 = vadd(T(1), hu);
     const T dntau = vmul(dn, itau), ntau = vfma(itau, a.n0, dntau), ai = vmul(vi, ut);
     // n0 v_i (E(sign v_i) + F^theta): the odd part changes sign with v_i, the even part does not
-    const T ci = vadd(dntau, vadd(x == 0 ? rt[E_NEB] : rt[E_NEA], vmul(a.n0 * vi, vadd(rt[E_EM], Ft)))), pF = vmul(a.n0, Fp);
+    const T ci = vadd(dntau, vmul(a.n0, vadd(x == 0 ? rt[E_NEB] : rt[E_NEA], vmul(vi, vadd(rt[E_EM], Ft))))), pF = vmul(a.n0, Fp);
     const T vc = vmul(pos ? vi : -vi, vmul(a.coef[(int64_t)C_CT * nt + q], dt * T(1.0 / 6.0)));
     const T* J = a.coef + (int64_t)C_J * nt;
     const T tf = -vmul(vc, J[pos ? qss : qnn]), tn = vmul(T(6) * vc, J[pos ? qs : qn]);
@@ -299,7 +298,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
       const T xi = vfma(dc.v[j], up, ai);
       const T pm1 = vfma(xi, vfma(xi, vfma(xi, T(1.0 / 6.0), T(0.5)), c0), hu);
       acc = vfma(dc.ww[i][j], vfma(ntau, pm1, vfma(dc.v[j], pF, ci)), acc);
-      update(4 * i + j, acc, U0[j], tf, tn, tm, td, rf, rn, rd, y, DF ? T(0) : vfma(T(-3), rt[E_PVB + y], ccx),
+      update(4 * i + j, acc, U0[j], tf, tn, tm, td, rf, rn, rd, y, DF ? T(0) : vfma(T(-3), rt[E_TH + 8 * y + TAP_PV], ccx),
              j >= 2 ? oww : oee, j >= 2 ? ow : oe, j >= 2 ? oe : ow);
     }
   }

@@ -16,6 +16,7 @@ struct vlb_handle {
   void* U[3];          // U^n, U^(1), U^(2)
   void* coefT;         // [NCOEF][n_theta] in state precision
   double* coefD;       // [NCOEF][n_theta] FP64
+  float* rows = nullptr;  // FP32 UW3: row table [n_theta][kRowTable] of the pair kernels
   double* staging;     // 17 N doubles
   double* partials;    // totals_blocks() * 8
   double* totals;      // 8 doubles (read-out)

@@ -58,12 +58,15 @@ struct VelocityConsts {
 };
 VelocityConsts velocity_consts();  // computed from the Hermite definitions in FP64
 
+constexpr int kRowTable = 32;  // FP32 entries per row of the row table
+
 template <typename T>
 struct StageArgs {
   const T* fin;     // state read by the right-hand side (17 arrays)
   const T* f0;      // U^n for the Runge-Kutta combination (NULL in the first stage)
   T* fout;          // output state (may alias f0 at the same node)
   const T* coef;    // [NCOEF][n_theta]
+  const T* rows = nullptr;  // FP32 pair kernels: row table [n_theta][kRowTable] (vlb_node.cuh)
   int nt, ns;
   int64_t stride;   // elements between consecutive arrays
   T b, dt;         // U_out = U0 + b (U_in - U0 + dt L(U_in)); without U0: U_in + dt L(U_in)
@@ -91,6 +94,7 @@ cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, i
 struct EnsembleMember {
   float* U[3];        // U^n, U^(1), U^(2)
   const float* coef;  // [NCOEF][n_theta]
+  const float* rows;  // [n_theta][kRowTable]
   int nt, ns;
   int64_t stride;
   float dt, inv_tau, M, A, kappa, gt, n0;

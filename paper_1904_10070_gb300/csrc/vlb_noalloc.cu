@@ -18,7 +18,7 @@
 
 #include <mutex>
 
-#include "vlb_internal.cuh"
+#include "vlb_node.cuh"
 
 namespace {
 
@@ -26,20 +26,36 @@ constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[VLB_NOALLOC_SCRATCH_BYTES];
 
+// Row table of the packed FP32 stages (vlb_node.cuh): they need at least 40 columns, so the scratch
+// bounds their rows.
+constexpr int kMaxPairRows = (int)(VLB_NOALLOC_SCRATCH_BYTES / (2 * sizeof(float) * (vlb::NARR + 1) * 40));
+static __device__ __align__(256) float g_noalloc_rows[kMaxPairRows * vlb::kRowTable];
+__device__ const vlb::RowRules<float> g_noalloc_rules = vlb::make_row_rules<float>();
+
+__global__ void noalloc_rows(vlb::StageArgs<float> a) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= a.nt * vlb::kRowTable) return;
+  const int q = x / vlb::kRowTable, e = x % vlb::kRowTable;
+  g_noalloc_rows[x] = vlb::row_entry(g_noalloc_rules.e[e], a, q, false);
+}
+
 std::mutex g_mu;
 void* g_scratch_ptr[kMaxDevices] = {};
+void* g_rows_ptr[kMaxDevices] = {};
 thread_local char g_noalloc_err[256] = "";
 
 // Device address of the scratch array on the current device (set-up on the first call per device).
-cudaError_t scratch_address(int dev, void** out) {
+cudaError_t scratch_address(int dev, void** out, void** rows) {
   std::lock_guard<std::mutex> lock(g_mu);
   if (!g_scratch_ptr[dev]) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&g_rows_ptr[dev], g_noalloc_rows);
     if (e != cudaSuccess) return e;
     g_scratch_ptr[dev] = p;
   }
   *out = g_scratch_ptr[dev];
+  *rows = g_rows_ptr[dev];
   return cudaSuccess;
 }
 
@@ -97,7 +113,7 @@ const char* check_params(const vlb_params* p) {
 
 template <typename T>
 cudaError_t run(const vlb_params* p, T* state, int64_t stride, double n0, int64_t nsteps, unsigned char* scratch,
-                cudaStream_t st) {
+                float* rows, cudaStream_t st) {
   const int nt = p->n_theta;
   T* coef = reinterpret_cast<T*>(scratch);
   T* U1 = reinterpret_cast<T*>(scratch + align256(sizeof(T) * vlb::NCOEF * nt));
@@ -118,6 +134,13 @@ cudaError_t run(const vlb_params* p, T* state, int64_t stride, double n0, int64_
   a.gt = (T)(1.0 / (2.0 * p->r * (2.0 * M_PI / nt)));
   a.n0 = (T)n0;
   a.err = nullptr;
+  if constexpr (sizeof(T) == 4) {
+    if (p->advection == VLB_UW3 && vlb::stage_maps_apply(nt, p->n_phi)) {
+      a.rows = rows;
+      noalloc_rows<<<(nt * vlb::kRowTable + 127) / 128, 128, 0, st>>>(a);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+  }
   for (int64_t n = 0; n < nsteps; ++n) {
     a.fin = state; a.f0 = nullptr; a.fout = U1; a.b = (T)1;
     if ((e = vlb::launch_stage<T>(a, p->advection, p->ch_mode, st)) != cudaSuccess) return e;
@@ -170,12 +193,12 @@ vlb_status vlb_step_noalloc(const vlb_params* p, void* d_state, int64_t stride, 
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return fail(VLB_ERR_CUDA, cudaGetErrorString(e));
   if (dev < 0 || dev >= kMaxDevices) return fail(VLB_ERR_CUDA, "device index out of range");
-  void* scratch = nullptr;
-  e = scratch_address(dev, &scratch);
+  void *scratch = nullptr, *rows = nullptr;
+  e = scratch_address(dev, &scratch, &rows);
   if (e != cudaSuccess) return fail(VLB_ERR_CUDA, cudaGetErrorString(e));
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  e = esize == 8 ? run<double>(p, (double*)d_state, stride, n0, nsteps, (unsigned char*)scratch, st)
-                 : run<float>(p, (float*)d_state, stride, n0, nsteps, (unsigned char*)scratch, st);
+  e = esize == 8 ? run<double>(p, (double*)d_state, stride, n0, nsteps, (unsigned char*)scratch, (float*)rows, st)
+                 : run<float>(p, (float*)d_state, stride, n0, nsteps, (unsigned char*)scratch, (float*)rows, st);
   if (e != cudaSuccess) return fail(VLB_ERR_CUDA, cudaGetErrorString(e));
   return VLB_OK;
 }

@@ -70,38 +70,42 @@ NodeConst<T> make_node_const() {
   return c;
 }
 
-// Row table: everything of the right-hand side that depends on the theta row alone, times dt, formed once
-// per CTA and row in shared memory (about 70 operations that every node would otherwise repeat).  Entry e of
-// row q is  S (c1 X1(q) Y + c2 X2(q))  -  [e >= E_CC] dt / tau,  with X1, X2 coefficient arrays, S one
-// of dt, n0 dt, M dt and Y one of 1, J(q - 2 .. q + 2), J(q +- 1/2).
+// Row table: everything of the right-hand side that depends on the theta row alone, times dt (about 70
+// operations that every node would otherwise repeat).  Entry e of row q is
+//   S (c1 X1(q) Y + c2 X2(q))  -  [e >= E_CC] dt / tau
+// with X1, X2 coefficient arrays, S one of dt, M dt, kappa and 1, and Y one of 1, J(q - 2 .. q + 2).
+// FP32 pair kernels read the 32-entry rows of a table in global memory, formed once per handle in FP64; the FP64
+// direct kernel forms the rows of its tile in shared memory.
 enum RowEntry : int {
   E_GBB = 0,  // Gamma v_b^2, Gamma v_b v_a, Gamma v_a^2
   E_GBA,
   E_GAA,
   E_EM,   // (E_pos + E_neg) / 2 of the rest-state residual
-  E_NEB,  // n0 v_x (E_pos - E_neg) / 2, x = b, a
+  E_NEB,  // v_x (E_pos - E_neg) / 2, x = b, a
   E_NEA,
   E_GP,   // 1 / (2 R J dvarphi)
-  E_PVB,  // v_x / (6 R J dvarphi), x = b, a
-  E_PVA,
-  E_LP,   // M times the Laplace-Beltrami coefficients: varphi, north, south
-  E_LN,
-  E_LS,
+  E_LP,   // M times the Laplace-Beltrami coefficients: varphi, theta
+  E_LT,
   E_XN,   // Cahn-Hilliard advection: J(q + 1), J(q - 1) over 2 r J dtheta; 1 / (2 R J dvarphi)
   E_XS,
   E_YP,
-  E_TH,   // theta taps of -v (flux difference), per x: far+, near+, down-, centre, near-, down+, far-
-  E_PV6 = E_TH + 14,  // FP64: 6 and -2 times E_PVx, then the sum of the three centre taps per (x, y)
+  E_JP,   // J(q + 1/2), J(q - 1/2) (not folded into E_LT, E_KT: neighbouring rows share the rounded value)
+  E_JM,
+  E_KT,   // kappa times the Laplace-Beltrami coefficients (for mu; not times dt): theta, varphi
+  E_KP,
+  E_TH,   // per x, 8 entries: theta taps of -v (flux difference) (RowTap), then v_x / (6 R J dvarphi)
+  E_PV6 = E_TH + 16,  // FP64: 6 and -2 times the varphi weight, then the sum of the centre taps per (x, y)
   E_PV2 = E_PV6 + 2,
   E_CC = E_PV2 + 2,
   NROW32 = E_PV6,
   NROW64 = E_CC + 4
 };
-enum RowTap : int { TAP_FARP = 0, TAP_NEARP, TAP_DOWNN, TAP_MID, TAP_NEARN, TAP_DOWNP, TAP_FARN };
+enum RowTap : int { TAP_FARP = 0, TAP_NEARP, TAP_DOWNN, TAP_MID, TAP_NEARN, TAP_DOWNP, TAP_FARN, TAP_PV };
 template <typename T>
 constexpr int row_entries() { return sizeof(T) == 8 ? NROW64 : NROW32; }
 
-// One entry's rule; y: 0 none, 1 .. 5 J(q - 2) .. J(q + 2), 6 J(q + 1/2), 7 J(q - 1/2); s: 0 dt, 1 n0 dt, 2 M dt.
+// One entry's rule; y: 0 none, 1 .. 5 J(q - 2) .. J(q + 2); s: 0 dt, 1 M dt,
+// 2 kappa, 3 one.
 // Compile-time tables in global memory: lanes of a warp read different entries, which a constant bank serialises.
 template <typename T>
 struct RowRule {
@@ -131,16 +135,19 @@ constexpr RowRules<T> make_row_rules() {
   set(E_GAA, v[1] * v[1], 0, C_GAM, 0);
   set(E_EM, 0.5, 0, C_EP, 0, 0.5, C_EN);
   set(E_GP, 1.0, 0, C_GP, 0);
-  set(E_LP, 1.0, 2, C_LP, 0);
-  set(E_LN, 1.0, 2, C_LT, 6);
-  set(E_LS, 1.0, 2, C_LT, 7);
+  set(E_LP, 1.0, 1, C_LP, 0);
+  set(E_LT, 1.0, 1, C_LT, 0);
+  set(E_JP, 1.0, 3, C_JP, 0);
+  set(E_JM, 1.0, 3, C_JM, 0);
+  set(E_KT, 1.0, 2, C_LT, 0);
+  set(E_KP, 1.0, 2, C_LP, 0);
   set(E_XN, 0.5, 0, C_CT, 4);
   set(E_XS, 0.5, 0, C_CT, 2);
   set(E_YP, 0.5, 0, C_CP, 0);
   for (int x = 0; x < 2; ++x) {
-    set(E_NEB + x, 0.5 * v[x], 1, C_EP, 0, -0.5 * v[x], C_EN);
-    set(E_PVB + x, v[x] / 6.0, 0, C_CP, 0);
-    const int t = E_TH + 7 * x;
+    set(E_NEB + x, 0.5 * v[x], 0, C_EP, 0, -0.5 * v[x], C_EN);
+    const int t = E_TH + 8 * x;
+    set(t + TAP_PV, v[x] / 6.0, 0, C_CP, 0);
     set(t + TAP_FARP, -v[x] / 6.0, 0, C_CT, 1);
     set(t + TAP_NEARP, v[x], 0, C_CT, 2);
     set(t + TAP_DOWNN, -v[x] / 3.0, 0, C_CT, 2);
@@ -159,17 +166,12 @@ constexpr RowRules<T> make_row_rules() {
 template <typename T>
 __device__ __forceinline__ T row_entry(const RowRule<T>& r, const StageArgs<T>& a, int q, bool centre) {
   const int nt = a.nt, y = r.y, s = r.s;
-  const T sc = vmul(a.dt, s == 0 ? T(1) : (s == 1 ? a.n0 : a.M));
+  const T sc = s == 3 ? T(1) : (s == 2 ? a.kappa : (s == 1 ? vmul(a.dt, a.M) : a.dt));
   T v = vmul(vmul(r.c1, sc), a.coef[(int64_t)r.x1 * nt + q]);
   if (y) {
-    int row = q, arr = C_J;
-    if (y <= 5) {
-      row += y - 3;
-      row += row < 0 ? nt : (row >= nt ? -nt : 0);
-    } else {
-      arr = y == 6 ? C_JP : C_JM;
-    }
-    v = vmul(v, a.coef[(int64_t)arr * nt + row]);
+    int row = q + y - 3;
+    row += row < 0 ? nt : (row >= nt ? -nt : 0);
+    v = vmul(v, a.coef[(int64_t)C_J * nt + row]);
   }
   if (r.c2 != T(0)) v = vfma(vmul(r.c2, sc), a.coef[(int64_t)r.x2 * nt + q], v);
   if (centre) v = vfma(-a.dt, a.inv_tau, v);
@@ -272,7 +274,7 @@ __device__ __forceinline__ void velocity_space(const V (&P)[16], V (&R)[16], con
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
     const V hA = vmul(bc<V>(nc.v2[x]), hut), nA = vmul(bc<V>(nc.v[x]), nut);
-    const V pre = vfma(ntau, vsub(hA, us), vadd(dntau, bc<V>(rt[E_NEB + x])));
+    const V pre = vfma(ntau, vsub(hA, us), vfma(bc<V>(n0), bc<V>(rt[E_NEB + x]), dntau));
     const V cx = vfma(third, hA, one), dx = vmul(bc<V>(nc.v[x]), tF), ox = vadd(hA, one);
 #pragma unroll
     for (int y = 0; y < 2; ++y) {
@@ -284,6 +286,32 @@ __device__ __forceinline__ void velocity_space(const V (&P)[16], V (&R)[16], con
     }
   }
   from_parity16(R);
+}
+
+// Fifth-order WENO-JS face value between g2 and g3 of the window g0..g4, upwind from g0's side.
+template <typename T>
+__device__ __forceinline__ T weno5(T g0, T g1, T g2, T g3, T g4) {
+  const T c13_12 = T(13) / T(12), sixth = T(1) / T(6), eps = T(1e-6);
+  T q0 = (T(2) * g0 - T(7) * g1 + T(11) * g2) * sixth;
+  T q1 = (-g1 + T(5) * g2 + T(2) * g3) * sixth;
+  T q2 = (T(2) * g2 + T(5) * g3 - g4) * sixth;
+  T d0 = g0 - T(2) * g1 + g2, e0 = g0 - T(4) * g1 + T(3) * g2;
+  T d1 = g1 - T(2) * g2 + g3, e1 = g1 - g3;
+  T d2 = g2 - T(2) * g3 + g4, e2 = T(3) * g2 - T(4) * g3 + g4;
+  T b0 = c13_12 * d0 * d0 + T(0.25) * e0 * e0;
+  T b1 = c13_12 * d1 * d1 + T(0.25) * e1 * e1;
+  T b2 = c13_12 * d2 * d2 + T(0.25) * e2 * e2;
+  T a0 = T(0.1) / ((eps + b0) * (eps + b0));
+  T a1 = T(0.6) / ((eps + b1) * (eps + b1));
+  T a2 = T(0.3) / ((eps + b2) * (eps + b2));
+  return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2);
+}
+
+// WENO5 flux difference face_{+1/2} - face_{-1/2} at the centre x[3] of a 7-point window.
+template <typename T, bool POS>
+__device__ __forceinline__ T weno_diff(const T (&x)[7]) {
+  if (POS) return weno5(x[1], x[2], x[3], x[4], x[5]) - weno5(x[0], x[1], x[2], x[3], x[4]);
+  return weno5(x[6], x[5], x[4], x[3], x[2]) - weno5(x[5], x[4], x[3], x[2], x[1]);
 }
 
 }  // namespace vlb

@@ -15,9 +15,13 @@
 //   2. computes the moments and mu on the tile plus a halo of 1;
 //   3. computes the right-hand sides and the Runge-Kutta combination and stores the tile.
 // One 256-thread CTA per 16 x 32 tile, two CTAs per SM.  For FP32 UW3 grids with n_phi % 4 == 0 (the
-// production path) step 3 runs on adjacent node pairs in packed FP32x2 arithmetic, two lanes of
-// one float2 per thread; every other case (FP64, WENO5, odd or tiny grids) runs step 3 in scalar
-// arithmetic, two nodes per thread.  A persistent double-buffered variant (next tile copied in
+// production path) steps 2 and 3 run on adjacent node pairs in packed FP32x2 arithmetic, two lanes of
+// one float2 per thread: a thread loads its pair once in step 2, keeps the parity combinations of the
+// populations (vlb_node.cuh) over the barrier and reads everything that depends on the row from a table.
+// The stage is bound by latency and the shared-memory pipe (58% busy) at 16 warps per SM, with HBM at about 75%;
+// against step 3 on the populations themselves the warp instructions of a launch at 1024 x 2048 fell from 44.0
+// to 34.0 M, its time from 82.6 to 76.1 us (stage 1: 77.7 to 68.6) and the step from 0.235 to 0.217 ms.
+// WENO5 grids and ragged ensemble members run steps 2 and 3 in scalar arithmetic, two nodes per thread.  A persistent double-buffered variant (next tile copied in
 // while the current one computes, one 384-thread CTA per SM) measured 1.6x slower on GB300: with
 // 12 warps per SM and all warps issuing copies and shared loads in the same phase, the memory-
 // input queue throttled issue to 30%.  FP64 UW3 grids and FP32 UW3 grids off the packed layout are stepped by
@@ -25,7 +29,7 @@
 // Periodic wrap-around is resolved on the copy addresses, so ragged tiles need no special case.
 #include <vector>
 
-#include "vlb_internal.cuh"
+#include "vlb_node.cuh"
 
 namespace vlb {
 
@@ -38,6 +42,7 @@ template <typename T>
 struct VConst {
   T v[4], w[4], K[4][4];
   T ww[4][4];  // w_i w_j
+  NodeConst<T> nc;
 };
 
 // Shared-memory layout of one CTA.  Offsets are in elements of T.
@@ -49,7 +54,9 @@ struct Lay {
   static constexpr int BQ = TQ + 2 * H, BS = TS + 2 * HS;
   static constexpr int BOX = NST * BQ * BS;          // populations, phi (, phi lo)
   static constexpr int MQ = TQ + 2, MS = TS + 4;     // moment / mu box: halo 1, column origin -2
-  static constexpr int CO = (NCT * BQ + 15) / 16 * 16;  // padded: sub-buffers stay 16-byte aligned
+  // row coefficients: NCT x BQ for the scalar step 3, or the row table of rows -1 .. TQ for packed pairs; padded:
+  // sub-buffers stay 128-byte aligned
+  static constexpr int CO = ((NCT * BQ > (TQ + 2) * kRowTable ? NCT * BQ : (TQ + 2) * kRowTable) + 31) / 32 * 32;
   static constexpr int VEC = 16 / sizeof(T);              // elements per 16-byte chunk
   // each box row starts HS columns left of the tile: shift the buffers so that the tile columns
   // (and every 16-byte chunk copied into them) start on a 16-byte boundary
@@ -148,32 +155,6 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, i
 
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
-
-// Fifth-order WENO-JS face value between g2 and g3 of the window g0..g4, upwind from g0's side.
-template <typename T>
-__device__ __forceinline__ T weno5(T g0, T g1, T g2, T g3, T g4) {
-  const T c13_12 = T(13) / T(12), sixth = T(1) / T(6), eps = T(1e-6);
-  T q0 = (T(2) * g0 - T(7) * g1 + T(11) * g2) * sixth;
-  T q1 = (-g1 + T(5) * g2 + T(2) * g3) * sixth;
-  T q2 = (T(2) * g2 + T(5) * g3 - g4) * sixth;
-  T d0 = g0 - T(2) * g1 + g2, e0 = g0 - T(4) * g1 + T(3) * g2;
-  T d1 = g1 - T(2) * g2 + g3, e1 = g1 - g3;
-  T d2 = g2 - T(2) * g3 + g4, e2 = T(3) * g2 - T(4) * g3 + g4;
-  T b0 = c13_12 * d0 * d0 + T(0.25) * e0 * e0;
-  T b1 = c13_12 * d1 * d1 + T(0.25) * e1 * e1;
-  T b2 = c13_12 * d2 * d2 + T(0.25) * e2 * e2;
-  T a0 = T(0.1) / ((eps + b0) * (eps + b0));
-  T a1 = T(0.6) / ((eps + b1) * (eps + b1));
-  T a2 = T(0.3) / ((eps + b2) * (eps + b2));
-  return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2);
-}
-
-// WENO5 flux difference face_{+1/2} - face_{-1/2} at the centre x[3] of a 7-point window.
-template <typename T, bool POS>
-__device__ __forceinline__ T weno_diff(const T (&x)[7]) {
-  if (POS) return weno5(x[1], x[2], x[3], x[4], x[5]) - weno5(x[0], x[1], x[2], x[3], x[4]);
-  return weno5(x[6], x[5], x[4], x[3], x[2]) - weno5(x[5], x[4], x[3], x[2], x[1]);
-}
 
 // Whether the chunked copy path applies: rows wrap at most once and columns come in aligned
 // 16-byte chunks that never straddle the periodic seam.
@@ -498,15 +479,9 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
 }
 
 // ---------------------------------------------------------------------------------------------
-// Step 3, packed FP32 pairs: two horizontally adjacent nodes per thread, one float2 lane each, so
-// the per-population arithmetic issues as FFMA2/FADD2/FMUL2 and shared/global accesses are 8 bytes.
-// Same arithmetic as phase3_node, lane by lane.
+// Packed FP32 pairs: two horizontally adjacent nodes per thread, one float2 lane each.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ float2 f2(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 
@@ -520,150 +495,146 @@ __device__ __forceinline__ void df_add(float base, float base_lo, float inc, flo
   lo = lo2 - (hi - s1);
 }
 
-// Step 2 on packed node pairs (FP32): moment-box positions (mr, mc) and (mr, mc + 1), mc even, in
-// FP32x2 arithmetic; lanes: bit 0 stores the first, bit 1 the second.
+// (0, r): the row table of row q0 + r - 1, r = 0 .. TQ + 1, by 16-byte copies
 template <typename L>
-__device__ __forceinline__ void pair_point(const StageArgs<float>& a, const VConst<float>& vc, const float* box,
-                                           const float* co, float* sm, int mr, int mc, int lanes) {
+__device__ __forceinline__ void issue_rows(const StageArgs<float>& a, float* co, int q0, int tid) {
+  for (int x = tid; x < (L::TQ + 2) * (kRowTable / 4); x += L::NTH) {
+    const int r = x / (kRowTable / 4), c = x % (kRowTable / 4);
+    cp_async16(co + r * kRowTable + 4 * c, a.rows + (int64_t)wrap(q0 + r - 1, a.nt) * kRowTable + 4 * c);
+  }
+}
+
+// Moments, mu and the parity combinations of a pair of adjacent nodes.
+struct PairNode {
+  float2 P[16], dn, inv, ut, up, ph, lo, mu;
+};
+
+static_assert(E_JP % 4 == 0 && E_KP == E_JP + 3 && E_TH % 8 == 0 && NROW32 == kRowTable, "16-byte groups of the row table");
+
+// Step 2 on packed node pairs (FP32): moment-box positions (mr, mc) and (mr, mc + 1), mc even.
+template <typename L>
+__device__ __forceinline__ void pair_point(const StageArgs<float>& a, const NodeConst<float>& nc, const float* box,
+                                           const float* rows, int mr, int mc, PairNode& o) {
   constexpr int H = L::H, BQ = L::BQ, BS = L::BS, HS = L::HS, MS = L::MS;
-  static_assert(HS % 2 == 0 && BS % 2 == 0 && MS % 2 == 0 && L::N_OFF % 2 == 0 && L::UT_OFF % 2 == 0 &&
-                    L::UP_OFF % 2 == 0 && L::MU_OFF % 2 == 0,
+  static_assert(HS % 2 == 0 && BS % 2 == 0 && MS % 2 == 0 && L::UT_OFF % 2 == 0 && L::UP_OFF % 2 == 0 &&
+                    L::MU_OFF % 2 == 0,
                 "pair alignment");
   const int bi = (mr + H - 1) * BS + (mc - 2 + HS);  // even
   const float* fp = box + bi;
-  float2 row[4] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)}, col[4] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 x = ld2(fp + (4 * i + j) * BQ * BS);
-      row[i] = add2(row[i], x);
-      col[j] = add2(col[j], x);
-    }
-  // n = n0 + sum g (the reference part carries no momentum); v_1 = -v_4, v_2 = -v_3
-  const float2 dn = add2(add2(row[0], row[1]), add2(row[2], row[3]));
-  const float2 mt = fma2(f2(vc.v[3]), sub2(row[3], row[0]), mul2(f2(vc.v[2]), sub2(row[2], row[1])));
-  const float2 mp = fma2(f2(vc.v[3]), sub2(col[3], col[0]), mul2(f2(vc.v[2]), sub2(col[2], col[1])));
-  const float2 nn = add2(f2(a.n0), dn);
-  const float2 inv_n = make_float2(__frcp_rn(nn.x), __frcp_rn(nn.y));
-  const float2 ut = mul2(mt, inv_n), up = mul2(mp, inv_n);
-  const int cr = mr + H - 1;
+  for (int k = 0; k < 16; ++k) o.P[k] = ld2(fp + k * BQ * BS);
   const float* pp = box + NPOP * BQ * BS + bi;
   const float* pl = box + (NPOP + 1) * BQ * BS + bi;
   const float2 ph = ld2(pp), lo = ld2(pl);
   const float2 phW = ld2(pp - 2), phE = ld2(pp + 2), loW = ld2(pl - 2), loE = ld2(pl + 2);
   // neighbour differences of phi = hi + lo: the hi differences are exact for nearby values
-  float2 dN = sub2(ld2(pp + BS), ph), dS = sub2(ph, ld2(pp - BS));
-  float2 dE = sub2(make_float2(ph.y, phE.x), ph), dW = sub2(ph, make_float2(phW.y, ph.x));
-  dN = add2(dN, sub2(ld2(pl + BS), lo));
-  dS = add2(dS, sub2(lo, ld2(pl - BS)));
-  dE = add2(dE, sub2(make_float2(lo.y, loE.x), lo));
-  dW = add2(dW, sub2(lo, make_float2(loW.y, lo.x)));
-  const float2 lap = fma2(f2(co[C_LP * BQ + cr]), sub2(dE, dW),
-                          mul2(f2(co[C_LT * BQ + cr]),
-                               sub2(mul2(f2(co[C_JP * BQ + cr]), dN), mul2(f2(co[C_JM * BQ + cr]), dS))));
+  float2 dN = vsub(ld2(pp + BS), ph), dS = vsub(ph, ld2(pp - BS));
+  float2 dE = vsub(make_float2(ph.y, phE.x), ph), dW = vsub(ph, make_float2(phW.y, ph.x));
+  dN = vadd(dN, vsub(ld2(pl + BS), lo));
+  dS = vadd(dS, vsub(lo, ld2(pl - BS)));
+  dE = vadd(dE, vsub(make_float2(lo.y, loE.x), lo));
+  dW = vadd(dW, vsub(lo, make_float2(loW.y, lo.x)));
+  const float4 c = *reinterpret_cast<const float4*>(rows + mr * kRowTable + E_JP);  // JP, JM, KT, KP
+  const float2 klap = vfma(f2(c.w), vsub(dE, dW), vmul(f2(c.z), vsub(vmul(f2(c.x), dN), vmul(f2(c.y), dS))));
   // phi (1 - phi^2) at hi + lo, to first order in lo
-  const float2 ph2 = mul2(ph, ph);
-  const float2 cubic = fma2(sub2(f2(1.0f), mul2(f2(3.0f), ph2)), lo, mul2(ph, sub2(f2(1.0f), ph2)));
-  const float2 mu = sub2(mul2(f2(-a.A), cubic), mul2(f2(a.kappa), lap));
-  const int mi = mr * MS + mc;  // even
-  if (lanes == 3) {
-    st2(sm + L::N_OFF + mi, dn);
-    st2(sm + L::UT_OFF + mi, ut);
-    st2(sm + L::UP_OFF + mi, up);
-    st2(sm + L::MU_OFF + mi, mu);
-  } else {
-    const int o = lanes == 1 ? 0 : 1;
-    sm[L::N_OFF + mi + o] = o ? dn.y : dn.x;
-    sm[L::UT_OFF + mi + o] = o ? ut.y : ut.x;
-    sm[L::UP_OFF + mi + o] = o ? up.y : up.x;
-    sm[L::MU_OFF + mi + o] = o ? mu.y : mu.x;
-  }
+  const float2 ph2 = vmul(ph, ph);
+  const float2 cubic = vfma(vfma(f2(-3.0f), ph2, f2(1.0f)), lo, vmul(ph, vsub(f2(1.0f), ph2)));
+  o.mu = vsub(vmul(f2(-a.A), cubic), klap);
+  to_parity16(o.P);
+  float2 mt, mp;
+  parity_moments(o.P, nc, o.dn, mt, mp);
+  const float2 nn = vadd(f2(a.n0), o.dn);
+  o.inv = make_float2(__frcp_rn(nn.x), __frcp_rn(nn.y));
+  o.ut = vmul(mt, o.inv);
+  o.up = vmul(mp, o.inv);
+  o.ph = ph;
+  o.lo = lo;
 }
 
-// Step 2 on packed node pairs: tile columns 0 .. TS-1 of every moment row two at a time; the halo
-// columns -1 and TS of the tile rows inside the aligned pairs (-2, -1) and (TS, TS + 1), keeping
-// one lane, so that every column takes the same sequence of FP32 operations (an axisymmetric
-// state stays bitwise axisymmetric).  The pairs' other lanes read box columns -4 .. TS + 3, inside
-// the HS = 4 halo.
+// Step 2 for the whole tile.  A thread's own pair of nodes stays in registers for step 3 (with its parity
+// combinations); the threads of the first warps also take the halo: rows -1 and TQ (mu, u^theta), and the
+// columns -1 and TS inside the aligned pairs (-2, -1) and (TS, TS + 1), keeping one lane (mu, u^phi), so
+// that every column takes the same sequence of FP32 operations (an axisymmetric state stays bitwise
+// axisymmetric).  The pairs' other lanes read box columns -4 .. TS + 3, inside the HS = 4 halo.
 template <typename L>
-__device__ __forceinline__ void phase2_pair(const StageArgs<float>& a, const VConst<float>& vc, const float* box,
-                                            const float* co, float* sm, int tid) {
-  constexpr int MQ = L::MQ, TQ = L::TQ, NP = MQ * (TS / 2), NSGL = 2 * TQ;
+__device__ __forceinline__ void phase2_pair(const StageArgs<float>& a, const NodeConst<float>& nc, const float* box,
+                                            const float* rows, float* sm, int tid, PairNode& own) {
+  constexpr int MQ = L::MQ, TQ = L::TQ, MS = L::MS, NROWS = TS;  // TS / 2 pairs in each of two halo rows
   static_assert(L::HS >= 4, "the halo pairs read two columns beyond the halo column");
-  for (int idx = tid; idx < NP + NSGL; idx += L::NTH) {
-    int mr, mc, lanes = 3;
-    if (idx < NP) {
-      mr = idx / (TS / 2);
-      mc = 2 + 2 * (idx - mr * (TS / 2));
-    } else {  // column TS: first lane of (TS, TS + 1); column -1: second lane of (-2, -1)
-      const int j = idx - NP;
-      mr = 1 + (j >> 1);
-      mc = (j & 1) ? TS + 2 : 0;
-      lanes = (j & 1) ? 1 : 2;
+  static_assert(L::NTH == TQ * (TS / 2) && NROWS + 2 * TQ <= L::NTH, "one node pair per thread, one halo item at most");
+  if (tid < NROWS + 2 * TQ) {
+    PairNode h;
+    if (tid < NROWS) {
+      const int mr = tid < TS / 2 ? 0 : MQ - 1, mc = 2 + 2 * (tid % (TS / 2));
+      pair_point<L>(a, nc, box, rows, mr, mc, h);
+      st2(sm + L::MU_OFF + mr * MS + mc, h.mu);
+      st2(sm + L::UT_OFF + mr * MS + mc, h.ut);
+    } else {
+      const int j = tid - NROWS, mr = 1 + (j >> 1);
+      const bool east = j & 1;
+      const int mc = east ? TS + 2 : 0, mi = mr * MS + mc + (east ? 0 : 1);
+      pair_point<L>(a, nc, box, rows, mr, mc, h);
+      sm[L::MU_OFF + mi] = east ? h.mu.x : h.mu.y;
+      sm[L::UP_OFF + mi] = east ? h.up.x : h.up.y;
     }
-    pair_point<L>(a, vc, box, co, sm, mr, mc, lanes);
   }
+  const int mr = 1 + tid / (TS / 2), mc = 2 + 2 * (tid % (TS / 2));
+  pair_point<L>(a, nc, box, rows, mr, mc, own);
+  st2(sm + L::MU_OFF + mr * MS + mc, own.mu);
+  st2(sm + L::UT_OFF + mr * MS + mc, own.ut);
+  st2(sm + L::UP_OFF + mr * MS + mc, own.up);
 }
 
+// Step 3 on a pair: right-hand sides and the Runge-Kutta combination (velocity-space terms in the parity basis,
+// vlb_node.cuh).  Two lanes of one float2, so the arithmetic issues as FFMA2 / FADD2 / FMUL2 and
+// shared and global accesses are 8 bytes; the two varphi taps that straddle a pair are scalar.
 template <typename L, int CH, bool F0>
-__device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const VConst<float>& vc, const float* box,
-                                            const float* co, const float* sm, int lr, int lc, int q, int s) {
+__device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const NodeConst<float>& nc, const float* box,
+                                            const float* rows, const float* sm, PairNode& n, int lr, int lc, int q,
+                                            int s) {
   constexpr int H = L::H, BQ = L::BQ, BS = L::BS, HS = L::HS, MS = L::MS, TQ = L::TQ;
-  static_assert(HS % 2 == 0 && BS % 2 == 0 && MS % 2 == 0, "pair alignment");
-  const float* sf = box;
   const float* sphi = box + NPOP * BQ * BS;
-  const float* sphl = box + (NPOP + 1) * BQ * BS;
   const float* su0 = sm + L::U0_OFF;
-  const float* sn = sm + L::N_OFF;
   const float* sut = sm + L::UT_OFF;
   const float* sup = sm + L::UP_OFF;
   const float* smu = sm + L::MU_OFF;
   const int64_t stride = a.stride;
-  const int fr = lr + H;
-  const int bi = fr * BS + lc + HS;       // even: 8-byte aligned pairs
-  const int mi = (lr + 1) * MS + lc + 2;  // even
+  const int bi = (lr + H) * BS + lc + HS;  // even: 8-byte aligned pairs
+  const int mi = (lr + 1) * MS + lc + 2;   // even
   const int ui = lr * TS + lc;
-  const float sixth = 1.0f / 6.0f;
+  const float itau = a.inv_tau * a.dt;
+  const float* row = rows + (lr + 1) * kRowTable;
+  float rt[16];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) reinterpret_cast<float4*>(rt)[c] = reinterpret_cast<const float4*>(row)[c];
 
-  const float2 dn = ld2(sn + mi), ut = ld2(sut + mi), up = ld2(sup + mi), ph = ld2(sphi + bi);
-  const float2 n = add2(dn, f2(a.n0));
-  const float ct = co[C_CT * BQ + fr], cp = co[C_CP * BQ + fr], gam = co[C_GAM * BQ + fr];
-  const float lt = co[C_LT * BQ + fr], lp = co[C_LP * BQ + fr];
-  const float Jp = co[C_JP * BQ + fr], Jm = co[C_JM * BQ + fr];
-  const float2 muC = ld2(smu + mi), muN = ld2(smu + mi + MS), muS = ld2(smu + mi - MS);
-  const float2 muL = ld2(smu + mi - 2), muR = ld2(smu + mi + 2);
-  const float2 muE = make_float2(muC.y, muR.x), muW = make_float2(muL.y, muC.x);
-
-  // Cahn-Hilliard: M Delta mu - div(u phi) (Eq. CH), flux form with mean face values
-  float2 lapmu = mul2(f2(lt), sub2(mul2(f2(Jp), sub2(muN, muC)), mul2(f2(Jm), sub2(muC, muS))));
-  lapmu = fma2(f2(lp), add2(sub2(muE, muC), sub2(muW, muC)), lapmu);
-  float2 Lphi = mul2(f2(a.M), lapmu);
-  float2 Ft = f2(0.0f), Fp = f2(0.0f);
+  const float2 muN = ld2(smu + mi + MS), muS = ld2(smu + mi - MS);
+  const float2 muE = make_float2(n.mu.y, smu[mi + 2]), muW = make_float2(smu[mi - 1], n.mu.x);
+  // Cahn-Hilliard: M Delta mu - div(u phi) (Eq. CH), flux form with mean face values, times dt
+  float2 Lp = vmul(f2(rt[E_LP]), vadd(vsub(muE, n.mu), vsub(muW, n.mu)));
+  Lp = vfma(f2(rt[E_LT]), vfma(f2(rt[E_JP]), vsub(muN, n.mu), vmul(f2(rt[E_JM]), vsub(muS, n.mu))), Lp);
+  float2 Ft = f2(0.0f), Fp = f2(0.0f);  // times dt
   if (CH == VLB_HYDRO) {
-    const float2 Xn = mul2(f2(co[C_J * BQ + fr + 1]), mul2(ld2(sut + mi + MS), ld2(sphi + bi + BS)));
-    const float2 Xs = mul2(f2(co[C_J * BQ + fr - 1]), mul2(ld2(sut + mi - MS), ld2(sphi + bi - BS)));
-    const float2 upL = ld2(sup + mi - 2), upR = ld2(sup + mi + 2);
-    const float2 phL = ld2(sphi + bi - 2), phR = ld2(sphi + bi + 2);
-    const float2 Ye = mul2(make_float2(up.y, upR.x), make_float2(ph.y, phR.x));
-    const float2 Yw = mul2(make_float2(upL.y, up.x), make_float2(phL.y, ph.x));
-    Lphi = sub2(Lphi, mul2(f2(0.5f), fma2(f2(ct), sub2(Xn, Xs), mul2(f2(cp), sub2(Ye, Yw)))));
+    const float2 upE = make_float2(n.up.y, sup[mi + 2]), upW = make_float2(sup[mi - 1], n.up.x);
+    const float2 phE = make_float2(n.ph.y, sphi[bi + 2]), phW = make_float2(sphi[bi - 1], n.ph.x);
+    Lp = vfma(f2(-rt[E_XN]), vmul(ld2(sut + mi + MS), ld2(sphi + bi + BS)), Lp);
+    Lp = vfma(f2(rt[E_XS]), vmul(ld2(sut + mi - MS), ld2(sphi + bi - BS)), Lp);
+    Lp = vfma(f2(-rt[E_YP]), vsub(vmul(upE, phE), vmul(upW, phW)), Lp);
     // n F = -phi grad mu (Eq. pbin), central differences
-    const float2 mpn = make_float2(-ph.x * __frcp_rn(n.x), -ph.y * __frcp_rn(n.y));
-    Ft = mul2(mul2(mpn, sub2(muN, muS)), f2(a.gt));
-    Fp = mul2(mul2(mpn, sub2(muE, muW)), f2(co[C_GP * BQ + fr]));
+    const float2 pn = vmul(n.ph, n.inv);
+    Ft = vmul(vmul(pn, vsub(muS, muN)), f2(a.gt * a.dt));
+    Fp = vmul(vmul(pn, vsub(muW, muE)), f2(rt[E_GP]));
   }
 
   const int64_t gidx = (int64_t)q * a.ns + s;  // even
   if (a.dphi) {
-    st2(a.dphi + gidx, mul2(Lphi, f2(a.dt)));  // the stabilised Cahn-Hilliard solve forms phi
+    st2(a.dphi + gidx, Lp);  // the stabilised Cahn-Hilliard solve forms phi
   } else {
-    const float2 lo = ld2(sphl + bi);
-    float2 base = ph, base_lo = lo, inc = mul2(Lphi, f2(a.dt));
+    float2 base = n.ph, base_lo = n.lo, inc = Lp;
     if (F0) {
       base = ld2(su0 + NPOP * TQ * TS + ui);
       base_lo = ld2(su0 + (NPOP + 1) * TQ * TS + ui);
-      inc = mul2(f2(a.b), fma2(Lphi, f2(a.dt), add2(sub2(ph, base), sub2(lo, base_lo))));
+      inc = vmul(f2(a.b), vadd(vadd(vsub(n.ph, base), vsub(n.lo, base_lo)), Lp));
     }
     float2 hi_o, lo_o;
     df_add(base.x, base_lo.x, inc.x, hi_o.x, lo_o.x);
@@ -672,79 +643,57 @@ __device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const VCo
     st2(a.fout + (NPOP + 1) * stride + gidx, lo_o);
   }
 
-  float2 g[NPOP];
-#pragma unroll
-  for (int k = 0; k < NPOP; ++k) g[k] = ld2(sf + k * BQ * BS + bi);
+  float2 R[NPOP];
+  velocity_space(n.P, R, nc, rt, Ft, Fp, itau, a.n0, n.dn, n.ut, n.up);
 
-  // UW3 theta weights with ct/6 folded in (same row for both lanes)
-  const float ct6 = ct * sixth, cp6 = cp * sixth;
-  const float Jm1 = co[C_J * BQ + fr - 1], J0 = co[C_J * BQ + fr], Jp1 = co[C_J * BQ + fr + 1];
-  const float wp0 = ct6 * co[C_J * BQ + fr - 2], wp1 = -6.0f * ct6 * Jm1, wp2 = 3.0f * ct6 * J0, wp3 = 2.0f * ct6 * Jp1;
-  const float wn0 = -2.0f * ct6 * Jm1, wn1 = -3.0f * ct6 * J0, wn2 = 6.0f * ct6 * Jp1, wn3 = -ct6 * co[C_J * BQ + fr + 2];
-
-  const float2 usq = fma2(ut, ut, mul2(up, up));
-  const float2 hu = mul2(f2(-0.5f), usq);
-  const float2 c0 = add2(f2(1.0f), hu);
-  const float2 ntau = mul2(n, f2(a.inv_tau)), dntau = mul2(dn, f2(a.inv_tau));
-  const float Ep = co[C_EP * BQ + fr], En = co[C_EN * BQ + fr];
-  float2 cj[4], nFp[4];
+  // advection, relaxation and update, two theta velocities of one magnitude (x = b: i = 3, 0; a: i = 2, 1)
+  // at a time.  UW3 seen from the upwind side has the weights 1, -6, 3, 2 on the far, near, centre and
+  // downwind nodes; the varphi difference keeps them whole so that its taps cancel on a uniform field.
+  const float2 pv[2] = {f2(-row[E_TH + TAP_PV]), f2(-row[E_TH + 8 + TAP_PV])};
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    cj[j] = sub2(f2(gam * vc.v[j] * vc.v[j]), Ft);  // Gamma v_j^2 - F^theta
-    nFp[j] = mul2(f2(a.n0 * vc.v[j]), Fp);           // n0 v_j F^phi
-  }
-
+  for (int x = 0; x < 2; ++x) {
+    float t[8];
+    reinterpret_cast<float4*>(t)[0] = reinterpret_cast<const float4*>(row + E_TH + 8 * x)[0];
+    reinterpret_cast<float4*>(t)[1] = reinterpret_cast<const float4*>(row + E_TH + 8 * x)[1];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    // h_m = (-F^phi - Gamma v_i v_m) g_{i m}  (K~ = K diag v, Sec. 2.3)
-    float2 h[4];
+    for (int sgn = 0; sgn < 2; ++sgn) {
+      const int i = sgn ? (x == 0 ? 0 : 1) : (x == 0 ? 3 : 2);
+      const float2 tf = f2(t[sgn ? TAP_FARN : TAP_FARP]), tn = f2(t[sgn ? TAP_NEARN : TAP_NEARP]);
+      const float2 td = f2(t[sgn ? TAP_DOWNN : TAP_DOWNP]), tm = f2(t[TAP_MID]);
+      constexpr int STEP = BS;
+      const int up = sgn ? STEP : -STEP;  // towards the upwind side
 #pragma unroll
-    for (int mm = 0; mm < 4; ++mm) h[mm] = mul2(sub2(f2(-gam * vc.v[i] * vc.v[mm]), Fp), g[4 * i + mm]);
-    const float2 ai = mul2(f2(vc.v[i]), ut);
-    // BGK relaxation and the closed-form reference part share w_i w_j
-    const float2 ci = fma2(f2(a.n0 * vc.v[i]), add2(f2(i >= 2 ? Ep : En), Ft), dntau);
-    // theta-advection weights of this velocity row with -v_i folded in (upwind side by sign(v_i))
-    const float mvi = -vc.v[i];
-    const float t0 = mvi * (i >= 2 ? wp0 : wn0), t1 = mvi * (i >= 2 ? wp1 : wn1);
-    const float t2 = mvi * (i >= 2 ? wp2 : wn2), t3 = mvi * (i >= 2 ? wp3 : wn3);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int k = 4 * i + j;
-      const float* fk = sf + k * BQ * BS + bi;
-      const float2 gk = g[k];
-      float2 rhs;  // -v_i (theta flux difference) - v_j (varphi flux difference) / (R J dvarphi)
-      if (i >= 2)
-        rhs = fma2(f2(t3), ld2(fk + BS), fma2(f2(t2), gk, fma2(f2(t1), ld2(fk - BS), mul2(f2(t0), ld2(fk - 2 * BS)))));
-      else
-        rhs = fma2(f2(t3), ld2(fk + 2 * BS), fma2(f2(t2), ld2(fk + BS), fma2(f2(t1), gk, mul2(f2(t0), ld2(fk - BS)))));
-      const float2 A = ld2(fk - 2), C = ld2(fk + 2);
-      const float2 M1 = make_float2(A.y, gk.x), M2 = make_float2(gk.y, C.x);
-      float2 Dp;
-      if (j >= 2)
-        Dp = fma2(f2(2.0f), M2, fma2(f2(3.0f), gk, fma2(f2(-6.0f), M1, A)));
-      else
-        Dp = sub2(fma2(f2(6.0f), M2, fma2(f2(-3.0f), gk, mul2(f2(-2.0f), M1))), C);
-      rhs = fma2(f2(-vc.v[j] * cp6), Dp, rhs);
-      float2 dvt = mul2(f2(vc.K[i][0]), g[j]);
-#pragma unroll
-      for (int mm = 1; mm < 4; ++mm) dvt = fma2(f2(vc.K[i][mm]), g[4 * mm + j], dvt);
-      rhs = fma2(cj[j], dvt, rhs);
-      // the K~ term accumulates straight into the right-hand side
-#pragma unroll
-      for (int mm = 0; mm < 4; ++mm) rhs = fma2(f2(vc.K[j][mm]), h[mm], rhs);
-      // BGK towards the third-order Hermite equilibrium (Eq. feq) plus the reference part
-      const float2 xi = fma2(f2(vc.v[j]), up, ai);
-      const float2 pm1 = fma2(xi, fma2(xi, fma2(xi, f2(sixth), f2(0.5f)), c0), hu);
-      const float2 X = fma2(ntau, pm1, add2(ci, nFp[j]));
-      rhs = fma2(f2(-a.inv_tau), gk, fma2(f2(vc.ww[i][j]), X, rhs));
-      float2 o;
-      if (F0) {
-        const float2 g0 = ld2(su0 + k * TQ * TS + ui);
-        o = fma2(f2(a.b), fma2(rhs, f2(a.dt), sub2(gk, g0)), g0);
-      } else {
-        o = fma2(rhs, f2(a.dt), gk);
+      for (int j = 0; j < 4; ++j) {
+        const int k = 4 * i + j;
+        const float* fk = box + k * BQ * BS + bi;
+        const float2 g = ld2(fk), A = ld2(fk - 2), C = ld2(fk + 2);
+        float2 acc = R[k], g0 = f2(0.0f);
+        if (F0) {
+          g0 = ld2(su0 + k * TQ * TS + ui);
+          acc = vadd(acc, vsub(g, g0));
+        }
+        acc = vfma(tf, ld2(fk + 2 * up), acc);
+        acc = vfma(tn, ld2(fk + up), acc);
+        acc = vfma(tm, g, acc);
+        acc = vfma(td, ld2(fk - up), acc);
+        float2 D;  // far + 3 centre - 6 near + 2 downwind along varphi
+        if (j >= 2) {
+          D = vfma(f2(3.0f), g, A);
+          D.x = __fmaf_rn(-6.0f, A.y, D.x);
+          D.y = __fmaf_rn(-6.0f, g.x, D.y);
+          D.x = __fmaf_rn(2.0f, g.y, D.x);
+          D.y = __fmaf_rn(2.0f, C.x, D.y);
+        } else {
+          D = vfma(f2(3.0f), g, C);
+          D.x = __fmaf_rn(-6.0f, g.y, D.x);
+          D.y = __fmaf_rn(-6.0f, C.x, D.y);
+          D.x = __fmaf_rn(2.0f, A.y, D.x);
+          D.y = __fmaf_rn(2.0f, g.x, D.y);
+        }
+        acc = vfma(pv[(j == 0 || j == 3) ? 0 : 1], D, acc);
+        acc = vfma(f2(-itau), g, acc);
+        st2(a.fout + k * stride + gidx, F0 ? vfma(f2(a.b), acc, g0) : vadd(acc, g));
       }
-      st2(a.fout + k * stride + gidx, o);
     }
   }
 }
@@ -760,35 +709,40 @@ __device__ __forceinline__ void tile_body(const StageArgs<T>& a, const VConst<T>
   T* box = sm + L::BOX_OFF;
   T* co = sm + L::CO_OFF;
   pdl_wait();  // the coefficients too may come from the previous kernel (the scratch tables of vlb_step_noalloc)
-  issue_co<L>(a, co, q0, tid);
+  constexpr bool CAN_PAIR = PM != 0 && sizeof(T) == 4 && ADV == VLB_UW3;
+  bool pair = PM == 1;
+  if constexpr (PM == 2) pair = chunked<L>(a.nt, a.ns);
+  if constexpr (CAN_PAIR) {
+    if (pair)
+      issue_rows<L>(a, co, q0, tid);
+    else
+      issue_co<L>(a, co, q0, tid);
+  } else {
+    issue_co<L>(a, co, q0, tid);
+  }
   issue_box<L>(a, box, co, q0, s0, tid);
   cp_async_commit();
   if (F0) issue_u0<L>(a, sm + L::U0_OFF, q0, s0, tid);
   cp_async_commit();
   cp_async_wait<1>();  // the box; U^n may still be in flight
   __syncthreads();
-  bool pair = PM == 1;
-  if constexpr (PM == 2) pair = chunked<L>(a.nt, a.ns);
-  if constexpr (PM != 0 && sizeof(T) == 4 && ADV == VLB_UW3) {
-    if (pair)
-      phase2_pair<L>(a, vc, box, co, sm, tid);
-    else
-      phase2<L>(a, vc, box, co, sm, tid);
-  } else {
-    phase2<L>(a, vc, box, co, sm, tid);
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  pdl_trigger();
-  if constexpr (PM != 0 && sizeof(T) == 4 && ADV == VLB_UW3) {
+  if constexpr (CAN_PAIR) {
     if (pair) {
-      static_assert(L::NTH == L::TQ * (TS / 2), "one node pair per thread");
+      PairNode own;
+      phase2_pair<L>(a, vc.nc, box, co, sm, tid, own);
+      cp_async_wait<0>();
+      __syncthreads();
+      pdl_trigger();
       const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
       const int q = q0 + lr, s = s0 + lc;  // n_phi is even, so s + 1 < n_phi whenever s < n_phi
-      if (q < a.nt && s < a.ns) phase3_pair<L, CH, F0>(a, vc, box, co, sm, lr, lc, q, s);
+      if (q < a.nt && s < a.ns) phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q, s);
       return;
     }
   }
+  phase2<L>(a, vc, box, co, sm, tid);
+  cp_async_wait<0>();
+  __syncthreads();
+  pdl_trigger();
   constexpr int ROWS = L::NTH / TS;  // thread rows; each thread takes TQ / ROWS nodes of its column
 #pragma unroll 1
   for (int m = 0; m < L::TQ / ROWS; ++m) {
@@ -824,7 +778,7 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
     __syncthreads();
   }
   pdl_wait();
-  issue_co<L>(a, co, q0, tid);
+  issue_rows<L>(a, co, q0, tid);
   cp_async_commit();
   if (tid == 0) {
     mbar_expect_tx(bar, BOX_BYTES);
@@ -853,7 +807,8 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
     }
     return;
   }
-  phase2_pair<L>(a, vc, box, co, sm, tid);
+  PairNode own;
+  phase2_pair<L>(a, vc.nc, box, co, sm, tid, own);
   ok = F0 ? mbar_wait(bar + 1, ph_u0) : true;
   if (__syncthreads_or(!ok)) {
     if (tid == 0) {
@@ -864,7 +819,7 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
   }
   pdl_trigger();
   const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
-  phase3_pair<L, CH, F0>(a, vc, box, co, sm, lr, lc, q0 + lr, s0 + lc);
+  phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q0 + lr, s0 + lc);
 }
 
 // One CTA per 16 x 32 tile.
@@ -914,6 +869,7 @@ __global__ void __launch_bounds__(TQR * (TS / 2)) ensemble_stage_kernel(const En
   a.f0 = F0 ? d.U[0] : nullptr;
   a.fout = d.U[stage == 2 ? 0 : stage + 1];
   a.coef = d.coef;
+  a.rows = d.rows;
   a.nt = d.nt;
   a.ns = d.ns;
   a.stride = d.stride;
@@ -1010,6 +966,7 @@ __device__ __forceinline__ StageArgs<float> member_args(const EnsembleMember& d,
   a.f0 = stage == 0 ? nullptr : d.U[0];
   a.fout = d.U[stage == 2 ? 0 : stage + 1];
   a.coef = d.coef;
+  a.rows = d.rows;
   a.nt = d.nt;
   a.ns = d.ns;
   a.stride = d.stride;
@@ -1486,6 +1443,7 @@ template <typename T>
 VConst<T> make_vconst() {
   const VelocityConsts d = velocity_consts();
   VConst<T> c;
+  c.nc = make_node_const<T>();
   for (int i = 0; i < 4; ++i) {
     c.v[i] = (T)d.v[i];
     c.w[i] = (T)d.w[i];
@@ -1532,8 +1490,8 @@ cudaError_t launch_generic(const StageArgs<T>& a, cudaStream_t st, const StageMa
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
       resident[dev] = per_sm * sms;
     }
-    // half a wave ahead (about the next tile started on the same SM) measured best on GB300: 0.237 ms
-    // per step on 1024 x 2048 against 0.244 (one wave), 0.268 (two) and 0.254 (no prefetch)
+    // half a wave ahead (about the next tile started on the same SM) measured best on GB300: 0.217 ms
+    // per step on 1024 x 2048 against 0.225 (one wave), 0.221 (a quarter) and 0.234 (no prefetch)
     args.ahead = dev < 32 ? resident[dev] / 2 : 0;
   }
   cudaLaunchConfig_t cfg = {};
