@@ -292,12 +292,12 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
   T* U1 = (T*)h->U[1];
   T* U2 = (T*)h->U[2];
   if (p.n_phi == 1 && p.n_theta <= vlb::kAxiMaxRows && !p.ch_stab) {
-    // axisymmetric grid: up to 256 steps per single-CTA launch, cut at the diagnostic steps
+    // axisymmetric grid: up to 256 steps per single-cluster launch, cut at the diagnostic steps
     int64_t n = 0;
     while (n < nsteps) {
       int64_t chunk = std::min<int64_t>(nsteps - n, 256);
       if (p.diag_every > 0) chunk = std::min<int64_t>(chunk, p.diag_every - h->steps_done % p.diag_every);
-      VLB_CUDA(h, vlb::launch_axi<T>(a, p.advection, p.ch_mode, U0, U1, U2, (int)chunk, h->stream));
+      VLB_CUDA(h, vlb::launch_axi<T>(a, p.advection, p.ch_mode, U0, (int)chunk, h->stream));
       h->steps_done += chunk;
       n += chunk;
       if (p.diag_every > 0 && (h->steps_done % p.diag_every == 0 || n == nsteps)) {

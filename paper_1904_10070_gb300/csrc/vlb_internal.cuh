@@ -143,13 +143,12 @@ cudaError_t launch_stage(const StageArgs<T>& a, int advection, int ch_mode, cuda
 // One UW3 stage without staging (vlb_direct.cu): FP64, and FP32 grids outside the packed layout.
 template <typename T>
 cudaError_t launch_direct(const StageArgs<T>& a, int ch_mode, cudaStream_t s);
-// Axisymmetric grids (n_phi = 1, n_theta <= kAxiMaxRows): `steps` whole SSP-RK3 steps of the
-// column in one single-CTA launch, on the buffers U0 (U^n, updated in place), U1, U2.  a.fin, a.f0,
-// a.fout and a.b are set per stage inside the kernel.
+// Axisymmetric grids (n_phi = 1, 4 <= n_theta <= kAxiMaxRows; vlb_axi.cu): `steps` whole SSP-RK3 steps of the
+// column in one launch of a single thread-block cluster, on the state U (updated in place).  a.fin, a.f0,
+// a.fout and a.b are not used.
 constexpr int kAxiMaxRows = 4096;
 template <typename T>
-cudaError_t launch_axi(const StageArgs<T>& a, int advection, int ch_mode, T* U0, T* U1, T* U2, int steps,
-                       cudaStream_t s);
+cudaError_t launch_axi(const StageArgs<T>& a, int advection, int ch_mode, T* U, int steps, cudaStream_t s);
 
 // Stabilised semi-implicit Cahn-Hilliard (vlb_chsolve.cu): phi_out = phi^n + b (phi_in - phi^n +
 // P(dphi)) with P = J^{-1} (I + dt M kappa D^2)^{-1} J (D: the constant-coefficient periodic Laplacian
