@@ -142,39 +142,12 @@ __global__ void fields_kernel(const T* state, int64_t stride, const double* coef
   mu[idx] = -A * p0 * (1.0 - p0 * p0) - kappa * lap;
 }
 
-// Per-block FP64 partial sums: mass, phi total, Psi (Eq. Landau), max |u|, non-finite count, L_I.
-template <typename T>
-__global__ void __launch_bounds__(TOTAL_THREADS) totals_kernel(const T* state, int64_t stride, const double* coefd,
-                                                               int nt, int ns, double r, double A, double kappa,
-                                                               double n0, double gt, double edge_p, double* partials,
-                                                               VD vd) {
-  const int64_t n = (int64_t)nt * ns;
-  double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
-    const int q = (int)(idx / ns), s = (int)(idx - (int64_t)q * ns);
-    double nn, a, b;
-    node_moments(state, stride, idx, vd, n0, nn, a, b);
-    const double dA = coefd[C_DA * nt + q];
-    const double p0 = load_phi(state, stride, idx);
-    const double pn = load_phi(state, stride, (int64_t)wrapi(q + 1, nt) * ns + s);
-    const double ps = load_phi(state, stride, (int64_t)wrapi(q - 1, nt) * ns + s);
-    const double pe = load_phi(state, stride, (int64_t)q * ns + wrapi(s + 1, ns));
-    const double pw = load_phi(state, stride, (int64_t)q * ns + wrapi(s - 1, ns));
-    const double g1 = (pn - ps) * gt, g2 = (pe - pw) * coefd[C_GP * nt + q];
-    const double om = 1.0 - p0 * p0;
-    acc[0] += nn * dA;
-    acc[1] += p0 * dA;
-    acc[2] += (0.25 * A * om * om + 0.5 * kappa * (g1 * g1 + g2 * g2)) * dA;
-    const double umag = sqrt(a * a + b * b);
-    acc[3] = fmax(acc[3], umag);
-    if (!isfinite(nn) || !isfinite(umag) || !isfinite(p0)) acc[4] += 1.0;
-    if (p0 * pe < 0.0) acc[5] += edge_p;                     // neighbour across varphi: r dtheta
-    if (p0 * pn < 0.0) acc[5] += coefd[C_EDGE * nt + q];     // neighbour across theta
-  }
-  // warp then block reduction in a fixed order
+// Per-block FP64 sums: mass, phi total, Psi (Eq. Landau), max |u|, non-finite count (slots 5 .. 7 unused).
+// Warp, then block reduction in a fixed order.
+__device__ __forceinline__ void reduce_totals(double (&acc)[NSUM], double* partials) {
   __shared__ double red[TOTAL_THREADS / 32][NSUM];
 #pragma unroll
-  for (int k = 0; k < NSUM; ++k) {
+  for (int k = 0; k < 5; ++k) {
     double x = acc[k];
     for (int o = 16; o > 0; o >>= 1) {
       const double y = __shfl_down_sync(0xffffffffu, x, o);
@@ -188,10 +161,185 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals_kernel(const T* state, i
   __syncthreads();
   if (threadIdx.x < NSUM) {
     const int k = threadIdx.x;
-    double x = (k == 3) ? 0.0 : 0.0;
+    double x = 0.0;
     for (int w = 0; w < TOTAL_THREADS / 32; ++w) x = (k == 3) ? fmax(x, red[w][k]) : x + red[w][k];
     partials[blockIdx.x * NSUM + k] = x;
   }
+}
+
+// One node's share of the totals in FP64; acc[3] collects |u|^2 (the root is taken once, after the maximum:
+// a correctly rounded root is monotone).
+template <typename T>
+__device__ __forceinline__ void node_totals(const T* state, int64_t stride, const double* coefd, int nt, int ns, int q,
+                                            int s, double A, double kappa, double n0, double gt, const VD& vd,
+                                            double (&acc)[NSUM]) {
+  const int64_t idx = (int64_t)q * ns + s;
+  double nn, a, b;
+  node_moments(state, stride, idx, vd, n0, nn, a, b);
+  const double dA = coefd[C_DA * nt + q];
+  const double p0 = load_phi(state, stride, idx);
+  const double pn = load_phi(state, stride, (int64_t)wrapi(q + 1, nt) * ns + s);
+  const double ps = load_phi(state, stride, (int64_t)wrapi(q - 1, nt) * ns + s);
+  const double pe = load_phi(state, stride, (int64_t)q * ns + wrapi(s + 1, ns));
+  const double pw = load_phi(state, stride, (int64_t)q * ns + wrapi(s - 1, ns));
+  const double g1 = (pn - ps) * gt, g2 = (pe - pw) * coefd[C_GP * nt + q];
+  const double om = 1.0 - p0 * p0;
+  acc[0] += nn * dA;
+  acc[1] += p0 * dA;
+  acc[2] += (0.25 * A * om * om + 0.5 * kappa * (g1 * g1 + g2 * g2)) * dA;
+  const double u2 = a * a + b * b;
+  acc[3] = fmax(acc[3], u2);
+  if (!isfinite(nn) || !isfinite(u2) || !isfinite(p0)) acc[4] += 1.0;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(TOTAL_THREADS) totals_kernel(const T* state, int64_t stride, const double* coefd,
+                                                               int nt, int ns, double A, double kappa, double n0,
+                                                               double gt, double* partials, VD vd) {
+  const int64_t n = (int64_t)nt * ns;
+  double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
+    const int q = (int)(idx / ns);
+    node_totals(state, stride, coefd, nt, ns, q, (int)(idx - (int64_t)q * ns), A, kappa, n0, gt, vd, acc);
+  }
+  acc[3] = sqrt(acc[3]);
+  reduce_totals(acc, partials);
+}
+
+// ---- Totals of an FP32 state in float pairs -----------------------------------------------------------
+// The FP64 units (one warp instruction per 19 cycles and SM) made the totals of 1024 x 2048 cost 558 us at
+// about 100 FP64 operations a node.  An FP32 state needs 48 bits, not 53: every quantity of a node is
+// formed as an unevaluated pair h + l of floats with error-free sums and products (Dekker 1971, Knuth),
+// 2^-47 relative per operation against the state's own 2^-24, a row's sums too; FP64 starts at the row
+// (times the area element) and does the rest.  About 520 FP32 operations a node: 86 us.  A node whose
+// values leave the range where the pairs cannot overflow or underflow takes the FP64 path.
+struct FF {
+  float h, l;
+};
+__device__ __forceinline__ FF quick_sum(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ FF two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ FF operator+(FF a, FF b) {
+  const FF s = two_sum(a.h, b.h);
+  return quick_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF operator-(FF a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ FF operator-(FF a, FF b) { return a + (-b); }
+__device__ __forceinline__ FF operator*(FF a, FF b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return quick_sum(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ FF operator/(FF a, FF b) {
+  const float q = __fdiv_rn(a.h, b.h);
+  const FF p = b * FF{q, 0.0f}, r = a - p;
+  return quick_sum(q, __fdiv_rn(r.h, b.h));
+}
+__device__ __forceinline__ FF to_ff(double x) {
+  const float h = (float)x;
+  return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ double to_d(FF a) { return (double)a.h + (double)a.l; }
+
+// W threads (a power of two) share a row.
+__global__ void __launch_bounds__(TOTAL_THREADS) totals32_kernel(const float* state, int64_t stride,
+                                                                 const double* coefd, int nt, int ns, int W, double A,
+                                                                 double kappa, double n0, double gt, double* partials,
+                                                                 VD vd) {
+  const int c = threadIdx.x & (W - 1), rb = TOTAL_THREADS / W;
+  const FF va = to_ff(vd.v[2]), vb = to_ff(vd.v[3]), gtf = to_ff(gt), A4 = to_ff(0.25 * A), k2 = to_ff(0.5 * kappa);
+  const FF n0f = to_ff(n0), one = {1.0f, 0.0f};
+  const float *hi = state + NPOP * stride, *lo = hi + stride;
+  double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
+  FF best = {0.0f, 0.0f};  // largest |u|^2
+  for (int q = blockIdx.x * rb + threadIdx.x / W; q < nt; q += gridDim.x * rb) {
+    const int64_t rn = (int64_t)(q + 1 < nt ? q + 1 : 0) * ns, rs = (int64_t)(q > 0 ? q - 1 : nt - 1) * ns;
+    const int64_t r0 = (int64_t)q * ns;
+    const FF gp = to_ff(coefd[C_GP * nt + q]);
+    FF m = {0.0f, 0.0f}, ph = m, psi = m;
+    int count = 0;
+    for (int s = c; s < ns; s += W) {
+      const int se = s + 1 < ns ? s + 1 : 0, sw = s > 0 ? s - 1 : ns - 1;
+      const float* f = state + r0 + s;
+      FF S[4], OB = {0.0f, 0.0f}, OA = OB;
+      float big = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float g0 = f[(4 * i) * stride], g1 = f[(4 * i + 1) * stride];
+        const float g2 = f[(4 * i + 2) * stride], g3 = f[(4 * i + 3) * stride];
+        big = fmaxf(fmaxf(big, fmaxf(fabsf(g0), fabsf(g1))), fmaxf(fabsf(g2), fabsf(g3)));
+        S[i] = two_sum(g3, g0) + two_sum(g2, g1);
+        OB = OB + two_sum(g3, -g0);
+        OA = OA + two_sum(g2, -g1);
+      }
+      const FF p0 = {hi[r0 + s], lo[r0 + s]};
+      const FF pn = {hi[rn + s], lo[rn + s]}, ps = {hi[rs + s], lo[rs + s]};
+      const FF pe = {hi[r0 + se], lo[r0 + se]}, pw = {hi[r0 + sw], lo[r0 + sw]};
+      const FF dn = (S[0] + S[3]) + (S[1] + S[2]), nn = n0f + dn;
+      const FF mt = vb * (S[3] - S[0]) + va * (S[2] - S[1]), mp = vb * OB + va * OA;
+      const FF u2 = (mt * mt + mp * mp) / (nn * nn);
+      const FF om = one - p0 * p0, g1 = (pn - ps) * gtf, g2 = (pe - pw) * gp;
+      const FF dens = A4 * (om * om) + k2 * (g1 * g1 + g2 * g2);
+      const float pm = fmaxf(fmaxf(fabsf(p0.h), fmaxf(fabsf(pn.h), fabsf(ps.h))), fmaxf(fabsf(pe.h), fabsf(pw.h)));
+      // the comparisons are false for NaN
+      if (nn.h >= 1e-6f && nn.h <= 1e6f && big <= 1e6f && pm <= 1e4f && u2.h <= 1e6f && dens.h <= 1e12f) {
+        m = m + dn;
+        ph = ph + p0;
+        psi = psi + dens;
+        ++count;
+        if (u2.h > best.h || (u2.h == best.h && u2.l > best.l)) best = u2;
+      } else {
+        node_totals(state, stride, coefd, nt, ns, q, s, A, kappa, n0, gt, vd, acc);
+      }
+    }
+    const double dA = coefd[C_DA * nt + q];
+    acc[0] += (to_d(m) + n0 * count) * dA;
+    acc[1] += to_d(ph) * dA;
+    acc[2] += to_d(psi) * dA;
+  }
+  acc[3] = sqrt(fmax(acc[3], to_d(best)));
+  reduce_totals(acc, partials);
+}
+
+// L_I: the interface edges of every row counted, then weighted in FP64 (r dtheta across varphi, the row's
+// edge length across theta).  Signs of an FP32 state come from the float pair's leading word that is not 0.
+__device__ __forceinline__ bool crosses(double a, double b) { return a * b < 0.0; }
+__device__ __forceinline__ bool crosses(float a, float b) { return (a < 0.0f && b > 0.0f) || (a > 0.0f && b < 0.0f); }
+__device__ __forceinline__ double phi_sign(const double* state, int64_t stride, int64_t idx) {
+  return state[NPOP * stride + idx];
+}
+__device__ __forceinline__ float phi_sign(const float* state, int64_t stride, int64_t idx) {
+  const float h = state[NPOP * stride + idx];
+  return h != 0.0f ? h : state[(NPOP + 1) * stride + idx];
+}
+template <typename T>
+__global__ void __launch_bounds__(TOTAL_THREADS) interface_kernel(const T* state, int64_t stride, const double* coefd,
+                                                                  int nt, int ns, int W, double edge_p,
+                                                                  double* partials) {
+  const int c = threadIdx.x & (W - 1), rb = TOTAL_THREADS / W;
+  double acc = 0.0;
+  for (int q = blockIdx.x * rb + threadIdx.x / W; q < nt; q += gridDim.x * rb) {
+    const int64_t r0 = (int64_t)q * ns, rn = (int64_t)(q + 1 < nt ? q + 1 : 0) * ns;
+    int np = 0, nn = 0;
+    for (int s = c; s < ns; s += W) {
+      const T p0 = phi_sign(state, stride, r0 + s);
+      np += crosses(p0, phi_sign(state, stride, r0 + (s + 1 < ns ? s + 1 : 0))) ? 1 : 0;
+      nn += crosses(p0, phi_sign(state, stride, rn + s)) ? 1 : 0;
+    }
+    if (np | nn) acc += edge_p * np + coefd[C_EDGE * nt + q] * nn;
+  }
+  __shared__ double red[TOTAL_THREADS];
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  for (int w = TOTAL_THREADS / 2; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) partials[blockIdx.x] = red[0];
 }
 
 // Fixed-order sum (or max) of part[b * stride + k] over b < nb by one warp: lane l takes b = l, l + 32,
@@ -208,6 +356,11 @@ __device__ __forceinline__ double warp_fold(const double* part, int nb, int stri
     x = is_max ? fmax(x, y) : x + y;
   }
   return x;
+}
+
+__global__ void interface_final_kernel(const double* partials, int nb, double* out) {
+  const double x = warp_fold(partials, nb, 1, 0, false);
+  if (threadIdx.x == 0) *out = x;
 }
 
 // one warp per output k (blockDim = 32 NSUM)
@@ -385,20 +538,41 @@ cudaError_t launch_fields(const T* state, int64_t stride, const double* coefd, i
   return cudaGetLastError();
 }
 
+// threads that share a row: a power of two up to a CTA
+static int row_threads(int ns) {
+  int w = 1;
+  while (w < TOTAL_THREADS && w < ns) w *= 2;
+  return w;
+}
+
 template <typename T>
-cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, int nt, int ns, double R, double r,
-                          double A, double kappa, double n0, int geometry, double* partials, int n_blocks,
-                          double* out, cudaStream_t s) {
-  (void)R;
-  (void)geometry;
-  const double dth = 2.0 * M_PI / nt;
-  const double gt = 1.0 / (2.0 * r * dth);
-  const double edge_p = r * dth;
-  totals_kernel<T><<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, r, A, kappa, n0, gt, edge_p,
-                                                      partials, make_vd());
+cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, int nt, int ns, double r, double A,
+                          double kappa, double n0, double* partials, int n_blocks, double* out, cudaStream_t s) {
+  const double gt = 1.0 / (2.0 * r * (2.0 * M_PI / nt));
+  if constexpr (sizeof(T) == 4) {
+    const int W = row_threads(ns), rb = TOTAL_THREADS / W;
+    n_blocks = (nt + rb - 1) / rb < n_blocks ? (nt + rb - 1) / rb : n_blocks;
+    totals32_kernel<<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, W, A, kappa, n0, gt, partials,
+                                                       make_vd());
+  } else {
+    totals_kernel<T><<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, A, kappa, n0, gt, partials,
+                                                        make_vd());
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   totals_final_kernel<<<1, 32 * NSUM, 0, s>>>(partials, n_blocks, out);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_interface(const T* state, int64_t stride, const double* coefd, int nt, int ns, double r,
+                             double* partials, int n_blocks, double* out, cudaStream_t s) {
+  const int W = row_threads(ns), rb = TOTAL_THREADS / W;
+  n_blocks = (nt + rb - 1) / rb < n_blocks ? (nt + rb - 1) / rb : n_blocks;
+  interface_kernel<T><<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, W, r * (2.0 * M_PI / nt), partials);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  interface_final_kernel<<<1, 32, 0, s>>>(partials, n_blocks, out);
   return cudaGetLastError();
 }
 
@@ -432,7 +606,9 @@ cudaError_t launch_snapshot_in(T* state, int64_t stride, int64_t n, double n0, c
   template cudaError_t launch_fields<T>(const T*, int64_t, const double*, int, int, double, double, double,     \
                                         double*, double*, double*, double*, double*, cudaStream_t);               \
   template cudaError_t launch_totals<T>(const T*, int64_t, const double*, int, int, double, double, double,      \
-                                        double, double, int, double*, int, double*, cudaStream_t);               \
+                                        double, double*, int, double*, cudaStream_t);                            \
+  template cudaError_t launch_interface<T>(const T*, int64_t, const double*, int, int, double, double*, int,     \
+                                           double*, cudaStream_t);                                                \
   template cudaError_t launch_snapshot_out<T>(const T*, int64_t, int64_t, double, float*, cudaStream_t);        \
   template cudaError_t launch_snapshot_in<T>(T*, int64_t, int64_t, double, const float*, const double*, int,   \
                                              cudaStream_t);

@@ -301,8 +301,8 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
       h->steps_done += chunk;
       n += chunk;
       if (p.diag_every > 0 && (h->steps_done % p.diag_every == 0 || n == nsteps)) {
-        VLB_CUDA(h, vlb::launch_totals<T>(U0, h->stride, h->coefD, p.n_theta, p.n_phi, p.R, p.r, p.A, p.kappa,
-                                          h->n0, p.geometry, h->partials, vlb::totals_blocks(), h->diag, h->stream));
+        VLB_CUDA(h, vlb::launch_totals<T>(U0, h->stride, h->coefD, p.n_theta, p.n_phi, p.r, p.A, p.kappa, h->n0,
+                                            h->partials, vlb::totals_blocks(), h->diag, h->stream));
         VLB_CUDA(h, vlb_internal_flag(h->diag, h->flag, h->stream));
       }
     }
@@ -331,8 +331,8 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
         h->steps_done += chunk;
         n += chunk;
         if (p.diag_every > 0 && (h->steps_done % p.diag_every == 0 || n == nsteps)) {
-          VLB_CUDA(h, vlb::launch_totals<T>(U0, h->stride, h->coefD, p.n_theta, p.n_phi, p.R, p.r, p.A, p.kappa,
-                                            h->n0, p.geometry, h->partials, vlb::totals_blocks(), h->diag, h->stream));
+          VLB_CUDA(h, vlb::launch_totals<T>(U0, h->stride, h->coefD, p.n_theta, p.n_phi, p.r, p.A, p.kappa, h->n0,
+                                            h->partials, vlb::totals_blocks(), h->diag, h->stream));
           VLB_CUDA(h, vlb_internal_flag(h->diag, h->flag, h->stream));
         }
       }
@@ -354,8 +354,8 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
     VLB_CUDA(h, solve(U2, U0, U0, (T)(2.0 / 3.0)));
     h->steps_done++;
     if (p.diag_every > 0 && (h->steps_done % p.diag_every == 0 || n + 1 == nsteps)) {
-      VLB_CUDA(h, vlb::launch_totals<T>(U0, h->stride, h->coefD, p.n_theta, p.n_phi, p.R, p.r, p.A, p.kappa,
-                                        h->n0, p.geometry, h->partials, vlb::totals_blocks(), h->diag, h->stream));
+      VLB_CUDA(h, vlb::launch_totals<T>(U0, h->stride, h->coefD, p.n_theta, p.n_phi, p.r, p.A, p.kappa, h->n0,
+                                            h->partials, vlb::totals_blocks(), h->diag, h->stream));
       VLB_CUDA(h, vlb_internal_flag(h->diag, h->flag, h->stream));
     }
   }
@@ -365,9 +365,8 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
 template <typename T>
 vlb_status totals_impl(vlb_handle* h) {
   const vlb_params& p = h->p;
-  VLB_CUDA(h, vlb::launch_totals<T>((const T*)h->U[0], h->stride, h->coefD, p.n_theta, p.n_phi, p.R, p.r, p.A,
-                                    p.kappa, h->n0, p.geometry, h->partials, vlb::totals_blocks(), h->totals,
-                                    h->stream));
+  VLB_CUDA(h, vlb::launch_totals<T>((const T*)h->U[0], h->stride, h->coefD, p.n_theta, p.n_phi, p.r, p.A, p.kappa,
+                                    h->n0, h->partials, vlb::totals_blocks(), h->totals, h->stream));
   return VLB_OK;
 }
 
@@ -795,12 +794,18 @@ vlb_status vlb_interface_length(vlb_handle* h, double* out) {
   vlb_status st = check_handle(h);
   if (st) return st;
   if (!out) return fail(h, VLB_ERR_ARG, "out is NULL");
-  st = h->esize == 8 ? totals_impl<double>(h) : totals_impl<float>(h);
-  if (st) return st;
-  double t[8];
-  VLB_CUDA(h, cudaMemcpyAsync(t, h->totals, sizeof t, cudaMemcpyDeviceToHost, h->stream));
+  const vlb_params& p = h->p;
+  double* d = h->totals + 5;
+  if (h->esize == 8)
+    VLB_CUDA(h, vlb::launch_interface<double>((const double*)h->U[0], h->stride, h->coefD, p.n_theta, p.n_phi, p.r,
+                                              h->partials, vlb::totals_blocks(), d, h->stream));
+  else
+    VLB_CUDA(h, vlb::launch_interface<float>((const float*)h->U[0], h->stride, h->coefD, p.n_theta, p.n_phi, p.r,
+                                             h->partials, vlb::totals_blocks(), d, h->stream));
+  double t = 0.0;
+  VLB_CUDA(h, cudaMemcpyAsync(&t, d, sizeof t, cudaMemcpyDeviceToHost, h->stream));
   st = sync_and_check(h, "vlb_interface_length", false);
-  *out = t[5];
+  *out = t;
   return st;
 }
 

@@ -34,25 +34,11 @@ struct C2 {
   T x, y;
 };
 
-__device__ __forceinline__ void sincospi_t(double a, double* s, double* c) { sincospi(a, s, c); }
-__device__ __forceinline__ void sincospi_t(float a, float* s, float* c) { sincospif(a, s, c); }
-
 __device__ __forceinline__ int bitrev(int i, int logn) { return (int)(__brev((unsigned)i) >> (32 - logn)); }
 
 // Twiddles stored level by level, so that the butterflies of one level read consecutive entries
 // (a single table indexed by j n / 2^l puts a warp's reads on one shared-memory bank at the middle
 // levels): tw[2^(l-1) - 1 + j] = exp(-2 pi i j / 2^l), j < 2^(l-1), l = 1 .. log2 n; n - 1 entries.
-template <typename T>
-__device__ void twiddles(C2<T>* tw, int n) {
-  for (int k = threadIdx.x; k < n - 1; k += blockDim.x) {
-    const int half = 1 << (31 - __clz(k + 1));  // 2^(l-1), the level's first entry is half - 1
-    const int j = k + 1 - half;
-    T s, c;
-    sincospi_t((T)(-(double)j / half), &s, &c);  // -2 pi j / 2^l = -pi j / half
-    tw[k].x = c;
-    tw[k].y = s;
-  }
-}
 
 // Shared-memory position of element e of a row transform: one pad element every 2^sh elements, so
 // that the bit-reversed scatter of 32 consecutive indices (multiples of n / 32) and the butterflies
@@ -386,52 +372,89 @@ cudaError_t launch_ch_stab(int nt, int ns, double dt_m_kappa, const double* J, c
 namespace {
 
 // ---- Structure factor S(m, n) = |F phi|^2 and its two sums (the L_S diagnostic) --------------------
-// The same radix-2 transforms in FP64 whatever the state's precision (phi in FP32 is the float pair
-// hi + lo, exact in a double): rows first, then strips of columns, whose CTA sums S and |k| S over its
-// strip (k = (m'/r, n'/R), m' and n' the signed frequencies; the mean mode m = n = 0 is left out) and
-// writes the two sums to part[2 b], part[2 b + 1].
+// The same transforms in FP64 whatever the state's precision (phi in FP32 is the float pair hi + lo, exact in a
+// double).  Bound by the FP64 units, so phi's realness is used throughout: two rows share one complex
+// transform, only the columns n = 0 .. N_phi / 2 are kept (columns 0 and N_phi / 2, real per row, packed
+// into one), the mirrored half enters by weight 2, and one root serves the modes m and -m.  A column CTA sums
+// S and |k| S over its strip (k = (m'/r, n'/R), m' and n' the signed frequencies; the mean mode m = n = 0 is left
+// out) and writes the two sums to part[2 b], part[2 b + 1].  The twiddles are tabulated once per call instead
+// of by every CTA.  1024 x 2048: 338 + 324 us for complex transforms with per-CTA twiddles, 123 + 145 us now.
 
-template <typename T>
-__global__ void __launch_bounds__(256) sf_row_kernel(int ns, int logns, const T* phi, const T* phi_lo,
-                                                     C2<double>* buf) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  C2<double>* a = reinterpret_cast<C2<double>*>(raw);
-  C2<double>* tw = a + ns;
-  const int q = blockIdx.x;
-  twiddles(tw, ns);
-  for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-    const int64_t g = (int64_t)q * ns + s;
-    const double v = (double)phi[g] + (phi_lo ? (double)phi_lo[g] : 0.0);
-    a[bitrev(s, logns)] = {v, 0.0};
-  }
-  __syncthreads();
-  fft_strided(a, ns, logns, 0, 31, tw, false);
-  for (int s = threadIdx.x; s < ns; s += blockDim.x) buf[(int64_t)q * ns + s] = a[s];
+__global__ void sf_twiddle_kernel(C2<double>* tw_s, int ns, C2<double>* tw_t, int nt) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool first = x < ns - 1;
+  const int k = first ? x : x - (ns - 1);
+  if (k >= nt - 1 && !first) return;
+  const int half = 1 << (31 - __clz(k + 1));  // a level's first entry is half - 1 (twiddle order of fft_strided)
+  double sn, cs;
+  sincospi(-(double)(k + 1 - half) / half, &sn, &cs);
+  (first ? tw_s : tw_t)[k] = {cs, sn};
 }
 
-__global__ void __launch_bounds__(256) sf_col_kernel(int nt, int lognt, int ns, int cw, double kt, double kp,
-                                                     const C2<double>* buf, double* part) {
+// Rows 2 b and 2 b + 1 -> their spectra at 0 .. N_phi / 2 - 1, entry 0 holding the real values at 0 and N_phi / 2.
+template <typename T>
+__global__ void __launch_bounds__(256) sf_row_kernel(int ns, int logns, const T* phi, const T* phi_lo,
+                                                     const C2<double>* tw_s, C2<double>* buf) {
   extern __shared__ __align__(16) unsigned char raw[];
   C2<double>* a = reinterpret_cast<C2<double>*>(raw);
-  C2<double>* tw = a + (size_t)nt * cw;
-  __shared__ double red[2][8];
-  const int n0 = blockIdx.x * cw;
-  twiddles(tw, nt);
-  for (int idx = threadIdx.x; idx < nt * cw; idx += blockDim.x) {
-    const int q = idx / cw, c = idx - q * cw;
-    a[bitrev(q, lognt) * cw + c] = buf[(int64_t)q * ns + n0 + c];
+  const int sh = row_pad_shift(logns), nh = ns / 2;
+  C2<double>* tw = a + padded(ns, sh);
+  const int64_t q = 2 * (int64_t)blockIdx.x;
+  for (int s = threadIdx.x; s < ns; s += blockDim.x) {
+    const int64_t g = q * ns + s, h = g + ns;
+    a[padded(bitrev(s, logns), sh)] = {(double)phi[g] + (phi_lo ? (double)phi_lo[g] : 0.0),
+                                       (double)phi[h] + (phi_lo ? (double)phi_lo[h] : 0.0)};
   }
+  load_twiddles(tw, tw_s, ns);
   __syncthreads();
-  fft_strided(a, nt, lognt, __ffs(cw) - 1, 31, tw, false);  // cw is a power of two
+  fft_strided(a, ns, logns, 0, sh, tw, false);
+  C2<double>*r0 = buf + q * nh, *r1 = r0 + nh;
+  for (int k = threadIdx.x; k < nh; k += blockDim.x) {
+    const C2<double> z = a[padded(k, sh)], y = a[padded(k ? ns - k : nh, sh)];
+    if (k == 0) {
+      r0[0] = {z.x, y.x};
+      r1[0] = {z.y, y.y};
+    } else {  // (z + conj y) / 2 and (z - conj y) / 2i
+      r0[k] = {0.5 * (z.x + y.x), 0.5 * (z.y - y.y)};
+      r1[k] = {0.5 * (z.y + y.y), 0.5 * (y.x - z.x)};
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) sf_col_kernel(int nt, int lognt, int ns, int lcw, double kt, double kp,
+                                                     const C2<double>* tw_t, const C2<double>* buf, double* part) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  C2<double>* a = reinterpret_cast<C2<double>*>(raw);
+  const int cw = 1 << lcw, nh = ns / 2, n0 = blockIdx.x << lcw;
+  C2<double>* tw = a + ((size_t)nt << lcw);
+  __shared__ double red[2][8];
+  for (int idx = threadIdx.x; idx < nt << lcw; idx += blockDim.x) {
+    const int q = idx >> lcw, c = idx & (cw - 1);
+    a[(bitrev(q, lognt) << lcw) + c] = buf[(int64_t)q * nh + n0 + c];
+  }
+  load_twiddles(tw, tw_t, nt);
+  __syncthreads();
+  fft_strided(a, nt, lognt, lcw, 31, tw, false);
   double s_sum = 0.0, k_sum = 0.0;
-  for (int idx = threadIdx.x; idx < nt * cw; idx += blockDim.x) {
-    const int m = idx / cw, n = n0 + idx - m * cw;
-    if (m == 0 && n == 0) continue;
-    const int ms = m <= nt / 2 ? m : m - nt, nsg = n <= ns / 2 ? n : n - ns;
-    const double S = a[idx].x * a[idx].x + a[idx].y * a[idx].y;
-    const double k = sqrt((ms * kt) * (ms * kt) + (nsg * kp) * (nsg * kp));
-    s_sum += S;
-    k_sum += k * S;
+  for (int idx = threadIdx.x; idx < (nt / 2 + 1) << lcw; idx += blockDim.x) {
+    const int m = idx >> lcw, c = idx & (cw - 1), n = n0 + c, mr = m ? nt - m : 0;
+    const C2<double> z = a[(m << lcw) + c], y = a[(mr << lcw) + c];
+    const double mk = (m * kt) * (m * kt);
+    if (n) {  // columns n and N_phi - n, rows m and -m
+      const double S = z.x * z.x + z.y * z.y + (mr != m ? y.x * y.x + y.y * y.y : 0.0);
+      s_sum += 2.0 * S;
+      k_sum += 2.0 * sqrt(mk + (n * kp) * (n * kp)) * S;
+    } else {  // the packed columns 0 and N_phi / 2: (z + conj y) / 2, (z - conj y) / 2i
+      const double w = mr != m ? 0.5 : 0.25;  // |.|^2 / 4, twice for the rows m and -m
+      const double ax = z.x + y.x, ay = z.y - y.y, bx = z.y + y.y, by = y.x - z.x;
+      const double S0 = w * (ax * ax + ay * ay), Sh = w * (bx * bx + by * by);
+      if (m) {
+        s_sum += S0;
+        k_sum += sqrt(mk) * S0;
+      }
+      s_sum += Sh;
+      k_sum += sqrt(mk + (nh * kp) * (nh * kp)) * Sh;
+    }
   }
   for (int o = 16; o > 0; o >>= 1) {
     s_sum += __shfl_xor_sync(0xffffffffu, s_sum, o);
@@ -454,32 +477,33 @@ __global__ void __launch_bounds__(256) sf_col_kernel(int nt, int lognt, int ns, 
   }
 }
 
+// columns per strip (log2): 32-byte segments of the spectrum's rows, and enough strips for every SM
+int sf_strip(int nt, int ns) { return ns / 2 >= 2 && nt <= 2048 ? 1 : 0; }
+
 }  // namespace
 
-int structure_blocks(int nt, int ns) {
-  int cw = 1;
-  while (cw < 32 && cw * 2 <= ns && (size_t)nt * cw * 2 * sizeof(C2<double>) <= kColBudget) cw *= 2;
-  return ns / cw;
-}
+int structure_blocks(int nt, int ns) { return (ns / 2) >> sf_strip(nt, ns); }
 
 template <typename T>
 cudaError_t launch_structure_sums(int nt, int ns, double r, double R, const T* phi, const T* phi_lo, void* buf,
                                   double* part, cudaStream_t st) {
   if (!ch_stab_shape_ok(nt, ns)) return cudaErrorInvalidValue;
-  const int lognt = ilog2(nt), logns = ilog2(ns);
-  const int cw = ns / structure_blocks(nt, ns);
+  const int lognt = ilog2(nt), logns = ilog2(ns), lcw = sf_strip(nt, ns);
   C2<double>* cb = reinterpret_cast<C2<double>*>(buf);
-  const size_t row_bytes = sizeof(C2<double>) * (size_t)ns * 2;
-  const size_t col_bytes = sizeof(C2<double>) * ((size_t)nt * cw + nt);
-  constexpr size_t row_max = sizeof(C2<double>) * 4096 * 2;
-  constexpr size_t col_max = kColBudget + sizeof(C2<double>) * 4096;
+  C2<double>*tw_s = cb + (size_t)nt * ns / 2, *tw_t = tw_s + (ns - 1);  // (nt - 2) (ns - 2) >= 0: they fit
+  const size_t row_bytes = sizeof(C2<double>) * ((size_t)ns * 2 + 32);
+  const size_t col_bytes = sizeof(C2<double>) * (((size_t)nt << lcw) + nt);
+  constexpr size_t row_max = sizeof(C2<double>) * (4096 * 2 + 32);
+  constexpr size_t col_max = sizeof(C2<double>) * 4096 * 2;
   static int m1 = 0, m2 = 0;
   cudaError_t e;
   if ((e = smem_attr(sf_row_kernel<T>, row_max, m1)) != cudaSuccess) return e;
   if ((e = smem_attr(sf_col_kernel, col_max, m2)) != cudaSuccess) return e;
-  sf_row_kernel<T><<<nt, 256, row_bytes, st>>>(ns, logns, phi, phi_lo, cb);
+  sf_twiddle_kernel<<<(ns + nt - 2 + 127) / 128, 128, 0, st>>>(tw_s, ns, tw_t, nt);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  sf_col_kernel<<<ns / cw, 256, col_bytes, st>>>(nt, lognt, ns, cw, 1.0 / r, 1.0 / R, cb, part);
+  sf_row_kernel<T><<<nt / 2, 256, row_bytes, st>>>(ns, logns, phi, phi_lo, tw_s, cb);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  sf_col_kernel<<<structure_blocks(nt, ns), 256, col_bytes, st>>>(nt, lognt, ns, lcw, 1.0 / r, 1.0 / R, tw_t, cb, part);
   return cudaGetLastError();
 }
 

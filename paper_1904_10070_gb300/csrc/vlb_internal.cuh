@@ -166,7 +166,7 @@ cudaError_t launch_ch_stab(int nt, int ns, double dt_m_kappa, const double* J, c
                            const T* phi0, T* phiout, int64_t lo_off, T b, cudaStream_t st);
 
 // Structure-factor sums (vlb_chsolve.cu, same power-of-two shapes): FP64 transform of phi (+ phi_lo
-// when not NULL) into buf (n_theta * n_phi complex doubles), then structure_blocks(nt, ns) CTAs write
+// when not NULL) into buf (n_theta * n_phi complex doubles, half of them spectrum), then structure_blocks(nt, ns) CTAs write
 // part[2 b] = sum S and part[2 b + 1] = sum |k| S over their strips (k = (m'/r, n'/R), mean mode left out).
 int structure_blocks(int nt, int ns);
 template <typename T>
@@ -188,11 +188,14 @@ cudaError_t launch_fields(const T* state, int64_t stride, const double* coefd, i
                           double kappa, double n0, double* rho, double* ut, double* up, double* phi, double* mu,
                           cudaStream_t s);
 // partials: n_blocks x 8 doubles; out: 8 doubles
-// out[0] mass, out[1] phi total, out[2] Psi, out[3] max|u|, out[4] non-finite count, out[5] L_I
+// out[0] mass, out[1] phi total, out[2] Psi, out[3] max|u|, out[4] non-finite count
 template <typename T>
-cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, int nt, int ns, double R,
-                          double r, double A, double kappa, double n0, int geometry, double* partials,
-                          int n_blocks, double* out, cudaStream_t s);
+cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, int nt, int ns, double r, double A,
+                          double kappa, double n0, double* partials, int n_blocks, double* out, cudaStream_t s);
+// *out = L_I; partials: n_blocks doubles
+template <typename T>
+cudaError_t launch_interface(const T* state, int64_t stride, const double* coefd, int nt, int ns, double r,
+                             double* partials, int n_blocks, double* out, cudaStream_t s);
 int totals_blocks();
 
 // Solver snapshots (vlb_aux.cu): FP32 [N][4] = (phi, n, u_theta, u_phi) on the device.
