@@ -1,5 +1,5 @@
-// Direct Runge-Kutta stage for UW3 grids without the packed FP32 layout: FP64, and FP32 grids with a
-// ragged n_phi or too small for a staged box.  Same stage as stage_kernel (vlb_stage.cu); the populations
+// Direct Runge-Kutta stage for FP64, for WENO5, and for FP32 UW3 grids without the packed layout (a
+// ragged n_phi, or too small for a staged box).  Same stage as stage_kernel (vlb_stage.cu); the populations
 // are read straight from global memory through L1 instead of being staged, so a tile can be small.
 //
 // FP64 is bound by the FP64 units (1.25 TFLOP/s nominal, pipe 99% active on the busiest SM): what counts is
@@ -9,7 +9,11 @@
 // of one thread per node do not trigger the next stage early: its CTAs would fill the free slots of
 // lightly loaded SMs and unbalance it (85 us a stage against 66 on 128 x 384).
 // FP32 grids off the packed layout are bound by latency (one wave); no staging with a modulo and a
-// 4-byte copy per element: 250 x 501 diffusive 57.6 -> 40 us per step.
+// 4-byte copy per element: 250 x 501 diffusive 57.6 -> 39 us per step.
+// WENO5 is bound by issue (about 50 instructions a face): a face is evaluated once for both its nodes instead
+// of once for each, with one approximate reciprocal instead of four divisions.  FP32, 256 x 512: 132 -> 72 us
+// per step (83 with the range check as a branch in every face); FP64, 128 x 256: 2399 -> 513 us.  At most 102
+// registers (five CTAs per SM): with seven and spills 75 us at 256 x 512, 517 against 537 us at 1024 x 1024.
 #include "vlb_node.cuh"
 
 namespace vlb {
@@ -68,13 +72,13 @@ __device__ __forceinline__ void slot_node(int it, int& mr, int& mc) {
 
 // One CTA per TQ x TSW tile.  Step 1 puts the moments and mu of the tile and a halo of 1 into shared memory
 // (dn, 1/n, u^theta, u^phi, mu); step 2 evaluates the right-hand side and the update.
-template <typename T, int CH, bool F0, int TQ, int TSW, bool SPLIT>
-__global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
+template <typename T, int ADV, int CH, bool F0, int TQ, int TSW, bool SPLIT>
+__global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && sizeof(T) == 4 ? 5 : 0)
     direct_kernel(StageArgs<T> a, const __grid_constant__ DirectConst<T> dc) {
   constexpr bool DF = sizeof(T) == 4;
   constexpr int MS = TSW + 2, MN = (TQ + 2) * MS, NTH = TQ * TSW * (SPLIT ? 4 : 1);
   constexpr int ITEMS = TQ * TSW + 2 * TSW + 2 * TQ;
-  constexpr bool HOLD = sizeof(T) == 8;  // hold U^n in registers over step 1
+  constexpr bool HOLD = sizeof(T) == 8 && ADV == VLB_UW3;  // hold U^n in registers over step 1
   constexpr bool TAB = !SPLIT && sizeof(T) == 8;  // row table in shared memory (FP64-bound), else per thread
   constexpr int NE = row_entries<T>(), RP = NE | 1;  // odd row pitch: two rows of a warp on different banks
   __shared__ T s_dn[MN], s_in[MN], s_ut[MN], s_up[MN], s_mu[MN], s_rt[TAB ? TQ * RP : 1];
@@ -86,6 +90,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
   constexpr uint32_t B = sizeof(T);
   const NodeConst<T>& nc = dc.nc;
   const T* phi = a.fin + NPOP * st;
+  constexpr bool KEEP = !SPLIT && ADV == VLB_UW3;  // the parity combinations stay in registers for step 2
   T P[SPLIT ? 1 : 16], U0[SPLIT ? 4 : 16];
   if (F0) {  // U^n of this thread's populations, in flight over step 1
     const int node = SPLIT ? tid >> 2 : tid, q = q0 + node / TSW, s = s0 + node % TSW;
@@ -140,7 +145,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
     T cubic = vmul(ph, vsub(T(1), ph2));
     if constexpr (DF) cubic = vfma(vsub(T(1), vmul(T(3), ph2)), lo, cubic);  // at hi + lo, to first order in lo
     s_mu[mi] = vsub(vmul(-a.A, cubic), vmul(a.kappa, lap));
-    if constexpr (!SPLIT) {
+    if constexpr (KEEP) {
       if (keep)
 #pragma unroll
         for (int k = 0; k < 16; ++k) P[k] = g[k];
@@ -154,6 +159,103 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
   }
   __syncthreads();
   if (SPLIT || sizeof(T) == 4) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+
+  constexpr bool WENO = ADV == VLB_WENO5;
+  __shared__ T s_adv[WENO ? 16 * TQ * TSW : 1], s_edge[WENO ? 16 * TQ : 1];
+  if constexpr (WENO) {
+    // Advection: -dt v (face difference) along both directions.  Warp i takes the four populations of theta
+    // velocity v_i, a lane a column.  Everything is seen from the upwind side (up = -1 for v > 0, +1 for
+    // v < 0), so that one face formula serves both signs.  Along theta a lane marches over the tile's rows,
+    // so a face is evaluated once for its two nodes (TQ + 1 faces for TQ nodes); along varphi a lane
+    // evaluates its downwind face and takes the upwind one from its neighbour, the tile's first lane from
+    // a face formed beforehand.
+    static_assert(!SPLIT && TSW == 32 && NTH == 4 * 32 && 16 * TQ <= NTH, "a warp per theta velocity");
+    const int i = tid >> 5, lane = tid & 31;
+    auto near = [](int x, int n) {
+      while (x < 0) x += n;
+      while (x >= n) x -= n;
+      return x;
+    };
+    auto col = [&](int c) { return B * (uint32_t)near(s0 + c, ns); };
+    bool bad = false;
+    if (tid < 16 * TQ) {  // the tile's first upwind face: at s0 - 1/2 (v > 0) or s0 + TSW - 1/2
+      const int k = tid / TQ, dn = (k & 3) >= 2 ? 1 : -1, first = dn > 0 ? -1 : TSW;
+      const uint32_t row = B * (uint32_t)(wrap_near(q0 + tid % TQ, nt) * ns);
+      T x[5];
+#pragma unroll
+      for (int d = 0; d < 5; ++d) x[d] = at(a.fin + k * st, row + col(first + dn * (d - 2)));
+      s_edge[tid] = weno5_face(x[0], x[1], x[2], x[3], x[4], bad);
+    }
+    __syncthreads();
+    const int dt_ = i >= 2 ? 1 : -1, top = i >= 2 ? 0 : TQ - 1;  // downwind step along theta; the first row of the march
+    uint32_t ro[TQ + 5], cs[5];  // rows of the march, columns lane - 2 .. lane + 2 (byte offsets)
+    T J[TQ + 5];
+#pragma unroll
+    for (int d = 0; d < TQ + 5; ++d) {
+      const int row = near(q0 + top + dt_ * (d - 3), nt);
+      ro[d] = B * (uint32_t)(row * ns);
+      J[d] = a.coef[(int64_t)C_J * nt + row];
+    }
+#pragma unroll
+    for (int d = 0; d < 5; ++d) cs[d] = col(lane + d - 2);
+    T vct[TQ], ccp[TQ];
+#pragma unroll
+    for (int r = 0; r < TQ; ++r) {
+      const int row = near(q0 + top + dt_ * r, nt);
+      vct[r] = -(dt_ > 0 ? dc.v[i] : -dc.v[i]) * (a.coef[(int64_t)C_CT * nt + row] * a.dt);
+      ccp[r] = a.coef[(int64_t)C_CP * nt + row] * a.dt;
+    }
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      const int k = 4 * i + j;
+      const T* f = a.fin + k * st;
+      const T fref = a.n0 * dc.ww[i][j];  // theta reconstructs the full J f
+      const int dp = j >= 2 ? 1 : -1;     // downwind step along varphi
+      const T vj = dp > 0 ? dc.v[j] : -dc.v[j];
+      const uint32_t c0 = dp > 0 ? cs[0] : cs[4], c1 = dp > 0 ? cs[1] : cs[3], c3 = dp > 0 ? cs[3] : cs[1];
+      const uint32_t c4 = dp > 0 ? cs[4] : cs[0];
+      T G[TQ + 5], x[TQ];
+#pragma unroll
+      for (int d = 0; d < TQ + 5; ++d) {
+        const T g = at(f, ro[d] + cs[2]);
+        if (d >= 3 && d < TQ + 3) x[d - 3] = g;
+        G[d] = J[d] * (g + fref);
+      }
+      T last = weno5_face(G[0], G[1], G[2], G[3], G[4], bad);
+#pragma unroll
+      for (int r = 0; r < TQ; ++r) {
+        const int lrow = top + dt_ * r;
+        const T F = weno5_face(G[r + 1], G[r + 2], G[r + 3], G[r + 4], G[r + 5], bad);
+        T adv = vct[r] * (F - last);  // -|v| (downwind - upwind face) in both directions
+        last = F;
+        const uint32_t o = ro[r + 3];
+        const T Fd = weno5_face(at(f, o + c0), at(f, o + c1), x[r], at(f, o + c3), at(f, o + c4), bad);
+        T Fu = __shfl_sync(0xffffffffu, Fd, (lane - dp) & 31);
+        if (lane == (dp > 0 ? 0 : 31)) Fu = s_edge[k * TQ + lrow];
+        adv -= vj * ccp[r] * (Fd - Fu);
+        s_adv[(k * TQ + lrow) * TSW + lane] = adv;
+      }
+    }
+    if (__syncthreads_or(bad)) {  // rare: the whole tile again with the plain face formula
+#pragma unroll 1
+      for (int x = lane; x < 4 * TQ * TSW; x += 32) {
+        const int j = x / (TQ * TSW), lrow = x / TSW % TQ, k = 4 * i + j, row = near(q0 + lrow, nt);
+        const T* f = a.fin + k * st;
+        T xt[7], xp[7];
+#pragma unroll
+        for (int d = 0; d < 7; ++d) {
+          const int rd = near(q0 + lrow + d - 3, nt);
+          xt[d] = a.coef[(int64_t)C_J * nt + rd] * (at(f, B * (uint32_t)(rd * ns) + cs[2]) + a.n0 * dc.ww[i][j]);
+          xp[d] = at(f, B * (uint32_t)(row * ns) + col(lane + d - 3));
+        }
+        const T Dt = i >= 2 ? weno_diff<T, true>(xt) : weno_diff<T, false>(xt);
+        const T Dp = j >= 2 ? weno_diff<T, true>(xp) : weno_diff<T, false>(xp);
+        s_adv[(k * TQ + lrow) * TSW + lane] = -(dc.v[i] * (a.coef[(int64_t)C_CT * nt + row] * a.dt)) * Dt -
+                                              (dc.v[j] * (a.coef[(int64_t)C_CP * nt + row] * a.dt)) * Dp;
+      }
+      __syncthreads();
+    }
+  }
 
   const int node = SPLIT ? tid >> 2 : tid;
   const int lr = node / TSW, lc = node % TSW;
@@ -223,10 +325,15 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
     const T g = at(f, id), pv = rt[E_TH + 8 * y + TAP_PV];
     if (F0 && !HOLD) g0 = at(a.f0 + k * st, id);
     if (F0) acc = vadd(acc, vsub(g, g0));
-    acc = vfma(tf, at(f, rf), acc);
-    acc = vfma(tn, at(f, rn), acc);
-    acc = vfma(td, at(f, rd), acc);
-    if constexpr (DF) {
+    if constexpr (!WENO) {
+      acc = vfma(tf, at(f, rf), acc);
+      acc = vfma(tn, at(f, rn), acc);
+      acc = vfma(td, at(f, rd), acc);
+    }
+    if constexpr (WENO) {
+      acc = vadd(acc, s_adv[(k * TQ + lr) * TSW + lc]);
+      acc = vfma(-itau, g, acc);
+    } else if constexpr (DF) {
       acc = vfma(tm, g, acc);
       const T D = vfma(T(2), at(f, cd), vfma(T(3), g, vfma(T(-6), at(f, cn), at(f, cf))));
       acc = vfma(-pv, D, acc);
@@ -242,6 +349,11 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1))
 
   if constexpr (!SPLIT) {
     T R[16];
+    if constexpr (!KEEP) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) P[k] = at(a.fin + k * st, id);
+      to_parity16(P);
+    }
     velocity_space(P, R, nc, rt, Ft, Fp, itau, a.n0, dn, ut, up);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -319,7 +431,7 @@ DirectConst<T> make_direct_const() {
   return c;
 }
 
-template <typename T, int CH, bool F0, int TQ, int TSW, bool SPLIT>
+template <typename T, int ADV, int CH, bool F0, int TQ, int TSW, bool SPLIT>
 cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
   static const DirectConst<T> dc = make_direct_const<T>();
   cudaLaunchConfig_t cfg = {};
@@ -331,7 +443,7 @@ cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, direct_kernel<T, CH, F0, TQ, TSW, SPLIT>, a, dc);
+  return cudaLaunchKernelEx(&cfg, direct_kernel<T, ADV, CH, F0, TQ, TSW, SPLIT>, a, dc);
 }
 
 // FP32: 4 x 32 tiles, one thread per node (8 x 32 tiles with 64 registers: 316 us against 304-320 on eight
@@ -342,26 +454,35 @@ cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
 // 72 / 93 us, 128 x 384 175 / 330 us.
 constexpr int64_t kSplitNodes = 32 * 152;
 
-template <typename T, int CH, bool F0>
+template <typename T, int ADV, int CH, bool F0>
 cudaError_t launch_direct_v(const StageArgs<T>& a, cudaStream_t st) {
-  if constexpr (sizeof(T) == 4) return launch_direct_t<T, CH, F0, 4, 32, false>(a, st);
-  if ((int64_t)a.nt * a.ns <= kSplitNodes) return launch_direct_t<T, CH, F0, 2, 8, true>(a, st);
-  return launch_direct_t<T, CH, F0, 8, 16, false>(a, st);
+  if constexpr (ADV == VLB_WENO5 || sizeof(T) == 4) {
+    return launch_direct_t<T, ADV, CH, F0, 4, 32, false>(a, st);
+  } else {
+    if ((int64_t)a.nt * a.ns <= kSplitNodes) return launch_direct_t<T, ADV, CH, F0, 2, 8, true>(a, st);
+    return launch_direct_t<T, ADV, CH, F0, 8, 16, false>(a, st);
+  }
+}
+
+template <typename T, int ADV>
+cudaError_t launch_direct_a(const StageArgs<T>& a, int ch_mode, cudaStream_t st) {
+  if (ch_mode == VLB_HYDRO)
+    return a.f0 ? launch_direct_v<T, ADV, VLB_HYDRO, true>(a, st) : launch_direct_v<T, ADV, VLB_HYDRO, false>(a, st);
+  return a.f0 ? launch_direct_v<T, ADV, VLB_DIFFUSIVE, true>(a, st)
+              : launch_direct_v<T, ADV, VLB_DIFFUSIVE, false>(a, st);
 }
 
 }  // namespace
 
 template <typename T>
-cudaError_t launch_direct(const StageArgs<T>& a, int ch_mode, cudaStream_t st) {
+cudaError_t launch_direct(const StageArgs<T>& a, int advection, int ch_mode, cudaStream_t st) {
   // 32-bit byte offsets within an array: 2^32 bytes per array would need over 200 GB for the three
   // states and as much again for the FP64 staging area, more than the device has
   if ((uint64_t)a.nt * a.ns * sizeof(T) >= ((uint64_t)1 << 32)) return cudaErrorInvalidValue;
-  if (ch_mode == VLB_HYDRO)
-    return a.f0 ? launch_direct_v<T, VLB_HYDRO, true>(a, st) : launch_direct_v<T, VLB_HYDRO, false>(a, st);
-  return a.f0 ? launch_direct_v<T, VLB_DIFFUSIVE, true>(a, st) : launch_direct_v<T, VLB_DIFFUSIVE, false>(a, st);
+  return advection == VLB_UW3 ? launch_direct_a<T, VLB_UW3>(a, ch_mode, st) : launch_direct_a<T, VLB_WENO5>(a, ch_mode, st);
 }
 
-template cudaError_t launch_direct<float>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_direct<double>(const StageArgs<double>&, int, cudaStream_t);
+template cudaError_t launch_direct<float>(const StageArgs<float>&, int, int, cudaStream_t);
+template cudaError_t launch_direct<double>(const StageArgs<double>&, int, int, cudaStream_t);
 
 }  // namespace vlb

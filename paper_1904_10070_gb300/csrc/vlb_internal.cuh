@@ -140,9 +140,9 @@ cudaError_t launch_wave(const StageArgs<float>& a, int ch_mode, float* U0, float
 template <typename T>
 cudaError_t launch_stage(const StageArgs<T>& a, int advection, int ch_mode, cudaStream_t s,
                          const StageMaps* maps = nullptr);
-// One UW3 stage without staging (vlb_direct.cu): FP64, and FP32 grids outside the packed layout.
+// One stage without staging (vlb_direct.cu): FP64, WENO5, and FP32 grids outside the packed layout.
 template <typename T>
-cudaError_t launch_direct(const StageArgs<T>& a, int ch_mode, cudaStream_t s);
+cudaError_t launch_direct(const StageArgs<T>& a, int advection, int ch_mode, cudaStream_t s);
 // Axisymmetric grids (n_phi = 1, 4 <= n_theta <= kAxiMaxRows; vlb_axi.cu): `steps` whole SSP-RK3 steps of the
 // column in one launch of a single thread-block cluster, on the state U (updated in place).  a.fin, a.f0,
 // a.fout and a.b are not used.

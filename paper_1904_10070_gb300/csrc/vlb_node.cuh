@@ -307,6 +307,29 @@ __device__ __forceinline__ T weno5(T g0, T g1, T g2, T g3, T g4) {
   return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2);
 }
 
+// a / b with b in the range of the weights: FP32 within 2 ulp (it scales a correction to g2)
+__device__ __forceinline__ float quotient(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double quotient(double a, double b) { return a * node_recip(b); }
+
+// The same face value with one reciprocal instead of four divisions: the weights d_k / s_k^2 times (s_0 s_1 s_2)^2.
+// Sets `bad` where the weights leave the range in which no product overflows (differences of about 3000 in
+// FP32, or a value that is not finite): the caller then takes weno5.
+template <typename T>
+__device__ __forceinline__ T weno5_face(T g0, T g1, T g2, T g3, T g4, bool& bad) {
+  const T c = T(13) / T(12), eps = T(1e-6);
+  const T f1 = g1 - g0, f2 = g2 - g1, f3 = g3 - g2, f4 = g4 - g3;
+  const T d0 = f2 - f1, d1 = f3 - f2, d2 = f4 - f3;
+  const T e0 = d0 + T(2) * f2, e1 = f2 + f3, e2 = d2 - T(2) * f3;  // g0 - 4 g1 + 3 g2, g3 - g1, 3 g2 - 4 g3 + g4
+  const T s0 = (c * d0) * d0 + ((T(0.25) * e0) * e0 + eps), s1 = (c * d1) * d1 + ((T(0.25) * e1) * e1 + eps);
+  const T s2 = (c * d2) * d2 + ((T(0.25) * e2) * e2 + eps);
+  const T p0 = s1 * s2, p1 = s0 * s2, p2 = s0 * s1;
+  const T w0 = (T(0.1) * p0) * p0, w1 = (T(0.6) * p1) * p1, w2 = (T(0.3) * p2) * p2, w = w0 + w1 + w2;
+  bad = bad || !(w <= (sizeof(T) == 4 ? T(1e30) : T(1e250)));
+  // face values relative to g2: (5 f2 - 2 f1) / 6, (f2 + 2 f3) / 6, (4 f3 - f4) / 6
+  const T num = w0 * (T(5) * f2 - T(2) * f1) + w1 * (f2 + T(2) * f3) + w2 * (T(4) * f3 - f4);
+  return g2 + quotient(num, w * T(6));
+}
+
 // WENO5 flux difference face_{+1/2} - face_{-1/2} at the centre x[3] of a 7-point window.
 template <typename T, bool POS>
 __device__ __forceinline__ T weno_diff(const T (&x)[7]) {

@@ -9,8 +9,8 @@
 // carried as an unevaluated float pair hi + lo (vlb_internal.cuh explains both).
 //
 // Work unit: a tile of TQ theta rows x 32 varphi columns.  For a tile the CTA
-//   1. stages, with asynchronous global->shared copies (cp.async), a box of H rows (2 for UW3,
-//      3 for WENO5) and HS columns around the tile for the 16 populations and phi, the tile's
+//   1. stages, with asynchronous global->shared copies (cp.async), a box of H = 2 rows
+//      and HS columns around the tile for the 16 populations and phi, the tile's
 //      U^n values and the per-row coefficients;
 //   2. computes the moments and mu on the tile plus a halo of 1;
 //   3. computes the right-hand sides and the Runge-Kutta combination and stores the tile.
@@ -21,11 +21,11 @@
 // The stage is bound by latency and the shared-memory pipe (58% busy) at 16 warps per SM, with HBM at about 75%;
 // against step 3 on the populations themselves the warp instructions of a launch at 1024 x 2048 fell from 44.0
 // to 34.0 M, its time from 82.6 to 76.1 us (stage 1: 77.7 to 68.6) and the step from 0.235 to 0.217 ms.
-// WENO5 grids and ragged ensemble members run steps 2 and 3 in scalar arithmetic, two nodes per thread.  A persistent double-buffered variant (next tile copied in
+// Ragged ensemble members run steps 2 and 3 in scalar arithmetic, two nodes per thread.  A persistent double-buffered variant (next tile copied in
 // while the current one computes, one 384-thread CTA per SM) measured 1.6x slower on GB300: with
 // 12 warps per SM and all warps issuing copies and shared loads in the same phase, the memory-
-// input queue throttled issue to 30%.  FP64 UW3 grids and FP32 UW3 grids off the packed layout are stepped by
-// direct_kernel (vlb_direct.cu).
+// input queue throttled issue to 30%.  FP64 and WENO5 grids and FP32 UW3 grids off the packed layout are stepped
+// by direct_kernel (vlb_direct.cu).
 // Periodic wrap-around is resolved on the copy addresses, so ragged tiles need no special case.
 #include <vector>
 
@@ -77,8 +77,7 @@ struct Lay {
   static_assert((CO_OFF * sizeof(T)) % 16 == 0 && (U0_OFF * sizeof(T)) % 16 == 0, "16-byte aligned sub-buffers");
 };
 
-template <typename T, int ADV>
-using GenericLay = Lay<T, (ADV == VLB_UW3 ? 2 : 3), 16, 4, 256, 1>;
+using StageLay = Lay<float, 2, 16, 4, 256, 1>;
 
 __device__ __forceinline__ int wrap(int x, int n) {
   x %= n;
@@ -154,7 +153,6 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, i
 }
 
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
 // Whether the chunked copy path applies: rows wrap at most once and columns come in aligned
 // 16-byte chunks that never straddle the periodic seam.
@@ -332,7 +330,7 @@ __device__ __forceinline__ void phase2(const StageArgs<T>& a, const VConst<T>& v
 // ---------------------------------------------------------------------------------------------
 // Step 3, scalar: right-hand sides and the Runge-Kutta combination for node (lr, lc) of the tile.
 // ---------------------------------------------------------------------------------------------
-template <typename L, typename T, int ADV, int CH, bool F0>
+template <typename L, typename T, int CH, bool F0>
 __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<T>& vc, const T* box, const T* co,
                                             const T* sm, int lr, int lc, int q, int s) {
   constexpr bool DF = L::DF;
@@ -432,27 +430,11 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
     for (int j = 0; j < 4; ++j) {
       const int k = 4 * i + j;
       const T* fk = sf + k * BQ * BS + bi;
-      T rhs;
-      if (ADV == VLB_UW3) {
-        const T Dt = (i >= 2) ? wp0 * fk[-2 * BS] + wp1 * fk[-BS] + wp2 * g[k] + wp3 * fk[BS]
-                              : wn0 * fk[-BS] + wn1 * g[k] + wn2 * fk[BS] + wn3 * fk[2 * BS];
-        const T Dp = (j >= 2) ? (fk[-2] - T(6) * fk[-1] + T(3) * g[k] + T(2) * fk[1])
-                              : (T(-2) * fk[-1] - T(3) * g[k] + T(6) * fk[1] - fk[2]);
-        rhs = -(vc.v[i] * Dt) - (vc.v[j] * cp6) * Dp;
-      } else {
-        // WENO5 is nonlinear: theta reconstruction of the full G = J (g + n0 w_i w_j); along
-        // varphi the reference part is a constant, which the reconstruction passes through.
-        const T fref = a.n0 * vc.ww[i][j];
-        T xt[7], xp[7];
-#pragma unroll
-        for (int d = 0; d < 7; ++d) {
-          xt[d] = co[C_J * BQ + fr + d - 3] * (fk[(d - 3) * BS] + fref);
-          xp[d] = fk[d - 3];
-        }
-        const T Dt = (i >= 2) ? weno_diff<T, true>(xt) : weno_diff<T, false>(xt);
-        const T Dp = (j >= 2) ? weno_diff<T, true>(xp) : weno_diff<T, false>(xp);
-        rhs = -(vc.v[i] * ct) * Dt - (vc.v[j] * cp) * Dp;
-      }
+      const T Dt = (i >= 2) ? wp0 * fk[-2 * BS] + wp1 * fk[-BS] + wp2 * g[k] + wp3 * fk[BS]
+                            : wn0 * fk[-BS] + wn1 * g[k] + wn2 * fk[BS] + wn3 * fk[2 * BS];
+      const T Dp = (j >= 2) ? (fk[-2] - T(6) * fk[-1] + T(3) * g[k] + T(2) * fk[1])
+                            : (T(-2) * fk[-1] - T(3) * g[k] + T(6) * fk[1] - fk[2]);
+      T rhs = -(vc.v[i] * Dt) - (vc.v[j] * cp6) * Dp;
       // force and inertial terms on the deviation: (Gamma v_j^2 - F^theta) dg/dv_theta + sum_m K_jm h_m
       T dvt = T(0), dvp = T(0);
 #pragma unroll
@@ -702,43 +684,37 @@ __device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const Nod
 // Kernels
 // ---------------------------------------------------------------------------------------------
 
-// Steps 1-3 for one tile.  PM: 0 = scalar step 3 (two or more nodes per thread), 1 = packed node
-// pairs, 2 = decided at run time from the grid (pairs when the chunked layout applies, FP32 UW3).
-template <typename L, typename T, int ADV, int CH, bool F0, int PM>
-__device__ __forceinline__ void tile_body(const StageArgs<T>& a, const VConst<T>& vc, T* sm, int tid, int q0, int s0) {
-  T* box = sm + L::BOX_OFF;
-  T* co = sm + L::CO_OFF;
+// Steps 1-3 for one tile: on packed node pairs (PAIRS: the grid is known to have the chunked layout), or in scalar
+// arithmetic, two or more nodes per thread (ensemble members with another layout).
+template <typename L, int CH, bool F0, bool PAIRS>
+__device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VConst<float>& vc, float* sm, int tid,
+                                          int q0, int s0) {
+  float* box = sm + L::BOX_OFF;
+  float* co = sm + L::CO_OFF;
   pdl_wait();  // the coefficients too may come from the previous kernel (the scratch tables of vlb_step_noalloc)
-  constexpr bool CAN_PAIR = PM != 0 && sizeof(T) == 4 && ADV == VLB_UW3;
-  bool pair = PM == 1;
-  if constexpr (PM == 2) pair = chunked<L>(a.nt, a.ns);
-  if constexpr (CAN_PAIR) {
-    if (pair)
-      issue_rows<L>(a, co, q0, tid);
-    else
-      issue_co<L>(a, co, q0, tid);
-  } else {
+  const bool pair = PAIRS || chunked<L>(a.nt, a.ns);
+  if (pair)
+    issue_rows<L>(a, co, q0, tid);
+  else
     issue_co<L>(a, co, q0, tid);
-  }
   issue_box<L>(a, box, co, q0, s0, tid);
   cp_async_commit();
   if (F0) issue_u0<L>(a, sm + L::U0_OFF, q0, s0, tid);
   cp_async_commit();
   cp_async_wait<1>();  // the box; U^n may still be in flight
   __syncthreads();
-  if constexpr (CAN_PAIR) {
-    if (pair) {
-      PairNode own;
-      phase2_pair<L>(a, vc.nc, box, co, sm, tid, own);
-      cp_async_wait<0>();
-      __syncthreads();
-      pdl_trigger();
-      const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
-      const int q = q0 + lr, s = s0 + lc;  // n_phi is even, so s + 1 < n_phi whenever s < n_phi
-      if (q < a.nt && s < a.ns) phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q, s);
-      return;
-    }
+  if (pair) {
+    PairNode own;
+    phase2_pair<L>(a, vc.nc, box, co, sm, tid, own);
+    cp_async_wait<0>();
+    __syncthreads();
+    pdl_trigger();
+    const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
+    const int q = q0 + lr, s = s0 + lc;  // n_phi is even, so s + 1 < n_phi whenever s < n_phi
+    if (q < a.nt && s < a.ns) phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q, s);
+    return;
   }
+  if constexpr (PAIRS) return;
   phase2<L>(a, vc, box, co, sm, tid);
   cp_async_wait<0>();
   __syncthreads();
@@ -748,7 +724,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<T>& a, const VConst<T>
   for (int m = 0; m < L::TQ / ROWS; ++m) {
     const int lr = tid / TS + ROWS * m, lc = tid % TS;
     const int q = q0 + lr, s = s0 + lc;
-    if (q < a.nt && s < a.ns) phase3_node<L, T, ADV, CH, F0>(a, vc, box, co, sm, lr, lc, q, s);
+    if (q < a.nt && s < a.ns) phase3_node<L, float, CH, F0>(a, vc, box, co, sm, lr, lc, q, s);
   }
 }
 
@@ -822,27 +798,25 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
   phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q0 + lr, s0 + lc);
 }
 
-// One CTA per 16 x 32 tile.
+// One CTA per 16 x 32 tile, on packed node pairs.
 // F0: the stage combines with U^n (stages 2 and 3); the first stage writes U_in + dt L(U_in).
-// PAIR: step 3 on packed node pairs (FP32, UW3, chunked layout); otherwise two scalar nodes per
-// thread (rows lr and lr + 8).
 // TMA: interior tiles are staged by tensor-map copies (tmb: the box of fin, tmu: the tile of f0);
 // tiles whose box wraps around the grid take the per-thread copies.
-template <typename T, int ADV, int CH, bool F0, bool PAIR, bool TMA>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
-    stage_kernel(StageArgs<T> a, VConst<T> vc, const __grid_constant__ CUtensorMap tmb,
+template <int CH, bool F0, bool TMA>
+__global__ void __launch_bounds__(256, 2)
+    stage_kernel(StageArgs<float> a, VConst<float> vc, const __grid_constant__ CUtensorMap tmb,
                  const __grid_constant__ CUtensorMap tmu) {
-  using L = GenericLay<T, ADV>;
+  using L = StageLay;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* sm = reinterpret_cast<T*>(smem_raw);
+  float* sm = reinterpret_cast<float*>(smem_raw);
   const int q0 = blockIdx.y * L::TQ, s0 = blockIdx.x * TS;
-  if constexpr (TMA && sizeof(T) == 4 && ADV == VLB_UW3 && PAIR) {
+  if constexpr (TMA) {
     if (q0 >= L::H && q0 + L::TQ + L::H <= a.nt && s0 >= L::HS && s0 + TS + L::HS <= a.ns) {
       tile_body_tma<L, CH, F0>(a, vc, sm, threadIdx.x, q0, s0, &tmb, &tmu);
       return;
     }
   }
-  tile_body<L, T, ADV, CH, F0, PAIR ? 1 : 0>(a, vc, sm, threadIdx.x, q0, s0);
+  tile_body<L, CH, F0, true>(a, vc, sm, threadIdx.x, q0, s0);
 }
 
 // Ensemble: one launch per stage over the tiles of every member (FP32, UW3).  Block b takes work
@@ -900,7 +874,7 @@ __global__ void __launch_bounds__(TQR * (TS / 2)) ensemble_stage_kernel(const En
       return;
     }
   }
-  tile_body<L, float, VLB_UW3, CH, F0, 2>(a, vc, sm, threadIdx.x, q0, s0);
+  tile_body<L, CH, F0, false>(a, vc, sm, threadIdx.x, q0, s0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1055,9 +1029,9 @@ __global__ void __launch_bounds__(TQR * (TS / 2), TQR == 16 ? 2 : 3) ensemble_pe
         }
         if (!tma) {
           if (stage == 0)
-            tile_body<L, float, VLB_UW3, CH, false, 2>(a, vc, sm, tid, q0, s0);
+            tile_body<L, CH, false, false>(a, vc, sm, tid, q0, s0);
           else
-            tile_body<L, float, VLB_UW3, CH, true, 2>(a, vc, sm, tid, q0, s0);
+            tile_body<L, CH, true, false>(a, vc, sm, tid, q0, s0);
         }
         if (tid == 0) s_next = after;
         __syncthreads();
@@ -1160,7 +1134,7 @@ __global__ void __launch_bounds__(256, 2) wave_kernel(StageArgs<float> base, flo
                                                       int nsteps, int lag, unsigned* cnt, int* err, long long budget,
                                                       int skip_cta, VConst<float> vc,
                                                       const __grid_constant__ WaveMaps maps) {
-  using L = GenericLay<float, VLB_UW3>;
+  using L = StageLay;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int s_item[2], s_go;
   float* sm = reinterpret_cast<float*>(smem_raw);
@@ -1230,9 +1204,9 @@ __global__ void __launch_bounds__(256, 2) wave_kernel(StageArgs<float> base, flo
       if (k > 0) ph_u0 ^= 1u;
     } else {
       if (k == 0)
-        tile_body<L, float, VLB_UW3, CH, false, 1>(a, vc, sm, tid, q0, s0);
+        tile_body<L, CH, false, true>(a, vc, sm, tid, q0, s0);
       else
-        tile_body<L, float, VLB_UW3, CH, true, 1>(a, vc, sm, tid, q0, s0);
+        tile_body<L, CH, true, true>(a, vc, sm, tid, q0, s0);
     }
     // this tile's stores, before the consumers' bulk copies; the CTA's shared-memory reads, before
     // the next tile's copies land
@@ -1277,16 +1251,16 @@ cudaError_t ensure_smem(K kernel, size_t bytes, int& mask) {
   return e;
 }
 
-template <typename T, int ADV, int CH, bool F0, bool PAIR, bool TMA>
-cudaError_t launch_generic(const StageArgs<T>& a, cudaStream_t st, const StageMaps* maps) {
-  using L = GenericLay<T, ADV>;
+template <int CH, bool F0, bool TMA>
+cudaError_t launch_pairs(const StageArgs<float>& a, cudaStream_t st, const StageMaps* maps) {
+  using L = StageLay;
   static int mask = 0;
-  cudaError_t e = ensure_smem(stage_kernel<T, ADV, CH, F0, PAIR, TMA>, L::BYTES, mask);
+  cudaError_t e = ensure_smem(stage_kernel<CH, F0, TMA>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
-  static const VConst<T> vc = make_vconst<T>();
+  static const VConst<float> vc = make_vconst<float>();
   static const StageMaps none = {};
   const StageMaps& m = maps ? *maps : none;
-  StageArgs<T> args = a;
+  StageArgs<float> args = a;
   args.ahead = 0;
   if (TMA) {
     static int resident[32] = {0};  // CTAs of this kernel resident at once, per device
@@ -1294,7 +1268,7 @@ cudaError_t launch_generic(const StageArgs<T>& a, cudaStream_t st, const StageMa
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if (dev < 32 && resident[dev] == 0) {
       int per_sm = 0, sms = 0;
-      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stage_kernel<T, ADV, CH, F0, PAIR, TMA>, 256,
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stage_kernel<CH, F0, TMA>, 256,
                                                              L::BYTES)) != cudaSuccess)
         return e;
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -1314,7 +1288,7 @@ cudaError_t launch_generic(const StageArgs<T>& a, cudaStream_t st, const StageMa
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, stage_kernel<T, ADV, CH, F0, PAIR, TMA>, args, vc, m.box, m.tile);
+  return cudaLaunchKernelEx(&cfg, stage_kernel<CH, F0, TMA>, args, vc, m.box, m.tile);
 }
 
 template <int TQR, int CH, bool F0>
@@ -1399,19 +1373,13 @@ cudaError_t launch_ens_rows(const EnsembleMember* members, const int2* items, in
 template <typename T, int ADV, int CH>
 cudaError_t launch_one(const StageArgs<T>& a, cudaStream_t st, const StageMaps* maps) {
   if constexpr (sizeof(T) == 4 && ADV == VLB_UW3) {
-    if (chunked<GenericLay<T, ADV>>(a.nt, a.ns)) {  // n_phi % 4 == 0: packed node pairs
+    if (chunked<StageLay>(a.nt, a.ns)) {  // n_phi % 4 == 0: packed node pairs
       if (maps)
-        return a.f0 ? launch_generic<T, ADV, CH, true, true, true>(a, st, maps)
-                    : launch_generic<T, ADV, CH, false, true, true>(a, st, maps);
-      return a.f0 ? launch_generic<T, ADV, CH, true, true, false>(a, st, nullptr)
-                  : launch_generic<T, ADV, CH, false, true, false>(a, st, nullptr);
+        return a.f0 ? launch_pairs<CH, true, true>(a, st, maps) : launch_pairs<CH, false, true>(a, st, maps);
+      return a.f0 ? launch_pairs<CH, true, false>(a, st, nullptr) : launch_pairs<CH, false, false>(a, st, nullptr);
     }
   }
-  if constexpr (ADV == VLB_UW3)
-    return launch_direct<T>(a, CH, st);  // FP64, and FP32 off the packed layout (vlb_direct.cu)
-  else
-    return a.f0 ? launch_generic<T, ADV, CH, true, false, false>(a, st, nullptr)
-                : launch_generic<T, ADV, CH, false, false, false>(a, st, nullptr);
+  return launch_direct<T>(a, ADV, CH, st);  // FP64, WENO5, and FP32 off the packed layout (vlb_direct.cu)
 }
 
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1448,10 +1416,10 @@ cudaError_t encode_state_map(CUtensorMap* m, const float* base, int nt, int ns, 
 
 }  // namespace
 
-bool stage_maps_apply(int nt, int ns) { return chunked<GenericLay<float, VLB_UW3>>(nt, ns); }
+bool stage_maps_apply(int nt, int ns) { return chunked<StageLay>(nt, ns); }
 
 cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, int64_t stride, StageMaps* out) {
-  using L = GenericLay<float, VLB_UW3>;
+  using L = StageLay;
   if (!stage_maps_apply(nt, ns) || stride % 4 != 0 || ((uintptr_t)fin) % 16 != 0 || ((uintptr_t)f0) % 16 != 0)
     return cudaErrorInvalidValue;
   cudaError_t e = encode_state_map(&out->box, fin, nt, ns, stride, L::BS, L::BQ);
@@ -1520,7 +1488,7 @@ bool wave_schedule_ok(int nb, int lag, int nsteps) {
 }
 
 bool wave_apply(int nt, int ns) {
-  using L = GenericLay<float, VLB_UW3>;
+  using L = StageLay;
   return stage_maps_apply(nt, ns) && nt % L::TQ == 0 && ns % TS == 0 && nt / L::TQ > 2 * kWaveLag + 2;
 }
 
@@ -1529,7 +1497,7 @@ int wave_counter_words(int nt) { return 3 * (nt / 16) + 1; }
 template <int CH>
 cudaError_t launch_wave_t(const StageArgs<float>& a, float* U0, float* U1, float* U2, int nsteps, unsigned* cnt,
                           long long budget, int skip_cta, cudaStream_t st, const WaveMaps& maps, int* grid_out) {
-  using L = GenericLay<float, VLB_UW3>;
+  using L = StageLay;
   static int mask = 0;
   cudaError_t e = ensure_smem(wave_kernel<CH>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
