@@ -9,16 +9,19 @@
 // a mode (m, n) is divided by 1 + dt M kappa lambda(m, n) with lambda = ((4/h_theta^2) sin^2(pi m/N_theta)
 // + (4/h_phi^2) sin^2(pi n/N_phi))^2; the mean (m = n = 0) is kept, so P conserves sum J x (the
 // integral of x sqrt(g)).  The stage kernel writes dt L_phi into a scratch array; three kernels then
-//   1. transform every theta row of J dt L_phi (complex FFT of real data, one CTA per row),
+//   1. transform the theta rows of J dt L_phi, two rows as one complex transform per CTA, and store the
+//      half spectrum n = 0 .. N_phi / 2 (the two real columns 0 and N_phi / 2 packed into one),
 //   2. transform strips of columns, divide by 1 + dt M kappa lambda and transform them back,
-//   3. transform every row back, take the real part / (N_theta N_phi J), and form phi_out (in FP32 as
+//   3. transform the rows back two at a time, divide by N_theta N_phi J and form phi_out (in FP32 as
 //      the float pair hi + lo with an error-free sum, as the stage kernel does).
-// The FFTs are in-place radix-2 (decimation in time, bit-reversed load) in shared memory, in the
-// state's precision, with twiddles from sincospi; N_theta and N_phi are powers of two <= 4096.  The
-// two factors of lambda, (4/h_theta^2) sin^2(pi m/N_theta) and (4/h_phi^2) sin^2(pi n/N_phi), are
-// tabulated once in FP64 on the host (ch_stab_tables) and rounded to the state precision, so the
-// division runs in that precision with no transcendental per mode; so are the twiddles of both
+// The FFTs are in place in shared memory, in the state's precision; N_theta and N_phi are powers of
+// two <= 4096.  The two factors of lambda, (4/h_theta^2) sin^2(pi m/N_theta) and (4/h_phi^2)
+// sin^2(pi n/N_phi), are tabulated once in FP64 on the host (ch_stab_tables) and rounded to the state
+// precision, so the division runs in that precision with no transcendental per mode; so are the twiddles of both
 // transform lengths, which each CTA copies from global memory (L2) into shared memory.
+// The kernels are bound by the shared-memory passes and the barriers of the transforms, so half the data is
+// half the time: per stage at 1024 x 2048 in FP32 20.5 + 41.7 + 26.9 us with complex transforms of every row,
+// 13.6 + 21.1 + 20.0 us now.
 #include <math.h>
 
 #include <vector>
@@ -103,6 +106,46 @@ __device__ void fft_strided(C2<T>* a, int n, int logn, int logw, int sh, const C
   }
 }
 
+// The adjoint of fft_strided (the unnormalised inverse transform) with the passes in reverse: natural order in,
+// bit-reversed order out (element e ends at position bitrev(e)), so that a transform and its inverse need no
+// reordering in between.
+template <typename T>
+__device__ void fft_adjoint(C2<T>* a, int n, int logn, int logw, int sh, const C2<T>* tw) {
+  const int w = 1 << logw, nq = (n >> 2) << logw;
+  for (int l = logn - 1; l >= 1 + (logn & 1); l -= 2) {
+    const int h = 1 << (l - 1);
+    for (int idx = threadIdx.x; idx < nq; idx += blockDim.x) {
+      const int g = idx >> logw, c = idx & (w - 1);
+      const int j = g & (h - 1);
+      const int i0 = ((g >> (l - 1)) << (l + 1)) + j;
+      const C2<T> t1 = {tw[h - 1 + j].x, -tw[h - 1 + j].y}, t2 = {tw[2 * h - 1 + j].x, -tw[2 * h - 1 + j].y};
+      const int e0 = padded((i0 << logw) + c, sh), e1 = padded(((i0 + h) << logw) + c, sh);
+      const int e2 = padded(((i0 + 2 * h) << logw) + c, sh), e3 = padded(((i0 + 3 * h) << logw) + c, sh);
+      const C2<T> y0 = a[e0], y1 = a[e1], y2 = a[e2], y3 = a[e3];
+      const C2<T> b0 = {y0.x + y2.x, y0.y + y2.y}, b1 = {y1.x + y3.x, y1.y + y3.y};
+      const C2<T> c2 = cmul(C2<T>{y0.x - y2.x, y0.y - y2.y}, t2);
+      C2<T> c3 = cmul(C2<T>{y1.x - y3.x, y1.y - y3.y}, t2);
+      c3 = {-c3.y, c3.x};  // times +i
+      a[e0] = {b0.x + b1.x, b0.y + b1.y};
+      a[e1] = cmul(C2<T>{b0.x - b1.x, b0.y - b1.y}, t1);
+      a[e2] = {c2.x + c3.x, c2.y + c3.y};
+      a[e3] = cmul(C2<T>{c2.x - c3.x, c2.y - c3.y}, t1);
+    }
+    __syncthreads();
+  }
+  if (logn & 1) {
+    const int nb = (n >> 1) << logw;
+    for (int idx = threadIdx.x; idx < nb; idx += blockDim.x) {
+      const int g = idx >> logw, c = idx & (w - 1);
+      const int e0 = padded(((2 * g) << logw) + c, sh), e1 = padded(((2 * g + 1) << logw) + c, sh);
+      const C2<T> u = a[e0], v = a[e1];
+      a[e0] = {u.x + v.x, u.y + v.y};
+      a[e1] = {u.x - v.x, u.y - v.y};
+    }
+    __syncthreads();
+  }
+}
+
 constexpr int kBatch = 8;  // global loads a thread keeps in flight before it stores them
 
 // the n - 1 per-level twiddles of a transform, from the host-computed table
@@ -123,39 +166,53 @@ __device__ __forceinline__ void load_twiddles(C2<T>* tw, const C2<T>* table, int
   }
 }
 
-// 1. Row q: F_phi[J_q dt L_phi(q, .)] -> buf row q.
+// 1. Rows q = 2 b and q + 1 of J dt L_phi, packed as the real and imaginary part of one transform, -> their
+// spectra at 0 .. N_phi / 2 - 1 (the others are their conjugates), entry 0 holding the real values at 0 and N_phi / 2.
 template <typename T>
 __global__ void __launch_bounds__(256) row_fwd_kernel(int ns, int logns, const T* dphi, const double* J,
                                                       const C2<T>* tw_s, C2<T>* buf) {
   extern __shared__ __align__(16) unsigned char raw[];
   C2<T>* a = reinterpret_cast<C2<T>*>(raw);
-  const int sh = row_pad_shift(logns);
+  const int sh = row_pad_shift(logns), nh = ns / 2;
   C2<T>* tw = a + padded(ns, sh);
-  const int q = blockIdx.x;
-  const T jq = (T)J[q];
-  const T* row = dphi + (int64_t)q * ns;
-  for (int s0 = threadIdx.x; s0 < ns; s0 += kBatch * blockDim.x) {
-    T v[kBatch];
+  const int64_t q = 2 * (int64_t)blockIdx.x;
+  const T j0 = (T)J[q], j1 = (T)J[q + 1];
+  const T *x0 = dphi + q * ns, *x1 = x0 + ns;
+  for (int s0 = threadIdx.x; s0 < ns; s0 += (kBatch / 2) * blockDim.x) {
+    T v[kBatch / 2], w[kBatch / 2];
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
+    for (int u = 0; u < kBatch / 2; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s < ns) v[u] = row[s];
+      if (s < ns) {
+        v[u] = x0[s];
+        w[u] = x1[s];
+      }
     }
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
+    for (int u = 0; u < kBatch / 2; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s < ns) a[padded(bitrev(s, logns), sh)] = {jq * v[u], T(0)};
+      if (s < ns) a[padded(bitrev(s, logns), sh)] = {j0 * v[u], j1 * w[u]};
     }
   }
   load_twiddles(tw, tw_s, ns);
   __syncthreads();
   fft_strided(a, ns, logns, 0, sh, tw, false);
-  for (int s = threadIdx.x; s < ns; s += blockDim.x) buf[(int64_t)q * ns + s] = a[padded(s, sh)];
+  C2<T>*r0 = buf + q * nh, *r1 = r0 + nh;
+  for (int k = threadIdx.x; k < nh; k += blockDim.x) {
+    const C2<T> z = a[padded(k, sh)], y = a[padded(k ? ns - k : nh, sh)];
+    if (k == 0) {
+      r0[0] = {z.x, y.x};
+      r1[0] = {z.y, y.y};
+    } else {  // (z + conj y) / 2 and (z - conj y) / 2i
+      r0[k] = {T(0.5) * (z.x + y.x), T(0.5) * (z.y - y.y)};
+      r1[k] = {T(0.5) * (z.y + y.y), T(0.5) * (y.x - z.x)};
+    }
+  }
 }
 
-// 2. Columns n0 .. n0 + cw - 1: F_theta, division by 1 + s lambda(m, n), inverse F_theta.
+// 2. Columns n0 .. n0 + cw - 1 of the half spectrum: F_theta, division by 1 + s lambda(m, n), inverse F_theta.
 template <typename T>
-__global__ void __launch_bounds__(256) col_solve_kernel(int nt, int lognt, int ns, int lcw, T sfac, const T* lam_t,
+__global__ void __launch_bounds__(512) col_solve_kernel(int nt, int lognt, int nh, int lcw, T sfac, const T* lam_t,
                                                         const T* lam_p, const C2<T>* tw_t, C2<T>* buf) {
   extern __shared__ __align__(16) unsigned char raw[];
   C2<T>* a = reinterpret_cast<C2<T>*>(raw);
@@ -168,7 +225,7 @@ __global__ void __launch_bounds__(256) col_solve_kernel(int nt, int lognt, int n
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       const int idx = i0 + u * blockDim.x;
-      if (idx < total) v[u] = buf[(int64_t)(idx >> lcw) * ns + n0 + (idx & (cw - 1))];
+      if (idx < total) v[u] = buf[(int64_t)(idx >> lcw) * nh + n0 + (idx & (cw - 1))];
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
@@ -179,29 +236,35 @@ __global__ void __launch_bounds__(256) col_solve_kernel(int nt, int lognt, int n
   load_twiddles(tw, tw_t, nt);
   __syncthreads();
   fft_strided(a, nt, lognt, lcw, 31, tw, false);
-  const T lp = lam_p[n0 + (threadIdx.x & (cw - 1))];  // a thread keeps its column (blockDim % cw == 0)
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    const int m = idx >> lcw;
+  auto damp = [&](int m, T lp) {
     const T lap = lam_t[m] + lp;
-    const T g = T(1) / (T(1) + sfac * lap * lap);
-    a[idx].x *= g;
-    a[idx].y *= g;
-  }
-  __syncthreads();
-  // back to bit-reversed order for the inverse transform: in-place swaps of the pairs (m, rev(m))
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    const int m = idx >> lcw, c = idx & (cw - 1), r = bitrev(m, lognt);
-    if (m < r) {
-      const C2<T> t = a[idx];
-      a[idx] = a[(r << lcw) + c];
-      a[(r << lcw) + c] = t;
+    return T(1) / (T(1) + sfac * lap * lap);
+  };
+  const int n = n0 + (threadIdx.x & (cw - 1));  // a thread keeps its column (blockDim % cw == 0)
+  const T lp = lam_p[n];
+  if (n) {
+    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+      const T g = damp(idx >> lcw, lp);
+      a[idx].x *= g;
+      a[idx].y *= g;
+    }
+  } else {
+    // the real columns 0 and N_phi / 2 packed as c = f + i h: g_0 f + i g_h h = (g_0 + g_h) / 2 c(m) +
+    // (g_0 - g_h) / 2 conj c(-m); the modes m and -m (the same damping) together
+    const T lh = lam_p[nh];
+    for (int idx = threadIdx.x; idx < (nt / 2 + 1) << lcw; idx += blockDim.x) {
+      const int m = idx >> lcw, mr = m ? nt - m : 0;
+      const T g0 = damp(m, lp), gh = damp(m, lh), p = T(0.5) * (g0 + gh), d = T(0.5) * (g0 - gh);
+      const C2<T> z = a[m << lcw], y = a[mr << lcw];
+      a[m << lcw] = {p * z.x + d * y.x, p * z.y - d * y.y};
+      if (mr != m) a[mr << lcw] = {p * y.x + d * z.x, p * y.y - d * z.y};
     }
   }
   __syncthreads();
-  fft_strided(a, nt, lognt, lcw, 31, tw, true);
+  fft_adjoint(a, nt, lognt, lcw, 31, tw);
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
     const int q = idx >> lcw, c = idx & (cw - 1);
-    buf[(int64_t)q * ns + n0 + c] = a[idx];
+    buf[(int64_t)q * nh + n0 + c] = a[(bitrev(q, lognt) << lcw) + c];
   }
 }
 
@@ -215,7 +278,8 @@ __device__ __forceinline__ void pair_add(float base, float base_lo, float inc, f
   lo = lo2 - (hi - s1);
 }
 
-// 3. Row q: inverse F_phi, y = Re / (N J_q), phi_out = phi^n + b (phi_in - phi^n + y).
+// 3. Rows q = 2 b and q + 1: inverse F_phi of both in one transform, y = Re (Im) / (N J), phi_out = phi^n +
+// b (phi_in - phi^n + y).
 template <typename T>
 __global__ void __launch_bounds__(256) row_inv_kernel(int ns, int logns, double inv_n, const double* J,
                                                       const C2<T>* tw_s, const C2<T>* buf, const T* phin,
@@ -224,34 +288,44 @@ __global__ void __launch_bounds__(256) row_inv_kernel(int ns, int logns, double 
   constexpr int U = 4;                 // nodes per batch of loads (four state words each)
   extern __shared__ __align__(16) unsigned char raw[];
   C2<T>* a = reinterpret_cast<C2<T>*>(raw);
-  const int sh = row_pad_shift(logns);
+  const int sh = row_pad_shift(logns), nh = ns / 2;
   C2<T>* tw = a + padded(ns, sh);
-  const int q = blockIdx.x;
-  const C2<T>* row = buf + (int64_t)q * ns;
-  for (int s0 = threadIdx.x; s0 < ns; s0 += kBatch * blockDim.x) {
-    C2<T> v[kBatch];
+  const int64_t q = 2 * (int64_t)blockIdx.x;
+  const C2<T>*r0 = buf + q * nh, *r1 = r0 + nh;
+  for (int s0 = threadIdx.x; s0 < nh; s0 += (kBatch / 2) * blockDim.x) {
+    C2<T> v[kBatch / 2], w[kBatch / 2];
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
+    for (int u = 0; u < kBatch / 2; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s < ns) v[u] = row[s];
+      if (s < nh) {
+        v[u] = r0[s];
+        w[u] = r1[s];
+      }
     }
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
+    for (int u = 0; u < kBatch / 2; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s < ns) a[padded(bitrev(s, logns), sh)] = v[u];
+      if (s >= nh) continue;
+      if (s == 0) {  // the packed real values at 0 and N_phi / 2
+        a[0] = {v[u].x, w[u].x};
+        a[padded(bitrev(nh, logns), sh)] = {v[u].y, w[u].y};
+      } else {  // x + i y and, at -s, conj x + i conj y
+        a[padded(bitrev(s, logns), sh)] = {v[u].x - w[u].y, v[u].y + w[u].x};
+        a[padded(bitrev(ns - s, logns), sh)] = {v[u].x + w[u].y, w[u].x - v[u].y};
+      }
     }
   }
   load_twiddles(tw, tw_s, ns);
   __syncthreads();
   fft_strided(a, ns, logns, 0, sh, tw, true);
-  const T scale = (T)(inv_n / J[q]);
-  for (int s0 = threadIdx.x; s0 < ns; s0 += U * blockDim.x) {
+  const T scale[2] = {(T)(inv_n / J[q]), (T)(inv_n / J[q + 1])};
+  for (int s0 = threadIdx.x; s0 < 2 * ns; s0 += U * blockDim.x) {  // the two rows follow each other
     T ph[U], lo[U], base[U], base_lo[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s < ns) {
-        const int64_t g = (int64_t)q * ns + s;
+      if (s < 2 * ns) {
+        const int64_t g = q * ns + s;
         ph[u] = phin[g];
         lo[u] = DF ? phin[g + lo_off] : T(0);
         base[u] = phi0 ? phi0[g] : ph[u];
@@ -261,9 +335,10 @@ __global__ void __launch_bounds__(256) row_inv_kernel(int ns, int logns, double 
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s >= ns) continue;
-      const int64_t g = (int64_t)q * ns + s;
-      const T y = a[padded(s, sh)].x * scale;
+      if (s >= 2 * ns) continue;
+      const int64_t g = q * ns + s;
+      const C2<T> z = a[padded(s & (ns - 1), sh)];
+      const T y = s < ns ? z.x * scale[0] : z.y * scale[1];
       const T inc = phi0 ? b * (((ph[u] - base[u]) + (lo[u] - base_lo[u])) + y) : y;
       if constexpr (DF) {
         float hi_o, lo_o;
@@ -345,12 +420,14 @@ cudaError_t launch_ch_stab(int nt, int ns, double dt_m_kappa, const double* J, c
   const C2<T>* tw_s = tw_t + (nt - 1);
   const size_t row_bytes = sizeof(C2<T>) * ((size_t)ns * 2 + 32);  // data (with its pads) and twiddles
   // column strips of 2^lcw columns: wide enough for whole 32-byte segments, narrow enough that the
-  // launch keeps at least 512 CTAs (about three per SM) when the grid allows
+  // launch keeps at least 256 CTAs of 512 threads (about two per SM) when the grid allows
+  const int nh = ns / 2;
   int lcw = 0;
-  while (lcw < 5 && (2 << lcw) <= ns && ((size_t)nt << lcw) * 2 * sizeof(C2<T>) <= kColBudget &&
-         (lcw < 2 || (ns >> (lcw + 1)) >= 512))
+  while (lcw < 5 && (2 << lcw) <= nh && ((size_t)nt << lcw) * 2 * sizeof(C2<T>) <= kColBudget &&
+         (lcw < 2 || (nh >> (lcw + 1)) >= 256))
     ++lcw;
   const size_t col_bytes = sizeof(C2<T>) * (((size_t)nt << lcw) + nt);
+  const int col_threads = ((size_t)nt << lcw) >= 2048 ? 512 : 256;
   // the attribute is set once per device to the largest size any grid needs (setting it to a
   // smaller size would cap later launches on larger grids)
   constexpr size_t row_max = sizeof(C2<T>) * (4096 * 2 + 32);
@@ -360,12 +437,13 @@ cudaError_t launch_ch_stab(int nt, int ns, double dt_m_kappa, const double* J, c
   if ((e = smem_attr(row_fwd_kernel<T>, row_max, m1)) != cudaSuccess) return e;
   if ((e = smem_attr(col_solve_kernel<T>, col_max, m2)) != cudaSuccess) return e;
   if ((e = smem_attr(row_inv_kernel<T>, row_max, m3)) != cudaSuccess) return e;
-  row_fwd_kernel<T><<<nt, 256, row_bytes, st>>>(ns, logns, dphi, J, tw_s, cb);
+  row_fwd_kernel<T><<<nt / 2, 256, row_bytes, st>>>(ns, logns, dphi, J, tw_s, cb);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  col_solve_kernel<T><<<ns >> lcw, 256, col_bytes, st>>>(nt, lognt, ns, lcw, (T)dt_m_kappa, lam, lam + nt, tw_t, cb);
+  col_solve_kernel<T><<<nh >> lcw, col_threads, col_bytes, st>>>(nt, lognt, nh, lcw, (T)dt_m_kappa, lam, lam + nt, tw_t,
+                                                                 cb);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  row_inv_kernel<T><<<nt, 256, row_bytes, st>>>(ns, logns, 1.0 / ((double)nt * ns), J, tw_s, cb, phin, phi0, phiout,
-                                               lo_off, b);
+  row_inv_kernel<T><<<nt / 2, 256, row_bytes, st>>>(ns, logns, 1.0 / ((double)nt * ns), J, tw_s, cb, phin, phi0, phiout,
+                                                   lo_off, b);
   return cudaGetLastError();
 }
 
