@@ -268,7 +268,7 @@ constexpr long long kWaveBudget = 1ll << 31;  // SM clock cycles per dependency 
 // has its counters and the stage tensor maps.  VLB_SCHED_AUTO takes the per-stage launches, which
 // measured faster on GB300 (0.236 against 0.469 ms per step at 1024 x 2048).
 bool wave_active(const vlb_handle* h) {
-  return h->kind == 0 && h->wave_cnt && h->maps && h->sched == VLB_SCHED_WAVE;
+  return h->kind == 0 && h->wave_cnt && h->wave_maps && h->sched == VLB_SCHED_WAVE;
 }
 
 template <typename T>
@@ -327,7 +327,7 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
         if (p.diag_every > 0) chunk = std::min<int64_t>(chunk, p.diag_every - h->steps_done % p.diag_every);
         VLB_CUDA(h, vlb::launch_wave(a, p.ch_mode, U0, U1, U2, (int)chunk, h->wave_cnt,
                                      h->wave_budget > 0 ? h->wave_budget : kWaveBudget, h->wave_skip, h->stream,
-                                     h->maps, nullptr));
+                                     h->wave_maps, nullptr));
         h->steps_done += chunk;
         n += chunk;
         if (p.diag_every > 0 && (h->steps_done % p.diag_every == 0 || n == nsteps)) {
@@ -645,13 +645,18 @@ vlb_status vlb_create(const vlb_params* p, void* d_workspace, size_t bytes, void
     return fail(nullptr, VLB_ERR_CUDA, "vlb_create upload: %s", cudaGetErrorString(e));
   }
   if (h->esize == 4 && p->advection == VLB_UW3 && vlb::stage_maps_apply(p->n_theta, p->n_phi)) {
-    h->maps = new (std::nothrow) vlb::StageMaps[3];
-    for (int k = 0; k < 3 && h->maps; ++k)
-      if (vlb::make_stage_maps((const float*)h->U[k], (const float*)h->U[0], p->n_theta, p->n_phi, h->stride,
-                               h->maps + k) != cudaSuccess) {
-        delete[] h->maps;  // the driver has no tensor-map encoder: per-thread copies only
-        h->maps = nullptr;
-      }
+    auto make = [&](int rows) -> vlb::StageMaps* {
+      vlb::StageMaps* m = new (std::nothrow) vlb::StageMaps[3];
+      for (int k = 0; k < 3 && m; ++k)
+        if (vlb::make_stage_maps((const float*)h->U[k], (const float*)h->U[0], p->n_theta, p->n_phi, h->stride, rows,
+                                 m + k) != cudaSuccess) {
+          delete[] m;  // the driver has no tensor-map encoder: per-thread copies only
+          m = nullptr;
+        }
+      return m;
+    };
+    h->maps = make(vlb::stage_rows(p->n_theta, p->n_phi));
+    if (h->wave_cnt) h->wave_maps = make(16);
   }
   *out = h;
   return VLB_OK;
@@ -668,7 +673,8 @@ vlb_status vlb_destroy(vlb_handle* h) {
     delete[] h->views;
   }
   delete[] h->maps;
-  delete h->ens_maps;
+  delete[] h->wave_maps;
+  delete[] h->ens_maps;
   delete h;
   return VLB_OK;
 }
@@ -814,7 +820,7 @@ vlb_status vlb_set_schedule(vlb_handle* h, int32_t schedule) {
   if (h->kind != 0) return fail(h, VLB_ERR_ARG, "vlb_set_schedule: solver handles only");
   if (schedule != VLB_SCHED_AUTO && schedule != VLB_SCHED_STAGES && schedule != VLB_SCHED_WAVE)
     return fail(h, VLB_ERR_ARG, "vlb_set_schedule: unknown schedule %d", (int)schedule);
-  if (schedule == VLB_SCHED_WAVE && !(h->wave_cnt && h->maps))
+  if (schedule == VLB_SCHED_WAVE && !(h->wave_cnt && h->wave_maps))
     return fail(h, VLB_ERR_ARG, "vlb_set_schedule: the wavefront schedule needs an FP32 UW3 explicit grid with "
                                 "n_theta a multiple of 16 (at least 176) and n_phi a multiple of 32");
   h->sched = schedule;
@@ -971,13 +977,13 @@ vlb_status ens_launch_steps(vlb_handle* h, int mode, int rows_idx, int nsteps, c
     VLB_CUDA(h, vlb::launch_ensemble_persistent(h->d_members, h->d_items[rows_idx], h->nitems[rows_idx], nsteps, 0,
                                                 kTileRows[rows_idx], h->p.ch_mode, h->ens_bar, h->flag,
                                                 h->ens_budget > 0 ? h->ens_budget : kBarrierBudget, h->ens_skip,
-                                                h->ens_ctas, st, h->ens_maps, &h->ens_grid));
+                                                h->ens_ctas, st, h->ens_maps + rows_idx, &h->ens_grid));
     return VLB_OK;
   }
   for (int n = 0; n < nsteps; ++n)
     for (int stage = 0; stage < 3; ++stage)
       VLB_CUDA(h, vlb::launch_ensemble_stage(h->d_members, h->d_items[rows_idx], h->nitems[rows_idx], stage,
-                                            kTileRows[rows_idx], h->p.ch_mode, h->flag, st, h->ens_maps));
+                                            kTileRows[rows_idx], h->p.ch_mode, h->flag, st, h->ens_maps + rows_idx));
   return VLB_OK;
 }
 
@@ -992,10 +998,10 @@ vlb_status ens_time(vlb_handle* h, int mode, int rows_idx, float* ms) {
     if (mode == 2)
       return vlb::launch_ensemble_persistent(h->d_members, h->d_items[rows_idx], h->nitems[rows_idx], reps, 1,
                                              kTileRows[rows_idx], h->p.ch_mode, h->ens_bar, h->flag, kBarrierBudget,
-                                             -1, h->ens_ctas, h->stream, h->ens_maps, nullptr);
+                                             -1, h->ens_ctas, h->stream, h->ens_maps + rows_idx, nullptr);
     for (int r = 0; r < reps; ++r) {
       cudaError_t e = vlb::launch_ensemble_stage(h->d_members, h->d_items[rows_idx], h->nitems[rows_idx], 0,
-                                                 kTileRows[rows_idx], h->p.ch_mode, h->flag, h->stream, h->ens_maps);
+                                                 kTileRows[rows_idx], h->p.ch_mode, h->flag, h->stream, h->ens_maps + rows_idx);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1223,7 +1229,7 @@ vlb_status vlb_ensemble_create(const vlb_params* p, int32_t count, void* d_works
     return fail(nullptr, VLB_ERR_ARG, "out of host memory");
   }
   std::vector<vlb::EnsembleMember> desc(count);
-  h->ens_maps = new (std::nothrow) vlb::EnsembleMaps();
+  h->ens_maps = new (std::nothrow) vlb::EnsembleMaps[2]();
   if (!h->ens_maps) {
     vlb_destroy(h);
     return fail(nullptr, VLB_ERR_ARG, "out of host memory");
@@ -1288,12 +1294,12 @@ vlb_status vlb_ensemble_create(const vlb_params* p, int32_t count, void* d_works
     d.maps = -1;  // members beyond kEnsMapMembers, or without an encoder, take per-thread copies
     if (m < vlb::kEnsMapMembers && vlb::stage_maps_apply(p[m].n_theta, p[m].n_phi)) {
       bool ok = true;
-      for (int k = 0; k < 3 && ok; ++k) {
+      for (int k = 0; k < 6 && ok; ++k) {
         vlb::StageMaps sm;
-        ok = vlb::make_stage_maps((const float*)v->U[k], (const float*)v->U[0], p[m].n_theta, p[m].n_phi, L.stride,
-                                  &sm) == cudaSuccess;
-        h->ens_maps->m[4 * m + k] = sm.box;
-        if (k == 0) h->ens_maps->m[4 * m + 3] = sm.tile;
+        ok = vlb::make_stage_maps((const float*)v->U[k % 3], (const float*)v->U[0], p[m].n_theta, p[m].n_phi, L.stride,
+                                  kTileRows[k / 3], &sm) == cudaSuccess;
+        h->ens_maps[k / 3].m[4 * m + k % 3] = sm.box;
+        if (k % 3 == 0) h->ens_maps[k / 3].m[4 * m + 3] = sm.tile;
       }
       if (ok) d.maps = 4 * m;
     }

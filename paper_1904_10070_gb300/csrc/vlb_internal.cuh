@@ -88,7 +88,12 @@ struct StageMaps {
 // Whether a grid takes the tensor-map path (FP32 UW3 with n_phi % 4 == 0 and a grid at least one
 // box large).
 bool stage_maps_apply(int nt, int ns);
-cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, int64_t stride, StageMaps* out);
+// rows: the tile height the maps serve (stage_rows for launch_stage, the work list's for ensembles, 16 for the
+// wavefront schedule).
+cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, int64_t stride, int rows,
+                            StageMaps* out);
+// Tile height of a solver's stage launches on this grid: 16 or 8 rows.
+int stage_rows(int nt, int ns);
 
 // Ensemble member as seen by the batched stage kernel (FP32 state).
 struct EnsembleMember {
@@ -103,7 +108,7 @@ struct EnsembleMember {
 
 // Tensor maps of the first kEnsMapMembers ensemble members, passed as one __grid_constant__ kernel
 // parameter (coherent for each launch, no proxy fence): per member the boxes of U^n, U^(1), U^(2)
-// and the U^n tile, for 16-row tiles.  28 KB, inside the 32 KB kernel-parameter limit.
+// and the U^n tile, for one tile height.  28 KB, inside the 32 KB kernel-parameter limit.
 constexpr int kEnsMapMembers = 56;
 struct EnsembleMaps {
   CUtensorMap m[4 * kEnsMapMembers];

@@ -14,15 +14,18 @@
 //      U^n values and the per-row coefficients;
 //   2. computes the moments and mu on the tile plus a halo of 1;
 //   3. computes the right-hand sides and the Runge-Kutta combination and stores the tile.
-// One 256-thread CTA per 16 x 32 tile, two CTAs per SM.  For FP32 UW3 grids with n_phi % 4 == 0 (the
+// One 128-thread CTA per 8 x 32 tile, four CTAs per SM, or one 256-thread CTA per 16 x 32 tile, two per SM
+// (stage_rows_rule).  For FP32 UW3 grids with n_phi % 4 == 0 (the
 // production path) steps 2 and 3 run on adjacent node pairs in packed FP32x2 arithmetic, two lanes of
 // one float2 per thread: a thread loads its pair once in step 2, keeps the parity combinations of the
 // populations (vlb_node.cuh) over the barrier and reads everything that depends on the row from a table.
-// The stage is bound by latency and the shared-memory pipe (58% busy) at 16 warps per SM, with HBM at about 75%;
-// against step 3 on the populations themselves the warp instructions of a launch at 1024 x 2048 fell from 44.0
-// to 34.0 M, its time from 82.6 to 76.1 us (stage 1: 77.7 to 68.6) and the step from 0.235 to 0.217 ms.
-// Ragged ensemble members run steps 2 and 3 in scalar arithmetic, two nodes per thread.  A persistent double-buffered variant (next tile copied in
-// while the current one computes, one 384-thread CTA per SM) measured 1.6x slower on GB300: with
+// The stage is bound by latency and the shared-memory pipe at 16 warps per SM (issue slots 45% busy), with HBM at
+// about 80%.  A stage at 1024 x 2048, first / later ones: 77.7 / 82.6 us on the populations themselves, 68.6 / 76.1
+// in the parity basis (44.0 against 34.0 M warp instructions), 62.8 / 73.5 with 8-row tiles, which fit four to an SM
+// because step 3 sums dn again and phi of U^n comes from L2; per step 0.235, 0.217 and 0.204 ms.
+// Ragged ensemble members run steps 2 and 3 in scalar arithmetic, two nodes per thread.  A persistent double-
+// buffered variant (next tile copied in while the current one computes, one 384-thread CTA per SM) measured 1.6x
+// slower on GB300: with
 // 12 warps per SM and all warps issuing copies and shared loads in the same phase, the memory-
 // input queue throttled issue to 30%.  FP64 and WENO5 grids and FP32 UW3 grids off the packed layout are stepped
 // by direct_kernel (vlb_direct.cu).
@@ -51,9 +54,11 @@ struct Lay {
   static constexpr bool DF = sizeof(T) == 4;       // phi as a float pair
   static constexpr int H = H_, TQ = TQ_, HS = HS_, NTH = NTH_, NBUF = NBUF_;
   static constexpr int NST = DF ? NARR + 1 : NARR;  // state arrays (= staged boxes)
+  static constexpr int NU0 = NPOP;                   // arrays of the staged U^n tile (phi comes from L2)
   static constexpr int BQ = TQ + 2 * H, BS = TS + 2 * HS;
   static constexpr int BOX = NST * BQ * BS;          // populations, phi (, phi lo)
-  static constexpr int MQ = TQ + 2, MS = TS + 4;     // moment / mu box: halo 1, column origin -2
+  // moment / mu box: halo 1, column origin -2; column TS of a row takes the next row's unused column -2
+  static constexpr int MQ = TQ + 2, MS = TS + 2, MN = MQ * MS + 2;
   // row coefficients: NCT x BQ for the scalar step 3, or the row table of rows -1 .. TQ for packed pairs; padded:
   // sub-buffers stay 128-byte aligned
   static constexpr int CO = ((NCT * BQ > (TQ + 2) * kRowTable ? NCT * BQ : (TQ + 2) * kRowTable) + 31) / 32 * 32;
@@ -63,11 +68,10 @@ struct Lay {
   static constexpr int BOX_OFF = (VEC - HS % VEC) % VEC;
   static constexpr int CO_OFF = (BOX_OFF + NBUF * BOX + VEC - 1) / VEC * VEC;
   static constexpr int U0_OFF = CO_OFF + NBUF * CO;
-  static constexpr int N_OFF = U0_OFF + NST * TQ * TS;
-  static constexpr int UT_OFF = N_OFF + MQ * MS;
-  static constexpr int UP_OFF = UT_OFF + MQ * MS;
-  static constexpr int MU_OFF = UP_OFF + MQ * MS;
-  static constexpr int MB_OFF = (MU_OFF + MQ * MS + 1) / 2 * 2;  // two 8-byte mbarriers
+  static constexpr int UT_OFF = U0_OFF + NU0 * TQ * TS;
+  static constexpr int UP_OFF = UT_OFF + MN;
+  static constexpr int MU_OFF = UP_OFF + MN;
+  static constexpr int MB_OFF = (MU_OFF + MN + 1) / 2 * 2;  // two 8-byte mbarriers
   static constexpr int TOTAL = MB_OFF + 16 / (int)sizeof(T);
   static constexpr size_t BYTES = sizeof(T) * (size_t)TOTAL;
   static_assert((BOX * sizeof(T)) % 16 == 0 && (BS * sizeof(T)) % 16 == 0 && (BQ * BS * sizeof(T)) % 16 == 0,
@@ -77,7 +81,9 @@ struct Lay {
   static_assert((CO_OFF * sizeof(T)) % 16 == 0 && (U0_OFF * sizeof(T)) % 16 == 0, "16-byte aligned sub-buffers");
 };
 
-using StageLay = Lay<float, 2, 16, 4, 256, 1>;
+template <int TQR>
+using StageLayR = Lay<float, 2, TQR, 4, TQR*(TS / 2), 1>;
+using StageLay = StageLayR<16>;
 
 __device__ __forceinline__ int wrap(int x, int n) {
   x %= n;
@@ -229,7 +235,7 @@ __device__ __forceinline__ void issue_u0(const StageArgs<T>& a, T* su0, int q0, 
     // TQ x TS/VEC chunk positions; the arrays are split between groups of threads
     constexpr int CT = TS / VEC, NPOS = TQ * CT;
     constexpr int GROUPS = L::NTH / NPOS > 0 ? L::NTH / NPOS : 1;
-    constexpr int PER = (L::NST + GROUPS - 1) / GROUPS;
+    constexpr int PER = (L::NU0 + GROUPS - 1) / GROUPS;
     for (int t = tid; t < NPOS * GROUPS; t += L::NTH) {
       const int pos = t % NPOS, grp = t / NPOS;
       const int r = pos / CT, ch = pos - r * CT;
@@ -237,13 +243,13 @@ __device__ __forceinline__ void issue_u0(const StageArgs<T>& a, T* su0, int q0, 
       if (gq < nt && gs < ns) {
         const T* src = a.f0 + (int64_t)gq * ns + gs;
         T* dst = su0 + r * TS + ch * VEC;
-        const int k0 = grp * PER, k1 = k0 + PER < L::NST ? k0 + PER : L::NST;
+        const int k0 = grp * PER, k1 = k0 + PER < L::NU0 ? k0 + PER : L::NU0;
 #pragma unroll 4
         for (int k = k0; k < k1; ++k) cp_async16(dst + k * TQ * TS, src + k * stride);
       }
     }
   } else {
-    for (int idx = tid; idx < L::NST * TQ * TS; idx += L::NTH) {
+    for (int idx = tid; idx < L::NU0 * TQ * TS; idx += L::NTH) {
       const int k = idx / (TQ * TS);
       const int rem = idx - k * (TQ * TS);
       const int r = rem / TS, c = rem - r * TS;
@@ -283,7 +289,6 @@ __device__ __forceinline__ void moment_point(const StageArgs<T>& a, const VConst
   const T mp = vc.v[3] * (col[3] - col[0]) + vc.v[2] * (col[2] - col[1]);
   const int mi = mr * MS + mc;
   const T inv_n = recip(a.n0 + dn);
-  sm[L::N_OFF + mi] = dn;
   sm[L::UT_OFF + mi] = mt * inv_n;
   sm[L::UP_OFF + mi] = mp * inv_n;
   const T* pp = sphi + bi;
@@ -339,7 +344,6 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
   const T* sphi = box + NPOP * BQ * BS;
   const T* sphl = box + (NPOP + 1) * BQ * BS;
   const T* su0 = sm + L::U0_OFF;
-  const T* sn = sm + L::N_OFF;
   const T* sut = sm + L::UT_OFF;
   const T* sup = sm + L::UP_OFF;
   const T* smu = sm + L::MU_OFF;
@@ -350,7 +354,14 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
   const int mi = (lr + 1) * MS + (lc + 2);
   const int ui = lr * TS + lc;
 
-  const T dn = sn[mi], ut = sut[mi], up = sup[mi], ph = sphi[bi];
+  // population deviations at the node, and their sum as in step 2
+  T g[NPOP], row[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+  for (int k = 0; k < NPOP; ++k) {
+    g[k] = sf[k * BQ * BS + bi];
+    row[k >> 2] += g[k];
+  }
+  const T dn = (row[0] + row[1]) + (row[2] + row[3]), ut = sut[mi], up = sup[mi], ph = sphi[bi];
   const T n = a.n0 + dn;
   const T ct = co[C_CT * BQ + fr], cp = co[C_CP * BQ + fr], gam = co[C_GAM * BQ + fr];
   const T mu_c = smu[mi], mu_n = smu[mi + MS], mu_s = smu[mi - MS], mu_e = smu[mi + 1], mu_w = smu[mi - 1];
@@ -378,8 +389,8 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
     const T lo = DF ? sphl[bi] : T(0);
     T base = ph, base_lo = lo, inc = Lphi * a.dt;
     if (F0) {
-      base = su0[NPOP * TQ * TS + ui];
-      base_lo = DF ? su0[(NPOP + 1) * TQ * TS + ui] : T(0);
+      base = __ldcg(a.f0 + NPOP * stride + gidx);
+      base_lo = DF ? __ldcg(a.f0 + (NPOP + 1) * stride + gidx) : T(0);
       inc = a.b * (((ph - base) + (lo - base_lo)) + inc);
     }
     if (DF) {
@@ -395,11 +406,6 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
       a.fout[NPOP * stride + gidx] = base + inc;
     }
   }
-
-  // population deviations at the node
-  T g[NPOP];
-#pragma unroll
-  for (int k = 0; k < NPOP; ++k) g[k] = sf[k * BQ * BS + bi];
 
   // UW3 advection weights: the theta flux difference of G = J g with ct/6 folded in, over
   // d = -2..1 (v > 0) and d = -1..2 (v < 0); the varphi difference is scaled by cp/6.
@@ -567,13 +573,24 @@ __device__ __forceinline__ void phase2_pair(const StageArgs<float>& a, const Nod
   st2(sm + L::UP_OFF + mr * MS + mc, own.up);
 }
 
+// phi of U^n at a thread's pair of nodes, loaded before step 2 so that it is in flight meanwhile; from L2, since
+// a persistent launch may hold a line of an earlier step in L1.
+template <bool F0>
+__device__ __forceinline__ void load_u0_phi(const StageArgs<float>& a, int q, int s, float2& hi, float2& lo) {
+  if (F0 && !a.dphi && q < a.nt && s < a.ns) {
+    const float* p = a.f0 + NPOP * a.stride + (int64_t)q * a.ns + s;
+    hi = __ldcg(reinterpret_cast<const float2*>(p));
+    lo = __ldcg(reinterpret_cast<const float2*>(p + a.stride));
+  }
+}
+
 // Step 3 on a pair: right-hand sides and the Runge-Kutta combination (velocity-space terms in the parity basis,
 // vlb_node.cuh).  Two lanes of one float2, so the arithmetic issues as FFMA2 / FADD2 / FMUL2 and
 // shared and global accesses are 8 bytes; the two varphi taps that straddle a pair are scalar.
 template <typename L, int CH, bool F0>
 __device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const NodeConst<float>& nc, const float* box,
-                                            const float* rows, const float* sm, PairNode& n, int lr, int lc, int q,
-                                            int s) {
+                                            const float* rows, const float* sm, PairNode& n, float2 u0_hi, float2 u0_lo,
+                                            int lr, int lc, int q, int s) {
   constexpr int H = L::H, BQ = L::BQ, BS = L::BS, HS = L::HS, MS = L::MS, TQ = L::TQ;
   const float* sphi = box + NPOP * BQ * BS;
   const float* su0 = sm + L::U0_OFF;
@@ -614,8 +631,8 @@ __device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const Nod
   } else {
     float2 base = n.ph, base_lo = n.lo, inc = Lp;
     if (F0) {
-      base = ld2(su0 + NPOP * TQ * TS + ui);
-      base_lo = ld2(su0 + (NPOP + 1) * TQ * TS + ui);
+      base = u0_hi;
+      base_lo = u0_lo;
       inc = vmul(f2(a.b), vadd(vadd(vsub(n.ph, base), vsub(n.lo, base_lo)), Lp));
     }
     float2 hi_o, lo_o;
@@ -701,6 +718,10 @@ __device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VCons
   cp_async_commit();
   if (F0) issue_u0<L>(a, sm + L::U0_OFF, q0, s0, tid);
   cp_async_commit();
+  const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));  // the thread's pair of nodes
+  const int q = q0 + lr, s = s0 + lc;                        // n_phi is even, so s + 1 < n_phi whenever s < n_phi
+  float2 u0_hi = f2(0.0f), u0_lo = f2(0.0f);
+  if (pair) load_u0_phi<F0>(a, q, s, u0_hi, u0_lo);
   cp_async_wait<1>();  // the box; U^n may still be in flight
   __syncthreads();
   if (pair) {
@@ -709,9 +730,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VCons
     cp_async_wait<0>();
     __syncthreads();
     pdl_trigger();
-    const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
-    const int q = q0 + lr, s = s0 + lc;  // n_phi is even, so s + 1 < n_phi whenever s < n_phi
-    if (q < a.nt && s < a.ns) phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q, s);
+    if (q < a.nt && s < a.ns) phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, u0_hi, u0_lo, lr, lc, q, s);
     return;
   }
   if constexpr (PAIRS) return;
@@ -722,9 +741,8 @@ __device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VCons
   constexpr int ROWS = L::NTH / TS;  // thread rows; each thread takes TQ / ROWS nodes of its column
 #pragma unroll 1
   for (int m = 0; m < L::TQ / ROWS; ++m) {
-    const int lr = tid / TS + ROWS * m, lc = tid % TS;
-    const int q = q0 + lr, s = s0 + lc;
-    if (q < a.nt && s < a.ns) phase3_node<L, float, CH, F0>(a, vc, box, co, sm, lr, lc, q, s);
+    const int nr = tid / TS + ROWS * m, nc = tid % TS;
+    if (q0 + nr < a.nt && s0 + nc < a.ns) phase3_node<L, float, CH, F0>(a, vc, box, co, sm, nr, nc, q0 + nr, s0 + nc);
   }
 }
 
@@ -738,7 +756,7 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
                                               int q0, int s0, const CUtensorMap* tmb, const CUtensorMap* tmu,
                                               bool init = true, unsigned ph_box = 0, unsigned ph_u0 = 0) {
   constexpr unsigned BOX_BYTES = sizeof(float) * L::NST * L::BQ * L::BS;
-  constexpr unsigned U0_BYTES = sizeof(float) * L::NST * L::TQ * TS;
+  constexpr unsigned U0_BYTES = sizeof(float) * L::NU0 * L::TQ * TS;
   static_assert((L::BOX_OFF * sizeof(float)) % 128 == 0 && (L::U0_OFF * sizeof(float)) % 128 == 0,
                 "tensor-map destinations are 128-byte aligned");
   static_assert((L::MB_OFF * sizeof(float)) % 8 == 0, "mbarriers are 8-byte aligned");
@@ -773,6 +791,9 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
       if (F0) tma_prefetch_3d(tmu, sn, qn, 0);
     }
   }
+  const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
+  float2 u0_hi = f2(0.0f), u0_lo = f2(0.0f);
+  load_u0_phi<F0>(a, q0 + lr, s0 + lc, u0_hi, u0_lo);
   cp_async_wait<0>();
   bool ok = mbar_wait(bar, ph_box);
   if (__syncthreads_or(!ok)) {  // a copy did not land: flag it, let the copies settle, skip the tile
@@ -794,19 +815,18 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
     return;
   }
   pdl_trigger();
-  const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
-  phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, lr, lc, q0 + lr, s0 + lc);
+  phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, u0_hi, u0_lo, lr, lc, q0 + lr, s0 + lc);
 }
 
 // One CTA per 16 x 32 tile, on packed node pairs.
 // F0: the stage combines with U^n (stages 2 and 3); the first stage writes U_in + dt L(U_in).
 // TMA: interior tiles are staged by tensor-map copies (tmb: the box of fin, tmu: the tile of f0);
 // tiles whose box wraps around the grid take the per-thread copies.
-template <int CH, bool F0, bool TMA>
-__global__ void __launch_bounds__(256, 2)
+template <int TQR, int CH, bool F0, bool TMA>
+__global__ void __launch_bounds__(TQR*(TS / 2), TQR == 16 ? 2 : 4)
     stage_kernel(StageArgs<float> a, VConst<float> vc, const __grid_constant__ CUtensorMap tmb,
                  const __grid_constant__ CUtensorMap tmu) {
-  using L = StageLay;
+  using L = StageLayR<TQR>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sm = reinterpret_cast<float*>(smem_raw);
   const int q0 = blockIdx.y * L::TQ, s0 = blockIdx.x * TS;
@@ -823,17 +843,15 @@ __global__ void __launch_bounds__(256, 2)
 // item items[b] = (member, tile index within the member); the member's buffers, grid and scalars
 // come from its descriptor, so members of different sizes, aspect ratios and time steps share the
 // launch.  TQR is the tile height chosen by the autotuner (16 or 8 rows).
-template <int TQR>
-using EnsLay = Lay<float, 2, TQR, 4, TQR * (TS / 2), 1>;
-
-// With 16-row tiles, interior tiles of members that have tensor maps are staged by the bulk copies
+// Interior tiles of members that have tensor maps (for this tile height) are staged by the bulk copies
 // of tile_body_tma, and each block prefetches into L2 the work item `ahead` blocks later.
 template <int TQR, int CH, bool F0>
-__global__ void __launch_bounds__(TQR * (TS / 2)) ensemble_stage_kernel(const EnsembleMember* members,
+__global__ void __launch_bounds__(TQR*(TS / 2), TQR == 16 ? 2 : 4) ensemble_stage_kernel(
+                                                                       const EnsembleMember* members,
                                                                        const int2* items, int nitems, int ahead,
                                                                        int stage, int* err, VConst<float> vc,
                                                                        const __grid_constant__ EnsembleMaps maps) {
-  using L = EnsLay<TQR>;
+  using L = StageLayR<TQR>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sm = reinterpret_cast<float*>(smem_raw);
   const int2 it = items[blockIdx.x];
@@ -859,20 +877,18 @@ __global__ void __launch_bounds__(TQR * (TS / 2)) ensemble_stage_kernel(const En
   a.ahead = 0;
   const int tiles_s = (d.ns + TS - 1) / TS;
   const int q0 = (it.y / tiles_s) * TQR, s0 = (it.y % tiles_s) * TS;
-  if constexpr (TQR == 16) {
-    if (threadIdx.x == 0 && ahead > 0 && blockIdx.x + ahead < nitems) {
-      const int2 nx = items[blockIdx.x + ahead];
-      const EnsembleMember& e = members[nx.x];
-      const int ts = (e.ns + TS - 1) / TS, qn = (nx.y / ts) * TQR, sn = (nx.y % ts) * TS;
-      if (e.maps >= 0 && qn >= L::H && qn + TQR + L::H <= e.nt && sn >= L::HS && sn + TS + L::HS <= e.ns) {
-        tma_prefetch_3d(&maps.m[e.maps + stage], sn - L::HS, qn - L::H, 0);
-        if (F0) tma_prefetch_3d(&maps.m[e.maps + 3], sn, qn, 0);
-      }
+  if (threadIdx.x == 0 && ahead > 0 && blockIdx.x + ahead < nitems) {
+    const int2 nx = items[blockIdx.x + ahead];
+    const EnsembleMember& e = members[nx.x];
+    const int ts = (e.ns + TS - 1) / TS, qn = (nx.y / ts) * TQR, sn = (nx.y % ts) * TS;
+    if (e.maps >= 0 && qn >= L::H && qn + TQR + L::H <= e.nt && sn >= L::HS && sn + TS + L::HS <= e.ns) {
+      tma_prefetch_3d(&maps.m[e.maps + stage], sn - L::HS, qn - L::H, 0);
+      if (F0) tma_prefetch_3d(&maps.m[e.maps + 3], sn, qn, 0);
     }
-    if (d.maps >= 0 && q0 >= L::H && q0 + TQR + L::H <= d.nt && s0 >= L::HS && s0 + TS + L::HS <= d.ns) {
-      tile_body_tma<L, CH, F0>(a, vc, sm, threadIdx.x, q0, s0, &maps.m[d.maps + stage], &maps.m[d.maps + 3]);
-      return;
-    }
+  }
+  if (d.maps >= 0 && q0 >= L::H && q0 + TQR + L::H <= d.nt && s0 >= L::HS && s0 + TS + L::HS <= d.ns) {
+    tile_body_tma<L, CH, F0>(a, vc, sm, threadIdx.x, q0, s0, &maps.m[d.maps + stage], &maps.m[d.maps + 3]);
+    return;
   }
   tile_body<L, CH, F0, false>(a, vc, sm, threadIdx.x, q0, s0);
 }
@@ -960,15 +976,15 @@ __device__ __forceinline__ StageArgs<float> member_args(const EnsembleMember& d,
 // nsteps whole steps, or with only0 nsteps passes of the first stage alone (which writes only the
 // scratch U^(1), so the autotuner can time it without advancing the state).
 template <int TQR, int CH>
-__global__ void __launch_bounds__(TQR * (TS / 2), TQR == 16 ? 2 : 3) ensemble_persistent_kernel(
+__global__ void __launch_bounds__(TQR * (TS / 2), TQR == 16 ? 2 : 4) ensemble_persistent_kernel(
     const EnsembleMember* members, const int2* items, int nitems, int nsteps, int only0, unsigned* bar, int* err,
     long long budget, int skip_cta, VConst<float> vc, const __grid_constant__ EnsembleMaps maps) {
-  using L = EnsLay<TQR>;
+  using L = StageLayR<TQR>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int s_ok;
   float* sm = reinterpret_cast<float*>(smem_raw);
   const int tid = threadIdx.x;
-  if (TQR == 16 && tid == 0) {
+  if (tid == 0) {
     uint64_t* mb = reinterpret_cast<uint64_t*>(sm + L::MB_OFF);
     mbar_init(mb, 1);
     mbar_init(mb + 1, 1);
@@ -1003,7 +1019,7 @@ __global__ void __launch_bounds__(TQR * (TS / 2), TQR == 16 ? 2 : 3) ensemble_pe
         int after = 0;
         if (tid == 0) {
           after = (int)atomicAdd(tickets, 1u);  // used only at the end of the tile
-          if (TQR == 16 && nxw < nitems) {      // the next tile of this CTA, into L2
+          if (nxw < nitems) {                   // the next tile of this CTA, into L2
             const int2 nx = items[nxw];
             const EnsembleMember& e = members[nx.x];
             const int ts = (e.ns + TS - 1) / TS, qn = (nx.y / ts) * TQR, sn = (nx.y % ts) * TS;
@@ -1013,19 +1029,16 @@ __global__ void __launch_bounds__(TQR * (TS / 2), TQR == 16 ? 2 : 3) ensemble_pe
             }
           }
         }
-        bool tma = false;
-        if constexpr (TQR == 16) {
-          tma = d.maps >= 0 && q0 >= L::H && q0 + TQR + L::H <= d.nt && s0 >= L::HS && s0 + TS + L::HS <= d.ns;
-          if (tma) {
-            if (stage == 0)
-              tile_body_tma<L, CH, false>(a, vc, sm, tid, q0, s0, &maps.m[d.maps], &maps.m[d.maps + 3], false, ph_box,
-                                          ph_u0);
-            else
-              tile_body_tma<L, CH, true>(a, vc, sm, tid, q0, s0, &maps.m[d.maps + stage], &maps.m[d.maps + 3], false,
-                                         ph_box, ph_u0);
-            ph_box ^= 1u;
-            if (stage > 0) ph_u0 ^= 1u;
-          }
+        const bool tma = d.maps >= 0 && q0 >= L::H && q0 + TQR + L::H <= d.nt && s0 >= L::HS && s0 + TS + L::HS <= d.ns;
+        if (tma) {
+          if (stage == 0)
+            tile_body_tma<L, CH, false>(a, vc, sm, tid, q0, s0, &maps.m[d.maps], &maps.m[d.maps + 3], false, ph_box,
+                                        ph_u0);
+          else
+            tile_body_tma<L, CH, true>(a, vc, sm, tid, q0, s0, &maps.m[d.maps + stage], &maps.m[d.maps + 3], false,
+                                       ph_box, ph_u0);
+          ph_box ^= 1u;
+          if (stage > 0) ph_u0 ^= 1u;
         }
         if (!tma) {
           if (stage == 0)
@@ -1239,6 +1252,18 @@ VConst<T> make_vconst() {
   return c;
 }
 
+// Tile height of a solver's stage launches.  8-row tiles take 56 KB and 128 threads, so four share an SM (16
+// warps, as two 16-row tiles) with finer-grained overlap of copies and arithmetic: us per step with 16 / 8
+// rows 22.6 / 21.3 (256 x 512), 45.2 / 37.5 (400 x 800), 69.7 / 57.9 (512 x 1024), 218.5 / 203.6 (1024 x 2048); small
+// grids too, where each SM holds at most one tile (64 x 128: 13.7 / 10.3).  In between, where one 16-row tile per SM
+// holds the grid but one 8-row tile does not, the second 8-row tile of an SM costs more than it saves (192 x 384:
+// 15.0 / 17.2, 256 x 256: 14.5 / 16.3).  4-row tiles are no better than 8 above 64 x 128.
+constexpr int kSms = 152;
+int stage_rows_rule(int nt, int ns) {
+  const int64_t cols = (ns + TS - 1) / TS, t8 = cols * ((nt + 7) / 8), t16 = cols * ((nt + 15) / 16);
+  return t8 > kSms && t16 <= kSms ? 16 : 8;
+}
+
 // Per-device, per-kernel one-time set-up (dynamic shared memory opt-in).
 template <typename K>
 cudaError_t ensure_smem(K kernel, size_t bytes, int& mask) {
@@ -1251,11 +1276,11 @@ cudaError_t ensure_smem(K kernel, size_t bytes, int& mask) {
   return e;
 }
 
-template <int CH, bool F0, bool TMA>
+template <int TQR, int CH, bool F0, bool TMA>
 cudaError_t launch_pairs(const StageArgs<float>& a, cudaStream_t st, const StageMaps* maps) {
-  using L = StageLay;
+  using L = StageLayR<TQR>;
   static int mask = 0;
-  cudaError_t e = ensure_smem(stage_kernel<CH, F0, TMA>, L::BYTES, mask);
+  cudaError_t e = ensure_smem(stage_kernel<TQR, CH, F0, TMA>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
   static const VConst<float> vc = make_vconst<float>();
   static const StageMaps none = {};
@@ -1268,7 +1293,7 @@ cudaError_t launch_pairs(const StageArgs<float>& a, cudaStream_t st, const Stage
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if (dev < 32 && resident[dev] == 0) {
       int per_sm = 0, sms = 0;
-      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stage_kernel<CH, F0, TMA>, 256,
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stage_kernel<TQR, CH, F0, TMA>, L::NTH,
                                                              L::BYTES)) != cudaSuccess)
         return e;
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -1280,7 +1305,7 @@ cudaError_t launch_pairs(const StageArgs<float>& a, cudaStream_t st, const Stage
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((a.ns + TS - 1) / TS, (a.nt + L::TQ - 1) / L::TQ);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(L::NTH);
   cfg.dynamicSmemBytes = L::BYTES;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -1288,13 +1313,13 @@ cudaError_t launch_pairs(const StageArgs<float>& a, cudaStream_t st, const Stage
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, stage_kernel<CH, F0, TMA>, args, vc, m.box, m.tile);
+  return cudaLaunchKernelEx(&cfg, stage_kernel<TQR, CH, F0, TMA>, args, vc, m.box, m.tile);
 }
 
 template <int TQR, int CH, bool F0>
 cudaError_t launch_ens(const EnsembleMember* members, const int2* items, int nitems, int stage, int* err,
                        cudaStream_t st, const EnsembleMaps& maps) {
-  using L = EnsLay<TQR>;
+  using L = StageLayR<TQR>;
   static int mask = 0;
   cudaError_t e = ensure_smem(ensemble_stage_kernel<TQR, CH, F0>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
@@ -1320,7 +1345,7 @@ template <int TQR, int CH>
 cudaError_t launch_pers(const EnsembleMember* members, const int2* items, int nitems, int nsteps, int only0,
                         unsigned* bar, int* err, long long budget, int skip_cta, int ctas_per_sm, cudaStream_t st,
                         const EnsembleMaps& maps, int* grid_out) {
-  using L = EnsLay<TQR>;
+  using L = StageLayR<TQR>;
   static int mask = 0;
   cudaError_t e = ensure_smem(ensemble_persistent_kernel<TQR, CH>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
@@ -1370,13 +1395,19 @@ cudaError_t launch_ens_rows(const EnsembleMember* members, const int2* items, in
 }
 
 
+template <int TQR, int CH>
+cudaError_t launch_rows(const StageArgs<float>& a, cudaStream_t st, const StageMaps* maps) {
+  if (maps)
+    return a.f0 ? launch_pairs<TQR, CH, true, true>(a, st, maps) : launch_pairs<TQR, CH, false, true>(a, st, maps);
+  return a.f0 ? launch_pairs<TQR, CH, true, false>(a, st, nullptr) : launch_pairs<TQR, CH, false, false>(a, st, nullptr);
+}
+
 template <typename T, int ADV, int CH>
 cudaError_t launch_one(const StageArgs<T>& a, cudaStream_t st, const StageMaps* maps) {
   if constexpr (sizeof(T) == 4 && ADV == VLB_UW3) {
     if (chunked<StageLay>(a.nt, a.ns)) {  // n_phi % 4 == 0: packed node pairs
-      if (maps)
-        return a.f0 ? launch_pairs<CH, true, true>(a, st, maps) : launch_pairs<CH, false, true>(a, st, maps);
-      return a.f0 ? launch_pairs<CH, true, false>(a, st, nullptr) : launch_pairs<CH, false, false>(a, st, nullptr);
+      const int rows = stage_rows(a.nt, a.ns);
+      return rows == 16 ? launch_rows<16, CH>(a, st, maps) : launch_rows<8, CH>(a, st, maps);
     }
   }
   return launch_direct<T>(a, ADV, CH, st);  // FP64, WENO5, and FP32 off the packed layout (vlb_direct.cu)
@@ -1400,13 +1431,14 @@ EncodeTiled encoder() {
   return fn;
 }
 
-// 3-D map over the 18 FP32 state arrays: (varphi, theta, array), box bx x by x 18.
-cudaError_t encode_state_map(CUtensorMap* m, const float* base, int nt, int ns, int64_t stride, int bx, int by) {
+// 3-D map over the 18 FP32 state arrays: (varphi, theta, array), box bx x by x arrays.
+cudaError_t encode_state_map(CUtensorMap* m, const float* base, int nt, int ns, int64_t stride, int bx, int by,
+                             int arrays) {
   EncodeTiled fn = encoder();
   if (!fn) return cudaErrorNotSupported;
   const cuuint64_t dims[3] = {(cuuint64_t)ns, (cuuint64_t)nt, (cuuint64_t)(NARR + 1)};
   const cuuint64_t strides[2] = {(cuuint64_t)ns * sizeof(float), (cuuint64_t)stride * sizeof(float)};
-  const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)(NARR + 1)};
+  const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)arrays};
   const cuuint32_t estr[3] = {1, 1, 1};
   const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1416,14 +1448,17 @@ cudaError_t encode_state_map(CUtensorMap* m, const float* base, int nt, int ns, 
 
 }  // namespace
 
+int stage_rows(int nt, int ns) { return stage_rows_rule(nt, ns); }
+
 bool stage_maps_apply(int nt, int ns) { return chunked<StageLay>(nt, ns); }
 
-cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, int64_t stride, StageMaps* out) {
+cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, int64_t stride, int rows,
+                            StageMaps* out) {
   using L = StageLay;
   if (!stage_maps_apply(nt, ns) || stride % 4 != 0 || ((uintptr_t)fin) % 16 != 0 || ((uintptr_t)f0) % 16 != 0)
     return cudaErrorInvalidValue;
-  cudaError_t e = encode_state_map(&out->box, fin, nt, ns, stride, L::BS, L::BQ);
-  if (e == cudaSuccess) e = encode_state_map(&out->tile, f0, nt, ns, stride, TS, L::TQ);
+  cudaError_t e = encode_state_map(&out->box, fin, nt, ns, stride, L::BS, rows + 2 * L::H, L::NST);
+  if (e == cudaSuccess) e = encode_state_map(&out->tile, f0, nt, ns, stride, TS, rows, L::NU0);
   return e;
 }
 
