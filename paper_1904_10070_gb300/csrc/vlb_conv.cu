@@ -36,10 +36,13 @@ __global__ void flip_kernel(int cin, int cout, const bf16* w, bf16* wf) {
 // dW[co][t][ci] = sum over groups of partial[group][t][co][ci] and db[co] = sum over groups of
 // bpart[group][co], in a fixed order.  A 256-thread block takes 32 consecutive entries (blocks past the
 // weights take the biases): warp j adds groups j, j + 8, ... (each load 128 contiguous bytes), and the
-// eight warp sums are folded in warp order through shared memory.
+// eight warp sums are folded in warp order through shared memory.  Launched programmatically, like the convolutions
+// before and after it: its blocks are placed while the last partial sums are written.
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(int groups, int cin, int cout, const float* partial,
                                                            float* dw, const float* bpart, float* db) {
   __shared__ float part[8][32];
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int nw = 9 * cout * cin, wblocks = (nw + 31) / 32, j = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool bias = (int)blockIdx.x >= wblocks;
   const int n = bias ? cout : nw;
@@ -103,8 +106,17 @@ cudaError_t conv_wgrad(int H, int W, int cin, int cout, const void* x, const voi
   cudaError_t e = conv_wgrad_tc(H, W, cin, cout, x, dy, partial, bpart, WG_SEGS, st);
   if (e != cudaSuccess) return e;
   const int blocks = (9 * cin * cout + 31) / 32 + (db ? (cout + 31) / 32 : 0);
-  wgrad_reduce_kernel<<<blocks, 256, 0, st>>>(groups, cin, cout, partial, dw, bpart, db);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, wgrad_reduce_kernel, groups, cin, cout, (const float*)partial, dw,
+                            (const float*)bpart, db);
 }
 
 bool conv_shape_ok(int H, int W, int cin, int cout, const char** why) { return shape_ok(H, W, cin, cout, why); }

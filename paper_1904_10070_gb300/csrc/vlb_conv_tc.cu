@@ -36,6 +36,7 @@ constexpr int TPR = 3, TPW = TPX + 2;    // patch rows, patch columns
 // buffer to the MMA warp), so that the latency of the fix-ups never delays the next copy.
 constexpr int TTHR = 224;
 constexpr int MMA_WARP = 4, LOAD_WARP = 5, FIX_WARP = 6;
+constexpr int FIX_AHEAD = 4;  // items (segments) whose wrapped pixels are in flight
 
 template <int CIN, int COUT>
 struct TcLay {
@@ -210,56 +211,101 @@ __device__ __forceinline__ bool fix_patch(unsigned char* dst, const bf16* x, int
   return true;
 }
 
-// Epilogue of work item `item` (row item % H, segment item / H: consecutive items of a CTA fall in
-// different segments) from the accumulator at column `col0`: thread (warp, lane) owns pixel
-// x0 + 32 warp + lane of the item's row; all C_out columns are read before one wait.
+// First pixel of work item `item` (row item % H, segment item / H: consecutive items of a CTA fall in different
+// segments).
+__device__ __forceinline__ size_t item_pixel(int H, int W, int item) {
+  return (size_t)(item % H) * W + (item / H) * TPX;
+}
+
+// 8 x 8 transpose of 16-byte chunks in each group of eight lanes: a[j] of lane l becomes a[l] of lane j.
+__device__ __forceinline__ void transpose_chunks(uint4* a, int lane) {
+#pragma unroll
+  for (int m = 1; m < 8; m <<= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j & m) continue;
+      uint32_t* lo = reinterpret_cast<uint32_t*>(a + j);
+      uint32_t* hi = reinterpret_cast<uint32_t*>(a + (j | m));
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t r = __shfl_xor_sync(~0u, up ? lo[i] : hi[i], m);
+        lo[i] = up ? r : lo[i];
+        hi[i] = up ? hi[i] : r;
+      }
+    }
+  }
+}
+
+// The mask of a thread's outputs, loaded before the accumulator is waited for.  64 channels: chunk lane % 8 of the
+// eight pixels of the lane's group (the order of the stores after the transpose); 16 channels: the thread's pixel.
 template <int COUT>
-__device__ __forceinline__ void epilogue(uint32_t tmem, uint32_t col0, int H, int W, int item, int warp, int lane,
-                                         const float* sbias, const bf16* mask, int relu, bf16* y, float* yf) {
-  const int row = item % H, x0 = (item / H) * TPX;
-  const size_t p = (size_t)row * W + x0 + 32 * warp + lane;
+__device__ __forceinline__ void load_mask(uint4* mk, const bf16* mask, size_t p0, int warp, int lane) {
+  const bf16* base = COUT == 64 ? mask + (p0 + 32 * warp + (lane & ~7)) * 64 + (lane & 7) * 8
+                                : mask + (p0 + 32 * warp + lane) * COUT;
+#pragma unroll
+  for (int i = 0; i < COUT / 8; ++i) mk[i] = *reinterpret_cast<const uint4*>(base + (COUT == 64 ? i * 64 : i * 8));
+}
+
+// bf16 outputs o whose mask is not > 0 become zero
+__device__ __forceinline__ void apply_mask(uint4& o, const uint4& mk) {
+  uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+  const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&mk);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    ow[i] &= (__low2float(mh[i]) > 0.0f ? 0x0000FFFFu : 0u) | (__high2float(mh[i]) > 0.0f ? 0xFFFF0000u : 0u);
+}
+
+// Epilogue of the work item whose first pixel is p0 from the accumulator at column `col0`: thread (warp, lane) owns
+// pixel p0 + 32 warp + lane; all C_out columns are read before one wait.  mk: load_mask, for the bf16 output.
+// The bf16 rows of 64 channels are transposed among eight lanes first, so that a store instruction writes four whole
+// 128-byte pixels instead of 16 bytes of 32 pixels.
+template <int COUT>
+__device__ __forceinline__ void epilogue(uint32_t tmem, uint32_t col0, size_t p0, int warp, int lane,
+                                         const float* sbias, const bf16* mask, const uint4* mk, int relu, bf16* y,
+                                         float* yf) {
+  const size_t p = p0 + 32 * warp + lane;
   uint32_t raw[COUT];
 #pragma unroll
   for (int j = 0; j < COUT / 16; ++j)
     tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + col0 + (uint32_t)(16 * j), raw + 16 * j);
   tmem_wait_ld();
+  uint4 o[COUT / 8];
 #pragma unroll
-  for (int j = 0; j < COUT / 16; ++j) {
-    float v[16];
-    const int co = 16 * j;
+  for (int j = 0; j < COUT / 8; ++j) {
+    float v[8];
+    const int co = 8 * j;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(raw[co + i]) + sbias[co + i];
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(raw[co + i]) + sbias[co + i];
     if (relu) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.0f);
+      for (int i = 0; i < 8; ++i) v[i] = fmaxf(v[i], 0.0f);
     }
-    if (mask) {
-      const uint4* mp = reinterpret_cast<const uint4*>(mask + p * COUT + co);
-      const uint4 m0 = mp[0], m1 = mp[1];
-      const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m0);
-      const __nv_bfloat162* mh1 = reinterpret_cast<const __nv_bfloat162*>(&m1);
+    __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(o + j);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (!(__low2float(mh[i]) > 0.0f)) v[2 * i] = 0.0f;
-        if (!(__high2float(mh[i]) > 0.0f)) v[2 * i + 1] = 0.0f;
-        if (!(__low2float(mh1[i]) > 0.0f)) v[8 + 2 * i] = 0.0f;
-        if (!(__high2float(mh1[i]) > 0.0f)) v[8 + 2 * i + 1] = 0.0f;
-      }
-    }
-    if (y) {
-      uint4 o[2];
-      __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(o);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) oh[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-      uint4* yp = reinterpret_cast<uint4*>(y + p * COUT + co);
-      yp[0] = o[0];
-      yp[1] = o[1];
-    }
+    for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
     if (yf) {
-      float4* fp = reinterpret_cast<float4*>(yf + p * COUT + co);
+      if (mask) {
+        const uint4 m0 = *reinterpret_cast<const uint4*>(mask + p * COUT + co);
+        const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) fp[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        for (int i = 0; i < 4; ++i) {
+          if (!(__low2float(mh[i]) > 0.0f)) v[2 * i] = 0.0f;
+          if (!(__high2float(mh[i]) > 0.0f)) v[2 * i + 1] = 0.0f;
+        }
+      }
+      float4* fp = reinterpret_cast<float4*>(yf + p * COUT + co);
+      fp[0] = make_float4(v[0], v[1], v[2], v[3]);
+      fp[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
+  }
+  if (!y) return;
+  if constexpr (COUT == 64) transpose_chunks(o, lane);
+  bf16* base = COUT == 64 ? y + (p0 + 32 * warp + (lane & ~7)) * 64 + (lane & 7) * 8 : y + p * COUT;
+#pragma unroll
+  for (int i = 0; i < COUT / 8; ++i) {
+    if (mask) apply_mask(o[i], mk[i]);
+    *reinterpret_cast<uint4*>(base + (COUT == 64 ? i * 64 : i * 8)) = o[i];
   }
 }
 
@@ -352,31 +398,44 @@ __global__ void __launch_bounds__(TTHR, 1)
     }
     if (L::SW && nmine == 0 && lane == 0) mbar_wait(wbar, 0);  // the weight copy lands before the CTA exits
   } else if (warp == FIX_WARP) {
-    for (int k = 0; k < nmine && ok; ++k) {
-      const int b = k % NB, item = blockIdx.x + k * gridDim.x;
-      const int row = item % H, x0 = (item / H) * TPX;
-      unsigned char* dst = sm + L::P_OFF + b * L::PATCH;
-      const bool left = x0 == 0, right = x0 + TPX == W;
-      const bool slow = row == 0 || row + 1 == H || (left && right);  // wrapped rows, or both sides wrap
-      // column wrap of an edge segment: the TPR x CH 16-byte chunks of the wrapped pixel, loaded into
-      // registers before the copy lands (their latency overlaps the copy), stored after it
-      uint4 v = make_uint4(0, 0, 0, 0);
-      const bool col_fix = (left || right) && !slow && lane < TPR * L::CH;
-      const int pr = lane / L::CH, c = lane % L::CH, pc = left ? 0 : TPW - 1;
-      if (col_fix) {
-        const int gx = left ? W - 1 : 0, gy = row + pr - 1;
-        v = *reinterpret_cast<const uint4*>(x + ((size_t)gy * W + gx) * CIN + c * 8);
+    // column wrap of an edge segment: the TPR x CH 16-byte chunks of the wrapped pixel, loaded into
+    // registers FIX_AHEAD items before they are stored (after the copy has landed)
+    const int pr = lane / L::CH, c = lane % L::CH;
+    auto col_fix = [&](int k) {
+      const int item = blockIdx.x + k * gridDim.x, row = item % H, x0 = (item / H) * TPX;
+      const bool left = x0 == 0, right = x0 + TPX == W, slow = row == 0 || row + 1 == H || (left && right);
+      return k < nmine && (left || right) && !slow && lane < TPR * L::CH;
+    };
+    auto wrapped = [&](int k) {
+      const int item = blockIdx.x + k * gridDim.x;
+      const int gx = item < H ? W - 1 : 0, gy = item % H + pr - 1;
+      return col_fix(k) ? *reinterpret_cast<const uint4*>(x + ((size_t)gy * W + gx) * CIN + c * 8)
+                        : make_uint4(0, 0, 0, 0);
+    };
+    uint4 v[FIX_AHEAD];
+#pragma unroll
+    for (int u = 0; u < FIX_AHEAD; ++u) v[u] = wrapped(u);
+    for (int k0 = 0; k0 < nmine && ok; k0 += FIX_AHEAD) {
+#pragma unroll
+      for (int u = 0; u < FIX_AHEAD; ++u) {
+        const int k = k0 + u;
+        if (k >= nmine || !ok) break;
+        const int b = k % NB, item = blockIdx.x + k * gridDim.x;
+        const int row = item % H, x0 = (item / H) * TPX;
+        unsigned char* dst = sm + L::P_OFF + b * L::PATCH;
+        const bool left = x0 == 0, right = x0 + TPX == W;
+        ok = __all_sync(~0u, mbar_wait(tma + b, (k / NB) & 1));
+        if (!ok) break;
+        if (row == 0 || row + 1 == H || (left && right)) {  // wrapped rows, or both sides wrap (rare)
+          if (fix_patch<CIN>(dst, x, H, W, row, x0, lane)) fence_async_smem();
+        } else if (left || right) {
+          if (col_fix(k)) *reinterpret_cast<uint4*>(dst + patch_off<CIN>(c, pr, left ? 0 : TPW - 1)) = v[u];
+          fence_async_smem();
+        }
+        v[u] = wrapped(k + FIX_AHEAD);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(pfull + b);
       }
-      ok = mbar_wait(tma + b, (k / NB) & 1);
-      if (!ok) break;
-      if (slow) {  // the first or last row of the grid, or a one-segment-wide grid (rare)
-        if (fix_patch<CIN>(dst, x, H, W, row, x0, lane)) fence_async_smem();
-      } else if (left || right) {
-        if (col_fix) *reinterpret_cast<uint4*>(dst + patch_off<CIN>(c, pr, pc)) = v;
-        fence_async_smem();
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(pfull + b);
     }
   } else if (warp == MMA_WARP) {
     if (lane == 0) {
@@ -415,11 +474,13 @@ __global__ void __launch_bounds__(TTHR, 1)
   } else {  // epilogue warps 0-3
     for (int k = 0; k < nmine && ok; ++k) {
       const int a = k & 1;
-      ok = mbar_wait(afull + a, (k >> 1) & 1);
+      const size_t p0 = item_pixel(H, W, blockIdx.x + k * gridDim.x);
+      uint4 mk[COUT / 8];
+      if (mask && y) load_mask<COUT>(mk, mask, p0, warp, lane);
+      ok = __all_sync(~0u, mbar_wait(afull + a, (k >> 1) & 1));
       if (!ok) break;
       tc_fence_after();
-      epilogue<COUT>(tmem, (uint32_t)(a * L::ACC), H, W, blockIdx.x + k * gridDim.x, warp, lane, sbias, mask, relu,
-                     y, yf);
+      epilogue<COUT>(tmem, (uint32_t)(a * L::ACC), p0, warp, lane, sbias, mask, mk, relu, y, yf);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(aempty + a);
@@ -471,6 +532,48 @@ __device__ __forceinline__ float dy_column_sum(const unsigned char* dyb, int t) 
     s += __bfloat162float(*reinterpret_cast<const bf16*>(dyb + j * (DC * 2) + (chunk << 4) + (c & 7) * 2));
   }
   return s;
+}
+
+// The edge pixels of wrapped segments in the weight-gradient kernels, stored after a segment's copy has landed:
+// lanes 0 .. CPP - 1 the left wrap (pixel j = 0 <- column W - 1), CPP .. 2 CPP - 1 the right wrap (j = TPW - 1 <-
+// column 0), CPP = 16-byte chunks of a pixel.  Chunk c of pixel j sits at chunk c ^ (j % 8) of its 128-byte row
+// (128-byte swizzle) or c ^ ((j / 4) % 2) of its 32-byte row (32-byte swizzle).  The loads run FIX_AHEAD segments
+// ahead: with four segments to a grid row every other one wraps, and their latency would be serial.
+template <int XC, int NS>
+__device__ __forceinline__ bool wgrad_fix(unsigned char* sx, int stage_bytes, const bf16* __restrict__ x, int H, int W,
+                                          int seg0, int nmine, int dyr, int lane, uint64_t* tma, uint64_t* full) {
+  constexpr int CPP = XC / 8;
+  const int segs_row = W / TPX, c = lane % CPP, side = lane / CPP, j = side == 0 ? 0 : TPW - 1;
+  const int cs = XC == 64 ? (c ^ (j & 7)) : (c ^ ((j >> 2) & 1));
+  auto mine = [&](int k) {
+    const int col = (seg0 + k) % segs_row;
+    return k < nmine && ((side == 0 && col == 0) || (side == 1 && col + 1 == segs_row));
+  };
+  auto wrapped = [&](int k) {
+    const int yy = (seg0 + k) / segs_row + dyr - 1, gy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+    return mine(k) ? *reinterpret_cast<const uint4*>(x + ((size_t)gy * W + (side == 0 ? W - 1 : 0)) * XC + c * 8)
+                   : make_uint4(0, 0, 0, 0);
+  };
+  uint4 v[FIX_AHEAD];
+#pragma unroll
+  for (int u = 0; u < FIX_AHEAD; ++u) v[u] = wrapped(u);
+  for (int k0 = 0; k0 < nmine; k0 += FIX_AHEAD) {
+#pragma unroll
+    for (int u = 0; u < FIX_AHEAD; ++u) {
+      const int k = k0 + u;
+      if (k >= nmine) break;
+      const int b = k % NS, col = (seg0 + k) % segs_row;
+      if (!__all_sync(~0u, mbar_wait(tma + b, (k / NS) & 1))) return false;
+      if (col == 0 || col + 1 == segs_row) {
+        if (mine(k)) *reinterpret_cast<uint4*>(sx + b * stage_bytes + j * (XC * 2) + (cs << 4)) = v[u];
+        fence_async_smem();
+      }
+      v[u] = wrapped(k + FIX_AHEAD);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + b);
+    }
+  }
+  return true;
 }
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;\n" ::: "memory"); }
@@ -563,27 +666,7 @@ __global__ void __launch_bounds__(TTHR)
       __syncwarp();
     }
   } else if (warp == FIX_WARP) {
-    for (int k = 0; k < nmine && ok; ++k) {
-      const int b = k % NS, use = k / NS, sg = seg0 + k, row = sg / segs_row, x0 = (sg % segs_row) * TPX;
-      unsigned char* xb = sm + b * L::STAGE + L::DY;
-      const int yy = row + dyr - 1, gy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
-      // the edge pixels of a wrapped segment (pixel j, chunk c at c ^ (j % 8)), loaded into registers
-      // before the copy lands so that their latency overlaps it: lanes 0-7 the left wrap (pixel
-      // j = 0 <- column W - 1), lanes 8-15 the right wrap (j = TPW - 1 <- column 0)
-      const bool left = x0 == 0, right = x0 + TPX == W;
-      const int c = lane % 8, side = lane / 8, j = side == 0 ? 0 : TPW - 1;
-      const bool mine = lane < 16 && ((side == 0 && left) || (side == 1 && right));
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (mine) v = *reinterpret_cast<const uint4*>(x + ((size_t)gy * W + (side == 0 ? W - 1 : 0)) * 64 + c * 8);
-      ok = mbar_wait(tma + b, use & 1);
-      if (!ok) break;
-      if (left || right) {
-        if (mine) *reinterpret_cast<uint4*>(xb + j * 128 + ((c ^ (j & 7)) << 4)) = v;
-        fence_async_smem();
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(full + b);
-    }
+    ok = wgrad_fix<64, NS>(sm + L::DY, L::STAGE, x, H, W, seg0, nmine, dyr, lane, tma, full);
   } else if (warp == MMA_WARP) {
     if (lane == 0) {
       constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((64u >> 3) << 17) |
@@ -720,30 +803,7 @@ __global__ void __launch_bounds__(TTHR)
       __syncwarp();
     }
   } else if (warp == FIX_WARP) {
-    constexpr int CPP = XROW / 16;  // 16-byte chunks per input pixel (2 or 8)
-    for (int k = 0; k < nmine && ok; ++k) {
-      const int b = k % NS, use = k / NS, sg = seg0 + k, row = sg / segs_row, x0 = (sg % segs_row) * TPX;
-      unsigned char* xb = sm + b * L::STAGE + L::DY;
-      const int yy = row + dyr - 1, gy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
-      // the edge pixels of a wrapped segment, loaded into registers before the copy lands: lanes
-      // 0 .. CPP-1 the left wrap (pixel j = 0 <- column W - 1), CPP .. 2 CPP - 1 the right wrap
-      // (j = TPW - 1 <- column 0).  Chunk c of pixel j sits at chunk c ^ (j % 8) of its 128-byte row
-      // (128-byte swizzle) or c ^ ((j / 4) % 2) of its 32-byte row (32-byte swizzle).
-      const bool left = x0 == 0, right = x0 + TPX == W;
-      const int c = lane % CPP, side = lane / CPP, j = side == 0 ? 0 : TPW - 1;
-      const bool mine = lane < 2 * CPP && ((side == 0 && left) || (side == 1 && right));
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (mine) v = *reinterpret_cast<const uint4*>(x + ((size_t)gy * W + (side == 0 ? W - 1 : 0)) * XC + c * 8);
-      ok = mbar_wait(tma + b, use & 1);
-      if (!ok) break;
-      if (left || right) {
-        const int cs = XC == 64 ? (c ^ (j & 7)) : (c ^ ((j >> 2) & 1));
-        if (mine) *reinterpret_cast<uint4*>(xb + j * XROW + (cs << 4)) = v;
-        fence_async_smem();
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(full + b);
-    }
+    ok = wgrad_fix<XC, NS>(sm + L::DY, L::STAGE, x, H, W, seg0, nmine, dyr, lane, tma, full);
   } else if (warp == MMA_WARP) {
     if (lane == 0) {
       // BF16 x BF16 -> F32, both operands MN-major (transpose bits 15, 16), N = 16, M = 64
