@@ -145,16 +145,22 @@ __host__ __device__ constexpr uint32_t idesc() {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TPX >> 4) << 24);
 }
 
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t accumulate) {
+// The MMA warp runs its loop as a whole, so that descriptors and addresses stay in uniform registers, and one lane
+// (lead) issues: with the loop inside `if (lane == 0)` the descriptors went through vector registers for every MMA.
+__device__ __forceinline__ void umma(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
+                                     uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-          d_tmem),
-      "l"(a), "l"(b), "r"(id), "r"(accumulate)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(id), "r"(accumulate), "r"(lead)
       : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(su32(bar))
-               : "memory");
+__device__ __forceinline__ void umma_commit(uint32_t lead, uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(su32(bar)),
+      "r"(lead)
+      : "memory");
 }
 
 // 16 consecutive FP32 columns of this thread's lane (asynchronous: tmem_wait_ld before use)
@@ -438,37 +444,34 @@ __global__ void __launch_bounds__(TTHR, 1)
       }
     }
   } else if (warp == MMA_WARP) {
-    if (lane == 0) {
-      constexpr uint32_t ID = idesc<COUT>();
-      if (L::SW && nmine > 0) ok = mbar_wait(wbar, 0);
-      const uint64_t bd0 = sdesc(su32(sm + L::W_OFF), L::LBO_B, 128);
-      for (int k = 0; k < nmine && ok; ++k) {
-        const int b = k % NB, a = k & 1;
-        ok = mbar_wait(pfull + b, (k / NB) & 1);
-        if (ok && k >= 2) ok = mbar_wait(aempty + a, ((k - 2) >> 1) & 1);  // epilogue of item k - 2
-        if (!ok) break;
-        tc_fence_after();
-        // descriptors differ only in the start address (low 14 bits, 16-byte units): constant offsets
-        const uint32_t pb = su32(sm + L::P_OFF + b * L::PATCH), wb = su32(sm + L::W_OFF);
-        const uint64_t ad0 = sdesc(pb, L::LBO_A, 128);
-        const uint32_t acc = tmem + (uint32_t)(a * L::ACC);
+    constexpr uint32_t ID = idesc<COUT>();
+    const uint32_t lead = lane == 0;
+    if (L::SW && nmine > 0) ok = __all_sync(~0u, mbar_wait(wbar, 0));
+    const uint64_t bd0 = L::SW ? sdesc_sw128(su32(sm + L::W_OFF)) : sdesc(su32(sm + L::W_OFF), L::LBO_B, 128);
+    for (int k = 0; k < nmine && ok; ++k) {
+      const int b = k % NB, a = k & 1;
+      ok = mbar_wait(pfull + b, (k / NB) & 1);
+      if (ok && k >= 2) ok = mbar_wait(aempty + a, ((k - 2) >> 1) & 1);  // epilogue of item k - 2
+      ok = __all_sync(~0u, ok);
+      if (!ok) break;
+      tc_fence_after();
+      // descriptors differ only in the start address (low 14 bits, 16-byte units): constant offsets
+      const uint32_t pb = su32(sm + L::P_OFF + b * L::PATCH);
+      const uint64_t ad0 = L::SW ? sdesc_sw128(pb) : sdesc(pb, L::LBO_A, 128);
+      const uint32_t acc = tmem + (uint32_t)(a * L::ACC);
 #pragma unroll
-        for (int t = 0; t < 9; ++t)
+      for (int t = 0; t < 9; ++t)
 #pragma unroll
-          for (int s2 = 0; s2 < CIN / 16; ++s2) {
-            uint64_t ad, bdd;
-            if constexpr (L::SW) {  // rows (t / 3) * TPW + t % 3 + m; K step s2 is 32 bytes into the row
-              ad = sdesc_sw128(pb + (uint32_t)(((t / 3) * TPW + t % 3) * 128 + 32 * s2));
-              bdd = sdesc_sw128(wb + (uint32_t)(t * COUT * 128 + 32 * s2));
-            } else {
-              ad = ad0 + (uint32_t)(((2 * s2) * TPR + t / 3) * TPW + t % 3);
-              bdd = bd0 + (uint32_t)((t * L::CH + 2 * s2) * COUT);
-            }
-            umma(acc, ad, bdd, ID, (t | s2) != 0);
-          }
-        umma_commit(pempty + b);
-        umma_commit(afull + a);
-      }
+        for (int s2 = 0; s2 < CIN / 16; ++s2) {
+          // swizzled: rows (t / 3) * TPW + t % 3 + m; K step s2 is 32 bytes into the row
+          const uint64_t ad = ad0 + (L::SW ? (uint32_t)(((t / 3) * TPW + t % 3) * 8 + 2 * s2)
+                                           : (uint32_t)(((2 * s2) * TPR + t / 3) * TPW + t % 3));
+          const uint64_t bd = bd0 + (L::SW ? (uint32_t)(t * COUT * 8 + 2 * s2)
+                                           : (uint32_t)((t * L::CH + 2 * s2) * COUT));
+          umma(lead, acc, ad, bd, ID, (t | s2) != 0);
+        }
+      umma_commit(lead, pempty + b);
+      umma_commit(lead, afull + a);
     }
     __syncwarp();
   } else {  // epilogue warps 0-3
@@ -668,25 +671,23 @@ __global__ void __launch_bounds__(TTHR)
   } else if (warp == FIX_WARP) {
     ok = wgrad_fix<64, NS>(sm + L::DY, L::STAGE, x, H, W, seg0, nmine, dyr, lane, tma, full);
   } else if (warp == MMA_WARP) {
-    if (lane == 0) {
-      constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((64u >> 3) << 17) |
-                              ((64u >> 4) << 24);
-      for (int k = 0; k < nmine && ok; ++k) {
-        const int b = k % NS;
-        ok = mbar_wait(full + b, (k / NS) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t dyb = su32(sm + b * L::STAGE), xb = dyb + L::DY;
+    constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((64u >> 3) << 17) |
+                            ((64u >> 4) << 24);
+    const uint32_t lead = lane == 0;
+    for (int k = 0; k < nmine && ok; ++k) {
+      const int b = k % NS;
+      ok = __all_sync(~0u, mbar_wait(full + b, (k / NS) & 1));
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t dyd = sdesc_mn_sw128(su32(sm + b * L::STAGE)), xd = dyd + (uint32_t)(L::DY >> 4);
+#pragma unroll
+      for (int s2 = 0; s2 < TPX / 16; ++s2)
 #pragma unroll
         for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-          for (int s2 = 0; s2 < TPX / 16; ++s2)
-            umma(tmem + 64u * dx, sdesc_mn_sw128(dyb + 2048u * s2), sdesc_mn_sw128(xb + 128u * dx + 2048u * s2), ID,
-                 (k | s2) != 0);
-        umma_commit(empty + b);
-      }
-      if (ok) umma_commit(done);
+          umma(lead, tmem + 64u * dx, dyd + 128u * s2, xd + (8u * dx + 128u * s2), ID, (k | s2) != 0);
+      umma_commit(lead, empty + b);
     }
+    if (ok) umma_commit(lead, done);
     __syncwarp();
   } else {  // warps 0-3: the bias sums as the segments arrive, then this group's partial sums
     float bacc = 0.0f;
@@ -805,34 +806,27 @@ __global__ void __launch_bounds__(TTHR)
   } else if (warp == FIX_WARP) {
     ok = wgrad_fix<XC, NS>(sm + L::DY, L::STAGE, x, H, W, seg0, nmine, dyr, lane, tma, full);
   } else if (warp == MMA_WARP) {
-    if (lane == 0) {
-      // BF16 x BF16 -> F32, both operands MN-major (transpose bits 15, 16), N = 16, M = 64
-      constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((16u >> 3) << 17) |
-                              ((64u >> 4) << 24);
-      for (int k = 0; k < nmine && ok; ++k) {
-        const int b = k % NS;
-        ok = mbar_wait(full + b, (k / NS) & 1);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t dyb = su32(sm + b * L::STAGE), xb = dyb + L::DY;
+    // BF16 x BF16 -> F32, both operands MN-major (transpose bits 15, 16), N = 16, M = 64
+    constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((16u >> 3) << 17) |
+                            ((64u >> 4) << 24);
+    const uint32_t lead = lane == 0;
+    for (int k = 0; k < nmine && ok; ++k) {
+      const int b = k % NS;
+      ok = __all_sync(~0u, mbar_wait(full + b, (k / NS) & 1));
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t dyb = su32(sm + b * L::STAGE), xb = dyb + L::DY;
+      // XC = 16: A = dY (64 channels), B = the shifted X window (16 channels); else A = X, B = dY
+      const uint64_t da = sdesc_mn_sw128(XC == 16 ? dyb : xb), db = sdesc_mn_sw32(XC == 16 ? xb : dyb);
+#pragma unroll
+      for (int s2 = 0; s2 < TPX / 16; ++s2)
 #pragma unroll
         for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-          for (int s2 = 0; s2 < TPX / 16; ++s2) {
-            uint64_t da, db;
-            if (XC == 16) {  // A = dY (64 channels), B = the shifted X window (16 channels)
-              da = sdesc_mn_sw128(dyb + 2048u * s2);
-              db = sdesc_mn_sw32(xb + 32u * dx + 512u * s2);
-            } else {         // A = the shifted X window (64 channels), B = dY (16 channels)
-              da = sdesc_mn_sw128(xb + 128u * dx + 2048u * s2);
-              db = sdesc_mn_sw32(dyb + 512u * s2);
-            }
-            umma(tmem + 16u * dx, da, db, ID, (k | s2) != 0);
-          }
-        umma_commit(empty + b);
-      }
-      if (ok) umma_commit(done);
+          umma(lead, tmem + 16u * dx, da + (128u * s2 + (XC == 16 ? 0u : 8u * dx)),
+               db + (32u * s2 + (XC == 16 ? 2u * dx : 0u)), ID, (k | s2) != 0);
+      umma_commit(lead, empty + b);
     }
+    if (ok) umma_commit(lead, done);
     __syncwarp();
   } else {  // warps 0-3: the bias sums as the segments arrive, then this group's partial sums
     float bacc = 0.0f;
