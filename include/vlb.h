@@ -345,6 +345,11 @@ vlb_status vlb_mse_loss(int64_t npix, const float* pred16, const float* target4,
  * the updated parameters rounded to bf16. */
 vlb_status vlb_adam_step(int64_t n, float* p, const float* g, float* m, float* v, int64_t t, float lr, float b1,
                          float b2, float eps, void* p_bf16, void* cuda_stream);
+/* The same step on `count` tensors in one launch (per 32): host arrays of `count` sizes and device
+ * pointers; p_bf16 may be NULL, and so may its entries. */
+vlb_status vlb_adam_step_many(int32_t count, const int64_t* n, float* const* p, const float* const* g, float* const* m,
+                              float* const* v, int64_t t, float lr, float b1, float b2, float eps,
+                              void* const* p_bf16, void* cuda_stream);
 vlb_status vlb_to_bf16(int64_t n, const float* x, void* y, void* cuda_stream);
 
 /* ---- Surrogate-accelerated stepping (not in the paper) ----

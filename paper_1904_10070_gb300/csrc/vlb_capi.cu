@@ -1572,7 +1572,23 @@ vlb_status vlb_mse_loss(int64_t npix, const float* pred16, const float* target4,
 vlb_status vlb_adam_step(int64_t n, float* p, const float* g, float* m, float* v, int64_t t, float lr, float b1,
                          float b2, float eps, void* p_bf16, void* cuda_stream) {
   if (n < 1 || !p || !g || !m || !v || t < 1) return fail(nullptr, VLB_ERR_ARG, "vlb_adam_step: bad argument");
-  VLB_CUDA(nullptr, vlb::sur_adam(n, p, g, m, v, t, lr, b1, b2, eps, p_bf16, (cudaStream_t)cuda_stream));
+  const vlb::AdamTensor a = {n, p, g, m, v, p_bf16};
+  VLB_CUDA(nullptr, vlb::sur_adam(1, &a, t, lr, b1, b2, eps, (cudaStream_t)cuda_stream));
+  return VLB_OK;
+}
+
+vlb_status vlb_adam_step_many(int32_t count, const int64_t* n, float* const* p, const float* const* g, float* const* m,
+                              float* const* v, int64_t t, float lr, float b1, float b2, float eps,
+                              void* const* p_bf16, void* cuda_stream) {
+  if (count < 1 || !n || !p || !g || !m || !v || t < 1)
+    return fail(nullptr, VLB_ERR_ARG, "vlb_adam_step_many: bad argument");
+  std::vector<vlb::AdamTensor> a(count);
+  for (int32_t k = 0; k < count; ++k) {
+    a[k] = {n[k], p[k], g[k], m[k], v[k], p_bf16 ? p_bf16[k] : nullptr};
+    if (n[k] < 1 || !p[k] || !g[k] || !m[k] || !v[k])
+      return fail(nullptr, VLB_ERR_ARG, "vlb_adam_step_many: bad tensor %d", (int)k);
+  }
+  VLB_CUDA(nullptr, vlb::sur_adam(count, a.data(), t, lr, b1, b2, eps, (cudaStream_t)cuda_stream));
   return VLB_OK;
 }
 

@@ -242,8 +242,16 @@ cudaError_t sur_apply(int64_t n, const float* before, const float* pred, const f
 cudaError_t sur_stats(int64_t n, int C, const float* x, double* part, double* out, cudaStream_t st);
 cudaError_t sur_mse(int64_t n, const float* pred, const float* target, void* grad, double* part, double* loss,
                     cudaStream_t st);
-cudaError_t sur_adam(int64_t n, float* p, const float* g, float* m, float* v, int64_t t, float lr, float b1, float b2,
-                     float eps, void* pb, cudaStream_t st);
+constexpr int kAdamTensors = 32;  // tensors of one launch
+struct AdamTensor {
+  int64_t n;
+  float* p;
+  const float* g;
+  float *m, *v;
+  void* p_bf16;
+};
+cudaError_t sur_adam(int count, const AdamTensor* tensors, int64_t t, float lr, float b1, float b2, float eps,
+                     cudaStream_t st);
 cudaError_t sur_to_bf16(int64_t n, const float* x, void* y, cudaStream_t st);
 size_t sur_reduce_doubles();
 

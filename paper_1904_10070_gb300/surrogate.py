@@ -100,11 +100,8 @@ class SurrogateNet:
     def adam(self, lr: float):
         st = _stream()
         self.t += 1
-        for li in range(len(LAYERS)):
-            vlb.vlb_adam_step(self.w32[li].numel(), self.w32[li], self.dw[li], self.mw[li], self.vw[li], self.t, lr,
-                              0.9, 0.999, 1e-8, self.wb[li], st)
-            vlb.vlb_adam_step(self.b32[li].numel(), self.b32[li], self.db[li], self.mb[li], self.vb[li], self.t, lr,
-                              0.9, 0.999, 1e-8, None, st)
+        vlb.vlb_adam_step_many(self.w32 + self.b32, self.dw + self.db, self.mw + self.mb, self.vw + self.vb, self.t, lr,
+                               0.9, 0.999, 1e-8, self.wb + [None] * len(self.b32), st)
 
     def parameters(self):
         return sum(int(w.numel()) + int(b.numel()) for w, b in zip(self.w32, self.b32))

@@ -26,10 +26,10 @@ EXPORTS = ["vlb_workspace_bytes", "vlb_max_stable_dt", "vlb_create", "vlb_destro
            "vlb_interface_length", "vlb_state_device", "vlb_steps_done", "vlb_last_error",
            "vlb_step_noalloc", "vlb_ensemble_workspace_bytes", "vlb_ensemble_create", "vlb_ensemble_step",
            "vlb_ensemble_member", "vlb_ensemble_tile_rows", "vlb_get_snapshot", "vlb_set_snapshot",
-           "vlb_conv3x3_fwd", "vlb_conv3x3_flip", "vlb_conv3x3_wgrad_workspace_bytes", "vlb_conv3x3_bwd_weight",
-           "vlb_reduce_workspace_bytes", "vlb_surrogate_norm", "vlb_surrogate_features", "vlb_surrogate_targets",
-           "vlb_surrogate_apply", "vlb_snapshot_compare", "vlb_channel_sums", "vlb_mse_loss", "vlb_adam_step", "vlb_to_bf16",
-           "vlb_conv_status", "vlb_test_raise_flag", "vlb_surrogate_workspace_bytes", "vlb_surrogate_create",
+           "vlb_conv3x3_fwd", "vlb_conv3x3_flip", "vlb_conv3x3_wgrad_workspace_bytes",
+           "vlb_conv3x3_bwd_weight", "vlb_reduce_workspace_bytes", "vlb_surrogate_norm", "vlb_surrogate_features", "vlb_surrogate_targets",
+           "vlb_surrogate_apply", "vlb_snapshot_compare", "vlb_channel_sums", "vlb_mse_loss", "vlb_adam_step",
+           "vlb_adam_step_many", "vlb_to_bf16", "vlb_conv_status", "vlb_test_raise_flag", "vlb_surrogate_workspace_bytes", "vlb_surrogate_create",
            "vlb_surrogate_advance", "vlb_surrogate_stats", "vlb_ensemble_configure", "vlb_ensemble_get_config",
            "vlb_structure_length", "vlb_set_schedule", "vlb_get_schedule", "vlb_test_wave_schedule",
            "vlb_test_wave_timeout"]
@@ -151,11 +151,13 @@ def lib() -> ctypes.CDLL:
     L.vlb_mse_loss.argtypes = [I64, P, P, P, P, P, P]
     L.vlb_adam_step.argtypes = [I64, P, P, P, P, I64, ctypes.c_float, ctypes.c_float, ctypes.c_float,
                                 ctypes.c_float, P, P]
+    L.vlb_adam_step_many.argtypes = [I32, P, P, P, P, P, I64, ctypes.c_float, ctypes.c_float, ctypes.c_float,
+                                     ctypes.c_float, P, P]
     L.vlb_to_bf16.argtypes = [I64, P, P, P]
     for name in ("vlb_conv3x3_fwd", "vlb_conv3x3_flip", "vlb_conv3x3_bwd_weight", "vlb_surrogate_norm",
                  "vlb_surrogate_features", "vlb_snapshot_compare",
                  "vlb_surrogate_targets", "vlb_surrogate_apply", "vlb_channel_sums", "vlb_mse_loss", "vlb_adam_step",
-                 "vlb_to_bf16"):
+                 "vlb_adam_step_many", "vlb_to_bf16"):
         getattr(L, name).restype = I32
     _lib = L
     return L
@@ -376,6 +378,14 @@ def vlb_mse_loss(npix, pred16, target4, grad16, work, loss, stream):
 def vlb_adam_step(n, p, g, m, v, t, lr, b1, b2, eps, p_bf16, stream):
     _check(lib().vlb_adam_step(n, _ptr(p), _ptr(g), _ptr(m), _ptr(v), t, lr, b1, b2, eps, _ptr(p_bf16),
                                ctypes.c_void_p(stream)))
+
+
+def vlb_adam_step_many(p, g, m, v, t, lr, b1, b2, eps, p_bf16, stream):
+    """One Adam step on a list of tensors; `p_bf16` has a tensor or None for each."""
+    k = len(p)
+    ptrs = [(ctypes.c_void_p * k)(*(x.data_ptr() if x is not None else None for x in xs)) for xs in (p, g, m, v, p_bf16)]
+    n = (ctypes.c_int64 * k)(*(x.numel() for x in p))
+    _check(lib().vlb_adam_step_many(k, n, *ptrs[:4], t, lr, b1, b2, eps, ptrs[4], ctypes.c_void_p(stream)))
 
 
 def vlb_to_bf16(n, x, y, stream):
