@@ -295,6 +295,10 @@ vlb_status vlb_conv3x3_fwd(int32_t H, int32_t W, int32_t cin, int32_t cout, cons
                            const float* bias, const void* mask, int32_t relu, void* y_bf16, float* y_f32,
                            void* cuda_stream);
 vlb_status vlb_conv3x3_flip(int32_t cin, int32_t cout, const void* w, void* w_flipped, void* cuda_stream);
+/* Backward data of the layer (C_in, C_out) straight from its weights, the same result as the flip and the call
+ * above: dx[p][ci] = sum_{t,co} dy[p - d_t][co] w[co][t][ci] in bf16, zeroed where mask <= 0 (mask may be NULL). */
+vlb_status vlb_conv3x3_bwd_data(int32_t H, int32_t W, int32_t cin, int32_t cout, const void* dy, const void* w,
+                                const void* mask, void* dx_bf16, void* cuda_stream);
 /* dw[co][t][ci] = sum_p dy[p][co] x[p + d_t][ci] and db[co] = sum_p dy[p][co] (db may be NULL), in
  * FP32, with partial sums reduced in a fixed order; workspace of vlb_conv3x3_wgrad_workspace_bytes. */
 size_t vlb_conv3x3_wgrad_workspace_bytes(int32_t H, int32_t W, int32_t cin, int32_t cout);

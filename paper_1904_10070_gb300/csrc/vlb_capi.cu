@@ -1464,6 +1464,15 @@ vlb_status vlb_conv3x3_fwd(int32_t H, int32_t W, int32_t cin, int32_t cout, cons
   return VLB_OK;
 }
 
+vlb_status vlb_conv3x3_bwd_data(int32_t H, int32_t W, int32_t cin, int32_t cout, const void* dy, const void* w,
+                                const void* mask, void* dx_bf16, void* cuda_stream) {
+  const char* why = nullptr;
+  if (!vlb::conv_shape_ok(H, W, cin, cout, &why)) return fail(nullptr, VLB_ERR_ARG, "vlb_conv3x3_bwd_data: %s", why);
+  if (!dy || !w || !dx_bf16) return fail(nullptr, VLB_ERR_ARG, "vlb_conv3x3_bwd_data: NULL tensor");
+  VLB_CUDA(nullptr, vlb::conv_bwd_data_tc(H, W, cin, cout, dy, w, mask, dx_bf16, (cudaStream_t)cuda_stream));
+  return VLB_OK;
+}
+
 vlb_status vlb_conv3x3_flip(int32_t cin, int32_t cout, const void* w, void* w_flipped, void* cuda_stream) {
   if (!w || !w_flipped || cin < 1 || cout < 1) return fail(nullptr, VLB_ERR_ARG, "vlb_conv3x3_flip: bad argument");
   VLB_CUDA(nullptr, vlb::conv_flip(cin, cout, w, w_flipped, (cudaStream_t)cuda_stream));

@@ -2,7 +2,8 @@
 // FP32 accumulators in tensor memory), for the learned surrogate.  Y[p][co] = act(sum_{t,ci}
 // X[p + d_t][ci] W[co][t][ci] + b[co]) on NHWC bf16 tensors, periodic in both directions, with the
 // optional bias, ReLU, mask (outputs where mask <= 0 are zeroed) and bf16 / f32 outputs.  The
-// backward-data convolution is this kernel on flipped weights.
+// backward-data convolution is this kernel on flipped weights, or on the layer's own weights read transposed with the
+// taps in reverse (TRB; a flip took 2.2 us a layer).
 //
 // Implicit GEMM.  A work item is one output row segment of 128 pixels: D[m][n] (m = pixel, n =
 // output channel, M = 128, N = C_out) accumulates over K = 9 taps x C_in,
@@ -11,12 +12,17 @@
 // same buffer with its descriptor start shifted by whole pixel rows, so a shifted window needs no
 // copy.  The weights are staged once per CTA (the CTA is persistent over work items).
 //
-// One 192-thread CTA per SM with six warps in fixed roles: warps 0-3 run the epilogue (warp w reads
-// tensor-memory lanes 32w .. 32w + 31, i.e. those pixels: bias, ReLU, mask, bf16/f32 stores), warp 4
-// allocates tensor memory and one of its threads issues the MMAs, warp 5 issues the copies (the
-// weights once, then one patch per item, three deep, and the periodic fix-ups of edge items).  Two
-// accumulators let the epilogue of one item overlap the MMAs of the next.  Hand-offs are mbarriers
-// and every wait is bounded.
+// One CTA per SM of twelve warps in fixed roles: warps 0-3 run the epilogue of even items, 4-7 of odd ones (warp w
+// reads tensor-memory lanes 32 (w % 4) .. + 31, i.e. those pixels: bias, ReLU, mask, bf16/f32 stores), warp 8 (for
+// C_out = 16 also 9) issues the MMAs, warp 10 the copies (the weights once, then one patch per item, three deep), and
+// warp 11 completes them (waits for a copy to land, applies the periodic fix-ups of edge items and hands the buffer to
+// the MMA warp), so that the latency of the fix-ups never delays the next copy.  Two accumulators let the epilogue of
+// one item overlap the MMAs of the next.  Hand-offs are mbarriers and every wait is bounded.
+//
+// At 256 x 512 an SM has 6.7 items; the MMAs keep the tensor pipe busy for 0.6 us of the 1.4 us an item takes.  What
+// counted, forward / masked us of a 64 -> 64 layer: start 14.3 / 20.0; mask loaded early, whole pixels stored, wrapped
+// columns loaded ahead 14.7 / 16.5; descriptors kept warp-uniform and a second set of epilogue warps 14.3 / 14.6.  A ring
+// of single rows (17 KB an item instead of 50) measured 16.1 / 16.7.
 #include <cuda_bf16.h>
 #include <string.h>
 
@@ -30,22 +36,18 @@ using bf16 = __nv_bfloat16;
 
 constexpr int TPX = 128;                 // pixels per work item (the MMA's M)
 constexpr int TPR = 3, TPW = TPX + 2;    // patch rows, patch columns
-// Warp roles: 0-3 epilogue (warp w reads tensor-memory lanes 32w .. 32w + 31), 4 MMA issue and
-// tensor-memory allocation, 5 issues the tensor-map copies (waiting only for a free buffer), 6
-// completes them (waits for a copy to land, applies the periodic fix-ups of edge items and hands the
-// buffer to the MMA warp), so that the latency of the fix-ups never delays the next copy.
-constexpr int TTHR = 224;
-constexpr int MMA_WARP = 4, LOAD_WARP = 5, FIX_WARP = 6;
 constexpr int FIX_AHEAD = 4;  // items (segments) whose wrapped pixels are in flight
 
-template <int CIN, int COUT>
+// TRB: weights [K channel][tap][N channel] (backward data), the B operand MN-major; else [N][tap][K], K-major.
+template <int CIN, int COUT, bool TRB>
 struct TcLay {
   // C_in = 64: 128-byte pixel rows in the 128-byte-swizzled K-major layout (fast row copies);
   // C_in = 16: the no-swizzle chunk-major layout [16-byte chunk][patch row][patch column]
   static constexpr bool SW = CIN == 64;
+  static constexpr bool WTMA = SW || TRB;                    // weights by tensor-map copies, swizzled
   static constexpr int CH = CIN / 8;                         // 16-byte channel chunks per pixel
   static constexpr int NBUF = 3;                             // patch buffers
-  static constexpr int WTS = 9 * CH * COUT * 16;             // weight bytes
+  static constexpr int TAP = CIN * COUT * 2, WTS = 9 * TAP;  // weight bytes
   static constexpr int PATCH_RAW = CH * TPR * TPW * 16;      // patch bytes
   static constexpr int PATCH = SW ? (PATCH_RAW + 1023) / 1024 * 1024 : (PATCH_RAW + 127) / 128 * 128;
   static constexpr int W_OFF = 0, P_OFF = WTS, BAR_OFF = WTS + NBUF * PATCH;
@@ -57,13 +59,17 @@ struct TcLay {
   static constexpr int COLS = 2 * ACC <= 32 ? 32 : (2 * ACC <= 64 ? 64 : (2 * ACC <= 128 ? 128 : 256));
   static constexpr uint32_t LBO_A = TPR * TPW * 16;          // next channel chunk of the patch
   static constexpr uint32_t LBO_B = COUT * 16;               // next channel chunk of a tap's weights
-  static_assert(SW ? (WTS % 1024 == 0 && PATCH % 1024 == 0) : (WTS % 128 == 0 && PATCH % 128 == 0),
+  static_assert(WTS % 1024 == 0 && (SW ? PATCH % 1024 == 0 : PATCH % 128 == 0),
                 "operand buffers stay aligned to the swizzle atom (1024 bytes) or the core matrix (128 bytes)");
   static_assert(BYTES <= 232448, "fits the opt-in shared memory of one CTA");
   static_assert(COUT % 16 == 0 && COUT <= 256 && CIN % 16 == 0, "MMA shape M = 128, N = C_out, K = 16");
 };
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// The warp's index as a warp-uniform value: what derives from threadIdx.x sends the MMA descriptors through vector
+// registers (64 -> 64 forward 15.7 us instead of 14.3).
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(~0u, threadIdx.x >> 5, 0); }
 
 // Programmatic dependent launch: the convolutions are launched so that a kernel's CTAs may start (tensor
 // memory, mbarriers) while the previous kernel of the stream drains; every global access comes after
@@ -136,6 +142,19 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
 __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// MN-major, 128-byte swizzle: groups of eight K rows (pixels, or input channels of the transposed weights),
+// 128-byte rows 1024 bytes from group to group (one 64-wide atom in MN)
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t addr) {
+  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// MN-major, 32-byte swizzle: 8-pixel groups of 32-byte rows 256 bytes apart (one 16-wide atom in MN)
+__device__ __forceinline__ uint64_t sdesc_mn_sw32(uint32_t addr) {
+  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
 }
 
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9, 10-12 = 1), both
@@ -320,15 +339,21 @@ __device__ __forceinline__ void epilogue(uint32_t tmem, uint32_t col0, size_t p0
 // works on earlier items and the epilogue warps drain the accumulator of item k - 2.  Hand-offs are
 // mbarriers: tma[b] (copy landed), pfull[b] (patch ready, fix-ups included), pempty[b] (its MMAs are
 // done), afull[a] (accumulator ready), aempty[a] (accumulator read, 4 arrivals), w (weights landed).
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(TTHR, 1)
+constexpr int FWD_THREADS = 384;
+// Warps that issue MMAs.  With N = 16 one warp issues more slowly than the tensor pipe works: 64 -> 16 at 256 x 512
+// takes 13.0 us with one and 10.0 with two, items in turn; with N = 64 one is as good (14.3 / 14.0, masked 15.3 / 15.7).
+template <int COUT>
+constexpr int kFwdMmas = COUT == 16 ? 2 : 1;
+template <int CIN, int COUT, bool TRB>
+__global__ void __launch_bounds__(FWD_THREADS, 1)
     conv_fwd_tc_kernel(int H, int W, const bf16* __restrict__ x, const bf16* __restrict__ w,
                        const float* __restrict__ bias, const bf16* __restrict__ mask, int relu, bf16* y, float* yf,
                        int* err, const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap) {
-  using L = TcLay<CIN, COUT>;
+  using L = TcLay<CIN, COUT, TRB>;
   constexpr int NB = L::NBUF;
+  constexpr int MMA_WARP = 8, LOAD_WARP = 10, FIX_WARP = 11, MMAS = kFwdMmas<COUT>;
   extern __shared__ __align__(1024) unsigned char sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF);
   uint64_t *tma = bars, *pfull = bars + NB, *pempty = bars + 2 * NB, *afull = bars + 3 * NB,
            *aempty = bars + 3 * NB + 2, *wbar = bars + 3 * NB + 4;
@@ -354,10 +379,10 @@ __global__ void __launch_bounds__(TTHR, 1)
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   pdl_wait_and_trigger();
-  for (int i = tid; i < COUT; i += TTHR) sbias[i] = bias ? bias[i] : 0.0f;
-  if constexpr (!L::SW) {
+  for (int i = tid; i < COUT; i += FWD_THREADS) sbias[i] = bias ? bias[i] : 0.0f;
+  if constexpr (!L::WTMA) {
     // 16-channel weights (18 KB), chunk-major [t][c][co]: per-thread copies before the roles split
-    for (int i = tid; i < COUT * 9 * L::CH; i += TTHR) {
+    for (int i = tid; i < COUT * 9 * L::CH; i += FWD_THREADS) {
       const int c = i % L::CH, t = (i / L::CH) % 9, co = i / (9 * L::CH);
       cp16(sm + L::W_OFF + ((t * L::CH + c) * COUT + co) * 16, w + ((size_t)co * 9 + t) * CIN + c * 8);
     }
@@ -373,19 +398,16 @@ __global__ void __launch_bounds__(TTHR, 1)
   const int nmine = blockIdx.x < nitems ? (nitems - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   bool ok = true;
   if (warp == LOAD_WARP) {
-    if constexpr (L::SW) {
-      // 64-channel weights (72 KB): nine tensor-map copies, one per tap, of the box (64 c_in, 1 tap,
-      // C_out), each landing as C_out rows of 128 bytes with the 128-byte swizzle at [tap][c_out]; they
-      // overlap the first patch copies
-      if (lane == 0) {
-        mbar_expect_tx(wbar, L::WTS);
-        for (int t = 0; t < 9; ++t)
-          asm volatile(
-              "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
-              "%5}], [%2];\n" ::"r"(su32(sm + L::W_OFF + t * COUT * 128)),
-              "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(su32(wbar)), "r"(0), "r"(t), "r"(0)
-              : "memory");
-      }
+    if (L::WTMA && lane == 0) {
+      // the weights, one box per tap: (64 c_in, 1 tap, C_out) landing as C_out rows of 128 bytes, or transposed
+      // (C_out, 1 tap, C_in) as C_in rows of 2 C_out bytes, tap 8 - t; they overlap the first patch copies
+      mbar_expect_tx(wbar, L::WTS);
+      for (int t = 0; t < 9; ++t)
+        asm volatile(
+            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
+            "%5}], [%2];\n" ::"r"(su32(sm + L::W_OFF + t * L::TAP)),
+            "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(su32(wbar)), "r"(0), "r"(TRB ? 8 - t : t), "r"(0)
+            : "memory");
     }
     for (int k = 0; k < nmine && ok; ++k) {
       const int b = k % NB, use = k / NB, item = blockIdx.x + k * gridDim.x;
@@ -402,7 +424,7 @@ __global__ void __launch_bounds__(TTHR, 1)
       }
       __syncwarp();
     }
-    if (L::SW && nmine == 0 && lane == 0) mbar_wait(wbar, 0);  // the weight copy lands before the CTA exits
+    if (L::WTMA && nmine == 0 && lane == 0) mbar_wait(wbar, 0);  // the weight copy lands before the CTA exits
   } else if (warp == FIX_WARP) {
     // column wrap of an edge segment: the TPR x CH 16-byte chunks of the wrapped pixel, loaded into
     // registers FIX_AHEAD items before they are stored (after the copy has landed)
@@ -443,12 +465,15 @@ __global__ void __launch_bounds__(TTHR, 1)
         if (lane == 0) mbar_arrive(pfull + b);
       }
     }
-  } else if (warp == MMA_WARP) {
-    constexpr uint32_t ID = idesc<COUT>();
-    const uint32_t lead = lane == 0;
-    if (L::SW && nmine > 0) ok = __all_sync(~0u, mbar_wait(wbar, 0));
-    const uint64_t bd0 = L::SW ? sdesc_sw128(su32(sm + L::W_OFF)) : sdesc(su32(sm + L::W_OFF), L::LBO_B, 128);
-    for (int k = 0; k < nmine && ok; ++k) {
+  } else if (warp >= MMA_WARP && warp < MMA_WARP + MMAS) {
+    constexpr uint32_t ID = idesc<COUT>() | (TRB ? 1u << 16 : 0u);
+    constexpr uint32_t BTAP = L::TAP / 16;  // 16-byte units of the weights: a tap, and a K step of 16
+    constexpr uint32_t BK = TRB ? COUT * 2 : (L::SW ? 2 : 2 * COUT);
+    const uint32_t lead = lane == 0, wb = su32(sm + L::W_OFF);
+    const uint64_t bd0 = TRB ? (COUT == 64 ? sdesc_mn_sw128(wb) : sdesc_mn_sw32(wb))
+                             : (L::SW ? sdesc_sw128(wb) : sdesc(wb, L::LBO_B, 128));
+    if (L::WTMA && nmine > 0) ok = __all_sync(~0u, mbar_wait(wbar, 0));
+    for (int k = warp - MMA_WARP; k < nmine && ok; k += MMAS) {
       const int b = k % NB, a = k & 1;
       ok = mbar_wait(pfull + b, (k / NB) & 1);
       if (ok && k >= 2) ok = mbar_wait(aempty + a, ((k - 2) >> 1) & 1);  // epilogue of item k - 2
@@ -466,24 +491,22 @@ __global__ void __launch_bounds__(TTHR, 1)
           // swizzled: rows (t / 3) * TPW + t % 3 + m; K step s2 is 32 bytes into the row
           const uint64_t ad = ad0 + (L::SW ? (uint32_t)(((t / 3) * TPW + t % 3) * 8 + 2 * s2)
                                            : (uint32_t)(((2 * s2) * TPR + t / 3) * TPW + t % 3));
-          const uint64_t bd = bd0 + (L::SW ? (uint32_t)(t * COUT * 8 + 2 * s2)
-                                           : (uint32_t)((t * L::CH + 2 * s2) * COUT));
-          umma(lead, acc, ad, bd, ID, (t | s2) != 0);
+          umma(lead, acc, ad, bd0 + (t * BTAP + s2 * BK), ID, (t | s2) != 0);
         }
       umma_commit(lead, pempty + b);
       umma_commit(lead, afull + a);
     }
     __syncwarp();
-  } else {  // epilogue warps 0-3
-    for (int k = 0; k < nmine && ok; ++k) {
-      const int a = k & 1;
+  } else if (warp < MMA_WARP) {  // epilogue: warps 0-3 even items, 4-7 odd ones
+    const int a = warp >> 2, quarter = warp & 3;
+    for (int k = a; k < nmine && ok; k += 2) {
       const size_t p0 = item_pixel(H, W, blockIdx.x + k * gridDim.x);
       uint4 mk[COUT / 8];
-      if (mask && y) load_mask<COUT>(mk, mask, p0, warp, lane);
+      if (mask && y) load_mask<COUT>(mk, mask, p0, quarter, lane);
       ok = __all_sync(~0u, mbar_wait(afull + a, (k >> 1) & 1));
       if (!ok) break;
       tc_fence_after();
-      epilogue<COUT>(tmem, (uint32_t)(a * L::ACC), p0, warp, lane, sbias, mask, mk, relu, y, yf);
+      epilogue<COUT>(tmem, (uint32_t)(a * L::ACC), p0, quarter, lane, sbias, mask, mk, relu, y, yf);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(aempty + a);
@@ -508,7 +531,11 @@ __global__ void __launch_bounds__(TTHR, 1)
 // K window of each of its taps lies in the single input row y + dy - 1, so a step copies the dY
 // segment and that one 130-pixel row (two tensor-map boxes, plus the periodic fix-ups), three deep.
 // Warps 0-3 read the three accumulators at the end and write the group's partial sums (reduced over
-// groups in a fixed order by a second kernel); warp 4 issues the MMAs; warp 5 copies.
+// groups in a fixed order by a second kernel).
+// Warps: 0-3 bias sums and epilogue, 4-6 the MMAs of taps dx = 0, 1, 2 (an accumulator each; one warp for all three
+// was slower than the tensor pipe), 7 copies, 8 wrapped columns.
+constexpr int WG_THREADS = 288, MMA_WARP = 4, LOAD_WARP = 7, FIX_WARP = 8;
+
 struct WgLay {
   static constexpr int NSTAGE = 3;
   static constexpr int DY = TPX * 128;                        // dY segment: 128 pixel rows of 128 B
@@ -524,12 +551,12 @@ struct WgLay {
 // once) the epilogue warps, idle until the accumulators are done, add up the staged dY segments.
 // Thread t (0 .. 127) sums channel t % DC over the pixels t / DC, t / DC + 128 / DC, ... of a segment
 // (DC = 64: 128-byte rows, chunk c at c ^ (j % 8); DC = 16: 32-byte rows, chunk c at c ^ ((j / 4) % 2)),
-// then releases the stage together with the MMAs (the stage's empty barrier counts both).
+// and each warp releases the stage together with the MMAs (the stage's empty barrier counts them all).
 template <int DC>
 __device__ __forceinline__ float dy_column_sum(const unsigned char* dyb, int t) {
   const int c = t % DC, j0 = t / DC;
   float s = 0.0f;
-#pragma unroll 8
+#pragma unroll 32
   for (int j = j0; j < TPX; j += 128 / DC) {
     const int chunk = DC == 64 ? ((c >> 3) ^ (j & 7)) : ((c >> 3) ^ ((j >> 2) & 1));
     s += __bfloat162float(*reinterpret_cast<const bf16*>(dyb + j * (DC * 2) + (chunk << 4) + (c & 7) * 2));
@@ -581,27 +608,38 @@ __device__ __forceinline__ bool wgrad_fix(unsigned char* sx, int stage_bytes, co
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;\n" ::: "memory"); }
 
-// the epilogue warps' share of a bias-gradient CTA: per segment, wait for its stage (one thread
-// waits, the outcome is broadcast), add it up, release it; returns false if a wait gave up
+// the epilogue warps' share of a bias-gradient CTA: per segment, wait for its stage, add it up, release it (each warp
+// for itself: a named barrier on both sides of a segment and one thread's wait took longer than its MMAs).  All four
+// warps come to the barrier at the end; returns, to all of them, whether no wait gave up.
 template <int DC, int NS>
 __device__ __forceinline__ bool bias_segments(const unsigned char* sm, int stage_bytes, uint64_t* full,
-                                              uint64_t* empty, int nmine, int tid, uint32_t* flag, float& acc) {
+                                              uint64_t* empty, int nmine, int tid, volatile uint32_t* gave_up,
+                                              float& acc) {
+  if (tid == 0) *gave_up = 0;
+  epi_sync();
   for (int k = 0; k < nmine; ++k) {
     const int b = k % NS;
-    if (tid == 0) *flag = mbar_wait(full + b, (k / NS) & 1) ? 1u : 0u;
-    epi_sync();
-    if (!*flag) return false;
+    if (!__all_sync(~0u, mbar_wait(full + b, (k / NS) & 1))) {
+      *gave_up = 1;
+      break;
+    }
     acc += dy_column_sum<DC>(sm + b * stage_bytes, tid);
-    epi_sync();
-    if (tid == 0) mbar_arrive(empty + b);
+    __syncwarp();
+    if (tid % 32 == 0) mbar_arrive(empty + b);
   }
-  return true;
+  epi_sync();
+  return *gave_up == 0;
 }
 
-// the CTA's partial bias sums, once every MMA is done (stage 0 serves as scratch): bpart[group][co]
+// the CTA's partial bias sums, once every MMA is done (stage 0 serves as scratch): bpart[group][co].
+// Returns, to all four warps, whether every thread came with ok.
 template <int DC>
-__device__ __forceinline__ void bias_store(unsigned char* sm, float acc, int tid, float* bpart) {
+__device__ __forceinline__ bool bias_store(unsigned char* sm, bool ok, float acc, int tid, volatile uint32_t* gave_up,
+                                           float* bpart) {
   float* red = reinterpret_cast<float*>(sm);
+  if (!ok) *gave_up = 1;
+  epi_sync();
+  if (*gave_up) return false;
   red[tid] = acc;
   epi_sync();
   if (tid < DC) {
@@ -609,15 +647,10 @@ __device__ __forceinline__ void bias_store(unsigned char* sm, float acc, int tid
     for (int r = 0; r < 128 / DC; ++r) t += red[r * DC + tid];
     bpart[(size_t)blockIdx.x * DC + tid] = t;
   }
+  return true;
 }
 
-// MN-major, 128-byte swizzle: 8-pixel groups of 128-byte rows 1024 bytes apart (one 64-wide atom in MN)
-__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-
-__global__ void __launch_bounds__(TTHR)
+__global__ void __launch_bounds__(WG_THREADS)
     conv_wgrad_tc_kernel(int H, int W, int segs_per_group, const bf16* __restrict__ x, float* partial, float* bpart,
                          int* err,
                          const __grid_constant__ CUtensorMap dymap, const __grid_constant__ CUtensorMap xmap) {
@@ -625,7 +658,7 @@ __global__ void __launch_bounds__(TTHR)
   constexpr int NS = L::NSTAGE;
   constexpr uint32_t COLS = 256;  // three 64-column accumulators
   extern __shared__ __align__(1024) unsigned char sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF);
   uint64_t *tma = bars, *full = bars + NS, *empty = bars + 2 * NS, *done = bars + 3 * NS;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + L::TSLOT_OFF);
@@ -640,9 +673,9 @@ __global__ void __launch_bounds__(TTHR)
     for (int b = 0; b < NS; ++b) {
       mbar_init(tma + b, 1);
       mbar_init(full + b, 1);
-      mbar_init(empty + b, bias ? 2 : 1);  // the MMAs (and the bias sums) release a stage
+      mbar_init(empty + b, bias ? 7 : 3);  // the three MMA warps (and the four of the bias sums) release a stage
     }
-    mbar_init(done, 1);
+    mbar_init(done, 3);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   pdl_wait_and_trigger();
@@ -670,10 +703,10 @@ __global__ void __launch_bounds__(TTHR)
     }
   } else if (warp == FIX_WARP) {
     ok = wgrad_fix<64, NS>(sm + L::DY, L::STAGE, x, H, W, seg0, nmine, dyr, lane, tma, full);
-  } else if (warp == MMA_WARP) {
+  } else if (warp >= MMA_WARP && warp < MMA_WARP + 3) {
     constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((64u >> 3) << 17) |
                             ((64u >> 4) << 24);
-    const uint32_t lead = lane == 0;
+    const uint32_t lead = lane == 0, dx = warp - MMA_WARP;
     for (int k = 0; k < nmine && ok; ++k) {
       const int b = k % NS;
       ok = __all_sync(~0u, mbar_wait(full + b, (k / NS) & 1));
@@ -682,9 +715,7 @@ __global__ void __launch_bounds__(TTHR)
       const uint64_t dyd = sdesc_mn_sw128(su32(sm + b * L::STAGE)), xd = dyd + (uint32_t)(L::DY >> 4);
 #pragma unroll
       for (int s2 = 0; s2 < TPX / 16; ++s2)
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx)
-          umma(lead, tmem + 64u * dx, dyd + 128u * s2, xd + (8u * dx + 128u * s2), ID, (k | s2) != 0);
+        umma(lead, tmem + 64u * dx, dyd + 128u * s2, xd + (8u * dx + 128u * s2), ID, (k | s2) != 0);
       umma_commit(lead, empty + b);
     }
     if (ok) umma_commit(lead, done);
@@ -693,8 +724,8 @@ __global__ void __launch_bounds__(TTHR)
     float bacc = 0.0f;
     if (bias) ok = bias_segments<64, NS>(sm, L::STAGE, full, empty, nmine, tid, tslot + 1, bacc);
     ok = ok && (nmine == 0 || mbar_wait(done, 0));
-    if (ok && bias) bias_store<64>(sm, bacc, tid, bpart);
-    if (ok && nmine > 0) {
+    if (bias) ok = bias_store<64>(sm, ok, bacc, tid, tslot + 1, bpart);
+    if (__all_sync(~0u, ok) && nmine > 0) {
       tc_fence_after();
       for (int dx = 0; dx < 3; ++dx) {
         uint32_t raw[64];
@@ -702,14 +733,22 @@ __global__ void __launch_bounds__(TTHR)
         for (int q = 0; q < 4; ++q)
           tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + 64u * dx + 16u * q, raw + 16 * q);
         tmem_wait_ld();
-        if (lane < 16) {  // lanes 0-15 of warp w hold output channels 16 w .. 16 w + 15
-          const int co = 16 * warp + lane;
-          float4* dst =
-              reinterpret_cast<float4*>(partial + (((size_t)blockIdx.x * 9 + 3 * dyr + dx) * 64 + co) * 64);
+        // lanes 0-15 of warp w hold output channels 16 w .. 16 w + 15, 256 bytes each; two transposes turn a store
+        // from 16 bytes of 16 rows into 128 bytes of two
+        float* tap = partial + ((size_t)blockIdx.x * 9 + 3 * dyr + dx) * 64 * 64;
 #pragma unroll
-          for (int q = 0; q < 16; ++q)
-            dst[q] = make_float4(__uint_as_float(raw[4 * q]), __uint_as_float(raw[4 * q + 1]),
-                                 __uint_as_float(raw[4 * q + 2]), __uint_as_float(raw[4 * q + 3]));
+        for (int h = 0; h < 2; ++h) {
+          uint4 o[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            o[q] = make_uint4(raw[32 * h + 4 * q], raw[32 * h + 4 * q + 1], raw[32 * h + 4 * q + 2],
+                              raw[32 * h + 4 * q + 3]);
+          transpose_chunks(o, lane);
+          if (lane < 16) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              *reinterpret_cast<uint4*>(tap + (16 * warp + (lane & 8) + q) * 64 + 32 * h + 4 * (lane & 7)) = o[q];
+          }
         }
       }
     }
@@ -744,14 +783,8 @@ struct Wg16Lay {
   static_assert((XC == 16 && DC == 64) || (XC == 64 && DC == 16), "one 16-channel and one 64-channel side");
 };
 
-// MN-major, 32-byte swizzle: 8-pixel groups of 32-byte rows 256 bytes apart (one 16-wide atom in MN)
-__device__ __forceinline__ uint64_t sdesc_mn_sw32(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
-}
-
 template <int XC, int DC>
-__global__ void __launch_bounds__(TTHR)
+__global__ void __launch_bounds__(WG_THREADS)
     conv_wgrad16_tc_kernel(int H, int W, int segs_per_group, const bf16* __restrict__ x, float* partial,
                            float* bpart, int* err,
                            const __grid_constant__ CUtensorMap dymap, const __grid_constant__ CUtensorMap xmap) {
@@ -760,7 +793,7 @@ __global__ void __launch_bounds__(TTHR)
   constexpr uint32_t COLS = 64;  // three 16-column accumulators
   constexpr int XROW = XC * 2;   // bytes of one input pixel row
   extern __shared__ __align__(1024) unsigned char sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF);
   uint64_t *tma = bars, *full = bars + NS, *empty = bars + 2 * NS, *done = bars + 3 * NS;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + L::TSLOT_OFF);
@@ -775,9 +808,9 @@ __global__ void __launch_bounds__(TTHR)
     for (int b = 0; b < NS; ++b) {
       mbar_init(tma + b, 1);
       mbar_init(full + b, 1);
-      mbar_init(empty + b, bias ? 2 : 1);  // the MMAs (and the bias sums) release a stage
+      mbar_init(empty + b, bias ? 7 : 3);  // the three MMA warps (and the four of the bias sums) release a stage
     }
-    mbar_init(done, 1);
+    mbar_init(done, 3);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   pdl_wait_and_trigger();
@@ -805,11 +838,11 @@ __global__ void __launch_bounds__(TTHR)
     }
   } else if (warp == FIX_WARP) {
     ok = wgrad_fix<XC, NS>(sm + L::DY, L::STAGE, x, H, W, seg0, nmine, dyr, lane, tma, full);
-  } else if (warp == MMA_WARP) {
+  } else if (warp >= MMA_WARP && warp < MMA_WARP + 3) {
     // BF16 x BF16 -> F32, both operands MN-major (transpose bits 15, 16), N = 16, M = 64
     constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((16u >> 3) << 17) |
                             ((64u >> 4) << 24);
-    const uint32_t lead = lane == 0;
+    const uint32_t lead = lane == 0, dx = warp - MMA_WARP;
     for (int k = 0; k < nmine && ok; ++k) {
       const int b = k % NS;
       ok = __all_sync(~0u, mbar_wait(full + b, (k / NS) & 1));
@@ -820,9 +853,7 @@ __global__ void __launch_bounds__(TTHR)
       const uint64_t da = sdesc_mn_sw128(XC == 16 ? dyb : xb), db = sdesc_mn_sw32(XC == 16 ? xb : dyb);
 #pragma unroll
       for (int s2 = 0; s2 < TPX / 16; ++s2)
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx)
-          umma(lead, tmem + 16u * dx, da + (128u * s2 + (XC == 16 ? 0u : 8u * dx)),
+        umma(lead, tmem + 16u * dx, da + (128u * s2 + (XC == 16 ? 0u : 8u * dx)),
                db + (32u * s2 + (XC == 16 ? 2u * dx : 0u)), ID, (k | s2) != 0);
       umma_commit(lead, empty + b);
     }
@@ -832,7 +863,7 @@ __global__ void __launch_bounds__(TTHR)
     float bacc = 0.0f;
     if (bias) ok = bias_segments<DC, NS>(sm, L::STAGE, full, empty, nmine, tid, tslot + 1, bacc);
     ok = ok && (nmine == 0 || mbar_wait(done, 0));
-    if (ok && bias) bias_store<DC>(sm, bacc, tid, bpart);
+    if (bias) ok = bias_store<DC>(sm, ok, bacc, tid, tslot + 1, bpart);
     if (ok && nmine > 0) {
       tc_fence_after();
       uint32_t raw[48];
@@ -888,10 +919,10 @@ EncodeTiled encoder() {
   return fn;
 }
 
-cudaLaunchConfig_t pdl_config(dim3 grid, size_t smem, cudaStream_t st) {
+cudaLaunchConfig_t pdl_config(dim3 grid, int threads, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(TTHR);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   return cfg;
@@ -904,10 +935,10 @@ void pdl_attr(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
   cfg.numAttrs = 1;
 }
 
-template <int CIN, int COUT>
+template <int CIN, int COUT, bool TRB>
 cudaError_t tc_launch(int H, int W, const void* x, const void* w, const float* b, const void* mask, int relu, void* y,
                       float* yf, cudaStream_t st) {
-  using L = TcLay<CIN, COUT>;
+  using L = TcLay<CIN, COUT, TRB>;
   static int ready[32] = {0};
   static int grid_max[32] = {0};
   static int* err[32] = {nullptr};
@@ -916,10 +947,10 @@ cudaError_t tc_launch(int H, int W, const void* x, const void* w, const float* b
   if (e != cudaSuccess) return e;
   if (dev >= 32) return cudaErrorInvalidDevice;
   if (!ready[dev]) {
-    e = cudaFuncSetAttribute(conv_fwd_tc_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::BYTES);
+    e = cudaFuncSetAttribute(conv_fwd_tc_kernel<CIN, COUT, TRB>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::BYTES);
     if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv_fwd_tc_kernel<CIN, COUT>, TTHR, L::BYTES);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv_fwd_tc_kernel<CIN, COUT, TRB>, FWD_THREADS, L::BYTES);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -934,26 +965,16 @@ cudaError_t tc_launch(int H, int W, const void* x, const void* w, const float* b
   alignas(64) CUtensorMap xmap, wmap;
   memset(&wmap, 0, sizeof wmap);
   CUresult r;
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
   if (L::SW) {
     // input (64 channels = one 128-byte row, W, H), box 64 x 130 x 3, 128-byte swizzle
-    const cuuint32_t estr[3] = {1, 1, 1};
     const cuuint64_t dims[3] = {(cuuint64_t)CIN, (cuuint64_t)W, (cuuint64_t)H};
     const cuuint64_t strides[2] = {(cuuint64_t)CIN * 2, (cuuint64_t)W * CIN * 2};
     const cuuint32_t box[3] = {(cuuint32_t)CIN, (cuuint32_t)TPW, (cuuint32_t)TPR};
     r = enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    // weights [c_out][tap][c_in] as (c_in, tap, c_out): the box (64, 1, C_out) of tap t lands as C_out
-    // rows of 128 bytes, 128-byte swizzle (the B operand of tap t)
-    const cuuint64_t wdims[3] = {(cuuint64_t)CIN, 9, (cuuint64_t)COUT};
-    const cuuint64_t wstrides[2] = {(cuuint64_t)CIN * 2, (cuuint64_t)9 * CIN * 2};
-    const cuuint32_t wbox[3] = {(cuuint32_t)CIN, 1, (cuuint32_t)COUT};
-    r = enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w), wdims, wstrides, wbox, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else {  // (8 channels of a chunk, W, H, chunk): the box 8 x 130 x 3 x CH lands chunk-major
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
     const cuuint64_t dims[4] = {8, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)L::CH};
     const cuuint64_t strides[3] = {(cuuint64_t)CIN * 2, (cuuint64_t)W * CIN * 2, 16};
     const cuuint32_t box[4] = {8, (cuuint32_t)TPW, (cuuint32_t)TPR, (cuuint32_t)L::CH};
@@ -962,12 +983,24 @@ cudaError_t tc_launch(int H, int W, const void* x, const void* w, const float* b
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
   if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  if (L::WTMA) {
+    // weights [N][tap][K] as (K, tap, N), or transposed [K][tap][N] as (N, tap, K): one tap per box, its rows
+    // swizzled over their own length (128 or 32 bytes)
+    constexpr int INNER = TRB ? COUT : CIN, OUTER = TRB ? CIN : COUT;
+    const cuuint64_t dims[3] = {(cuuint64_t)INNER, 9, (cuuint64_t)OUTER};
+    const cuuint64_t strides[2] = {(cuuint64_t)INNER * 2, (cuuint64_t)9 * INNER * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)INNER, 1, (cuuint32_t)OUTER};
+    r = enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, INNER == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  }
   const int nitems = H * (W / TPX);
   const int grid = nitems < grid_max[dev] ? nitems : grid_max[dev];
-  cudaLaunchConfig_t cfg = pdl_config(dim3(grid), L::BYTES, st);
+  cudaLaunchConfig_t cfg = pdl_config(dim3(grid), FWD_THREADS, L::BYTES, st);
   cudaLaunchAttribute attr[1];
   pdl_attr(cfg, attr);
-  return cudaLaunchKernelEx(&cfg, conv_fwd_tc_kernel<CIN, COUT>, H, W, (const bf16*)x, (const bf16*)w, b,
+  return cudaLaunchKernelEx(&cfg, conv_fwd_tc_kernel<CIN, COUT, TRB>, H, W, (const bf16*)x, (const bf16*)w, b,
                             (const bf16*)mask, relu, (bf16*)y, yf, err[dev], xmap, wmap);
 }
 
@@ -1000,7 +1033,7 @@ cudaError_t wg64_launch(int H, int W, const void* x, const void* dy, float* part
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   const int nseg = H * (W / TPX), groups = (nseg + segs_per_group - 1) / segs_per_group;
-  cudaLaunchConfig_t cfg = pdl_config(dim3(groups, 3), WgLay::BYTES, st);
+  cudaLaunchConfig_t cfg = pdl_config(dim3(groups, 3), WG_THREADS, WgLay::BYTES, st);
   cudaLaunchAttribute attr[1];
   pdl_attr(cfg, attr);
   return cudaLaunchKernelEx(&cfg, conv_wgrad_tc_kernel, H, W, segs_per_group, (const bf16*)x, partial, bpart, err[dev],
@@ -1042,7 +1075,7 @@ cudaError_t wg16_launch(int H, int W, const void* x, const void* dy, float* part
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   const int nseg = H * (W / TPX), groups = (nseg + segs_per_group - 1) / segs_per_group;
-  cudaLaunchConfig_t cfg = pdl_config(dim3(groups, 3), L::BYTES, st);
+  cudaLaunchConfig_t cfg = pdl_config(dim3(groups, 3), WG_THREADS, L::BYTES, st);
   cudaLaunchAttribute attr[1];
   pdl_attr(cfg, attr);
   return cudaLaunchKernelEx(&cfg, conv_wgrad16_tc_kernel<XC, DC>, H, W, segs_per_group, (const bf16*)x, partial, bpart,
@@ -1053,9 +1086,16 @@ cudaError_t wg16_launch(int H, int W, const void* x, const void* dy, float* part
 
 cudaError_t conv_fwd_tc(int H, int W, int cin, int cout, const void* x, const void* w, const float* b,
                         const void* mask, int relu, void* y, float* yf, cudaStream_t st) {
-  if (cin == 16) return tc_launch<16, 64>(H, W, x, w, b, mask, relu, y, yf, st);
-  if (cout == 64) return tc_launch<64, 64>(H, W, x, w, b, mask, relu, y, yf, st);
-  return tc_launch<64, 16>(H, W, x, w, b, mask, relu, y, yf, st);
+  if (cin == 16) return tc_launch<16, 64, false>(H, W, x, w, b, mask, relu, y, yf, st);
+  if (cout == 64) return tc_launch<64, 64, false>(H, W, x, w, b, mask, relu, y, yf, st);
+  return tc_launch<64, 16, false>(H, W, x, w, b, mask, relu, y, yf, st);
+}
+
+cudaError_t conv_bwd_data_tc(int H, int W, int cin, int cout, const void* dy, const void* w, const void* mask, void* dx,
+                             cudaStream_t st) {
+  if (cin == 16) return tc_launch<64, 16, true>(H, W, dy, w, nullptr, mask, 0, dx, nullptr, st);
+  if (cout == 64) return tc_launch<64, 64, true>(H, W, dy, w, nullptr, mask, 0, dx, nullptr, st);
+  return tc_launch<16, 64, true>(H, W, dy, w, nullptr, mask, 0, dx, nullptr, st);
 }
 
 cudaError_t conv_wgrad_tc(int H, int W, int cin, int cout, const void* x, const void* dy, float* partial, float* bpart,

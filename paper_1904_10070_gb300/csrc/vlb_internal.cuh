@@ -219,6 +219,9 @@ size_t conv_wgrad_workspace_bytes(int H, int W, int cin, int cout);
 // the forward on the tcgen05 tensor cores (vlb_conv_tc.cu)
 cudaError_t conv_fwd_tc(int H, int W, int cin, int cout, const void* x, const void* w, const float* b,
                         const void* mask, int relu, void* y, float* yf, cudaStream_t st);
+// dX = mask * (transposed convolution of dY with w[co][tap][ci]), (cin, cout) those of the layer
+cudaError_t conv_bwd_data_tc(int H, int W, int cin, int cout, const void* dy, const void* w, const void* mask, void* dx,
+                             cudaStream_t st);
 // partial[group][tap][co][ci] of a weight gradient on tcgen05 (vlb_conv_tc.cu; (c_in, c_out) = (64, 64),
 // (16, 64) or (64, 16)); group g covers row segments (128 pixels) g * segs_per_group ..  With bpart,
 // also bpart[group][co] = the group's sum of dY[p][co] (the bias gradient's partials).

@@ -35,7 +35,7 @@ class SurrogateNet:
         self.H, self.W = H, W
         rng = np.random.default_rng(seed)
         dev = "cuda"
-        self.w32, self.b32, self.wb, self.wf = [], [], [], []
+        self.w32, self.b32, self.wb = [], [], []
         self.mw, self.vw, self.mb, self.vb, self.dw, self.db = [], [], [], [], [], []
         for li, (cin, cout) in enumerate(LAYERS):
             fan_in = 9 * (N_IN if li == 0 else cin)
@@ -50,7 +50,6 @@ class SurrogateNet:
             self.b32.append(torch.zeros(cout, dtype=torch.float32, device=dev))
             self.wb.append(torch.empty((cout, 3, 3, cin), dtype=torch.bfloat16, device=dev))
             vlb.vlb_to_bf16(t.numel(), t, self.wb[-1], _stream())
-            self.wf.append(torch.empty((cin, 3, 3, cout), dtype=torch.bfloat16, device=dev))
             for lst, shape in ((self.mw, t.shape), (self.vw, t.shape), (self.dw, t.shape)):
                 lst.append(torch.zeros(shape, dtype=torch.float32, device=dev))
             for lst in (self.mb, self.vb, self.db):
@@ -90,11 +89,9 @@ class SurrogateNet:
             vlb.vlb_conv3x3_bwd_weight(self.H, self.W, cin, cout, self.acts[li], dz, self.dw[li], self.db[li],
                                        self.wg_ws, st)
             if li > 0:
-                vlb.vlb_conv3x3_flip(cin, cout, self.wb[li], self.wf[li], st)
                 nxt = self.dz[li % 2]
-                # dZ_{l-1} = (W_l^T dZ_l) * (A_{l-1} > 0): the forward kernel with flipped weights and mask
-                vlb.vlb_conv3x3_fwd(self.H, self.W, cout, cin, dz, self.wf[li], None, self.acts[li], 0, nxt, None,
-                                    st)
+                # dZ_{l-1} = (W_l^T dZ_l) * (A_{l-1} > 0)
+                vlb.vlb_conv3x3_bwd_data(self.H, self.W, cin, cout, dz, self.wb[li], self.acts[li], nxt, st)
                 dz = nxt
 
     def adam(self, lr: float):

@@ -26,7 +26,7 @@ EXPORTS = ["vlb_workspace_bytes", "vlb_max_stable_dt", "vlb_create", "vlb_destro
            "vlb_interface_length", "vlb_state_device", "vlb_steps_done", "vlb_last_error",
            "vlb_step_noalloc", "vlb_ensemble_workspace_bytes", "vlb_ensemble_create", "vlb_ensemble_step",
            "vlb_ensemble_member", "vlb_ensemble_tile_rows", "vlb_get_snapshot", "vlb_set_snapshot",
-           "vlb_conv3x3_fwd", "vlb_conv3x3_flip", "vlb_conv3x3_wgrad_workspace_bytes",
+           "vlb_conv3x3_fwd", "vlb_conv3x3_flip", "vlb_conv3x3_bwd_data", "vlb_conv3x3_wgrad_workspace_bytes",
            "vlb_conv3x3_bwd_weight", "vlb_reduce_workspace_bytes", "vlb_surrogate_norm", "vlb_surrogate_features", "vlb_surrogate_targets",
            "vlb_surrogate_apply", "vlb_snapshot_compare", "vlb_channel_sums", "vlb_mse_loss", "vlb_adam_step",
            "vlb_adam_step_many", "vlb_to_bf16", "vlb_conv_status", "vlb_test_raise_flag", "vlb_surrogate_workspace_bytes", "vlb_surrogate_create",
@@ -138,6 +138,7 @@ def lib() -> ctypes.CDLL:
     L.vlb_test_raise_flag.argtypes, L.vlb_test_raise_flag.restype = [P, I32], I32
     L.vlb_conv3x3_fwd.argtypes = [I32, I32, I32, I32, P, P, P, P, I32, P, P, P]
     L.vlb_conv3x3_flip.argtypes = [I32, I32, P, P, P]
+    L.vlb_conv3x3_bwd_data.argtypes, L.vlb_conv3x3_bwd_data.restype = [I32, I32, I32, I32, P, P, P, P, P], I32
     L.vlb_conv3x3_wgrad_workspace_bytes.argtypes = [I32, I32, I32, I32]
     L.vlb_conv3x3_wgrad_workspace_bytes.restype = S
     L.vlb_conv3x3_bwd_weight.argtypes = [I32, I32, I32, I32, P, P, P, P, P, S, P]
@@ -313,6 +314,11 @@ def vlb_conv3x3_fwd(H, W, cin, cout, x, w, bias, mask, relu, y_bf16, y_f32, stre
 
 def vlb_conv3x3_flip(cin, cout, w, w_flipped, stream):
     _check(lib().vlb_conv3x3_flip(cin, cout, _ptr(w), _ptr(w_flipped), ctypes.c_void_p(stream)))
+
+
+def vlb_conv3x3_bwd_data(H, W, cin, cout, dy, w, mask, dx, stream):
+    _check(lib().vlb_conv3x3_bwd_data(H, W, cin, cout, _ptr(dy), _ptr(w), _ptr(mask), _ptr(dx),
+                                      ctypes.c_void_p(stream)))
 
 
 def vlb_conv3x3_wgrad_workspace_bytes(H, W, cin, cout) -> int:
