@@ -147,14 +147,14 @@ vlb_status vlb_test_raise_flag(vlb_handle* h, int32_t value);
 vlb_status vlb_get_fields(vlb_handle* h, double* rho, double* u_th, double* u_ph, double* phi,
                           double* mu);
 
-/* Conserved totals and diagnostics, reduced in FP64 on the GPU:
+/* Conserved totals and diagnostics, reduced on the GPU in FP64 (FP32 states: in float pairs of about 48 bits):
  * out[0] = sum n sqrt(g) dtheta dvarphi, out[1] = sum phi sqrt(g) dtheta dvarphi,
  * out[2] = Psi (Eq. Landau, central differences), out[3] = max |u|.  Synchronous. */
 vlb_status vlb_get_totals(vlb_handle* h, double out[4]);
 
 /* Total interface length L_I (Sec. 4: every neighbour pair with phi phi' < 0 adds the shared
- * edge, r dtheta across varphi and (R + r cos theta_{q+1/2}) dvarphi across theta), reduced in
- * FP64 on the GPU; the domain length is L_d = 4 pi^2 r R / L_I (Eq. cart_scaling_L0).  Synchronous. */
+ * edge, r dtheta across varphi and (R + r cos theta_{q+1/2}) dvarphi across theta), sign changes counted
+ * on the GPU and weighted in FP64; the domain length is L_d = 4 pi^2 r R / L_I (Eq. cart_scaling_L0).  Synchronous. */
 vlb_status vlb_interface_length(vlb_handle* h, double* out);
 
 /* Structure-factor length L_S = 2 pi sum S(k) / sum |k| S(k) over k != 0 (a Fourier measure of the
@@ -186,8 +186,8 @@ vlb_status vlb_steps_done(const vlb_handle* h, int64_t* out);
  * stages are read back from L2 and only the state itself crosses HBM; it needs an FP32 UW3
  * explicit grid with N_theta a multiple of 16 and >= 176 and N_phi a multiple of 32 (VLB_ERR_ARG
  * otherwise).  VLB_SCHED_AUTO (the default) takes the per-stage launches: the stage is bound by
- * instruction issue rather than HBM, and the wavefront's per-tile dependency waits cost more than the
- * HBM traffic it saves (measured on GB300: 0.469 against 0.236 ms per step at 1024 x 2048).
+ * latency rather than HBM, and the wavefront's per-tile dependency waits cost more than the
+ * HBM traffic it saves (measured on GB300: 0.498 against 0.204 ms per step at 1024 x 2048).
  * vlb_get_schedule writes the schedule vlb_step takes (STAGES or WAVE). */
 enum { VLB_SCHED_AUTO = 0, VLB_SCHED_STAGES = 1, VLB_SCHED_WAVE = 2 };
 vlb_status vlb_set_schedule(vlb_handle* h, int32_t schedule);
@@ -435,7 +435,8 @@ vlb_status vlb_surrogate_stats(const vlb_handle* sur, int64_t out[4]);
  * resolution).  diag_every is ignored; nothing is read back.
  *
  * The two intermediate Runge-Kutta states and the row coefficients live in one file-scope device
- * array of VLB_NOALLOC_SCRATCH_BYTES that every device loading the library holds until exit; the
+ * array of VLB_NOALLOC_SCRATCH_BYTES (the row table of the FP32 stage in a second, smaller one) that every device
+ * loading the library holds until exit; the
  * call needs 2 * (17 or 18) * stride * element-size bytes plus the tables, and a larger grid is
  * rejected with VLB_ERR_ARG (about 170 k nodes in FP32, 90 k in FP64), and so is a stride beyond
  * that limit, before any size arithmetic.  The first call on each device does the one-time set-up:

@@ -20,7 +20,7 @@
 // one item overlap the MMAs of the next.  Hand-offs are mbarriers and every wait is bounded.
 //
 // At 256 x 512 an SM has 6.7 items; the MMAs keep the tensor pipe busy for 0.6 us of the 1.4 us an item takes.  What
-// counted, forward / masked us of a 64 -> 64 layer: start 14.3 / 20.0; mask loaded early, whole pixels stored, wrapped
+// counted, forward / masked us of a 64 -> 64 layer: 14.3 / 20.0 at first; mask loaded early, whole pixels stored, wrapped
 // columns loaded ahead 14.7 / 16.5; descriptors kept warp-uniform and a second set of epilogue warps 14.3 / 14.6.  A ring
 // of single rows (17 KB an item instead of 50) measured 16.1 / 16.7.
 #include <cuda_bf16.h>
