@@ -30,7 +30,7 @@ constexpr int kAxiThreads = 256;
 
 template <typename T>
 struct AxiConst {
-  T v[4], K[4][4], ww[4][4];
+  T v[4], K[4][4], ww[4][4], fix;  // fix: of node_velocity
 };
 
 // everything a row needs, times dt where it multiplies a rate
@@ -125,8 +125,7 @@ __host__ __device__ __forceinline__ int axi_pitch(int rows, int H) {
   return p;
 }
 
-// FP32 UW3 columns read the handle's row table (rounded once from FP64, which halves the error of coefficients
-// multiplied together in FP32); the others form an AxiRow from the coefficient arrays
+// FP32 UW3 columns read the handle's row table; the others form an AxiRow from the coefficient arrays
 template <typename T, int ADV>
 __host__ __device__ constexpr bool row_table() { return sizeof(T) == 4 && ADV == VLB_UW3; }
 
@@ -185,6 +184,7 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
   const bool pos = i >= 2;
   const T vi = ac.v[i], K0 = ac.K[i][0], K1 = ac.K[i][1], K2 = ac.K[i][2], K3 = ac.K[i][3];
   const T itau = a.inv_tau * a.dt, av = pos ? vi : -vi;
+  const T ivb = T(1) / ac.v[3], iva = T(1) / ac.v[2];
   for (int n = 0; n < steps && ok; ++n) {
 #pragma unroll 1
     for (int st = 0; st < 3; ++st, ++stage) {
@@ -233,12 +233,12 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
           jm = rv.jm;
         }
         if (i == 0 && (it >> 2) <= R + 1) {
-          const T inv_n = node_recip(a.n0 + dn);
+          const T inv_n = node_recip(vadd(a.n0, dn));
           const T cubic = p0 * (T(1) - p0 * p0) + (T(1) - T(3) * p0 * p0) * lo;  // at hi + lo, first order in lo
           s_dn[row] = dn;
           s_in[row] = inv_n;
-          s_ut[row] = mt * inv_n;
-          s_up[row] = mp * inv_n;
+          s_ut[row] = node_velocity(mt, inv_n, ac.fix);
+          s_up[row] = node_velocity(mp, inv_n, ac.fix);
           s_mu[row] = -a.A * cubic - kt * (jp * dN - jm * dS);
         }
       }
@@ -258,8 +258,10 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
         T g[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) g[k] = in[k * P + H + row];
+        // n / tau from the density that was inverted for u: n0 / tau rounded on its own would be off by the same amount
+        // at every node and stage, and the momentum would drift by it
         const T usq = ut * ut + up * up, c0 = T(1) - T(0.5) * usq, hu = T(-0.5) * usq;
-        const T dntau = dn * itau, ntau = a.n0 * itau + dntau, ai = vi * ut;
+        const T dntau = vmul(dn, itau), ntau = vmul(vadd(a.n0, dn), itau), ai = vmul(vi, ut);
         const bool big = i == 0 || i == 3;
         const T em = RT ? rt[E_EM] : rv.em, ne = RT ? (big ? rt[E_NEB] : rt[E_NEA]) : av * rv.ed;
         const T ci = dntau + a.n0 * (vi * (em + Ft) + ne);
@@ -270,12 +272,13 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
         hb = pos ? hb : -hb;
         ha = pos ? ha : -ha;
         T tf, tn, tm, td;
-        if constexpr (RT) {
+        if constexpr (RT) {  // tm: the sum of the four taps, v_i (E + Gamma)
           const T* t = rt + E_TH + (big ? 0 : 8);
           tf = t[pos ? TAP_FARP : TAP_FARN];
           tn = t[pos ? TAP_NEARP : TAP_NEARN];
-          tm = t[TAP_MID];
           td = t[pos ? TAP_DOWNP : TAP_DOWNN];
+          const T gv = big ? gb2 * ivb : ga2 * iva;
+          tm = vadd(vfma(vi, em, ne), pos ? gv : -gv);
         } else {
           tf = -av * (pos ? rv.w[0] : rv.w[4]);
           tn = T(6) * av * (pos ? rv.w[1] : rv.w[3]);
@@ -290,7 +293,10 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
           T acc;
           if (ADV == VLB_UW3) {
             const int s = pos ? 1 : -1;
-            acc = (tf * fk[-2 * s] + tn * fk[-s]) + (tm * gk + td * fk[s]);
+            if constexpr (RT)  // the taps nearly cancel: on differences the products stay small, and so do their roundings
+              acc = vfma(tm, gk, vfma(tn, vsub(fk[-s], gk), vfma(tf, vsub(fk[-2 * s], gk), vmul(td, vsub(fk[s], gk)))));
+            else
+              acc = (tf * fk[-2 * s] + tn * fk[-s]) + (tm * gk + td * fk[s]);
           } else {  // WENO5 reconstructs the full J f; its rows of J come from the coefficient table
             const T fref = a.n0 * ac.ww[i][j];
             T x[7];
@@ -306,9 +312,9 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
           const T dvp = (ac.K[j][0] * (hb * fi[0]) + ac.K[j][1] * (ha * fi[P])) -
                         (ac.K[j][2] * (ha * fi[2 * P]) + ac.K[j][3] * (hb * fi[3 * P]));
           acc += (((j == 0 || j == 3) ? gb2 : ga2) - Ft) * dvt + dvp;
-          const T xi = ai + ac.v[j] * up;
-          const T pm1 = xi * (c0 + xi * (T(0.5) + xi * T(1.0 / 6.0))) + hu;
-          acc += ac.ww[i][j] * (ntau * pm1 + ci) - itau * gk;
+          const T xi = vfma(ac.v[j], up, ai);
+          const T pm1 = vfma(xi, vfma(xi, vfma(xi, T(1.0 / 6.0), T(0.5)), c0), hu);
+          acc = vadd(acc, vfma(-itau, gk, vmul(ac.ww[i][j], vfma(ntau, pm1, ci))));
           const T g0 = u0[(k0 + j) * P];
           o[j] = st == 0 ? gk + acc : g0 + b * ((gk - g0) + acc);
         }
@@ -393,8 +399,11 @@ __global__ void __launch_bounds__(512) axi16_kernel(StageArgs<float> a, const __
   const float* rt = a.rows + (int64_t)axi_wrap(r0 + grp - 1, nt) * kRowTable;
   const bool bi = i == 0 || i == 3, bj = j == 0 || j == 3;
   const float* t = rt + E_TH + (bi ? 0 : 8);
-  const float tf = t[pos ? TAP_FARP : TAP_FARN], tn = t[pos ? TAP_NEARP : TAP_NEARN], tm = t[TAP_MID];
+  const float tf = t[pos ? TAP_FARP : TAP_FARN], tn = t[pos ? TAP_NEARP : TAP_NEARN];
   const float td = t[pos ? TAP_DOWNP : TAP_DOWNN];
+  // the sum of the four taps, v_i (E + Gamma)
+  const float gv = bi ? rt[E_GBB] / ac.v[3] : rt[E_GAA] / ac.v[2];
+  const float ts = __fadd_rn(__fmaf_rn(vi, rt[E_EM], bi ? rt[E_NEB] : rt[E_NEA]), pos ? gv : -gv);
   const float gvj = bj ? rt[E_GBB] : rt[E_GAA], nv = a.n0 * vi, ce = a.n0 * (vi * rt[E_EM] + (bi ? rt[E_NEB] : rt[E_NEA]));
   const float lt = rt[E_LT], xn = rt[E_XN], xs = rt[E_XS], kt = rt[E_KT], jp = rt[E_JP], jm = rt[E_JM];
   const float avj = bj ? ac.v[3] : ac.v[2];
@@ -446,7 +455,8 @@ __global__ void __launch_bounds__(512) axi16_kernel(StageArgs<float> a, const __
       dn += __shfl_xor_sync(0xffffffffu, dn, 4);
       mt += __shfl_xor_sync(0xffffffffu, mt, 4);
       mp += __shfl_xor_sync(0xffffffffu, mp, 4);
-      const float inv_n = __frcp_rn(a.n0 + dn), ut = mt * inv_n, up = mp * inv_n;
+      const float nn = __fadd_rn(a.n0, dn), inv_n = __frcp_rn(nn);
+      const float ut = node_velocity(mt, inv_n, ac.fix), up = node_velocity(mp, inv_n, ac.fix);
       const float cubic = p0 * (1.0f - p0 * p0) + (1.0f - 3.0f * p0 * p0) * lo;  // at hi + lo, first order in lo
       const float mu_c = -a.A * cubic - kt * (jp * dN - jm * dS);
       if (k == 0) {
@@ -465,19 +475,22 @@ __global__ void __launch_bounds__(512) axi16_kernel(StageArgs<float> a, const __
         if (CH == VLB_HYDRO) Ft = p0 * inv_n * (mu_s - mu_n) * gt;  // n F^theta = -phi d_theta mu (Eq. pbin)
         const float* fk = in + at;
         const float* fr = in + H + grp - 1;
-        float acc = tf * fk[-2 * sgn] + tn * fk[-sgn];
-        float ac2 = tm * g + td * fk[sgn];
+        // the taps nearly cancel: on differences the products stay small, and so do their roundings
+        float acc = __fmaf_rn(tn, __fsub_rn(fk[-sgn], g), __fmul_rn(tf, __fsub_rn(fk[-2 * sgn], g)));
+        float ac2 = __fmaf_rn(ts, g, __fmul_rn(td, __fsub_rn(fk[sgn], g)));
         // force and inertial terms: (Gamma v_j^2 - F^theta) dg/dv_theta - Gamma v_i sum_m K_jm v_m g_im
         const float dvt = (Kt[0] * fr[j * P] + Kt[1] * fr[(4 + j) * P]) + (Kt[2] * fr[(8 + j) * P] + Kt[3] * fr[(12 + j) * P]);
         const float* fi = fr + 4 * i * P;
         acc += Kp[0] * fi[0] + Kp[1] * fi[P];
         ac2 += Kp[2] * fi[2 * P] + Kp[3] * fi[3 * P];
-        const float usq = ut * ut + up * up, hu = -0.5f * usq, xi = vi * ut + vj * up;
-        const float dntau = dn * itau, ntau = a.n0 * itau + dntau;
-        const float pm1 = xi * ((1.0f + hu) + xi * (0.5f + xi * (1.0f / 6.0f))) + hu;
-        acc += (gvj - Ft) * dvt;
-        ac2 += ww * (ntau * pm1 + (dntau + (ce + nv * Ft))) - itau * g;
-        acc += ac2;
+        // n / tau from the density that was inverted for u: n0 / tau rounded on its own would be off by the same amount
+        // at every node and stage, and the momentum would drift by it.  F^theta, the last to arrive, enters late.
+        const float usq = ut * ut + up * up, hu = -0.5f * usq, xi = __fmaf_rn(vj, up, __fmul_rn(vi, ut));
+        const float dntau = __fmul_rn(dn, itau), ntau = __fmul_rn(nn, itau);
+        const float pm1 = __fmaf_rn(xi, __fmaf_rn(xi, __fmaf_rn(xi, 1.0f / 6.0f, 0.5f), 1.0f + hu), hu);
+        const float X = __fmaf_rn(nv, Ft, __fmaf_rn(ntau, pm1, __fadd_rn(dntau, ce)));
+        acc = __fmaf_rn(-Ft, dvt, __fmaf_rn(gvj, dvt, acc));
+        acc = __fadd_rn(acc, __fmaf_rn(ww, X, __fmaf_rn(-itau, g, ac2)));
         const float o = st == 0 ? g + acc : u0 + b * ((g - u0) + acc);
         // Cahn-Hilliard (Eq. CH): M Delta mu - div(u phi), theta parts only (every lane; 0 and 1 store hi, lo)
         float L = lt * (jp * (mu_n - mu_c) - jm * (mu_c - mu_s));
@@ -521,6 +534,7 @@ AxiConst<T> make_axi_const() {
       c.ww[i][m] = (T)(d.w[i] * d.w[m]);
     }
   }
+  c.fix = make_node_const<T>().fix;
   return c;
 }
 
