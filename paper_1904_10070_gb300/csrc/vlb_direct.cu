@@ -138,8 +138,8 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     const int mi = mr * MS + mc;
     s_dn[mi] = dn;
     s_in[mi] = inv_n;
-    s_ut[mi] = vmul(mt, inv_n);
-    s_up[mi] = vmul(mp, inv_n);
+    s_ut[mi] = node_velocity(mt, inv_n, nc.fix);
+    s_up[mi] = node_velocity(mp, inv_n, nc.fix);
     const T lap = vfma(lp, vsub(dE, dW), vmul(lt, vsub(vmul(jp, dN), vmul(jm, dS))));
     const T ph2 = vmul(ph, ph);
     T cubic = vmul(ph, vsub(T(1), ph2));

@@ -289,8 +289,8 @@ __device__ __forceinline__ void moment_point(const StageArgs<T>& a, const VConst
   const T mp = vc.v[3] * (col[3] - col[0]) + vc.v[2] * (col[2] - col[1]);
   const int mi = mr * MS + mc;
   const T inv_n = recip(a.n0 + dn);
-  sm[L::UT_OFF + mi] = mt * inv_n;
-  sm[L::UP_OFF + mi] = mp * inv_n;
+  sm[L::UT_OFF + mi] = node_velocity(mt, inv_n, vc.nc.fix);
+  sm[L::UP_OFF + mi] = node_velocity(mp, inv_n, vc.nc.fix);
   const T* pp = sphi + bi;
   const int cr = mr + H - 1;
   const T ph = pp[0];
@@ -533,8 +533,8 @@ __device__ __forceinline__ void pair_point(const StageArgs<float>& a, const Node
   parity_moments(o.P, nc, o.dn, mt, mp);
   const float2 nn = vadd(f2(a.n0), o.dn);
   o.inv = make_float2(__frcp_rn(nn.x), __frcp_rn(nn.y));
-  o.ut = vmul(mt, o.inv);
-  o.up = vmul(mp, o.inv);
+  o.ut = node_velocity(mt, o.inv, nc.fix);
+  o.up = node_velocity(mp, o.inv, nc.fix);
   o.ph = ph;
   o.lo = lo;
 }
