@@ -1257,10 +1257,12 @@ VConst<T> make_vconst() {
 // rows 22.6 / 21.3 (256 x 512), 45.2 / 37.5 (400 x 800), 69.7 / 57.9 (512 x 1024), 218.5 / 203.6 (1024 x 2048); small
 // grids too, where each SM holds at most one tile (64 x 128: 13.7 / 10.3).  In between, where one 16-row tile per SM
 // holds the grid but one 8-row tile does not, the second 8-row tile of an SM costs more than it saves (192 x 384:
-// 15.0 / 17.2, 256 x 256: 14.5 / 16.3).  4-row tiles are no better than 8 above 64 x 128.
-constexpr int kSms = 152;
+// 15.0 / 17.2, 256 x 256: 14.5 / 16.3).  4-row tiles are no better than 8 above 64 x 128.  Grids with more 8-row
+// tiles along theta than a grid dimension holds take 16 rows too (vlb_create admits 65535 x 16 rows).
+constexpr int kSms = 152, kGridRows = 65535;
 int stage_rows_rule(int nt, int ns) {
   const int64_t cols = (ns + TS - 1) / TS, t8 = cols * ((nt + 7) / 8), t16 = cols * ((nt + 15) / 16);
+  if ((nt + 7) / 8 > kGridRows) return 16;
   return t8 > kSms && t16 <= kSms ? 16 : 8;
 }
 
