@@ -206,6 +206,11 @@ vlb_status vlb_test_wave_schedule(int32_t n_bands, int32_t lag, int32_t nsteps);
  * normal operation. */
 vlb_status vlb_test_wave_timeout(vlb_handle* h, int32_t skip_cta, int64_t budget);
 
+/* Test hook (not part of the method): the steps of solver h take paths that otherwise only other grids or devices
+ * reach; the results are the same.  routes: a sum of VLB_TEST_*, 0 restores normal operation. */
+enum { VLB_TEST_WIDE_OFFSETS = 1 /* FP64 stages: the 64-bit offsets of grids of 2^29 nodes and more */ };
+vlb_status vlb_test_route(vlb_handle* h, int32_t routes);
+
 /* Message of the last failure on h (or of the calling thread's last handle-less failure when
  * h is NULL).  Never NULL; empty when there was none. */
 const char* vlb_last_error(const vlb_handle* h);

@@ -277,6 +277,7 @@ vlb_status run_steps(vlb_handle* h, int64_t nsteps) {
   vlb::StageArgs<T> a;
   a.coef = (const T*)h->coefT;
   if constexpr (sizeof(T) == 4) a.rows = h->rows;
+  a.route = h->route;
   a.nt = p.n_theta;
   a.ns = p.n_phi;
   a.stride = h->stride;
@@ -840,6 +841,13 @@ vlb_status vlb_test_wave_timeout(vlb_handle* h, int32_t skip_cta, int64_t budget
   if (budget < 0) return fail(h, VLB_ERR_ARG, "vlb_test_wave_timeout: budget < 0");
   h->wave_skip = skip_cta < 0 ? -1 : skip_cta;
   h->wave_budget = budget;
+  return VLB_OK;
+}
+
+vlb_status vlb_test_route(vlb_handle* h, int32_t routes) {
+  if (!h) return fail(nullptr, VLB_ERR_ARG, "handle is NULL");
+  if (h->kind != 0) return fail(h, VLB_ERR_ARG, "vlb_test_route: solver handles only");
+  h->route = routes;
   return VLB_OK;
 }
 

@@ -37,12 +37,12 @@ struct DirectConst {
 };
 
 // Element at byte offset `off` of an array whose base is uniform over the CTA.
-template <typename T>
-__device__ __forceinline__ T at(const T* base, uint32_t off) {
+template <typename T, typename Off>
+__device__ __forceinline__ T at(const T* base, Off off) {
   return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
 }
-template <typename T>
-__device__ __forceinline__ void put(T* base, uint32_t off, T v) {
+template <typename T, typename Off>
+__device__ __forceinline__ void put(T* base, Off off, T v) {
   *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off) = v;
 }
 
@@ -71,8 +71,9 @@ __device__ __forceinline__ void slot_node(int it, int& mr, int& mc) {
 }
 
 // One CTA per TQ x TSW tile.  Step 1 puts the moments and mu of the tile and a halo of 1 into shared memory
-// (dn, 1/n, u^theta, u^phi, mu); step 2 evaluates the right-hand side and the update.
-template <typename T, int ADV, int CH, bool F0, int TQ, int TSW, bool SPLIT>
+// (dn, 1/n, u^theta, u^phi, mu); step 2 evaluates the right-hand side and the update.  Off: the type of a byte offset
+// within one array.
+template <typename T, int ADV, int CH, bool F0, int TQ, int TSW, bool SPLIT, typename Off>
 __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && sizeof(T) == 4 ? 5 : 0)
     direct_kernel(StageArgs<T> a, const __grid_constant__ DirectConst<T> dc) {
   constexpr bool DF = sizeof(T) == 4;
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
   const int tiles_s = (ns + TSW - 1) / TSW;  // 1-D grid: a column grid has more tile rows than gridDim.y may hold
   const int q0 = (int)(blockIdx.x / tiles_s) * TQ, s0 = (int)(blockIdx.x % tiles_s) * TSW;
   const int64_t st = a.stride;
-  constexpr uint32_t B = sizeof(T);
+  constexpr Off B = sizeof(T);
   const NodeConst<T>& nc = dc.nc;
   const T* phi = a.fin + NPOP * st;
   constexpr bool KEEP = !SPLIT && ADV == VLB_UW3;  // the parity combinations stay in registers for step 2
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
 #pragma unroll
       for (int k = 0; k < (SPLIT ? 4 : 16); ++k)
         U0[k] = SPLIT ? a.f0[(k + 4 * (tid & 3)) * st + (int64_t)q * ns + s]
-                      : at(a.f0 + k * st, (uint32_t)sizeof(T) * (uint32_t)(q * ns + s));
+                      : at(a.f0 + k * st, B * (uint32_t)(q * ns + s));
   }
   if constexpr (TAB) {
     for (int e = tid; e < TQ * NE; e += NTH)
@@ -110,13 +111,13 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     slot_node<TQ, TSW>(it, mr, mc);
     if (q0 + mr - 1 > nt || s0 + mc - 1 > ns) return;  // beyond the halo of the last node
     const int q = wrap_near(q0 + mr - 1, nt), s = wrap_near(s0 + mc - 1, ns);
-    const uint32_t id = B * (uint32_t)(q * ns + s);
+    const Off id = B * (uint32_t)(q * ns + s);
     T g[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) g[k] = at(a.fin + k * st, id);
-    const uint32_t in_ = B * (uint32_t)((q + 1 < nt ? q + 1 : 0) * ns + s);
-    const uint32_t is = B * (uint32_t)((q > 0 ? q - 1 : nt - 1) * ns + s);
-    const uint32_t ie = B * (uint32_t)(q * ns + (s + 1 < ns ? s + 1 : 0));
+    const Off in_ = B * (uint32_t)((q + 1 < nt ? q + 1 : 0) * ns + s);
+    const Off is = B * (uint32_t)((q > 0 ? q - 1 : nt - 1) * ns + s);
+    const Off ie = B * (uint32_t)(q * ns + (s + 1 < ns ? s + 1 : 0));
     const uint32_t iw = B * (uint32_t)(q * ns + (s > 0 ? s - 1 : ns - 1));
     const T ph = at(phi, id);
     T dN = vsub(at(phi, in_), ph), dS = vsub(ph, at(phi, is)), lo = T(0);
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     bool bad = false;
     if (tid < 16 * TQ) {  // the tile's first upwind face: at s0 - 1/2 (v > 0) or s0 + TSW - 1/2
       const int k = tid / TQ, dn = (k & 3) >= 2 ? 1 : -1, first = dn > 0 ? -1 : TSW;
-      const uint32_t row = B * (uint32_t)(wrap_near(q0 + tid % TQ, nt) * ns);
+      const Off row = B * (uint32_t)(wrap_near(q0 + tid % TQ, nt) * ns);
       T x[5];
 #pragma unroll
       for (int d = 0; d < 5; ++d) x[d] = at(a.fin + k * st, row + col(first + dn * (d - 2)));
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     }
     __syncthreads();
     const int dt_ = i >= 2 ? 1 : -1, top = i >= 2 ? 0 : TQ - 1;  // downwind step along theta; the first row of the march
-    uint32_t ro[TQ + 5], cs[5];  // rows of the march, columns lane - 2 .. lane + 2 (byte offsets)
+    Off ro[TQ + 5], cs[5];  // rows of the march, columns lane - 2 .. lane + 2 (byte offsets)
     T J[TQ + 5];
 #pragma unroll
     for (int d = 0; d < TQ + 5; ++d) {
@@ -212,8 +213,8 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
       const T fref = a.n0 * dc.ww[i][j];  // theta reconstructs the full J f
       const int dp = j >= 2 ? 1 : -1;     // downwind step along varphi
       const T vj = dp > 0 ? dc.v[j] : -dc.v[j];
-      const uint32_t c0 = dp > 0 ? cs[0] : cs[4], c1 = dp > 0 ? cs[1] : cs[3], c3 = dp > 0 ? cs[3] : cs[1];
-      const uint32_t c4 = dp > 0 ? cs[4] : cs[0];
+      const Off c0 = dp > 0 ? cs[0] : cs[4], c1 = dp > 0 ? cs[1] : cs[3], c3 = dp > 0 ? cs[3] : cs[1];
+      const Off c4 = dp > 0 ? cs[4] : cs[0];
       T G[TQ + 5], x[TQ];
 #pragma unroll
       for (int d = 0; d < TQ + 5; ++d) {
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
         const T F = weno5_face(G[r + 1], G[r + 2], G[r + 3], G[r + 4], G[r + 5], bad);
         T adv = vct[r] * (F - last);  // -|v| (downwind - upwind face) in both directions
         last = F;
-        const uint32_t o = ro[r + 3];
+        const Off o = ro[r + 3];
         const T Fd = weno5_face(at(f, o + c0), at(f, o + c1), x[r], at(f, o + c3), at(f, o + c4), bad);
         T Fu = __shfl_sync(0xffffffffu, Fd, (lane - dp) & 31);
         if (lane == (dp > 0 ? 0 : 31)) Fu = s_edge[k * TQ + lrow];
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
   T rl[TAB ? 1 : NE];
   if constexpr (!TAB) row_all<T>(rl, a, q);
   const T* rt = TAB ? s_rt + lr * RP : rl;
-  const uint32_t id = B * (uint32_t)(q * ns + s);  // byte offsets within one array (launch_direct checks the range)
+  const Off id = B * (uint32_t)(q * ns + s);  // byte offsets within one array (launch_direct checks the range)
   const int qn = q + 1 < nt ? q + 1 : 0, qs = q > 0 ? q - 1 : nt - 1;
   const int qnn = wrap_near(q + 2, nt), qss = wrap_near(q - 2, nt);
   const int se = s + 1 < ns ? s + 1 : 0, sw = s > 0 ? s - 1 : ns - 1;
@@ -279,10 +280,10 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     Ft = vmul(vmul(pn, vsub(mu_s, mu_n)), a.gt * dt);
     Fp = vmul(vmul(pn, vsub(mu_w, mu_e)), rt[E_GP]);
   }
-  const uint32_t on = B * (uint32_t)(qn * ns + s), os = B * (uint32_t)(qs * ns + s);
-  const uint32_t onn = B * (uint32_t)(qnn * ns + s), oss = B * (uint32_t)(qss * ns + s);
-  const uint32_t oe = B * (uint32_t)(q * ns + se), ow = B * (uint32_t)(q * ns + sw);
-  const uint32_t oee = B * (uint32_t)(q * ns + see), oww = B * (uint32_t)(q * ns + sww);
+  const Off on = B * (uint32_t)(qn * ns + s), os = B * (uint32_t)(qs * ns + s);
+  const Off onn = B * (uint32_t)(qnn * ns + s), oss = B * (uint32_t)(qss * ns + s);
+  const Off oe = B * (uint32_t)(q * ns + se), ow = B * (uint32_t)(q * ns + sw);
+  const Off oee = B * (uint32_t)(q * ns + see), oww = B * (uint32_t)(q * ns + sww);
   const int i_split = SPLIT ? tid & 3 : 0;
   if (!SPLIT || i_split == 0) {
     // Cahn-Hilliard: M Delta mu - div(u phi) (Eq. CH), flux form with mean face values, times dt
@@ -319,8 +320,8 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
   // weights 1, -6, 3, 2 on the far, near, centre and downwind nodes (tf .. td: theta, on J g; pv: varphi).
   // FP64 folds the three centre taps into one coefficient, whose rounding is far below the scheme's;
   // FP32 keeps the varphi difference on whole-number weights, which cancel on a uniform field.
-  auto update = [&](int k, T acc, T g0, T tf, T tn, T tm, T td, uint32_t rf, uint32_t rn, uint32_t rd, int y, T cc,
-                    uint32_t cf, uint32_t cn, uint32_t cd) {
+  auto update = [&](int k, T acc, T g0, T tf, T tn, T tm, T td, Off rf, Off rn, Off rd, int y, T cc,
+                    Off cf, Off cn, Off cd) {
     const T* f = a.fin + k * st;
     const T g = at(f, id), pv = rt[E_TH + 8 * y + TAP_PV];
     if (F0 && !HOLD) g0 = at(a.f0 + k * st, id);
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     const T tf = -vmul(vc, J[pos ? qss : qnn]), tn = vmul(T(6) * vc, J[pos ? qs : qn]);
     const T td = vmul(T(-2) * vc, J[pos ? qn : qs]), tm = vmul(T(-3) * vc, J[q]);
     const T ccx = vsub(tm, itau);
-    const uint32_t rf = pos ? oss : onn, rn = pos ? os : on, rd = pos ? on : os;
+    const Off rf = pos ? oss : onn, rn = pos ? os : on, rd = pos ? on : os;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int y = (j == 0 || j == 3) ? 0 : 1;
@@ -431,7 +432,7 @@ DirectConst<T> make_direct_const() {
   return c;
 }
 
-template <typename T, int ADV, int CH, bool F0, int TQ, int TSW, bool SPLIT>
+template <typename T, int ADV, int CH, bool F0, int TQ, int TSW, bool SPLIT, typename Off = uint32_t>
 cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
   static const DirectConst<T> dc = make_direct_const<T>();
   cudaLaunchConfig_t cfg = {};
@@ -443,7 +444,7 @@ cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, direct_kernel<T, ADV, CH, F0, TQ, TSW, SPLIT>, a, dc);
+  return cudaLaunchKernelEx(&cfg, direct_kernel<T, ADV, CH, F0, TQ, TSW, SPLIT, Off>, a, dc);
 }
 
 // FP32: 4 x 32 tiles, one thread per node (8 x 32 tiles with 64 registers: 316 us against 304-320 on eight
@@ -453,9 +454,17 @@ cudaError_t launch_direct_t(const StageArgs<T>& a, cudaStream_t st) {
 // threads share a node (2 x 8 nodes a CTA).  Per step, one / four threads a node: 32 x 64 72 / 34 us, 64 x 128
 // 72 / 93 us, 128 x 384 175 / 330 us.
 constexpr int64_t kSplitNodes = 32 * 152;
+// Byte offsets within one array are 32 bits up to 2^32 bytes.  An FP32 array cannot be larger (its grid would need
+// 360 GB: 352 bytes a node with the staging area); FP64 grids of 2^29 nodes and more take 64-bit offsets (544 bytes a
+// node: 272 GiB, which the device holds up to about 547 million nodes).
+constexpr uint64_t kWideNodes = (uint64_t)1 << 29;
 
 template <typename T, int ADV, int CH, bool F0>
 cudaError_t launch_direct_v(const StageArgs<T>& a, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if ((uint64_t)a.nt * a.ns >= kWideNodes || (a.route & VLB_TEST_WIDE_OFFSETS))
+      return launch_direct_t<T, ADV, CH, F0, ADV == VLB_WENO5 ? 4 : 8, ADV == VLB_WENO5 ? 32 : 16, false, uint64_t>(a, st);
+  }
   if constexpr (ADV == VLB_WENO5 || sizeof(T) == 4) {
     return launch_direct_t<T, ADV, CH, F0, 4, 32, false>(a, st);
   } else {
@@ -476,9 +485,6 @@ cudaError_t launch_direct_a(const StageArgs<T>& a, int ch_mode, cudaStream_t st)
 
 template <typename T>
 cudaError_t launch_direct(const StageArgs<T>& a, int advection, int ch_mode, cudaStream_t st) {
-  // 32-bit byte offsets within an array: 2^32 bytes per array would need over 200 GB for the three
-  // states and as much again for the FP64 staging area, more than the device has
-  if ((uint64_t)a.nt * a.ns * sizeof(T) >= ((uint64_t)1 << 32)) return cudaErrorInvalidValue;
   return advection == VLB_UW3 ? launch_direct_a<T, VLB_UW3>(a, ch_mode, st) : launch_direct_a<T, VLB_WENO5>(a, ch_mode, st);
 }
 

@@ -27,6 +27,7 @@ struct vlb_handle {
   vlb::StageMaps* maps = nullptr;  // FP32 UW3: tensor maps of the three stage inputs (NULL: per-thread copies)
   vlb::StageMaps* wave_maps = nullptr;  // the same for the 16-row tiles of the wavefront schedule
   unsigned* wave_cnt = nullptr;    // FP32 UW3: counters of the wavefront schedule (NULL: not available)
+  int route = 0;                   // VLB_TEST_* paths taken regardless of size and device (vlb_test_route)
   int sched = 0;                   // VLB_SCHED_AUTO / STAGES / WAVE (vlb_set_schedule)
   int wave_skip = -1;              // test hook: a wavefront CTA that never reports its tiles
   long long wave_budget = 0;       // wavefront dependency-wait budget in SM cycles (0 = default)

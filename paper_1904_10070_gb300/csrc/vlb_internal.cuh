@@ -74,6 +74,7 @@ struct StageArgs {
   T n0;             // reference density of the stored deviations
   int* err;         // device flag raised if a bounded wait on a bulk copy gives up (may be NULL)
   int ahead;        // tensor-map path: CTAs resident at once; each prefetches the tile this many ahead
+  int route = 0;    // VLB_TEST_* (vlb_test_route)
   T* dphi = nullptr;  // stabilised Cahn-Hilliard: receives dt L_phi per node, and phi is not written
                       // (launch_ch_stab forms it); NULL: the stage writes phi itself
 };

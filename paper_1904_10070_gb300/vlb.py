@@ -32,7 +32,7 @@ EXPORTS = ["vlb_workspace_bytes", "vlb_max_stable_dt", "vlb_create", "vlb_destro
            "vlb_adam_step_many", "vlb_to_bf16", "vlb_conv_status", "vlb_test_raise_flag", "vlb_surrogate_workspace_bytes", "vlb_surrogate_create",
            "vlb_surrogate_advance", "vlb_surrogate_stats", "vlb_ensemble_configure", "vlb_ensemble_get_config",
            "vlb_structure_length", "vlb_set_schedule", "vlb_get_schedule", "vlb_test_wave_schedule",
-           "vlb_test_wave_timeout"]
+           "vlb_test_wave_timeout", "vlb_test_route"]
 
 NOALLOC_SCRATCH_BYTES = 24 * 1024 * 1024
 
@@ -107,6 +107,7 @@ def lib() -> ctypes.CDLL:
     L.vlb_test_wave_schedule.argtypes = [ctypes.c_int32, ctypes.c_int32, ctypes.c_int32]
     L.vlb_test_wave_schedule.restype = I32
     L.vlb_test_wave_timeout.argtypes, L.vlb_test_wave_timeout.restype = [P, ctypes.c_int32, I64], I32
+    L.vlb_test_route.argtypes, L.vlb_test_route.restype = [P, ctypes.c_int32], I32
     L.vlb_state_device.argtypes, L.vlb_state_device.restype = [P, ctypes.POINTER(P), ctypes.POINTER(I64)], I32
     L.vlb_steps_done.argtypes, L.vlb_steps_done.restype = [P, ctypes.POINTER(I64)], I32
     L.vlb_last_error.argtypes, L.vlb_last_error.restype = [P], ctypes.c_char_p
@@ -240,6 +241,7 @@ def vlb_interface_length(h) -> float:
 
 
 SCHED_AUTO, SCHED_STAGES, SCHED_WAVE = 0, 1, 2
+TEST_WIDE_OFFSETS = 1
 
 
 def vlb_set_schedule(h, schedule: int):
@@ -259,6 +261,10 @@ def vlb_test_wave_schedule(n_bands: int, lag: int, nsteps: int) -> bool:
 
 def vlb_test_wave_timeout(h, skip_cta: int, budget: int):
     _check(lib().vlb_test_wave_timeout(h, int(skip_cta), int(budget)), h)
+
+
+def vlb_test_route(h, routes: int):
+    _check(lib().vlb_test_route(h, int(routes)), h)
 
 
 def vlb_structure_length(h) -> float:
