@@ -245,24 +245,27 @@ __device__ __forceinline__ FF to_ff(double x) {
 }
 __device__ __forceinline__ double to_d(FF a) { return (double)a.h + (double)a.l; }
 
-// W threads (a power of two) share a row.
+// W threads (a power of two) share a segment of `len` nodes of a row; `segs` segments a row.
 __global__ void __launch_bounds__(TOTAL_THREADS) totals32_kernel(const float* state, int64_t stride,
-                                                                 const double* coefd, int nt, int ns, int W, double A,
-                                                                 double kappa, double n0, double gt, double* partials,
-                                                                 VD vd) {
+                                                                 const double* coefd, int nt, int ns, int W, int segs,
+                                                                 int len, double A, double kappa, double n0, double gt,
+                                                                 double* partials, VD vd) {
   const int c = threadIdx.x & (W - 1), rb = TOTAL_THREADS / W;
   const FF va = to_ff(vd.v[2]), vb = to_ff(vd.v[3]), gtf = to_ff(gt), A4 = to_ff(0.25 * A), k2 = to_ff(0.5 * kappa);
   const FF n0f = to_ff(n0), one = {1.0f, 0.0f};
   const float *hi = state + NPOP * stride, *lo = hi + stride;
   double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
   FF best = {0.0f, 0.0f};  // largest |u|^2
-  for (int q = blockIdx.x * rb + threadIdx.x / W; q < nt; q += gridDim.x * rb) {
+  for (int64_t unit = blockIdx.x * (int64_t)rb + threadIdx.x / W; unit < (int64_t)nt * segs;
+       unit += (int64_t)gridDim.x * rb) {
+    const int q = (int)(unit / segs), first = (int)(unit - (int64_t)q * segs) * len;
+    const int last = first + len < ns ? first + len : ns;
     const int64_t rn = (int64_t)(q + 1 < nt ? q + 1 : 0) * ns, rs = (int64_t)(q > 0 ? q - 1 : nt - 1) * ns;
     const int64_t r0 = (int64_t)q * ns;
     const FF gp = to_ff(coefd[C_GP * nt + q]);
     FF m = {0.0f, 0.0f}, ph = m, psi = m;
     int count = 0;
-    for (int s = c; s < ns; s += W) {
+    for (int s = first + c; s < last; s += W) {
       const int se = s + 1 < ns ? s + 1 : 0, sw = s > 0 ? s - 1 : ns - 1;
       const float* f = state + r0 + s;
       FF S[4], OB = {0.0f, 0.0f}, OA = OB;
@@ -318,14 +321,17 @@ __device__ __forceinline__ float phi_sign(const float* state, int64_t stride, in
 }
 template <typename T>
 __global__ void __launch_bounds__(TOTAL_THREADS) interface_kernel(const T* state, int64_t stride, const double* coefd,
-                                                                  int nt, int ns, int W, double edge_p,
-                                                                  double* partials) {
+                                                                  int nt, int ns, int W, int segs, int len,
+                                                                  double edge_p, double* partials) {
   const int c = threadIdx.x & (W - 1), rb = TOTAL_THREADS / W;
   double acc = 0.0;
-  for (int q = blockIdx.x * rb + threadIdx.x / W; q < nt; q += gridDim.x * rb) {
+  for (int64_t unit = blockIdx.x * (int64_t)rb + threadIdx.x / W; unit < (int64_t)nt * segs;
+       unit += (int64_t)gridDim.x * rb) {
+    const int q = (int)(unit / segs), first = (int)(unit - (int64_t)q * segs) * len;
+    const int last = first + len < ns ? first + len : ns;
     const int64_t r0 = (int64_t)q * ns, rn = (int64_t)(q + 1 < nt ? q + 1 : 0) * ns;
     int np = 0, nn = 0;
-    for (int s = c; s < ns; s += W) {
+    for (int s = first + c; s < last; s += W) {
       const T p0 = phi_sign(state, stride, r0 + s);
       np += crosses(p0, phi_sign(state, stride, r0 + (s + 1 < ns ? s + 1 : 0))) ? 1 : 0;
       nn += crosses(p0, phi_sign(state, stride, rn + s)) ? 1 : 0;
@@ -538,11 +544,25 @@ cudaError_t launch_fields(const T* state, int64_t stride, const double* coefd, i
   return cudaGetLastError();
 }
 
-// threads that share a row: a power of two up to a CTA
-static int row_threads(int ns) {
-  int w = 1;
-  while (w < TOTAL_THREADS && w < ns) w *= 2;
-  return w;
+// How the sums over rows are shared out: W threads (a power of two up to a CTA) to a segment, and rows cut into
+// segments of whole passes of W nodes where they alone would leave CTAs idle (few long rows: 8 x 262144 is 8 CTAs
+// of 1024 passes otherwise).
+struct RowSplit {
+  int W, segs, len, blocks;
+};
+static RowSplit row_split(int nt, int ns, int n_blocks) {
+  RowSplit r;
+  r.W = 1;
+  while (r.W < TOTAL_THREADS && r.W < ns) r.W *= 2;
+  const int rb = TOTAL_THREADS / r.W;
+  const int64_t units = (int64_t)n_blocks * rb, passes = (ns + r.W - 1) / r.W;
+  const int64_t want = units / nt > 1 ? (units / nt < passes ? units / nt : passes) : 1;
+  const int64_t per = (passes + want - 1) / want;
+  r.len = (int)(per * r.W);
+  r.segs = (int)((passes + per - 1) / per);
+  const int64_t blocks = ((int64_t)nt * r.segs + rb - 1) / rb;
+  r.blocks = (int)(blocks < n_blocks ? blocks : n_blocks);
+  return r;
 }
 
 template <typename T>
@@ -550,10 +570,10 @@ cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, i
                           double kappa, double n0, double* partials, int n_blocks, double* out, cudaStream_t s) {
   const double gt = 1.0 / (2.0 * r * (2.0 * M_PI / nt));
   if constexpr (sizeof(T) == 4) {
-    const int W = row_threads(ns), rb = TOTAL_THREADS / W;
-    n_blocks = (nt + rb - 1) / rb < n_blocks ? (nt + rb - 1) / rb : n_blocks;
-    totals32_kernel<<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, W, A, kappa, n0, gt, partials,
-                                                       make_vd());
+    const RowSplit r = row_split(nt, ns, n_blocks);
+    n_blocks = r.blocks;
+    totals32_kernel<<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, r.W, r.segs, r.len, A, kappa, n0,
+                                                       gt, partials, make_vd());
   } else {
     totals_kernel<T><<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, A, kappa, n0, gt, partials,
                                                         make_vd());
@@ -567,9 +587,10 @@ cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, i
 template <typename T>
 cudaError_t launch_interface(const T* state, int64_t stride, const double* coefd, int nt, int ns, double r,
                              double* partials, int n_blocks, double* out, cudaStream_t s) {
-  const int W = row_threads(ns), rb = TOTAL_THREADS / W;
-  n_blocks = (nt + rb - 1) / rb < n_blocks ? (nt + rb - 1) / rb : n_blocks;
-  interface_kernel<T><<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, W, r * (2.0 * M_PI / nt), partials);
+  const RowSplit w = row_split(nt, ns, n_blocks);
+  n_blocks = w.blocks;
+  interface_kernel<T><<<n_blocks, TOTAL_THREADS, 0, s>>>(state, stride, coefd, nt, ns, w.W, w.segs, w.len,
+                                                         r * (2.0 * M_PI / nt), partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   interface_final_kernel<<<1, 32, 0, s>>>(partials, n_blocks, out);
