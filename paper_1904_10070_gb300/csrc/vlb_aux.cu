@@ -142,12 +142,13 @@ __global__ void fields_kernel(const T* state, int64_t stride, const double* coef
   mu[idx] = -A * p0 * (1.0 - p0 * p0) - kappa * lap;
 }
 
-// Per-block FP64 sums: mass, phi total, Psi (Eq. Landau), max |u|, non-finite count (slots 5 .. 7 unused).
+// Per-block FP64 sums: mass, phi total, Psi (Eq. Landau), max |u|, non-finite count (NTOT of a block's NSUM slots).
 // Warp, then block reduction in a fixed order.
+constexpr int NTOT = 5;
 __device__ __forceinline__ void reduce_totals(double (&acc)[NSUM], double* partials) {
   __shared__ double red[TOTAL_THREADS / 32][NSUM];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {
+  for (int k = 0; k < NTOT; ++k) {
     double x = acc[k];
     for (int o = 16; o > 0; o >>= 1) {
       const double y = __shfl_down_sync(0xffffffffu, x, o);
@@ -159,7 +160,7 @@ __device__ __forceinline__ void reduce_totals(double (&acc)[NSUM], double* parti
   if (lane == 0)
     for (int k = 0; k < NSUM; ++k) red[wid][k] = acc[k];
   __syncthreads();
-  if (threadIdx.x < NSUM) {
+  if (threadIdx.x < NTOT) {
     const int k = threadIdx.x;
     double x = 0.0;
     for (int w = 0; w < TOTAL_THREADS / 32; ++w) x = (k == 3) ? fmax(x, red[w][k]) : x + red[w][k];
@@ -208,11 +209,12 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals_kernel(const T* state, i
 
 // ---- Totals of an FP32 state in float pairs -----------------------------------------------------------
 // The FP64 units (one warp instruction per 19 cycles and SM) made the totals of 1024 x 2048 cost 558 us at
-// about 100 FP64 operations a node.  An FP32 state needs 48 bits, not 53: every quantity of a node is
-// formed as an unevaluated pair h + l of floats with error-free sums and products (Dekker 1971, Knuth),
-// 2^-47 relative per operation against the state's own 2^-24, a row's sums too; FP64 starts at the row
-// (times the area element) and does the rest.  About 520 FP32 operations a node: 86 us.  A node whose
-// values leave the range where the pairs cannot overflow or underflow takes the FP64 path.
+// about 100 FP64 operations a node.  Here a node's quantities are unevaluated pairs h + l of floats with error-free
+// sums and products (Dekker 1971, Knuth), 2^-46 relative each, and FP64 takes over at the row.  What a sum over
+// many nodes averages out may stay at that; what it does not is done as exactly as in FP64: differences keep their
+// relative accuracy (diff, 1 - phi^2 as a product), phi is summed with the rounding of its low words carried, and
+// the node of the largest |u| is evaluated again in FP64.  About 560 FP32 operations a node.  A node whose values
+// leave the range in which the pairs neither overflow nor lose bits to underflow takes the FP64 path.
 struct FF {
   float h, l;
 };
@@ -230,6 +232,12 @@ __device__ __forceinline__ FF operator+(FF a, FF b) {
 }
 __device__ __forceinline__ FF operator-(FF a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ FF operator-(FF a, FF b) { return a + (-b); }
+// a - b, accurate relative to the difference
+__device__ __forceinline__ FF diff(FF a, FF b) {
+  const FF s = two_sum(a.h, -b.h), t = two_sum(a.l, -b.l), r = quick_sum(s.h, __fadd_rn(s.l, t.h));
+  return quick_sum(r.h, __fadd_rn(r.l, t.l));
+}
+__device__ __forceinline__ bool exceeds(FF a, FF b) { return a.h > b.h || (a.h == b.h && a.l > b.l); }
 __device__ __forceinline__ FF operator*(FF a, FF b) {
   const float p = __fmul_rn(a.h, b.h);
   return quick_sum(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p))));
@@ -255,7 +263,8 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals32_kernel(const float* st
   const FF n0f = to_ff(n0), one = {1.0f, 0.0f};
   const float *hi = state + NPOP * stride, *lo = hi + stride;
   double acc[NSUM] = {0, 0, 0, 0, 0, 0, 0, 0};
-  FF best = {0.0f, 0.0f};  // largest |u|^2
+  FF best = {0.0f, 0.0f};  // largest |u|^2, and its node
+  int64_t best_at = -1;
   for (int64_t unit = blockIdx.x * (int64_t)rb + threadIdx.x / W; unit < (int64_t)nt * segs;
        unit += (int64_t)gridDim.x * rb) {
     const int q = (int)(unit / segs), first = (int)(unit - (int64_t)q * segs) * len;
@@ -264,6 +273,7 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals32_kernel(const float* st
     const int64_t r0 = (int64_t)q * ns;
     const FF gp = to_ff(coefd[C_GP * nt + q]);
     FF m = {0.0f, 0.0f}, ph = m, psi = m;
+    float ph3 = 0.0f;  // rounding of ph's low word
     int count = 0;
     for (int s = first + c; s < last; s += W) {
       const int se = s + 1 < ns ? s + 1 : 0, sw = s > 0 ? s - 1 : ns - 1;
@@ -285,26 +295,62 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals32_kernel(const float* st
       const FF dn = (S[0] + S[3]) + (S[1] + S[2]), nn = n0f + dn;
       const FF mt = vb * (S[3] - S[0]) + va * (S[2] - S[1]), mp = vb * OB + va * OA;
       const FF u2 = (mt * mt + mp * mp) / (nn * nn);
-      const FF om = one - p0 * p0, g1 = (pn - ps) * gtf, g2 = (pe - pw) * gp;
+      const FF om = diff(one, p0) * (one + p0), g1 = diff(pn, ps) * gtf, g2 = diff(pe, pw) * gp;
       const FF dens = A4 * (om * om) + k2 * (g1 * g1 + g2 * g2);
       const float pm = fmaxf(fmaxf(fabsf(p0.h), fmaxf(fabsf(pn.h), fabsf(ps.h))), fmaxf(fabsf(pe.h), fabsf(pw.h)));
-      // the comparisons are false for NaN
-      if (nn.h >= 1e-6f && nn.h <= 1e6f && big <= 1e6f && pm <= 1e4f && u2.h <= 1e6f && dens.h <= 1e12f) {
+      // the comparisons are false for NaN; products below 1e-23 lose bits of their low word, which matters where they
+      // are the largest |u|^2 so far, or the density of Psi itself
+      if (nn.h >= 1e-6f && nn.h <= 1e6f && big <= 1e6f && pm <= 1e4f && u2.h <= 1e6f && dens.h <= 1e12f &&
+          (u2.h >= 1e-23f || best.h >= 1e-23f || (mt.h == 0.0f && mp.h == 0.0f)) &&
+          (dens.h >= 1e-23f || ((A4.h == 0.0f || om.h == 0.0f) && (k2.h == 0.0f || (g1.h == 0.0f && g2.h == 0.0f))))) {
         m = m + dn;
-        ph = ph + p0;
+        const FF sh = two_sum(ph.h, p0.h), sl = two_sum(ph.l, p0.l), st = two_sum(sh.l, sl.h);
+        ph = quick_sum(sh.h, st.h);
+        ph3 = __fadd_rn(ph3, __fadd_rn(sl.l, st.l));
         psi = psi + dens;
         ++count;
-        if (u2.h > best.h || (u2.h == best.h && u2.l > best.l)) best = u2;
+        if (exceeds(u2, best)) {
+          best = u2;
+          best_at = r0 + s;
+        }
       } else {
         node_totals(state, stride, coefd, nt, ns, q, s, A, kappa, n0, gt, vd, acc);
       }
     }
     const double dA = coefd[C_DA * nt + q];
     acc[0] += (to_d(m) + n0 * count) * dA;
-    acc[1] += to_d(ph) * dA;
+    acc[1] += (to_d(ph) + (double)ph3) * dA;
     acc[2] += to_d(psi) * dA;
   }
-  acc[3] = sqrt(fmax(acc[3], to_d(best)));
+  // the CTA's node of the largest |u|^2 again in FP64, by one thread
+  __shared__ FF s_best[TOTAL_THREADS / 32];
+  __shared__ int64_t s_at[TOTAL_THREADS / 32];
+  for (int o = 16; o > 0; o >>= 1) {
+    const FF x = {__shfl_down_sync(0xffffffffu, best.h, o), __shfl_down_sync(0xffffffffu, best.l, o)};
+    const int64_t at = __shfl_down_sync(0xffffffffu, best_at, o);
+    if (exceeds(x, best)) {
+      best = x;
+      best_at = at;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    s_best[threadIdx.x >> 5] = best;
+    s_at[threadIdx.x >> 5] = best_at;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < TOTAL_THREADS / 32; ++w)
+      if (exceeds(s_best[w], best)) {
+        best = s_best[w];
+        best_at = s_at[w];
+      }
+    if (best_at >= 0) {
+      double nn, a, b;
+      node_moments(state, stride, best_at, vd, n0, nn, a, b);
+      acc[3] = fmax(acc[3], a * a + b * b);
+    }
+  }
+  acc[3] = sqrt(acc[3]);
   reduce_totals(acc, partials);
 }
 
@@ -369,7 +415,7 @@ __global__ void interface_final_kernel(const double* partials, int nb, double* o
   if (threadIdx.x == 0) *out = x;
 }
 
-// one warp per output k (blockDim = 32 NSUM)
+// one warp per output k (blockDim = 32 NTOT)
 __global__ void totals_final_kernel(const double* partials, int nb, double* out) {
   const int k = threadIdx.x >> 5;
   const double x = warp_fold(partials, nb, NSUM, k, k == 3);
@@ -580,7 +626,7 @@ cudaError_t launch_totals(const T* state, int64_t stride, const double* coefd, i
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  totals_final_kernel<<<1, 32 * NSUM, 0, s>>>(partials, n_blocks, out);
+  totals_final_kernel<<<1, 32 * NTOT, 0, s>>>(partials, n_blocks, out);
   return cudaGetLastError();
 }
 
