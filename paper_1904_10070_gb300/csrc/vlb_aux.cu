@@ -355,7 +355,8 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals32_kernel(const float* st
 }
 
 // L_I: the interface edges of every row counted, then weighted in FP64 (r dtheta across varphi, the row's
-// edge length across theta).  Signs of an FP32 state come from the float pair's leading word that is not 0.
+// edge length across theta).  The sign of an FP32 phi is that of the float pair's high word, or of the sum where that
+// word alone does not tell (0; an infinity, whose low word is NaN in a state that has diverged).
 __device__ __forceinline__ bool crosses(double a, double b) { return a * b < 0.0; }
 __device__ __forceinline__ bool crosses(float a, float b) { return (a < 0.0f && b > 0.0f) || (a > 0.0f && b < 0.0f); }
 __device__ __forceinline__ double phi_sign(const double* state, int64_t stride, int64_t idx) {
@@ -363,7 +364,7 @@ __device__ __forceinline__ double phi_sign(const double* state, int64_t stride, 
 }
 __device__ __forceinline__ float phi_sign(const float* state, int64_t stride, int64_t idx) {
   const float h = state[NPOP * stride + idx];
-  return h != 0.0f ? h : state[(NPOP + 1) * stride + idx];
+  return h != 0.0f && isfinite(h) ? h : h + state[(NPOP + 1) * stride + idx];
 }
 template <typename T>
 __global__ void __launch_bounds__(TOTAL_THREADS) interface_kernel(const T* state, int64_t stride, const double* coefd,
