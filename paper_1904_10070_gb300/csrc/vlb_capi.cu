@@ -1599,13 +1599,18 @@ vlb_status vlb_adam_step_many(int32_t count, const int64_t* n, float* const* p, 
                               void* const* p_bf16, void* cuda_stream) {
   if (count < 1 || !n || !p || !g || !m || !v || t < 1)
     return fail(nullptr, VLB_ERR_ARG, "vlb_adam_step_many: bad argument");
-  std::vector<vlb::AdamTensor> a(count);
-  for (int32_t k = 0; k < count; ++k) {
-    a[k] = {n[k], p[k], g[k], m[k], v[k], p_bf16 ? p_bf16[k] : nullptr};
+  for (int32_t k = 0; k < count; ++k)
     if (n[k] < 1 || !p[k] || !g[k] || !m[k] || !v[k])
       return fail(nullptr, VLB_ERR_ARG, "vlb_adam_step_many: bad tensor %d", (int)k);
+  for (int64_t k0 = 0; k0 < count; k0 += vlb::kAdamTensors) {  // one launch's worth at a time, on the stack
+    vlb::AdamTensor a[vlb::kAdamTensors];
+    const int c = (int)std::min<int64_t>(count - k0, vlb::kAdamTensors);
+    for (int j = 0; j < c; ++j) {
+      const int64_t k = k0 + j;
+      a[j] = {n[k], p[k], g[k], m[k], v[k], p_bf16 ? p_bf16[k] : nullptr};
+    }
+    VLB_CUDA(nullptr, vlb::sur_adam(c, a, t, lr, b1, b2, eps, (cudaStream_t)cuda_stream));
   }
-  VLB_CUDA(nullptr, vlb::sur_adam(count, a.data(), t, lr, b1, b2, eps, (cudaStream_t)cuda_stream));
   return VLB_OK;
 }
 
