@@ -7,6 +7,7 @@ the CUDA runtime linked statically (no torch types cross the C ABI).  Usage:
 """
 from __future__ import annotations
 
+import hashlib
 import os
 import subprocess
 import sys
@@ -28,9 +29,20 @@ def nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
+def stage_tag() -> str:
+    """64-bit hash of the sources of the packed FP32 stage: the key of kept autotune choices and of measured traffic."""
+    h = hashlib.sha256()
+    for name in ("vlb_stage.cu", "vlb_node.cuh", "vlb_internal.cuh"):
+        with open(os.path.join(CSRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def _compile(src: str, verbose_ptxas: bool) -> str:
     obj = os.path.join(BUILD, src.replace(".cu", ".o"))
     cmd = [nvcc(), *ARCH, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+    if src == "vlb_capi.cu":
+        cmd.append(f"-DVLB_ENSEMBLE_TAG=0x{stage_tag()}ull")
     if verbose_ptxas:
         cmd += ["-Xptxas", "-v"]
     res = subprocess.run(cmd, capture_output=True, text=True)

@@ -1027,8 +1027,13 @@ vlb_status ens_time(vlb_handle* h, int mode, int rows_idx, float* ms) {
   return VLB_OK;
 }
 
-// ---- autotune cache: one JSON object per line, keyed by the members' grids, ch_mode and SM count.
-// The file is VLB_AUTOTUNE_CACHE if that is set; every process also keeps its own entries.
+// Tag of the ensemble kernels' sources, set by the build.
+#ifndef VLB_ENSEMBLE_TAG
+#define VLB_ENSEMBLE_TAG 0
+#endif
+
+// ---- autotune cache: one JSON object per line, keyed by the kernels' sources (another build's timings decide
+// nothing here), the members' grids, ch_mode and SM count.  The file is VLB_AUTOTUNE_CACHE if that is set; every process also keeps its own entries.
 struct EnsChoice {
   int mode, rows, ctas;
   float ms[4];
@@ -1044,6 +1049,7 @@ std::string ens_key(const vlb_handle* h, int sms) {
       x *= 1099511628211ull;
     }
   };
+  mix((uint64_t)VLB_ENSEMBLE_TAG);
   mix((uint64_t)h->count);
   mix((uint64_t)h->p.ch_mode);
   for (int m = 0; m < h->count; ++m) {
