@@ -15,7 +15,6 @@ no collective).  Rank 0 prints one JSON line.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -38,7 +37,6 @@ BYTES_PER_NODE_STEP = {"f32": 544, "f64": 1088}
 # the FP32 path also carries the low word of phi (an 18th array) for precision: 576 B moved per node-step
 BYTES_PER_NODE_STEP_MOVED_F32 = 576
 PKEYS = ["R", "r", "n_theta", "n_phi", "dt", "tau", "M", "A", "kappa", "geometry", "advection", "ch_mode"]
-STAGE_SRC = os.path.join(ROOT, "paper_1904_10070_gb300", "csrc", "vlb_stage.cu")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "stage_kernel_fp32_uw3_coarsen_1024x2048.md")
 
 
@@ -68,18 +66,18 @@ def _peaks():
 
 
 def _traffic_per_launch():
-    """DRAM bytes per stage launch from the committed ncu summary, if it was taken on this source."""
+    """DRAM bytes per stage launch from the committed ncu summary, if it was taken on these sources."""
+    from paper_1904_10070_gb300 import build
     try:
         txt = open(TRAFFIC_FILE).read()
     except OSError:
         return None
-    src_hash = hashlib.sha256(open(STAGE_SRC, "rb").read()).hexdigest()[:16]
     vals = {}
     for line in txt.splitlines():
         if ":" in line and line.startswith("- "):
             k, v = line[2:].split(":", 1)
             vals[k.strip()] = v.strip().strip("`")
-    if vals.get("stage_source_sha256_16") != src_hash:
+    if vals.get("stage_source_sha256_16") != build.stage_tag():
         return None
     try:
         return float(vals["dram_bytes_per_launch"])
