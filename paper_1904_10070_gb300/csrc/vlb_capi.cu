@@ -20,7 +20,6 @@
 #include <vector>
 
 #include "vlb_handle.cuh"
-#include "vlb_node.cuh"
 
 // Raises the handle's device flag when a diagnostic vector shows an unstable state.
 cudaError_t vlb_internal_flag(const double* diag, int* flag, cudaStream_t s);
@@ -165,20 +164,6 @@ void row_tables(const vlb_params* p, double* out) {
   }
 }
 
-// Row table of the FP32 pair kernels (RowEntry in vlb_node.cuh) from the FP64 coefficient tables.
-void pair_rows(const vlb_params* p, const double* tab, float* out) {
-  constexpr vlb::RowRules<double> rules = vlb::make_row_rules<double>();
-  const int nt = p->n_theta;
-  for (int q = 0; q < nt; ++q)
-    for (int e = 0; e < vlb::kRowTable; ++e) {
-      const vlb::RowRule<double>& r = rules.e[e];
-      double y = 1.0;
-      if (r.y) y = tab[vlb::C_J * nt + (q + r.y - 3 + nt) % nt];
-      const double s = r.s == 3 ? 1.0 : r.s == 2 ? p->kappa : (r.s == 1 ? p->dt * p->M : p->dt);
-      out[(size_t)q * vlb::kRowTable + e] = (float)(s * (r.c1 * tab[r.x1 * nt + q] * y + r.c2 * tab[r.x2 * nt + q]));
-    }
-}
-
 // The reference density n0 of the stored deviations from the row sums of n: the area-weighted mean
 // sum_q J_q row_q / sum_q J_q N_phi (J_q = 1 + (r/R) cos theta_q), rounded to 20 significant bits so
 // that it is exact in FP32.  False if it is not finite and positive.
@@ -236,15 +221,11 @@ vlb_status upload_tables(vlb_handle* h) {
     else
       ((float*)tabT)[i] = (float)tab[i];
   }
-  std::vector<float> rows;
   cudaError_t e = cudaMemcpyAsync(h->coefD, tab, sizeof(double) * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->coefT, tabT, h->esize * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess && h->rows) {
-    rows.resize((size_t)nt * vlb::kRowTable);
-    pair_rows(p, tab, rows.data());
-    e = cudaMemcpyAsync(h->rows, rows.data(), sizeof(float) * rows.size(), cudaMemcpyHostToDevice, h->stream);
-  }
+  if (e == cudaSuccess && h->rows)
+    e = vlb::launch_pair_rows(h->coefD, nt, p->dt, p->M, p->kappa, h->rows, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   free(tab);
   free(tabT);
@@ -619,12 +600,8 @@ vlb_status vlb_create(const vlb_params* p, void* d_workspace, size_t bytes, void
   e = cudaMemcpyAsync(h->coefD, tab, sizeof(double) * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->coefT, tabT, L.esize * vlb::NCOEF * nt, cudaMemcpyHostToDevice, h->stream);
-  std::vector<float> rows;
-  if (e == cudaSuccess && h->rows) {
-    rows.resize((size_t)nt * vlb::kRowTable);
-    pair_rows(p, tab, rows.data());
-    e = cudaMemcpyAsync(h->rows, rows.data(), sizeof(float) * rows.size(), cudaMemcpyHostToDevice, h->stream);
-  }
+  if (e == cudaSuccess && h->rows)
+    e = vlb::launch_pair_rows(h->coefD, nt, p->dt, p->M, p->kappa, h->rows, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.off_U[0], 0, L.off_staging - L.off_U[0], h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream);
   std::vector<double> lam;

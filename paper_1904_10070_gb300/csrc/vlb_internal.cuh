@@ -180,6 +180,8 @@ cudaError_t launch_structure_sums(int nt, int ns, double r, double R, const T* p
                                   double* part, cudaStream_t st);
 
 // Auxiliary kernels (vlb_aux.cu).  Staging arrays are FP64 [n_theta][n_phi].
+// rows = the row table [n_theta][kRowTable] of the FP32 pair kernels (RowEntry in vlb_node.cuh) from the FP64 coefficients.
+cudaError_t launch_pair_rows(const double* coefd, int nt, double dt, double M, double kappa, float* rows, cudaStream_t s);
 // out[q] = the sum of row q of x (FP64 [nt][ns]), in a fixed order.
 cudaError_t launch_row_sums(const double* x, int nt, int ns, double* out, cudaStream_t s);
 template <typename T>
