@@ -27,17 +27,10 @@ constexpr int kMaxDevices = 64;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[VLB_NOALLOC_SCRATCH_BYTES];
 
 // Row table of the packed FP32 stages (vlb_node.cuh): they need at least 40 columns, so the scratch
-// bounds their rows.
+// bounds their rows.  Formed in FP64 and rounded once, as the handle API forms it.
 constexpr int kMaxPairRows = (int)(VLB_NOALLOC_SCRATCH_BYTES / (2 * sizeof(float) * (vlb::NARR + 1) * 40));
 static __device__ __align__(256) float g_noalloc_rows[kMaxPairRows * vlb::kRowTable];
-__device__ const vlb::RowRules<float> g_noalloc_rules = vlb::make_row_rules<float>();
-
-__global__ void noalloc_rows(vlb::StageArgs<float> a) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= a.nt * vlb::kRowTable) return;
-  const int q = x / vlb::kRowTable, e = x % vlb::kRowTable;
-  g_noalloc_rows[x] = vlb::row_entry(g_noalloc_rules.e[e], a, q, false);
-}
+__device__ const vlb::RowRules<double> g_noalloc_rules = vlb::make_row_rules<double>();
 
 std::mutex g_mu;
 void* g_scratch_ptr[kMaxDevices] = {};
@@ -61,38 +54,50 @@ cudaError_t scratch_address(int dev, void** out, void** rows) {
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Row coefficient tables (the same quantities the handle API precomputes on the host), evaluated
-// in FP64 on the device and rounded once to T.
+// Row coefficient tables (the same quantities the handle API precomputes on the host), evaluated in FP64 on the
+// device and rounded once to T, and with `rows` the row table.  A warp per row: lanes 0 .. 6 evaluate J at q - 2 .. q + 2
+// and q +- 1/2, then a lane a coefficient, then a lane an entry, so that the chain is one sine and cosine, one
+// division and a few products long (a thread per row and a second kernel for the table took 2 us more).
 template <typename T>
-__global__ void noalloc_tables(T* coef, int nt, int nphi, int geometry, int advection, double R, double r) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nt) return;
+__global__ void __launch_bounds__(64) noalloc_tables(T* coef, int nt, int nphi, int geometry, int advection, double R,
+                                                     double r, float* rows, double dt, double M, double kappa) {
+  const int q = (blockIdx.x * blockDim.x + threadIdx.x) / 32, k = threadIdx.x % 32;
+  if (q >= nt) return;  // whole warps
   const double pi = 3.14159265358979323846;
   const double dth = 2.0 * pi / nt, dph = 2.0 * pi / nphi;
   const bool torus = geometry == VLB_TORUS;
   const double a = torus ? r / R : 0.0;
-  const double th = q * dth;
-  auto Jat = [&](int d) { return 1.0 + a * cos(th + d * dth); };
-  const double J = Jat(0);
-  const double gam = torus ? sin(th) / (R * J) : 0.0;
-  coef[vlb::C_J * nt + q] = (T)J;
-  coef[vlb::C_JP * nt + q] = (T)(1.0 + a * cos(th + 0.5 * dth));
-  coef[vlb::C_JM * nt + q] = (T)(1.0 + a * cos(th - 0.5 * dth));
-  coef[vlb::C_CT * nt + q] = (T)(1.0 / (r * J * dth));
-  coef[vlb::C_CP * nt + q] = (T)(1.0 / (R * J * dph));
-  coef[vlb::C_GAM * nt + q] = (T)gam;
-  coef[vlb::C_LT * nt + q] = (T)(1.0 / (r * r * J * dth * dth));
-  coef[vlb::C_LP * nt + q] = (T)(1.0 / (R * R * J * J * dph * dph));
-  coef[vlb::C_GP * nt + q] = (T)(1.0 / (2.0 * R * J * dph));
-  if (advection == VLB_UW3) {
-    const double dpos = (Jat(-2) - 6.0 * Jat(-1) + 3.0 * Jat(0) + 2.0 * Jat(1)) / 6.0;
-    const double dneg = (-2.0 * Jat(-1) - 3.0 * Jat(0) + 6.0 * Jat(1) - Jat(2)) / 6.0;
-    coef[vlb::C_EP * nt + q] = (T)(-dpos / (r * J * dth) - gam);
-    coef[vlb::C_EN * nt + q] = (T)(-dneg / (r * J * dth) - gam);
-  } else {
-    coef[vlb::C_EP * nt + q] = (T)(-gam);
-    coef[vlb::C_EN * nt + q] = (T)(-gam);
+  const double off = k < 5 ? k - 2 : (k == 5 ? 0.5 : (k == 6 ? -0.5 : 0.0));
+  double sn, cs;
+  sincos(q * dth + off * dth, &sn, &cs);
+  const double own = 1.0 + a * cs;
+  auto J = [&](int lane) { return __shfl_sync(0xffffffffu, own, lane); };
+  const double J0 = J(2), Jm1 = J(1), Jm2 = J(0), Jp1 = J(3), Jp2 = J(4), Jp = J(5), Jm = J(6);
+  sn = __shfl_sync(0xffffffffu, sn, 2);
+  double num = 1.0, den = 1.0;
+  switch (k) {
+    case vlb::C_J: num = J0; break;
+    case vlb::C_JP: num = Jp; break;
+    case vlb::C_JM: num = Jm; break;
+    case vlb::C_CT: den = r * J0 * dth; break;
+    case vlb::C_CP: den = R * J0 * dph; break;
+    case vlb::C_GAM: num = torus ? sn : 0.0; den = R * J0; break;
+    case vlb::C_LT: den = r * r * J0 * dth * dth; break;
+    case vlb::C_LP: den = R * R * J0 * J0 * dph * dph; break;
+    case vlb::C_GP: den = 2.0 * R * J0 * dph; break;
+    case vlb::C_EP: num = -(Jm2 - 6.0 * Jm1 + 3.0 * J0 + 2.0 * Jp1) / 6.0; den = r * J0 * dth; break;
+    case vlb::C_EN: num = -(-2.0 * Jm1 - 3.0 * J0 + 6.0 * Jp1 - Jp2) / 6.0; den = r * J0 * dth; break;
   }
+  double c = num / den;
+  const double gam = __shfl_sync(0xffffffffu, c, vlb::C_GAM);
+  if (k == vlb::C_EP || k == vlb::C_EN) c = (advection == VLB_UW3 ? c : 0.0) - gam;
+  if (k <= vlb::C_EN) coef[k * nt + q] = (T)c;
+  if (!rows) return;
+  const vlb::RowRule<double> e = g_noalloc_rules.e[k];
+  const double x1 = __shfl_sync(0xffffffffu, c, e.x1), x2 = __shfl_sync(0xffffffffu, c, e.x2);
+  const double y = __shfl_sync(0xffffffffu, own, e.y ? e.y - 1 : 0);
+  const double s = e.s == 3 ? 1.0 : e.s == 2 ? kappa : (e.s == 1 ? dt * M : dt);
+  rows[q * vlb::kRowTable + k] = (float)(s * (e.c1 * x1 * (e.y ? y : 1.0) + e.c2 * x2));
 }
 
 const char* check_params(const vlb_params* p) {
@@ -118,7 +123,9 @@ cudaError_t run(const vlb_params* p, T* state, int64_t stride, double n0, int64_
   T* coef = reinterpret_cast<T*>(scratch);
   T* U1 = reinterpret_cast<T*>(scratch + align256(sizeof(T) * vlb::NCOEF * nt));
   T* U2 = U1 + (size_t)vlb::state_arrays(sizeof(T)) * stride;
-  noalloc_tables<T><<<(nt + 127) / 128, 128, 0, st>>>(coef, nt, p->n_phi, p->geometry, p->advection, p->R, p->r);
+  const bool pairs = sizeof(T) == 4 && p->advection == VLB_UW3 && vlb::stage_maps_apply(nt, p->n_phi);
+  noalloc_tables<T><<<(nt + 1) / 2, 64, 0, st>>>(coef, nt, p->n_phi, p->geometry, p->advection, p->R, p->r,
+                                                 pairs ? rows : nullptr, p->dt, p->M, p->kappa);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   vlb::StageArgs<T> a;
@@ -135,11 +142,7 @@ cudaError_t run(const vlb_params* p, T* state, int64_t stride, double n0, int64_
   a.n0 = (T)n0;
   a.err = nullptr;
   if constexpr (sizeof(T) == 4) {
-    if (p->advection == VLB_UW3 && vlb::stage_maps_apply(nt, p->n_phi)) {
-      a.rows = rows;
-      noalloc_rows<<<(nt * vlb::kRowTable + 127) / 128, 128, 0, st>>>(a);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    if (pairs) a.rows = rows;
   }
   for (int64_t n = 0; n < nsteps; ++n) {
     a.fin = state; a.f0 = nullptr; a.fout = U1; a.b = (T)1;
