@@ -54,7 +54,9 @@ struct Lay {
   static constexpr bool DF = sizeof(T) == 4;       // phi as a float pair
   static constexpr int H = H_, TQ = TQ_, HS = HS_, NTH = NTH_, NBUF = NBUF_;
   static constexpr int NST = DF ? NARR + 1 : NARR;  // state arrays (= staged boxes)
-  static constexpr int NU0 = NPOP;                   // arrays of the staged U^n tile (phi comes from L2)
+  // arrays of the staged U^n tile: with 16 rows phi too (two CTAs per SM either way; from L2 it is a wait of its own in
+  // every tile, 0.50 against 0.45 ms a step in the wavefront schedule), with 8 rows from L2, to fit four CTAs
+  static constexpr int NU0 = TQ == 16 ? NST : NPOP;
   static constexpr int BQ = TQ + 2 * H, BS = TS + 2 * HS;
   static constexpr int BOX = NST * BQ * BS;          // populations, phi (, phi lo)
   // moment / mu box: halo 1, column origin -2; column TS of a row takes the next row's unused column -2
@@ -389,8 +391,8 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
     const T lo = DF ? sphl[bi] : T(0);
     T base = ph, base_lo = lo, inc = Lphi * a.dt;
     if (F0) {
-      base = __ldcg(a.f0 + NPOP * stride + gidx);
-      base_lo = DF ? __ldcg(a.f0 + (NPOP + 1) * stride + gidx) : T(0);
+      base = L::NU0 > NPOP ? su0[NPOP * TQ * TS + ui] : __ldcg(a.f0 + NPOP * stride + gidx);
+      base_lo = L::NU0 > NPOP ? su0[(NPOP + 1) * TQ * TS + ui] : __ldcg(a.f0 + (NPOP + 1) * stride + gidx);
       inc = a.b * (((ph - base) + (lo - base_lo)) + inc);
     }
     if (DF) {
@@ -574,10 +576,10 @@ __device__ __forceinline__ void phase2_pair(const StageArgs<float>& a, const Nod
 }
 
 // phi of U^n at a thread's pair of nodes, loaded before step 2 so that it is in flight meanwhile; from L2, since
-// a persistent launch may hold a line of an earlier step in L1.
-template <bool F0>
+// a persistent launch may hold a line of an earlier step in L1.  Not where the staged tile has it.
+template <typename L, bool F0>
 __device__ __forceinline__ void load_u0_phi(const StageArgs<float>& a, int q, int s, float2& hi, float2& lo) {
-  if (F0 && !a.dphi && q < a.nt && s < a.ns) {
+  if (L::NU0 == NPOP && F0 && !a.dphi && q < a.nt && s < a.ns) {
     const float* p = a.f0 + NPOP * a.stride + (int64_t)q * a.ns + s;
     hi = __ldcg(reinterpret_cast<const float2*>(p));
     lo = __ldcg(reinterpret_cast<const float2*>(p + a.stride));
@@ -631,8 +633,8 @@ __device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const Nod
   } else {
     float2 base = n.ph, base_lo = n.lo, inc = Lp;
     if (F0) {
-      base = u0_hi;
-      base_lo = u0_lo;
+      base = L::NU0 > NPOP ? ld2(su0 + NPOP * TQ * TS + ui) : u0_hi;
+      base_lo = L::NU0 > NPOP ? ld2(su0 + (NPOP + 1) * TQ * TS + ui) : u0_lo;
       inc = vmul(f2(a.b), vadd(vadd(vsub(n.ph, base), vsub(n.lo, base_lo)), Lp));
     }
     float2 hi_o, lo_o;
@@ -721,7 +723,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VCons
   const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));  // the thread's pair of nodes
   const int q = q0 + lr, s = s0 + lc;                        // n_phi is even, so s + 1 < n_phi whenever s < n_phi
   float2 u0_hi = f2(0.0f), u0_lo = f2(0.0f);
-  if (pair) load_u0_phi<F0>(a, q, s, u0_hi, u0_lo);
+  if (pair) load_u0_phi<L, F0>(a, q, s, u0_hi, u0_lo);
   cp_async_wait<1>();  // the box; U^n may still be in flight
   __syncthreads();
   if (pair) {
@@ -793,7 +795,7 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
   }
   const int lr = tid / (TS / 2), lc = 2 * (tid % (TS / 2));
   float2 u0_hi = f2(0.0f), u0_lo = f2(0.0f);
-  load_u0_phi<F0>(a, q0 + lr, s0 + lc, u0_hi, u0_lo);
+  load_u0_phi<L, F0>(a, q0 + lr, s0 + lc, u0_hi, u0_lo);
   cp_async_wait<0>();
   bool ok = mbar_wait(bar, ph_box);
   if (__syncthreads_or(!ok)) {  // a copy did not land: flag it, let the copies settle, skip the tile
@@ -1460,7 +1462,7 @@ cudaError_t make_stage_maps(const float* fin, const float* f0, int nt, int ns, i
   if (!stage_maps_apply(nt, ns) || stride % 4 != 0 || ((uintptr_t)fin) % 16 != 0 || ((uintptr_t)f0) % 16 != 0)
     return cudaErrorInvalidValue;
   cudaError_t e = encode_state_map(&out->box, fin, nt, ns, stride, L::BS, rows + 2 * L::H, L::NST);
-  if (e == cudaSuccess) e = encode_state_map(&out->tile, f0, nt, ns, stride, TS, rows, L::NU0);
+  if (e == cudaSuccess) e = encode_state_map(&out->tile, f0, nt, ns, stride, TS, rows, rows == 16 ? StageLayR<16>::NU0 : StageLayR<8>::NU0);
   return e;
 }
 
