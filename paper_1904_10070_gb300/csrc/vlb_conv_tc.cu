@@ -262,14 +262,17 @@ __device__ __forceinline__ void transpose_chunks(uint4* a, int lane) {
   }
 }
 
-// The mask of a thread's outputs, loaded before the accumulator is waited for.  64 channels: chunk lane % 8 of the
-// eight pixels of the lane's group (the order of the stores after the transpose); 16 channels: the thread's pixel.
+// The mask of a thread's outputs, loaded before the accumulator is waited for.  64 channels in bf16: chunk lane % 8 of the
+// eight pixels of the lane's group (the order of the stores after the transpose); 16 channels, or FP32 outputs alone
+// (`own`): the thread's pixel.
 template <int COUT>
-__device__ __forceinline__ void load_mask(uint4* mk, const bf16* mask, size_t p0, int warp, int lane) {
-  const bf16* base = COUT == 64 ? mask + (p0 + 32 * warp + (lane & ~7)) * 64 + (lane & 7) * 8
-                                : mask + (p0 + 32 * warp + lane) * COUT;
+__device__ __forceinline__ void load_mask(uint4* mk, const bf16* mask, size_t p0, int warp, int lane, bool own) {
+  const bool turned = COUT == 64 && !own;
+  const bf16* base = turned ? mask + (p0 + 32 * warp + (lane & ~7)) * 64 + (lane & 7) * 8
+                            : mask + (p0 + 32 * warp + lane) * COUT;
+  const int step = turned ? 64 : 8;
 #pragma unroll
-  for (int i = 0; i < COUT / 8; ++i) mk[i] = *reinterpret_cast<const uint4*>(base + (COUT == 64 ? i * 64 : i * 8));
+  for (int i = 0; i < COUT / 8; ++i) mk[i] = *reinterpret_cast<const uint4*>(base + i * step);
 }
 
 // bf16 outputs o whose mask is not > 0 become zero
@@ -282,7 +285,8 @@ __device__ __forceinline__ void apply_mask(uint4& o, const uint4& mk) {
 }
 
 // Epilogue of the work item whose first pixel is p0 from the accumulator at column `col0`: thread (warp, lane) owns
-// pixel p0 + 32 warp + lane; all C_out columns are read before one wait.  mk: load_mask, for the bf16 output.
+// pixel p0 + 32 warp + lane; all C_out columns are read before one wait.  mk: load_mask, for the bf16 output, or for the
+// FP32 output where it is the only one.
 // The bf16 rows of 64 channels are transposed among eight lanes first, so that a store instruction writes four whole
 // 128-byte pixels instead of 16 bytes of 32 pixels.
 template <int COUT>
@@ -311,7 +315,7 @@ __device__ __forceinline__ void epilogue(uint32_t tmem, uint32_t col0, size_t p0
     for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
     if (yf) {
       if (mask) {
-        const uint4 m0 = *reinterpret_cast<const uint4*>(mask + p * COUT + co);
+        const uint4 m0 = y ? *reinterpret_cast<const uint4*>(mask + p * COUT + co) : mk[j];
         const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m0);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -502,7 +506,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
     for (int k = a; k < nmine && ok; k += 2) {
       const size_t p0 = item_pixel(H, W, blockIdx.x + k * gridDim.x);
       uint4 mk[COUT / 8];
-      if (mask && y) load_mask<COUT>(mk, mask, p0, quarter, lane);
+      if (mask) load_mask<COUT>(mk, mask, p0, quarter, lane, !y);
       ok = __all_sync(~0u, mbar_wait(afull + a, (k >> 1) & 1));
       if (!ok) break;
       tc_fence_after();
