@@ -456,17 +456,29 @@ namespace {
 // into one), the mirrored half enters by weight 2, and one root serves the modes m and -m.  A column CTA sums
 // S and |k| S over its strip (k = (m'/r, n'/R), m' and n' the signed frequencies; the mean mode m = n = 0 is left
 // out) and writes the two sums to part[2 b], part[2 b + 1].  The twiddles are tabulated once per call instead
-// of by every CTA.  1024 x 2048: 338 + 324 us for complex transforms with per-CTA twiddles, 123 + 145 us now.
+// of by every CTA.  1024 x 2048: 338 + 324 us for complex transforms with per-CTA twiddles, 123 + 145 us now.  On grids
+// of at most kOwnTwiddles rows and columns a CTA forms its own: two values a thread at most, less than the launch.
+
+constexpr int kOwnTwiddles = 64;
+
+// entry k of a per-level twiddle table
+__device__ __forceinline__ C2<double> sf_twiddle(int k) {
+  const int half = 1 << (31 - __clz(k + 1));  // a level's first entry is half - 1 (twiddle order of fft_strided)
+  double sn, cs;
+  sincospi(-(double)(k + 1 - half) / half, &sn, &cs);
+  return {cs, sn};
+}
+__device__ __forceinline__ void sf_twiddles(C2<double>* tw, const C2<double>* table, int n) {
+  if (table) return load_twiddles(tw, table, n);
+  for (int k = threadIdx.x; k < n - 1; k += blockDim.x) tw[k] = sf_twiddle(k);
+}
 
 __global__ void sf_twiddle_kernel(C2<double>* tw_s, int ns, C2<double>* tw_t, int nt) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const bool first = x < ns - 1;
   const int k = first ? x : x - (ns - 1);
   if (k >= nt - 1 && !first) return;
-  const int half = 1 << (31 - __clz(k + 1));  // a level's first entry is half - 1 (twiddle order of fft_strided)
-  double sn, cs;
-  sincospi(-(double)(k + 1 - half) / half, &sn, &cs);
-  (first ? tw_s : tw_t)[k] = {cs, sn};
+  (first ? tw_s : tw_t)[k] = sf_twiddle(k);
 }
 
 // Rows 2 b and 2 b + 1 -> their spectra at 0 .. N_phi / 2 - 1, entry 0 holding the real values at 0 and N_phi / 2.
@@ -483,7 +495,7 @@ __global__ void __launch_bounds__(256) sf_row_kernel(int ns, int logns, const T*
     a[padded(bitrev(s, logns), sh)] = {(double)phi[g] + (phi_lo ? (double)phi_lo[g] : 0.0),
                                        (double)phi[h] + (phi_lo ? (double)phi_lo[h] : 0.0)};
   }
-  load_twiddles(tw, tw_s, ns);
+  sf_twiddles(tw, tw_s, ns);
   __syncthreads();
   fft_strided(a, ns, logns, 0, sh, tw, false);
   C2<double>*r0 = buf + q * nh, *r1 = r0 + nh;
@@ -510,7 +522,7 @@ __global__ void __launch_bounds__(256) sf_col_kernel(int nt, int lognt, int ns, 
     const int q = idx >> lcw, c = idx & (cw - 1);
     a[(bitrev(q, lognt) << lcw) + c] = buf[(int64_t)q * nh + n0 + c];
   }
-  load_twiddles(tw, tw_t, nt);
+  sf_twiddles(tw, tw_t, nt);
   __syncthreads();
   fft_strided(a, nt, lognt, lcw, 31, tw, false);
   double s_sum = 0.0, k_sum = 0.0;
@@ -569,6 +581,7 @@ cudaError_t launch_structure_sums(int nt, int ns, double r, double R, const T* p
   const int lognt = ilog2(nt), logns = ilog2(ns), lcw = sf_strip(nt, ns);
   C2<double>* cb = reinterpret_cast<C2<double>*>(buf);
   C2<double>*tw_s = cb + (size_t)nt * ns / 2, *tw_t = tw_s + (ns - 1);  // (nt - 2) (ns - 2) >= 0: they fit
+  if (nt <= kOwnTwiddles && ns <= kOwnTwiddles) tw_s = tw_t = nullptr;
   const size_t row_bytes = sizeof(C2<double>) * ((size_t)ns * 2 + 32);
   const size_t col_bytes = sizeof(C2<double>) * (((size_t)nt << lcw) + nt);
   constexpr size_t row_max = sizeof(C2<double>) * (4096 * 2 + 32);
@@ -577,8 +590,10 @@ cudaError_t launch_structure_sums(int nt, int ns, double r, double R, const T* p
   cudaError_t e;
   if ((e = smem_attr(sf_row_kernel<T>, row_max, m1)) != cudaSuccess) return e;
   if ((e = smem_attr(sf_col_kernel, col_max, m2)) != cudaSuccess) return e;
-  sf_twiddle_kernel<<<(ns + nt - 2 + 127) / 128, 128, 0, st>>>(tw_s, ns, tw_t, nt);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (tw_s) {
+    sf_twiddle_kernel<<<(ns + nt - 2 + 127) / 128, 128, 0, st>>>(tw_s, ns, tw_t, nt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   sf_row_kernel<T><<<nt / 2, 256, row_bytes, st>>>(ns, logns, phi, phi_lo, tw_s, cb);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   sf_col_kernel<<<structure_blocks(nt, ns), 256, col_bytes, st>>>(nt, lognt, ns, lcw, 1.0 / r, 1.0 / R, tw_t, cb, part);
