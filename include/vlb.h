@@ -208,7 +208,10 @@ vlb_status vlb_test_wave_timeout(vlb_handle* h, int32_t skip_cta, int64_t budget
 
 /* Test hook (not part of the method): the steps of solver h take paths that otherwise only other grids or devices
  * reach; the results are the same.  routes: a sum of VLB_TEST_*, 0 restores normal operation. */
-enum { VLB_TEST_WIDE_OFFSETS = 1 /* FP64 stages: the 64-bit offsets of grids of 2^29 nodes and more */ };
+enum {
+  VLB_TEST_WIDE_OFFSETS = 1,     /* FP64 stages: the 64-bit offsets of grids of 2^29 nodes and more */
+  VLB_TEST_PORTABLE_CLUSTER = 2  /* columns (n_phi = 1): clusters of eight CTAs, of a device that refuses sixteen */
+};
 vlb_status vlb_test_route(vlb_handle* h, int32_t routes);
 
 /* Message of the last failure on h (or of the calling thread's last handle-less failure when

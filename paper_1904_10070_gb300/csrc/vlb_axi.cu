@@ -112,17 +112,21 @@ __device__ __forceinline__ void push(uint32_t addr, double v, uint32_t bar) {
 }
 
 // rows of CTA c of nc: the first nt % nc CTAs own one row more
-__host__ __device__ __forceinline__ int axi_first(int nt, int nc, int c) {
+__host__ __device__ constexpr int axi_first(int nt, int nc, int c) {
   return c * (nt / nc) + (c < nt % nc ? c : nt % nc);
 }
-__host__ __device__ __forceinline__ int axi_count(int nt, int nc, int c) { return nt / nc + (c < nt % nc ? 1 : 0); }
+__host__ __device__ constexpr int axi_count(int nt, int nc, int c) { return nt / nc + (c < nt % nc ? 1 : 0); }
+
+constexpr size_t kSmemMax = 232448;  // opt-in shared memory of one CTA
 
 // pitch of one array of a state buffer: the rows and their halos, padded so that the four velocity rows
-// of a warp (4 pitch apart) fall on different banks
-__host__ __device__ __forceinline__ int axi_pitch(int rows, int H) {
+// of a warp (4 pitch apart) fall on different banks, unless the padding is what does not fit (the longest FP64
+// columns on eight CTAs)
+template <typename T>
+__host__ __device__ constexpr int axi_pitch(int rows, int H) {
   int p = rows + 2 * H;
   while (p % 8 != 2) ++p;
-  return p;
+  return 32 + sizeof(T) * ((size_t)3 * state_arrays(sizeof(T)) * p + 5 * (size_t)(rows + 2)) <= kSmemMax ? p : rows + 2 * H;
 }
 
 // FP32 UW3 columns read the handle's row table; the others form an AxiRow from the coefficient arrays
@@ -130,12 +134,17 @@ template <typename T, int ADV>
 __host__ __device__ constexpr bool row_table() { return sizeof(T) == 4 && ADV == VLB_UW3; }
 
 template <typename T, int ADV>
-size_t axi_smem(int nt, int nc, bool table) {
+constexpr size_t axi_smem(int nt, int nc, bool table) {
   const int rmax = axi_count(nt, nc, 0), H = ADV == VLB_UW3 ? 2 : 3;
-  const size_t elems = (size_t)3 * state_arrays(sizeof(T)) * axi_pitch(rmax, H) + 5 * (size_t)(rmax + 2) +
+  const size_t elems = (size_t)3 * state_arrays(sizeof(T)) * axi_pitch<T>(rmax, H) + 5 * (size_t)(rmax + 2) +
                        (table ? (size_t)(rmax + 2) * (row_table<T, ADV>() ? kRowVals : sizeof(AxiRow<T>) / sizeof(T)) : 0);
   return 32 + elems * sizeof(T);
 }
+static_assert(axi_smem<double, VLB_UW3>(kAxiMaxRows, kAxiPortable, false) <= kSmemMax &&
+                  axi_smem<double, VLB_WENO5>(kAxiMaxRows, kAxiPortable, false) <= kSmemMax &&
+                  axi_smem<float, VLB_UW3>(kAxiMaxRows, kAxiPortable, true) <= kSmemMax &&
+                  axi_smem<float, VLB_WENO5>(kAxiMaxRows, kAxiPortable, false) <= kSmemMax,
+              "every column fits a cluster of the portable size");
 
 // `steps` SSP-RK3 steps in the Shu-Osher form of run_steps: U1 = U + dt L(U); U2 = U + 1/4 (U1 - U + dt L(U1));
 // U <- U + 2/3 (U2 - U + dt L(U2)).  The third stage writes U in place: a thread reads its own U before it
@@ -148,7 +157,7 @@ __global__ void __launch_bounds__(kAxiThreads) axi_kernel(StageArgs<T> a, const 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nt = a.nt, nc = gridDim.x, c = blockIdx.x, tid = threadIdx.x;  // one cluster: rank = blockIdx.x
   const int r0 = axi_first(nt, nc, c), R = axi_count(nt, nc, c), rmax = axi_count(nt, nc, 0);
-  const int P = axi_pitch(rmax, H), SZ = NST * P;
+  const int P = axi_pitch<T>(rmax, H), SZ = NST * P;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);  // [from prev, from next][parity of the stage]
   T* buf = reinterpret_cast<T*>(smem_raw + 32);  // three states, array k of state s at buf + s SZ + k P, row r at H + r
   T *s_dn = buf + 3 * SZ, *s_in = s_dn + rmax + 2, *s_ut = s_in + rmax + 2, *s_up = s_ut + rmax + 2;
@@ -372,7 +381,7 @@ constexpr int kAxi16Rows = 30;
 
 __host__ __device__ __forceinline__ size_t axi16_smem(int nt, int nc) {
   const int rmax = axi_count(nt, nc, 0);
-  return sizeof(float) * (8 + (size_t)3 * (NARR + 1) * axi_pitch(rmax, 2) + 2 * (size_t)(rmax + 2));
+  return sizeof(float) * (8 + (size_t)3 * (NARR + 1) * axi_pitch<float>(rmax, 2) + 2 * (size_t)(rmax + 2));
 }
 
 template <int CH>
@@ -382,7 +391,7 @@ __global__ void __launch_bounds__(512) axi16_kernel(StageArgs<float> a, const __
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nt = a.nt, nc = gridDim.x, c = blockIdx.x, tid = threadIdx.x;  // one cluster: rank = blockIdx.x
   const int r0 = axi_first(nt, nc, c), R = axi_count(nt, nc, c), rmax = axi_count(nt, nc, 0);
-  const int P = axi_pitch(rmax, H), SZ = NST * P;
+  const int P = axi_pitch<float>(rmax, H), SZ = NST * P;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);  // [from prev, from next][parity of the stage]
   float* buf = reinterpret_cast<float*>(smem_raw) + 8;
   float *s_mu = buf + 3 * SZ, *s_ut = s_mu + rmax + 2;
@@ -538,8 +547,6 @@ AxiConst<T> make_axi_const() {
   return c;
 }
 
-constexpr size_t kSmemMax = 232448;  // opt-in shared memory of one CTA
-
 cudaLaunchConfig_t axi_config(int nc, int threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nc);
@@ -587,6 +594,7 @@ cudaError_t launch_axi_t(const StageArgs<T>& a, T* U, int steps, cudaStream_t st
   if constexpr (sizeof(T) == 4 && ADV == VLB_UW3) {
     static int most16[32] = {0};
     if ((e = axi_most(axi16_kernel<CH>, most16, &nc)) != cudaSuccess) return e;
+    if (a.route & VLB_TEST_PORTABLE_CLUSTER) nc = kAxiPortable;
     nc = std::min(nc, std::max(1, a.nt / 8));
     const int rows = axi_count(a.nt, nc, 0);
     if (rows <= kAxi16Rows) {
@@ -596,10 +604,11 @@ cudaError_t launch_axi_t(const StageArgs<T>& a, T* U, int steps, cudaStream_t st
   }
   static int most[32] = {0};
   if ((e = axi_most(axi_kernel<T, ADV, CH>, most, &nc)) != cudaSuccess) return e;
+  if (a.route & VLB_TEST_PORTABLE_CLUSTER) nc = kAxiPortable;
   nc = std::min(nc, std::max(1, a.nt / 4));
   const bool table = axi_smem<T, ADV>(a.nt, nc, true) <= kSmemMax;
   const size_t smem = axi_smem<T, ADV>(a.nt, nc, table);
-  if (smem > kSmemMax) return cudaErrorInvalidValue;  // kAxiMaxRows rows fit a portable cluster
+  if (smem > kSmemMax) return cudaErrorInvalidValue;  // never: see the assertion at axi_smem
   const cudaLaunchConfig_t cfg = axi_config(nc, kAxiThreads, smem, st, attr);
   return cudaLaunchKernelEx(&cfg, axi_kernel<T, ADV, CH>, a, ac, U, steps, table ? 1 : 0);
 }

@@ -241,7 +241,7 @@ def vlb_interface_length(h) -> float:
 
 
 SCHED_AUTO, SCHED_STAGES, SCHED_WAVE = 0, 1, 2
-TEST_WIDE_OFFSETS = 1
+TEST_WIDE_OFFSETS, TEST_PORTABLE_CLUSTER = 1, 2
 
 
 def vlb_set_schedule(h, schedule: int):
