@@ -203,17 +203,19 @@ __global__ void sum_final_kernel(int nb, const double* part, double scale, doubl
 }
 
 // Adam (Kingma & Ba 2015) on FP32 master parameters; optionally refreshes a BF16 copy.
-// One Adam step on up to kAdamTensors tensors: block b works on the tensor whose blocks first[t] .. first[t + 1] - 1
-// hold it.  The update is a few KB to a few hundred KB per tensor, so a launch each was all latency: the sixteen
+// One Adam step on up to N tensors: block b works on the tensor whose blocks first[t] .. first[t + 1] - 1 hold it.  The update is a few KB to a few hundred KB per tensor, so a launch each was all latency: the sixteen
 // tensors of the surrogate network took 16 x 3.5 us, one launch of them all brought a training
-// iteration at 256 x 512 from 575 to 516 us.
+// iteration at 256 x 512 from 575 to 516 us.  A single tensor has a launch of its own with N = 1: 1.7 KB of
+// parameters cost the call about 1 us.
+template <int N>
 struct AdamBatch {
   int count;
-  int first[kAdamTensors + 1];
-  AdamTensor t[kAdamTensors];
+  int first[N + 1];
+  AdamTensor t[N];
 };
 
-__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamBatch a, float lr, float b1, float b2,
+template <int N>
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamBatch<N> a, float lr, float b1, float b2,
                                                    float eps, float c1, float c2) {
   int k = 0;
   while (k + 1 < a.count && (int)blockIdx.x >= a.first[k + 1]) ++k;
@@ -301,14 +303,19 @@ cudaError_t sur_mse(int64_t n, const float* pred, const float* target, void* gra
 cudaError_t sur_adam(int count, const AdamTensor* tensors, int64_t t, float lr, float b1, float b2, float eps,
                      cudaStream_t st) {
   const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
+  if (count == 1) {
+    AdamBatch<1> a = {1, {0, blocks_for(tensors[0].n)}, {tensors[0]}};
+    adam_kernel<1><<<a.first[1], 256, 0, st>>>(a, lr, b1, b2, eps, c1, c2);
+    return cudaGetLastError();
+  }
   for (int k0 = 0; k0 < count; k0 += kAdamTensors) {
-    AdamBatch a = {};
+    AdamBatch<kAdamTensors> a = {};
     a.count = count - k0 < kAdamTensors ? count - k0 : kAdamTensors;
     for (int k = 0; k < a.count; ++k) {
       a.t[k] = tensors[k0 + k];
       a.first[k + 1] = a.first[k] + blocks_for(a.t[k].n);
     }
-    adam_kernel<<<a.first[a.count], 256, 0, st>>>(a, lr, b1, b2, eps, c1, c2);
+    adam_kernel<kAdamTensors><<<a.first[a.count], 256, 0, st>>>(a, lr, b1, b2, eps, c1, c2);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
