@@ -41,50 +41,39 @@ namespace {
 constexpr int TS = 32;   // tile width along varphi
 constexpr int NCT = 11;  // coefficient rows staged in shared memory (C_J .. C_EN)
 
-template <typename T>
 struct VConst {
-  T v[4], w[4], K[4][4];
-  T ww[4][4];  // w_i w_j
-  NodeConst<T> nc;
+  float v[4], w[4], K[4][4];
+  float ww[4][4];  // w_i w_j
+  NodeConst<float> nc;
 };
 
-// Shared-memory layout of one CTA.  Offsets are in elements of T.
-template <typename T, int H_, int TQ_, int HS_, int NTH_, int NBUF_>
-struct Lay {
-  static constexpr bool DF = sizeof(T) == 4;       // phi as a float pair
-  static constexpr int H = H_, TQ = TQ_, HS = HS_, NTH = NTH_, NBUF = NBUF_;
-  static constexpr int NST = DF ? NARR + 1 : NARR;  // state arrays (= staged boxes)
+// Shared-memory layout of one CTA of TQ rows.  Offsets are in floats.
+template <int TQ_>
+struct StageLayR {
+  static constexpr int H = 2, TQ = TQ_, HS = 4, NTH = TQ * (TS / 2);  // halo rows, halo columns staged, threads
+  static constexpr int NST = NARR + 1;  // state arrays (= staged boxes): populations, phi, phi lo
   // arrays of the staged U^n tile: with 16 rows phi too (two CTAs per SM either way; from L2 it is a wait of its own in
   // every tile, 0.50 against 0.45 ms a step in the wavefront schedule), with 8 rows from L2, to fit four CTAs
   static constexpr int NU0 = TQ == 16 ? NST : NPOP;
   static constexpr int BQ = TQ + 2 * H, BS = TS + 2 * HS;
-  static constexpr int BOX = NST * BQ * BS;          // populations, phi (, phi lo)
+  static constexpr int BOX = NST * BQ * BS;
   // moment / mu box: halo 1, column origin -2; column TS of a row takes the next row's unused column -2
   static constexpr int MQ = TQ + 2, MS = TS + 2, MN = MQ * MS + 2;
   // row coefficients: NCT x BQ for the scalar step 3, or the row table of rows -1 .. TQ for packed pairs; padded:
   // sub-buffers stay 128-byte aligned
   static constexpr int CO = ((NCT * BQ > (TQ + 2) * kRowTable ? NCT * BQ : (TQ + 2) * kRowTable) + 31) / 32 * 32;
-  static constexpr int VEC = 16 / sizeof(T);              // elements per 16-byte chunk
-  // each box row starts HS columns left of the tile: shift the buffers so that the tile columns
-  // (and every 16-byte chunk copied into them) start on a 16-byte boundary
-  static constexpr int BOX_OFF = (VEC - HS % VEC) % VEC;
-  static constexpr int CO_OFF = (BOX_OFF + NBUF * BOX + VEC - 1) / VEC * VEC;
-  static constexpr int U0_OFF = CO_OFF + NBUF * CO;
+  static constexpr int VEC = 4;  // floats per 16-byte chunk
+  static constexpr int CO_OFF = BOX;
+  static constexpr int U0_OFF = CO_OFF + CO;
   static constexpr int UT_OFF = U0_OFF + NU0 * TQ * TS;
   static constexpr int UP_OFF = UT_OFF + MN;
   static constexpr int MU_OFF = UP_OFF + MN;
   static constexpr int MB_OFF = (MU_OFF + MN + 1) / 2 * 2;  // two 8-byte mbarriers
-  static constexpr int TOTAL = MB_OFF + 16 / (int)sizeof(T);
-  static constexpr size_t BYTES = sizeof(T) * (size_t)TOTAL;
-  static_assert((BOX * sizeof(T)) % 16 == 0 && (BS * sizeof(T)) % 16 == 0 && (BQ * BS * sizeof(T)) % 16 == 0,
-                "box rows and arrays keep 16-byte alignment");
-  static_assert(((BOX_OFF + HS) * sizeof(T)) % 16 == 0, "tile columns start on a 16-byte boundary");
-  static_assert((BOX_OFF * sizeof(T)) % 8 == 0, "edge chunks are 8-byte aligned");
-  static_assert((CO_OFF * sizeof(T)) % 16 == 0 && (U0_OFF * sizeof(T)) % 16 == 0, "16-byte aligned sub-buffers");
+  static constexpr int TOTAL = MB_OFF + 4;
+  static constexpr size_t BYTES = sizeof(float) * (size_t)TOTAL;
+  static_assert(BOX % VEC == 0 && BS % VEC == 0 && HS % VEC == 0 && CO_OFF % VEC == 0 && U0_OFF % VEC == 0,
+                "box rows, tile columns and sub-buffers start on a 16-byte boundary");
 };
-
-template <int TQR>
-using StageLayR = Lay<float, 2, TQR, 4, TQR*(TS / 2), 1>;
 using StageLay = StageLayR<16>;
 
 __device__ __forceinline__ int wrap(int x, int n) {
@@ -98,9 +87,8 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst)), "l"(src));
 }
 
-template <int BYTES>
-__device__ __forceinline__ void cp_async_small(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES));
+__device__ __forceinline__ void cp_async_small(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src));
 }
 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
@@ -166,56 +154,39 @@ __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 // 16-byte chunks that never straddle the periodic seam.
 template <typename L>
 __host__ __device__ inline bool chunked(int nt, int ns) {
-  constexpr int VEC = 16 / (L::DF ? 4 : 8);
-  return ns % VEC == 0 && ns >= L::BS && nt >= L::BQ;
+  return ns % L::VEC == 0 && ns >= L::BS && nt >= L::BQ;
 }
 
 // ---------------------------------------------------------------------------------------------
 // Step 1: asynchronous copies of the box (populations and phi of U_in) with its row coefficients,
 // and of the tile's U^n.
 // ---------------------------------------------------------------------------------------------
-template <typename L, typename T>
-__device__ __forceinline__ void issue_co(const StageArgs<T>& a, T* co, int q0, int tid) {
+template <typename L>
+__device__ __forceinline__ void issue_co(const StageArgs<float>& a, float* co, int q0, int tid) {
   for (int idx = tid; idx < NCT * L::BQ; idx += L::NTH) {
     const int k = idx / L::BQ, r = idx - k * L::BQ;
-    cp_async_small<sizeof(T)>(co + idx, a.coef + (int64_t)k * a.nt + wrap(q0 + r - L::H, a.nt));
+    cp_async_small(co + idx, a.coef + (int64_t)k * a.nt + wrap(q0 + r - L::H, a.nt));
   }
 }
 
-template <typename L, typename T>
-__device__ __forceinline__ void issue_box(const StageArgs<T>& a, T* box, T* co, int q0, int s0, int tid) {
+template <typename L>
+__device__ __forceinline__ void issue_box(const StageArgs<float>& a, float* box, float* co, int q0, int s0, int tid) {
   constexpr int H = L::H, BQ = L::BQ, BS = L::BS, HS = L::HS;
-  constexpr int VEC = 16 / sizeof(T);
+  constexpr int VEC = L::VEC;
   const int nt = a.nt, ns = a.ns;
   const int64_t stride = a.stride;
   if (chunked<L>(nt, ns)) {
-    // chunk c of a box row: with HS % VEC == 0 all chunks are VEC wide; otherwise the two edge
-    // chunks are HS wide (8-byte copies) and the interior ones VEC wide.
-    constexpr bool EDGE = HS % VEC != 0;
-    constexpr int CPR = EDGE ? TS / VEC + 2 : BS / VEC;
+    constexpr int CPR = BS / VEC;  // 16-byte chunks of a box row
     for (int pos = tid; pos < BQ * CPR; pos += L::NTH) {
-      const int r = pos / CPR, ch = pos - r * CPR;
+      const int r = pos / CPR, col = (pos - r * CPR) * VEC;
       int gq = q0 + r - H;
       gq += gq < 0 ? nt : (gq >= nt ? -nt : 0);
-      int col, width;
-      if (EDGE) {
-        col = ch == 0 ? 0 : (ch == CPR - 1 ? HS + TS : HS + (ch - 1) * VEC);
-        width = (ch == 0 || ch == CPR - 1) ? HS : VEC;
-      } else {
-        col = ch * VEC;
-        width = VEC;
-      }
       int gs = s0 - HS + col;
       gs += gs < 0 ? ns : (gs >= ns ? -ns : 0);
-      const T* src = a.fin + (int64_t)gq * ns + gs;
-      T* dst = box + r * BS + col;
-      if (width == VEC) {
+      const float* src = a.fin + (int64_t)gq * ns + gs;
+      float* dst = box + r * BS + col;
 #pragma unroll
-        for (int k = 0; k < L::NST; ++k) cp_async16(dst + k * BQ * BS, src + k * stride);
-      } else {
-#pragma unroll
-        for (int k = 0; k < L::NST; ++k) cp_async_small<8>(dst + k * BQ * BS, src + k * stride);
-      }
+      for (int k = 0; k < L::NST; ++k) cp_async16(dst + k * BQ * BS, src + k * stride);
     }
   } else {
     for (int idx = tid; idx < L::NST * BQ * BS; idx += L::NTH) {
@@ -223,14 +194,14 @@ __device__ __forceinline__ void issue_box(const StageArgs<T>& a, T* box, T* co, 
       const int rem = idx - k * (BQ * BS);
       const int r = rem / BS, c = rem - r * BS;
       const int gq = wrap(q0 + r - H, nt), gs = wrap(s0 + c - HS, ns);
-      cp_async_small<sizeof(T)>(box + (k * BQ + r) * BS + c, a.fin + k * stride + (int64_t)gq * ns + gs);
+      cp_async_small(box + (k * BQ + r) * BS + c, a.fin + k * stride + (int64_t)gq * ns + gs);
     }
   }
 }
 
-template <typename L, typename T>
-__device__ __forceinline__ void issue_u0(const StageArgs<T>& a, T* su0, int q0, int s0, int tid) {
-  constexpr int TQ = L::TQ, VEC = 16 / sizeof(T);
+template <typename L>
+__device__ __forceinline__ void issue_u0(const StageArgs<float>& a, float* su0, int q0, int s0, int tid) {
+  constexpr int TQ = L::TQ, VEC = L::VEC;
   const int nt = a.nt, ns = a.ns;
   const int64_t stride = a.stride;
   if (chunked<L>(nt, ns)) {
@@ -243,8 +214,8 @@ __device__ __forceinline__ void issue_u0(const StageArgs<T>& a, T* su0, int q0, 
       const int r = pos / CT, ch = pos - r * CT;
       const int gq = q0 + r, gs = s0 + ch * VEC;
       if (gq < nt && gs < ns) {
-        const T* src = a.f0 + (int64_t)gq * ns + gs;
-        T* dst = su0 + r * TS + ch * VEC;
+        const float* src = a.f0 + (int64_t)gq * ns + gs;
+        float* dst = su0 + r * TS + ch * VEC;
         const int k0 = grp * PER, k1 = k0 + PER < L::NU0 ? k0 + PER : L::NU0;
 #pragma unroll 4
         for (int k = k0; k < k1; ++k) cp_async16(dst + k * TQ * TS, src + k * stride);
@@ -257,7 +228,7 @@ __device__ __forceinline__ void issue_u0(const StageArgs<T>& a, T* su0, int q0, 
       const int r = rem / TS, c = rem - r * TS;
       const int gq = q0 + r, gs = s0 + c;
       if (gq < nt && gs < ns)
-        cp_async_small<sizeof(T)>(su0 + (k * TQ + r) * TS + c, a.f0 + k * stride + (int64_t)gq * ns + gs);
+        cp_async_small(su0 + (k * TQ + r) * TS + c, a.f0 + k * stride + (int64_t)gq * ns + gs);
     }
   }
 }
@@ -267,55 +238,53 @@ __device__ __forceinline__ void issue_u0(const StageArgs<T>& a, T* su0, int q0, 
 // Moment-box position (mr, mc) is tile node (mr - 1, mc - 2).
 // ---------------------------------------------------------------------------------------------
 // Moments and mu at moment-box position (mr, mc).
-template <typename L, typename T>
-__device__ __forceinline__ void moment_point(const StageArgs<T>& a, const VConst<T>& vc, const T* box, const T* co,
-                                             T* sm, int mr, int mc) {
+template <typename L>
+__device__ __forceinline__ void moment_point(const StageArgs<float>& a, const VConst& vc, const float* box, const float* co,
+                                             float* sm, int mr, int mc) {
   constexpr int H = L::H, BQ = L::BQ, BS = L::BS, HS = L::HS, MS = L::MS;
-  const T* sf = box;
-  const T* sphi = box + NPOP * BQ * BS;
-  const T* sphl = box + (NPOP + 1) * BQ * BS;
+  const float* sf = box;
+  const float* sphi = box + NPOP * BQ * BS;
+  const float* sphl = box + (NPOP + 1) * BQ * BS;
   const int bi = (mr + H - 1) * BS + (mc - 2 + HS);  // box index of this position
-  const T* fp = sf + bi;
-  T row[4] = {T(0), T(0), T(0), T(0)}, col[4] = {T(0), T(0), T(0), T(0)};
+  const float* fp = sf + bi;
+  float row[4] = {0.0f, 0.0f, 0.0f, 0.0f}, col[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const T x = fp[(4 * i + j) * BQ * BS];
+      const float x = fp[(4 * i + j) * BQ * BS];
       row[i] += x;
       col[j] += x;
     }
   // n = n0 + sum g (the reference part carries no momentum); v_1 = -v_4, v_2 = -v_3
-  const T dn = (row[0] + row[1]) + (row[2] + row[3]);
-  const T mt = vc.v[3] * (row[3] - row[0]) + vc.v[2] * (row[2] - row[1]);
-  const T mp = vc.v[3] * (col[3] - col[0]) + vc.v[2] * (col[2] - col[1]);
+  const float dn = (row[0] + row[1]) + (row[2] + row[3]);
+  const float mt = vc.v[3] * (row[3] - row[0]) + vc.v[2] * (row[2] - row[1]);
+  const float mp = vc.v[3] * (col[3] - col[0]) + vc.v[2] * (col[2] - col[1]);
   const int mi = mr * MS + mc;
-  const T inv_n = recip(a.n0 + dn);
+  const float inv_n = recip(a.n0 + dn);
   sm[L::UT_OFF + mi] = node_velocity(mt, inv_n, vc.nc.fix);
   sm[L::UP_OFF + mi] = node_velocity(mp, inv_n, vc.nc.fix);
-  const T* pp = sphi + bi;
+  const float* pp = sphi + bi;
   const int cr = mr + H - 1;
-  const T ph = pp[0];
+  const float ph = pp[0];
   // neighbour differences of phi = hi + lo: the hi differences are exact for nearby values
-  T dN = pp[BS] - ph, dS = ph - pp[-BS], dE = pp[1] - ph, dW = ph - pp[-1], lo = T(0);
-  if (L::DF) {
-    const T* pl = sphl + bi;
-    lo = pl[0];
-    dN += pl[BS] - lo;
-    dS += lo - pl[-BS];
-    dE += pl[1] - lo;
-    dW += lo - pl[-1];
-  }
-  const T lap = co[C_LT * BQ + cr] * (co[C_JP * BQ + cr] * dN - co[C_JM * BQ + cr] * dS) +
-                co[C_LP * BQ + cr] * (dE - dW);
+  float dN = pp[BS] - ph, dS = ph - pp[-BS], dE = pp[1] - ph, dW = ph - pp[-1];
+  const float* pl = sphl + bi;
+  const float lo = pl[0];
+  dN += pl[BS] - lo;
+  dS += lo - pl[-BS];
+  dE += pl[1] - lo;
+  dW += lo - pl[-1];
+  const float lap = co[C_LT * BQ + cr] * (co[C_JP * BQ + cr] * dN - co[C_JM * BQ + cr] * dS) +
+                    co[C_LP * BQ + cr] * (dE - dW);
   // phi (1 - phi^2) at hi + lo, to first order in lo
-  const T cubic = ph * (T(1) - ph * ph) + (T(1) - T(3) * ph * ph) * lo;
+  const float cubic = ph * (1.0f - ph * ph) + (1.0f - 3.0f * ph * ph) * lo;
   sm[L::MU_OFF + mi] = -a.A * cubic - a.kappa * lap;
 }
 
-template <typename L, typename T>
-__device__ __forceinline__ void phase2(const StageArgs<T>& a, const VConst<T>& vc, const T* box, const T* co,
-                                       T* sm, int tid) {
+template <typename L>
+__device__ __forceinline__ void phase2(const StageArgs<float>& a, const VConst& vc, const float* box, const float* co,
+                                       float* sm, int tid) {
   constexpr int MQ = L::MQ, TQ = L::TQ;
   constexpr int MS2 = TS + 2;  // tile columns -1 .. TS in the rows of the tile
   constexpr int PA = TQ * MS2;
@@ -337,49 +306,48 @@ __device__ __forceinline__ void phase2(const StageArgs<T>& a, const VConst<T>& v
 // ---------------------------------------------------------------------------------------------
 // Step 3, scalar: right-hand sides and the Runge-Kutta combination for node (lr, lc) of the tile.
 // ---------------------------------------------------------------------------------------------
-template <typename L, typename T, int CH, bool F0>
-__device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<T>& vc, const T* box, const T* co,
-                                            const T* sm, int lr, int lc, int q, int s) {
-  constexpr bool DF = L::DF;
+template <typename L, int CH, bool F0>
+__device__ __forceinline__ void phase3_node(const StageArgs<float>& a, const VConst& vc, const float* box, const float* co,
+                                            const float* sm, int lr, int lc, int q, int s) {
   constexpr int H = L::H, BQ = L::BQ, BS = L::BS, HS = L::HS, MS = L::MS, TQ = L::TQ;
-  const T* sf = box;
-  const T* sphi = box + NPOP * BQ * BS;
-  const T* sphl = box + (NPOP + 1) * BQ * BS;
-  const T* su0 = sm + L::U0_OFF;
-  const T* sut = sm + L::UT_OFF;
-  const T* sup = sm + L::UP_OFF;
-  const T* smu = sm + L::MU_OFF;
+  const float* sf = box;
+  const float* sphi = box + NPOP * BQ * BS;
+  const float* sphl = box + (NPOP + 1) * BQ * BS;
+  const float* su0 = sm + L::U0_OFF;
+  const float* sut = sm + L::UT_OFF;
+  const float* sup = sm + L::UP_OFF;
+  const float* smu = sm + L::MU_OFF;
   const int64_t stride = a.stride;
-  const T sixth = T(1) / T(6);
+  const float sixth = 1.0f / 6.0f;
   const int fr = lr + H, fc = lc + HS;
   const int bi = fr * BS + fc;
   const int mi = (lr + 1) * MS + (lc + 2);
   const int ui = lr * TS + lc;
 
   // population deviations at the node, and their sum as in step 2
-  T g[NPOP], row[4] = {T(0), T(0), T(0), T(0)};
+  float g[NPOP], row[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
   for (int k = 0; k < NPOP; ++k) {
     g[k] = sf[k * BQ * BS + bi];
     row[k >> 2] += g[k];
   }
-  const T dn = (row[0] + row[1]) + (row[2] + row[3]), ut = sut[mi], up = sup[mi], ph = sphi[bi];
-  const T n = a.n0 + dn;
-  const T ct = co[C_CT * BQ + fr], cp = co[C_CP * BQ + fr], gam = co[C_GAM * BQ + fr];
-  const T mu_c = smu[mi], mu_n = smu[mi + MS], mu_s = smu[mi - MS], mu_e = smu[mi + 1], mu_w = smu[mi - 1];
+  const float dn = (row[0] + row[1]) + (row[2] + row[3]), ut = sut[mi], up = sup[mi], ph = sphi[bi];
+  const float n = a.n0 + dn;
+  const float ct = co[C_CT * BQ + fr], cp = co[C_CP * BQ + fr], gam = co[C_GAM * BQ + fr];
+  const float mu_c = smu[mi], mu_n = smu[mi + MS], mu_s = smu[mi - MS], mu_e = smu[mi + 1], mu_w = smu[mi - 1];
 
   // Cahn-Hilliard: M Delta mu - div(u phi) (Eq. CH), flux form with mean face values
-  T Lphi = a.M * (co[C_LT * BQ + fr] * (co[C_JP * BQ + fr] * (mu_n - mu_c) - co[C_JM * BQ + fr] * (mu_c - mu_s)) +
-                  co[C_LP * BQ + fr] * (mu_e - T(2) * mu_c + mu_w));
-  T Ft = T(0), Fp = T(0);
+  float Lphi = a.M * (co[C_LT * BQ + fr] * (co[C_JP * BQ + fr] * (mu_n - mu_c) - co[C_JM * BQ + fr] * (mu_c - mu_s)) +
+                  co[C_LP * BQ + fr] * (mu_e - 2.0f * mu_c + mu_w));
+  float Ft = 0.0f, Fp = 0.0f;
   if (CH == VLB_HYDRO) {
-    const T Xn = co[C_J * BQ + fr + 1] * sut[mi + MS] * sphi[bi + BS];
-    const T Xs = co[C_J * BQ + fr - 1] * sut[mi - MS] * sphi[bi - BS];
-    const T Ye = sup[mi + 1] * sphi[bi + 1];
-    const T Yw = sup[mi - 1] * sphi[bi - 1];
-    Lphi -= T(0.5) * (ct * (Xn - Xs) + cp * (Ye - Yw));
+    const float Xn = co[C_J * BQ + fr + 1] * sut[mi + MS] * sphi[bi + BS];
+    const float Xs = co[C_J * BQ + fr - 1] * sut[mi - MS] * sphi[bi - BS];
+    const float Ye = sup[mi + 1] * sphi[bi + 1];
+    const float Yw = sup[mi - 1] * sphi[bi - 1];
+    Lphi -= 0.5f * (ct * (Xn - Xs) + cp * (Ye - Yw));
     // n F = -phi grad mu (Eq. pbin), central differences
-    const T pn = ph * recip(n);
+    const float pn = ph * recip(n);
     Ft = -pn * (mu_n - mu_s) * a.gt;
     Fp = -pn * (mu_e - mu_w) * co[C_GP * BQ + fr];
   }
@@ -388,63 +356,59 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
   if (a.dphi) {
     a.dphi[gidx] = Lphi * a.dt;  // the stabilised Cahn-Hilliard solve forms phi
   } else {
-    const T lo = DF ? sphl[bi] : T(0);
-    T base = ph, base_lo = lo, inc = Lphi * a.dt;
+    const float lo = sphl[bi];
+    float base = ph, base_lo = lo, inc = Lphi * a.dt;
     if (F0) {
       base = L::NU0 > NPOP ? su0[NPOP * TQ * TS + ui] : __ldcg(a.f0 + NPOP * stride + gidx);
       base_lo = L::NU0 > NPOP ? su0[(NPOP + 1) * TQ * TS + ui] : __ldcg(a.f0 + (NPOP + 1) * stride + gidx);
       inc = a.b * (((ph - base) + (lo - base_lo)) + inc);
     }
-    if (DF) {
-      // (hi, lo) <- (base, base_lo) + inc with an error-free sum, then renormalised
-      const T s1 = base + inc;
-      const T bb = s1 - base;
-      const T err = (base - (s1 - bb)) + (inc - bb);
-      const T lo2 = base_lo + err;
-      const T hi_out = s1 + lo2;
-      a.fout[NPOP * stride + gidx] = hi_out;
-      a.fout[(NPOP + 1) * stride + gidx] = lo2 - (hi_out - s1);
-    } else {
-      a.fout[NPOP * stride + gidx] = base + inc;
-    }
+    // (hi, lo) <- (base, base_lo) + inc with an error-free sum, then renormalised
+    const float s1 = base + inc;
+    const float bb = s1 - base;
+    const float err = (base - (s1 - bb)) + (inc - bb);
+    const float lo2 = base_lo + err;
+    const float hi_out = s1 + lo2;
+    a.fout[NPOP * stride + gidx] = hi_out;
+    a.fout[(NPOP + 1) * stride + gidx] = lo2 - (hi_out - s1);
   }
 
   // UW3 advection weights: the theta flux difference of G = J g with ct/6 folded in, over
   // d = -2..1 (v > 0) and d = -1..2 (v < 0); the varphi difference is scaled by cp/6.
-  const T ct6 = ct * sixth, cp6 = cp * sixth;
-  const T Jm1 = co[C_J * BQ + fr - 1], J0 = co[C_J * BQ + fr], Jp1 = co[C_J * BQ + fr + 1];
-  const T wp0 = ct6 * co[C_J * BQ + fr - 2], wp1 = T(-6) * ct6 * Jm1, wp2 = T(3) * ct6 * J0, wp3 = T(2) * ct6 * Jp1;
-  const T wn0 = T(-2) * ct6 * Jm1, wn1 = T(-3) * ct6 * J0, wn2 = T(6) * ct6 * Jp1, wn3 = -ct6 * co[C_J * BQ + fr + 2];
+  const float ct6 = ct * sixth, cp6 = cp * sixth;
+  const float Jm1 = co[C_J * BQ + fr - 1], J0 = co[C_J * BQ + fr], Jp1 = co[C_J * BQ + fr + 1];
+  const float wp0 = ct6 * co[C_J * BQ + fr - 2], wp1 = -6.0f * ct6 * Jm1, wp2 = 3.0f * ct6 * J0, wp3 = 2.0f * ct6 * Jp1;
+  const float wn0 = -2.0f * ct6 * Jm1, wn1 = -3.0f * ct6 * J0, wn2 = 6.0f * ct6 * Jp1, wn3 = -ct6 * co[C_J * BQ + fr + 2];
 
-  const T usq = ut * ut + up * up;
-  const T c0 = T(1) - T(0.5) * usq;
-  const T hu = T(-0.5) * usq;
-  const T ntau = n * a.inv_tau, dntau = dn * a.inv_tau;
-  const T Ep = co[C_EP * BQ + fr], En = co[C_EN * BQ + fr];
+  const float usq = ut * ut + up * up;
+  const float c0 = 1.0f - 0.5f * usq;
+  const float hu = -0.5f * usq;
+  const float ntau = n * a.inv_tau, dntau = dn * a.inv_tau;
+  const float Ep = co[C_EP * BQ + fr], En = co[C_EN * BQ + fr];
 
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     // varphi-derivative operands h_m = (-F^phi - Gamma v_i v_m) g_{i m}; K~ = K diag(v) (Sec. 2.3)
-    const T gvi = gam * vc.v[i];
-    T h[4];
+    const float gvi = gam * vc.v[i];
+    float h[4];
 #pragma unroll
     for (int mm = 0; mm < 4; ++mm) h[mm] = (-Fp - gvi * vc.v[mm]) * g[4 * i + mm];
-    const T ai = vc.v[i] * ut;
+    const float ai = vc.v[i] * ut;
     // The BGK relaxation and the closed-form reference part share the factor w_i w_j:
     //   (f^eq - n0 w w)/tau + n0 w w [v_i (E(q) + F^theta) + v_j F^phi]
     //   = w_i w_j [ (dn + n (poly - 1))/tau + n0 v_i (E + F^theta) + n0 v_j F^phi ]
-    const T ci = dntau + a.n0 * vc.v[i] * ((i >= 2 ? Ep : En) + Ft);
+    const float ci = dntau + a.n0 * vc.v[i] * ((i >= 2 ? Ep : En) + Ft);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int k = 4 * i + j;
-      const T* fk = sf + k * BQ * BS + bi;
-      const T Dt = (i >= 2) ? wp0 * fk[-2 * BS] + wp1 * fk[-BS] + wp2 * g[k] + wp3 * fk[BS]
+      const float* fk = sf + k * BQ * BS + bi;
+      const float Dt = (i >= 2) ? wp0 * fk[-2 * BS] + wp1 * fk[-BS] + wp2 * g[k] + wp3 * fk[BS]
                             : wn0 * fk[-BS] + wn1 * g[k] + wn2 * fk[BS] + wn3 * fk[2 * BS];
-      const T Dp = (j >= 2) ? (fk[-2] - T(6) * fk[-1] + T(3) * g[k] + T(2) * fk[1])
-                            : (T(-2) * fk[-1] - T(3) * g[k] + T(6) * fk[1] - fk[2]);
-      T rhs = -(vc.v[i] * Dt) - (vc.v[j] * cp6) * Dp;
+      const float Dp = (j >= 2) ? (fk[-2] - 6.0f * fk[-1] + 3.0f * g[k] + 2.0f * fk[1])
+                            : (-2.0f * fk[-1] - 3.0f * g[k] + 6.0f * fk[1] - fk[2]);
+      float rhs = -(vc.v[i] * Dt) - (vc.v[j] * cp6) * Dp;
       // force and inertial terms on the deviation: (Gamma v_j^2 - F^theta) dg/dv_theta + sum_m K_jm h_m
-      T dvt = T(0), dvp = T(0);
+      float dvt = 0.0f, dvp = 0.0f;
 #pragma unroll
       for (int mm = 0; mm < 4; ++mm) {
         dvt += vc.K[i][mm] * g[4 * mm + j];
@@ -452,13 +416,13 @@ __device__ __forceinline__ void phase3_node(const StageArgs<T>& a, const VConst<
       }
       rhs += (gam * vc.v[j] * vc.v[j] - Ft) * dvt + dvp;
       // BGK towards the third-order Hermite equilibrium (Eq. feq) plus the reference part
-      const T xi = ai + vc.v[j] * up;
-      const T pm1 = xi * (c0 + xi * (T(0.5) + xi * sixth)) + hu;
-      const T X = ntau * pm1 + (ci + a.n0 * vc.v[j] * Fp);
+      const float xi = ai + vc.v[j] * up;
+      const float pm1 = xi * (c0 + xi * (0.5f + xi * sixth)) + hu;
+      const float X = ntau * pm1 + (ci + a.n0 * vc.v[j] * Fp);
       rhs += vc.ww[i][j] * X - a.inv_tau * g[k];
-      T o;
+      float o;
       if (F0) {
-        const T g0 = su0[k * TQ * TS + ui];
+        const float g0 = su0[k * TQ * TS + ui];
         o = g0 + a.b * ((g[k] - g0) + rhs * a.dt);
       } else {
         o = rhs * a.dt + g[k];
@@ -706,9 +670,9 @@ __device__ __forceinline__ void phase3_pair(const StageArgs<float>& a, const Nod
 // Steps 1-3 for one tile: on packed node pairs (PAIRS: the grid is known to have the chunked layout), or in scalar
 // arithmetic, two or more nodes per thread (ensemble members with another layout).
 template <typename L, int CH, bool F0, bool PAIRS>
-__device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VConst<float>& vc, float* sm, int tid,
+__device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VConst& vc, float* sm, int tid,
                                           int q0, int s0) {
-  float* box = sm + L::BOX_OFF;
+  float* box = sm;
   float* co = sm + L::CO_OFF;
   pdl_wait();  // the coefficients too may come from the previous kernel (the scratch tables of vlb_step_noalloc)
   const bool pair = PAIRS || chunked<L>(a.nt, a.ns);
@@ -744,7 +708,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VCons
 #pragma unroll 1
   for (int m = 0; m < L::TQ / ROWS; ++m) {
     const int nr = tid / TS + ROWS * m, nc = tid % TS;
-    if (q0 + nr < a.nt && s0 + nc < a.ns) phase3_node<L, float, CH, F0>(a, vc, box, co, sm, nr, nc, q0 + nr, s0 + nc);
+    if (q0 + nr < a.nt && s0 + nc < a.ns) phase3_node<L, CH, F0>(a, vc, box, co, sm, nr, nc, q0 + nr, s0 + nc);
   }
 }
 
@@ -754,15 +718,15 @@ __device__ __forceinline__ void tile_body(const StageArgs<float>& a, const VCons
 // A persistent CTA (which stages many tiles) initialises the two mbarriers once and passes init =
 // false with the parity of each barrier's current phase.
 template <typename L, int CH, bool F0>
-__device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const VConst<float>& vc, float* sm, int tid,
+__device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const VConst& vc, float* sm, int tid,
                                               int q0, int s0, const CUtensorMap* tmb, const CUtensorMap* tmu,
                                               bool init = true, unsigned ph_box = 0, unsigned ph_u0 = 0) {
   constexpr unsigned BOX_BYTES = sizeof(float) * L::NST * L::BQ * L::BS;
   constexpr unsigned U0_BYTES = sizeof(float) * L::NU0 * L::TQ * TS;
-  static_assert((L::BOX_OFF * sizeof(float)) % 128 == 0 && (L::U0_OFF * sizeof(float)) % 128 == 0,
+  static_assert((L::U0_OFF * sizeof(float)) % 128 == 0,
                 "tensor-map destinations are 128-byte aligned");
   static_assert((L::MB_OFF * sizeof(float)) % 8 == 0, "mbarriers are 8-byte aligned");
-  float* box = sm + L::BOX_OFF;
+  float* box = sm;
   float* co = sm + L::CO_OFF;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + L::MB_OFF);
   if (init) {
@@ -826,7 +790,7 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
 // tiles whose box wraps around the grid take the per-thread copies.
 template <int TQR, int CH, bool F0, bool TMA>
 __global__ void __launch_bounds__(TQR*(TS / 2), TQR == 16 ? 2 : 4)
-    stage_kernel(StageArgs<float> a, VConst<float> vc, const __grid_constant__ CUtensorMap tmb,
+    stage_kernel(StageArgs<float> a, VConst vc, const __grid_constant__ CUtensorMap tmb,
                  const __grid_constant__ CUtensorMap tmu) {
   using L = StageLayR<TQR>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -851,7 +815,7 @@ template <int TQR, int CH, bool F0>
 __global__ void __launch_bounds__(TQR*(TS / 2), TQR == 16 ? 2 : 4) ensemble_stage_kernel(
                                                                        const EnsembleMember* members,
                                                                        const int2* items, int nitems, int ahead,
-                                                                       int stage, int* err, VConst<float> vc,
+                                                                       int stage, int* err, VConst vc,
                                                                        const __grid_constant__ EnsembleMaps maps) {
   using L = StageLayR<TQR>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -980,7 +944,7 @@ __device__ __forceinline__ StageArgs<float> member_args(const EnsembleMember& d,
 template <int TQR, int CH>
 __global__ void __launch_bounds__(TQR * (TS / 2), TQR == 16 ? 2 : 4) ensemble_persistent_kernel(
     const EnsembleMember* members, const int2* items, int nitems, int nsteps, int only0, unsigned* bar, int* err,
-    long long budget, int skip_cta, VConst<float> vc, const __grid_constant__ EnsembleMaps maps) {
+    long long budget, int skip_cta, VConst vc, const __grid_constant__ EnsembleMaps maps) {
   using L = StageLayR<TQR>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int s_ok;
@@ -1147,7 +1111,7 @@ __device__ __forceinline__ void discard_tile(const float* U, int64_t stride, int
 template <int CH>
 __global__ void __launch_bounds__(256, 2) wave_kernel(StageArgs<float> base, float* U0, float* U1, float* U2,
                                                       int nsteps, int lag, unsigned* cnt, int* err, long long budget,
-                                                      int skip_cta, VConst<float> vc,
+                                                      int skip_cta, VConst vc,
                                                       const __grid_constant__ WaveMaps maps) {
   using L = StageLay;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1238,17 +1202,16 @@ __global__ void __launch_bounds__(256, 2) wave_kernel(StageArgs<float> base, flo
   }
 }
 
-template <typename T>
-VConst<T> make_vconst() {
+VConst make_vconst() {
   const VelocityConsts d = velocity_consts();
-  VConst<T> c;
-  c.nc = make_node_const<T>();
+  VConst c;
+  c.nc = make_node_const<float>();
   for (int i = 0; i < 4; ++i) {
-    c.v[i] = (T)d.v[i];
-    c.w[i] = (T)d.w[i];
+    c.v[i] = (float)d.v[i];
+    c.w[i] = (float)d.w[i];
     for (int m = 0; m < 4; ++m) {
-      c.K[i][m] = (T)d.K[i][m];
-      c.ww[i][m] = (T)(d.w[i] * d.w[m]);
+      c.K[i][m] = (float)d.K[i][m];
+      c.ww[i][m] = (float)(d.w[i] * d.w[m]);
     }
   }
   return c;
@@ -1286,7 +1249,7 @@ cudaError_t launch_pairs(const StageArgs<float>& a, cudaStream_t st, const Stage
   static int mask = 0;
   cudaError_t e = ensure_smem(stage_kernel<TQR, CH, F0, TMA>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
-  static const VConst<float> vc = make_vconst<float>();
+  static const VConst vc = make_vconst();
   static const StageMaps none = {};
   const StageMaps& m = maps ? *maps : none;
   StageArgs<float> args = a;
@@ -1327,7 +1290,7 @@ cudaError_t launch_ens(const EnsembleMember* members, const int2* items, int nit
   static int mask = 0;
   cudaError_t e = ensure_smem(ensemble_stage_kernel<TQR, CH, F0>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
-  static const VConst<float> vc = make_vconst<float>();
+  static const VConst vc = make_vconst();
   static int resident[32] = {0};  // blocks of this kernel resident at once, per device
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1353,7 +1316,7 @@ cudaError_t launch_pers(const EnsembleMember* members, const int2* items, int ni
   static int mask = 0;
   cudaError_t e = ensure_smem(ensemble_persistent_kernel<TQR, CH>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
-  static const VConst<float> vc = make_vconst<float>();
+  static const VConst vc = make_vconst();
   static int occ[32] = {0}, sms[32] = {0};
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1540,7 +1503,7 @@ cudaError_t launch_wave_t(const StageArgs<float>& a, float* U0, float* U1, float
   static int mask = 0;
   cudaError_t e = ensure_smem(wave_kernel<CH>, L::BYTES, mask);
   if (e != cudaSuccess) return e;
-  static const VConst<float> vc = make_vconst<float>();
+  static const VConst vc = make_vconst();
   static int occ[32] = {0}, sms[32] = {0};
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
