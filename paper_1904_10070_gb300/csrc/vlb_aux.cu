@@ -549,12 +549,12 @@ __device__ const RowRules<double> g_pair_rules = make_row_rules<double>();
 __global__ void __launch_bounds__(128) pair_rows_kernel(const double* coefd, int nt, double dt, double M, double kappa,
                                                         float* rows) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= nt * kRowTable) return;
+  if (x >= nt * kRowTable) return;  // whole warps: a row each
   const int q = x / kRowTable;
   const RowRule<double> r = g_pair_rules.e[x % kRowTable];
   const double s = r.s == 3 ? 1.0 : r.s == 2 ? kappa : (r.s == 1 ? dt * M : dt);
   const double y = r.y ? coefd[C_J * nt + (q + r.y - 3 + nt) % nt] : 1.0;
-  rows[x] = (float)(s * (r.c1 * coefd[r.x1 * nt + q] * y + r.c2 * coefd[r.x2 * nt + q]));
+  rows[x] = row_table_entry(s * (r.c1 * coefd[r.x1 * nt + q] * y + r.c2 * coefd[r.x2 * nt + q]), x % kRowTable);
 }
 
 cudaError_t launch_pair_rows(const double* coefd, int nt, double dt, double M, double kappa, float* rows,

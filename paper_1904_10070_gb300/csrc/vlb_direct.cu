@@ -318,8 +318,10 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
 
   // population k: acc (dt times the other terms) -> stored update.  UW3 seen from the upwind side has the
   // weights 1, -6, 3, 2 on the far, near, centre and downwind nodes (tf .. td: theta, on J g; pv: varphi).
-  // FP64 folds the three centre taps into one coefficient, whose rounding is far below the scheme's;
-  // FP32 keeps the varphi difference on whole-number weights, which cancel on a uniform field.
+  // FP64 folds the three centre taps into one coefficient, whose rounding is far below the scheme's.
+  // FP32 keeps the varphi difference on whole-number weights, which cancel on a uniform field, and takes the theta
+  // taps on differences to the node, with their sum as the coefficient tm: they nearly cancel, so the products
+  // stay small (tau = 0.1, 401 x 63: 1.05e-7 -> 0.96e-7; 250 x 501, 8 steps: 314 -> 308 us).
   auto update = [&](int k, T acc, T g0, T tf, T tn, T tm, T td, Off rf, Off rn, Off rd, int y, T cc,
                     Off cf, Off cn, Off cd) {
     const T* f = a.fin + k * st;
@@ -327,9 +329,15 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     if (F0 && !HOLD) g0 = at(a.f0 + k * st, id);
     if (F0) acc = vadd(acc, vsub(g, g0));
     if constexpr (!WENO) {
-      acc = vfma(tf, at(f, rf), acc);
-      acc = vfma(tn, at(f, rn), acc);
-      acc = vfma(td, at(f, rd), acc);
+      if constexpr (DF) {
+        acc = vfma(tf, vsub(at(f, rf), g), acc);
+        acc = vfma(tn, vsub(at(f, rn), g), acc);
+        acc = vfma(td, vsub(at(f, rd), g), acc);
+      } else {
+        acc = vfma(tf, at(f, rf), acc);
+        acc = vfma(tn, at(f, rn), acc);
+        acc = vfma(td, at(f, rd), acc);
+      }
     }
     if constexpr (WENO) {
       acc = vadd(acc, s_adv[(k * TQ + lr) * TSW + lc]);
@@ -360,7 +368,12 @@ __global__ void __launch_bounds__(TQ* TSW*(SPLIT ? 4 : 1), ADV == VLB_WENO5 && s
     for (int i = 0; i < 4; ++i) {
       const int x = (i == 0 || i == 3) ? 0 : 1;
       const T* t = rt + E_TH + 8 * x;
-      const T tf = t[i >= 2 ? TAP_FARP : TAP_FARN], tn = t[i >= 2 ? TAP_NEARP : TAP_NEARN], tm = t[TAP_MID];
+      const T tf = t[i >= 2 ? TAP_FARP : TAP_FARN], tn = t[i >= 2 ? TAP_NEARP : TAP_NEARN];
+      T tm = t[TAP_MID];
+      if constexpr (DF) {  // the sum of the four taps, v_i (E + Gamma)
+        const T gv = x == 0 ? rt[E_GBB] * (T(1) / nc.v[0]) : rt[E_GAA] * (T(1) / nc.v[1]);
+        tm = vadd(vfma(i >= 2 ? nc.v[x] : -nc.v[x], rt[E_EM], rt[E_NEB + x]), i >= 2 ? gv : -gv);
+      }
       const T td = t[i >= 2 ? TAP_DOWNP : TAP_DOWNN];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {

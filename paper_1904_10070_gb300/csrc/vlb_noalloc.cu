@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(64) noalloc_tables(T* coef, int nt, int nphi, 
   const double x1 = __shfl_sync(0xffffffffu, c, e.x1), x2 = __shfl_sync(0xffffffffu, c, e.x2);
   const double y = __shfl_sync(0xffffffffu, own, e.y ? e.y - 1 : 0);
   const double s = e.s == 3 ? 1.0 : e.s == 2 ? kappa : (e.s == 1 ? dt * M : dt);
-  rows[q * vlb::kRowTable + k] = (float)(s * (e.c1 * x1 * (e.y ? y : 1.0) + e.c2 * x2));
+  rows[q * vlb::kRowTable + k] = vlb::row_table_entry(s * (e.c1 * x1 * (e.y ? y : 1.0) + e.c2 * x2), k);
 }
 
 const char* check_params(const vlb_params* p) {
