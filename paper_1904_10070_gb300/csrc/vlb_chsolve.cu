@@ -12,7 +12,7 @@
 //   1. transform the theta rows of J dt L_phi, two rows as one complex transform per CTA, and store the
 //      half spectrum n = 0 .. N_phi / 2 (the two real columns 0 and N_phi / 2 packed into one),
 //   2. transform strips of columns, divide by 1 + dt M kappa lambda and transform them back,
-//   3. transform the rows back two at a time, divide by N_theta N_phi J and form phi_out (in FP32 as
+//   3. transform the rows back (FP64: two at a time), divide by N_theta N_phi J and form phi_out (in FP32 as
 //      the float pair hi + lo with an error-free sum, as the stage kernel does).
 // The FFTs are in place in shared memory, in the state's precision; N_theta and N_phi are powers of
 // two <= 4096.  The two factors of lambda, (4/h_theta^2) sin^2(pi m/N_theta) and (4/h_phi^2)
@@ -53,6 +53,11 @@ template <typename T>
 __device__ __forceinline__ C2<T> cmul(C2<T> v, C2<T> t) {
   return {v.x * t.x - v.y * t.y, v.x * t.y + v.y * t.x};
 }
+// c + a b
+template <typename T>
+__device__ __forceinline__ C2<T> cfma(C2<T> a, C2<T> b, C2<T> c) {
+  return {fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y))};
+}
 
 // In-place FFT along the first index of a[i * w + c] (w = 2^logw interleaved sequences of length n,
 // loaded in bit-reversed order of i; element e stored at padded(e, sh)), decimation in time: the
@@ -92,15 +97,15 @@ __device__ void fft_strided(C2<T>* a, int n, int logn, int logw, int sh, const C
       }
       const int e0 = padded((i0 << logw) + c, sh), e1 = padded(((i0 + h) << logw) + c, sh);
       const int e2 = padded(((i0 + 2 * h) << logw) + c, sh), e3 = padded(((i0 + 3 * h) << logw) + c, sh);
-      const C2<T> a0 = a[e0], a1 = cmul(a[e1], t1), a2 = a[e2], a3 = cmul(a[e3], t1);
-      const C2<T> b0 = {a0.x + a1.x, a0.y + a1.y}, b1 = {a0.x - a1.x, a0.y - a1.y};
-      const C2<T> b2 = cmul(C2<T>{a2.x + a3.x, a2.y + a3.y}, t2);
-      C2<T> b3 = cmul(C2<T>{a2.x - a3.x, a2.y - a3.y}, t2);
-      b3 = inverse ? C2<T>{-b3.y, b3.x} : C2<T>{b3.y, -b3.x};  // times +i / -i
-      a[e0] = {b0.x + b2.x, b0.y + b2.y};
-      a[e2] = {b0.x - b2.x, b0.y - b2.y};
-      a[e1] = {b1.x + b3.x, b1.y + b3.y};
-      a[e3] = {b1.x - b3.x, b1.y - b3.y};
+      // multiply-adds throughout: as many operations as products and sums apart, two roundings instead of three
+      const C2<T> a0 = a[e0], a1 = a[e1], a2 = a[e2], a3 = a[e3];
+      const C2<T> n1 = {-t1.x, -t1.y}, b0 = cfma(a1, t1, a0), b1 = cfma(a1, n1, a0);
+      const C2<T> b2 = cfma(a3, t1, a2), b3 = cfma(a3, n1, a2);
+      const C2<T> t3 = inverse ? C2<T>{-t2.y, t2.x} : C2<T>{t2.y, -t2.x};  // +i t2 / -i t2
+      a[e0] = cfma(b2, t2, b0);
+      a[e2] = cfma(b2, C2<T>{-t2.x, -t2.y}, b0);
+      a[e1] = cfma(b3, t3, b1);
+      a[e3] = cfma(b3, C2<T>{-t3.x, -t3.y}, b1);
     }
     __syncthreads();
   }
@@ -278,32 +283,38 @@ __device__ __forceinline__ void pair_add(float base, float base_lo, float inc, f
   lo = lo2 - (hi - s1);
 }
 
-// 3. Rows q = 2 b and q + 1: inverse F_phi of both in one transform, y = Re (Im) / (N J), phi_out = phi^n +
-// b (phi_in - phi^n + y).
+// Rows that share an inverse transform.  In FP64 two, as real and imaginary part.  In FP32 one: the rounding of this
+// transform is what phi keeps undamped, and with a row alone half of it goes with the imaginary part (populations at
+// 1024 x 2048 after two steps: error 2.2e-7 with two rows, 1.9e-7 with one).
+template <typename T>
+constexpr int inv_rows() { return sizeof(T) == 8 ? 2 : 1; }
+
+// 3. Rows q .. q + inv_rows - 1: inverse F_phi in one transform, y = Re (Im) / (N J), phi_out = phi^n + b (phi_in - phi^n + y).
 template <typename T>
 __global__ void __launch_bounds__(256) row_inv_kernel(int ns, int logns, double inv_n, const double* J,
                                                       const C2<T>* tw_s, const C2<T>* buf, const T* phin,
                                                       const T* phi0, T* phiout, int64_t lo_off, T b) {
   constexpr bool DF = sizeof(T) == 4;  // phi as a float pair
   constexpr int U = 4;                 // nodes per batch of loads (four state words each)
+  constexpr int ROWS = inv_rows<T>(), NB = kBatch / ROWS;
   extern __shared__ __align__(16) unsigned char raw[];
   C2<T>* a = reinterpret_cast<C2<T>*>(raw);
   const int sh = row_pad_shift(logns), nh = ns / 2;
   C2<T>* tw = a + padded(ns, sh);
-  const int64_t q = 2 * (int64_t)blockIdx.x;
+  const int64_t q = ROWS * (int64_t)blockIdx.x;
   const C2<T>*r0 = buf + q * nh, *r1 = r0 + nh;
-  for (int s0 = threadIdx.x; s0 < nh; s0 += (kBatch / 2) * blockDim.x) {
-    C2<T> v[kBatch / 2], w[kBatch / 2];
+  for (int s0 = threadIdx.x; s0 < nh; s0 += NB * blockDim.x) {
+    C2<T> v[NB], w[NB];
 #pragma unroll
-    for (int u = 0; u < kBatch / 2; ++u) {
+    for (int u = 0; u < NB; ++u) {
       const int s = s0 + u * blockDim.x;
       if (s < nh) {
         v[u] = r0[s];
-        w[u] = r1[s];
+        w[u] = ROWS == 2 ? r1[s] : C2<T>{T(0), T(0)};
       }
     }
 #pragma unroll
-    for (int u = 0; u < kBatch / 2; ++u) {
+    for (int u = 0; u < NB; ++u) {
       const int s = s0 + u * blockDim.x;
       if (s >= nh) continue;
       if (s == 0) {  // the packed real values at 0 and N_phi / 2
@@ -318,13 +329,13 @@ __global__ void __launch_bounds__(256) row_inv_kernel(int ns, int logns, double 
   load_twiddles(tw, tw_s, ns);
   __syncthreads();
   fft_strided(a, ns, logns, 0, sh, tw, true);
-  const T scale[2] = {(T)(inv_n / J[q]), (T)(inv_n / J[q + 1])};
-  for (int s0 = threadIdx.x; s0 < 2 * ns; s0 += U * blockDim.x) {  // the two rows follow each other
+  const T scale[2] = {(T)(inv_n / J[q]), (T)(inv_n / J[q + ROWS - 1])};
+  for (int s0 = threadIdx.x; s0 < ROWS * ns; s0 += U * blockDim.x) {  // two rows follow each other
     T ph[U], lo[U], base[U], base_lo[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s < 2 * ns) {
+      if (s < ROWS * ns) {
         const int64_t g = q * ns + s;
         ph[u] = phin[g];
         lo[u] = DF ? phin[g + lo_off] : T(0);
@@ -335,10 +346,10 @@ __global__ void __launch_bounds__(256) row_inv_kernel(int ns, int logns, double 
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int s = s0 + u * blockDim.x;
-      if (s >= 2 * ns) continue;
+      if (s >= ROWS * ns) continue;
       const int64_t g = q * ns + s;
       const C2<T> z = a[padded(s & (ns - 1), sh)];
-      const T y = s < ns ? z.x * scale[0] : z.y * scale[1];
+      const T y = ROWS == 1 || s < ns ? z.x * scale[0] : z.y * scale[1];
       const T inc = phi0 ? b * (((ph[u] - base[u]) + (lo[u] - base_lo[u])) + y) : y;
       if constexpr (DF) {
         float hi_o, lo_o;
@@ -442,7 +453,7 @@ cudaError_t launch_ch_stab(int nt, int ns, double dt_m_kappa, const double* J, c
   col_solve_kernel<T><<<nh >> lcw, col_threads, col_bytes, st>>>(nt, lognt, nh, lcw, (T)dt_m_kappa, lam, lam + nt, tw_t,
                                                                  cb);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  row_inv_kernel<T><<<nt / 2, 256, row_bytes, st>>>(ns, logns, 1.0 / ((double)nt * ns), J, tw_s, cb, phin, phi0, phiout,
+  row_inv_kernel<T><<<nt / inv_rows<T>(), 256, row_bytes, st>>>(ns, logns, 1.0 / ((double)nt * ns), J, tw_s, cb, phin, phi0, phiout,
                                                    lo_off, b);
   return cudaGetLastError();
 }
