@@ -856,11 +856,17 @@ vlb_status vlb_structure_length(vlb_handle* h, double* out) {
   std::vector<double> sums((size_t)2 * nb);
   VLB_CUDA(h, cudaMemcpyAsync(sums.data(), part, sums.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   st = sync_and_check(h, "vlb_structure_length", false);
-  double s_sum = 0.0, k_sum = 0.0;
-  for (int b = 0; b < nb; ++b) {
-    s_sum += sums[2 * b];
-    k_sum += sums[2 * b + 1];
-  }
+  // compensated: up to 2048 strips, most of them far smaller than the first ones
+  auto total = [&](int k) {
+    double s = 0.0, c = 0.0;
+    for (int b = 0; b < nb; ++b) {
+      const double x = sums[2 * b + k], t = s + x;
+      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+      s = t;
+    }
+    return s + c;
+  };
+  const double s_sum = total(0), k_sum = total(1);
   // a uniform phi has no domains: its length is infinite
   *out = k_sum > 0.0 ? 2.0 * M_PI * s_sum / k_sum : INFINITY;
   return st;
