@@ -868,7 +868,7 @@ __global__ void __launch_bounds__(WG_THREADS)
     if (bias) ok = bias_segments<DC, NS>(sm, L::STAGE, full, empty, nmine, tid, tslot + 1, bacc);
     ok = ok && (nmine == 0 || mbar_wait(done, 0));
     if (bias) ok = bias_store<DC>(sm, ok, bacc, tid, tslot + 1, bpart);
-    if (ok && nmine > 0) {
+    if (__all_sync(~0u, ok) && nmine > 0) {
       tc_fence_after();
       uint32_t raw[48];
 #pragma unroll
