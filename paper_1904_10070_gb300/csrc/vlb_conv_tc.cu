@@ -262,17 +262,14 @@ __device__ __forceinline__ void transpose_chunks(uint4* a, int lane) {
   }
 }
 
-// The mask of a thread's outputs, loaded before the accumulator is waited for.  64 channels in bf16: chunk lane % 8 of the
-// eight pixels of the lane's group (the order of the stores after the transpose); 16 channels, or FP32 outputs alone
-// (`own`): the thread's pixel.
+// The mask of a thread's bf16 outputs, loaded before the accumulator is waited for.  64 channels: chunk lane % 8 of the
+// eight pixels of the lane's group (the order of the stores after the transpose); 16 channels: the thread's pixel.
 template <int COUT>
-__device__ __forceinline__ void load_mask(uint4* mk, const bf16* mask, size_t p0, int warp, int lane, bool own) {
-  const bool turned = COUT == 64 && !own;
-  const bf16* base = turned ? mask + (p0 + 32 * warp + (lane & ~7)) * 64 + (lane & 7) * 8
-                            : mask + (p0 + 32 * warp + lane) * COUT;
-  const int step = turned ? 64 : 8;
+__device__ __forceinline__ void load_mask(uint4* mk, const bf16* mask, size_t p0, int warp, int lane) {
+  const bf16* base = COUT == 64 ? mask + (p0 + 32 * warp + (lane & ~7)) * 64 + (lane & 7) * 8
+                                : mask + (p0 + 32 * warp + lane) * COUT;
 #pragma unroll
-  for (int i = 0; i < COUT / 8; ++i) mk[i] = *reinterpret_cast<const uint4*>(base + i * step);
+  for (int i = 0; i < COUT / 8; ++i) mk[i] = *reinterpret_cast<const uint4*>(base + (COUT == 64 ? i * 64 : i * 8));
 }
 
 // bf16 outputs o whose mask is not > 0 become zero
@@ -285,8 +282,8 @@ __device__ __forceinline__ void apply_mask(uint4& o, const uint4& mk) {
 }
 
 // Epilogue of the work item whose first pixel is p0 from the accumulator at column `col0`: thread (warp, lane) owns
-// pixel p0 + 32 warp + lane; all C_out columns are read before one wait.  mk: load_mask, for the bf16 output, or for the
-// FP32 output where it is the only one.
+// pixel p0 + 32 warp + lane; all C_out columns are read before one wait.  mk: load_mask, for the bf16 output.  An FP32
+// output's mask is read 16 columns at a time (8 at a time its stores wait twice as often: 64 -> 64 at 256 x 512 26.9 us).
 // The bf16 rows of 64 channels are transposed among eight lanes first, so that a store instruction writes four whole
 // 128-byte pixels instead of 16 bytes of 32 pixels.
 template <int COUT>
@@ -299,11 +296,15 @@ __device__ __forceinline__ void epilogue(uint32_t tmem, uint32_t col0, size_t p0
   for (int j = 0; j < COUT / 16; ++j)
     tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + col0 + (uint32_t)(16 * j), raw + 16 * j);
   tmem_wait_ld();
-  uint4 o[COUT / 8];
+  uint4 o[COUT / 8], mf[2];
 #pragma unroll
   for (int j = 0; j < COUT / 8; ++j) {
     float v[8];
     const int co = 8 * j;
+    if (yf && mask && j % 2 == 0) {
+      mf[0] = *reinterpret_cast<const uint4*>(mask + p * COUT + co);
+      mf[1] = *reinterpret_cast<const uint4*>(mask + p * COUT + co + 8);
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(raw[co + i]) + sbias[co + i];
     if (relu) {
@@ -315,8 +316,7 @@ __device__ __forceinline__ void epilogue(uint32_t tmem, uint32_t col0, size_t p0
     for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
     if (yf) {
       if (mask) {
-        const uint4 m0 = y ? *reinterpret_cast<const uint4*>(mask + p * COUT + co) : mk[j];
-        const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m0);
+        const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(mf + j % 2);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (!(__low2float(mh[i]) > 0.0f)) v[2 * i] = 0.0f;
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
     for (int k = a; k < nmine && ok; k += 2) {
       const size_t p0 = item_pixel(H, W, blockIdx.x + k * gridDim.x);
       uint4 mk[COUT / 8];
-      if (mask) load_mask<COUT>(mk, mask, p0, quarter, lane, !y);
+      if (mask && y) load_mask<COUT>(mk, mask, p0, quarter, lane);
       ok = __all_sync(~0u, mbar_wait(afull + a, (k >> 1) & 1));
       if (!ok) break;
       tc_fence_after();
