@@ -120,8 +120,8 @@ vlb_status vlb_set_state(vlb_handle* h, const double* f16, const double* phi);
 vlb_status vlb_get_state(vlb_handle* h, double* f16, double* phi);
 
 /* Advance nsteps SSP-RK3 steps (3 fused-stage launches per step), asynchronously on the stream.
- * Axisymmetric grids (N_phi = 1, N_theta <= 4096) run up to 256 whole steps per launch of a
- * single-CTA kernel instead.  With the wavefront schedule (vlb_set_schedule) up to 4096 whole steps
+ * Axisymmetric grids (N_phi = 1, N_theta <= 4096) run up to 256 whole steps per launch of one
+ * thread-block cluster instead.  With the wavefront schedule (vlb_set_schedule) up to 4096 whole steps
  * run per persistent launch, whose bounded dependency waits raise the same flag as the bulk-copy
  * waits below.  The result does not depend on how the steps are grouped or scheduled (bit for bit).
  * With diag_every > 0 the totals are checked every diag_every steps and at the end, the
@@ -147,7 +147,8 @@ vlb_status vlb_test_raise_flag(vlb_handle* h, int32_t value);
 vlb_status vlb_get_fields(vlb_handle* h, double* rho, double* u_th, double* u_ph, double* phi,
                           double* mu);
 
-/* Conserved totals and diagnostics, reduced on the GPU in FP64 (FP32 states: in float pairs of about 48 bits):
+/* Conserved totals and diagnostics, reduced on the GPU in FP64 (FP32 states: a node's share in float pairs, as
+ * accurate in the totals as FP64):
  * out[0] = sum n sqrt(g) dtheta dvarphi, out[1] = sum phi sqrt(g) dtheta dvarphi,
  * out[2] = Psi (Eq. Landau, central differences), out[3] = max |u|.  Synchronous. */
 vlb_status vlb_get_totals(vlb_handle* h, double out[4]);
@@ -187,7 +188,7 @@ vlb_status vlb_steps_done(const vlb_handle* h, int64_t* out);
  * explicit grid with N_theta a multiple of 16 and >= 176 and N_phi a multiple of 32 (VLB_ERR_ARG
  * otherwise).  VLB_SCHED_AUTO (the default) takes the per-stage launches: the stage is bound by
  * latency rather than HBM, and the wavefront's per-tile dependency waits cost more than the
- * HBM traffic it saves (measured on GB300: 0.498 against 0.204 ms per step at 1024 x 2048).
+ * HBM traffic it saves (measured on GB300: 0.45 against 0.204 ms per step at 1024 x 2048).
  * vlb_get_schedule writes the schedule vlb_step takes (STAGES or WAVE). */
 enum { VLB_SCHED_AUTO = 0, VLB_SCHED_STAGES = 1, VLB_SCHED_WAVE = 2 };
 vlb_status vlb_set_schedule(vlb_handle* h, int32_t schedule);

@@ -247,7 +247,7 @@ constexpr long long kWaveBudget = 1ll << 31;  // SM clock cycles per dependency 
 
 // Whether vlb_step takes the wavefront schedule: only when asked for (VLB_SCHED_WAVE) on a grid that
 // has its counters and the stage tensor maps.  VLB_SCHED_AUTO takes the per-stage launches, which
-// measured faster on GB300 (0.204 against 0.498 ms per step at 1024 x 2048).
+// measured faster on GB300 (0.204 against 0.45 ms per step at 1024 x 2048).
 bool wave_active(const vlb_handle* h) {
   return h->kind == 0 && h->wave_cnt && h->wave_maps && h->sched == VLB_SCHED_WAVE;
 }

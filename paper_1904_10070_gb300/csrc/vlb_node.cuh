@@ -10,9 +10,9 @@
 // themselves; the step kernels are bound by the floating-point units, so this is their main saving.
 // Moments are sums of the same combinations.
 //
-// V is the lane type: double, float, or float2 (two nodes in packed FP32x2 arithmetic).  All
-// operations are explicitly rounded (no contraction), so that every kernel and every column of a
-// grid evaluates the same sequence of roundings.
+// V is the lane type: double, float, or float2 (two nodes in packed FP32x2 arithmetic).  The
+// operations of the UW3 step are explicitly rounded (no contraction), so that every kernel and every column of a
+// grid evaluates the same sequence of roundings; those of the WENO functions are left to the compiler.
 #pragma once
 
 #include "vlb_internal.cuh"
@@ -51,7 +51,7 @@ __device__ __forceinline__ double node_recip(double x) { return __drcp_rn(x); }
 // fix: 1 - sum w v v with the constants as they are rounded (FP32: -4.0e-8, nearly all from a, which rounds up by a
 // third of an ulp).
 template <typename T>
-struct NodeConst {
+struct alignas(16) NodeConst {  // 16-byte loads of what follows it in a kernel's parameters
   T v[2], v2[2], kap[2][2], lam[2][2], ww[2][2], fix;
 };
 
@@ -89,8 +89,8 @@ __device__ __forceinline__ V node_velocity(V m, V inv, T fix) {
 // operations that every node would otherwise repeat).  Entry e of row q is
 //   S (c1 X1(q) Y + c2 X2(q))  -  [e >= E_CC] dt / tau
 // with X1, X2 coefficient arrays, S one of dt, M dt, kappa and 1, and Y one of 1, J(q - 2 .. q + 2).
-// FP32 pair kernels read the 32-entry rows of a table in global memory, formed once per handle in FP64; the FP64
-// direct kernel forms the rows of its tile in shared memory.
+// FP32 pair kernels read the 32-entry rows of a table in global memory, formed once per handle in FP64
+// (row_table_entry rounds it); the FP64 direct kernel forms the rows of its tile in shared memory.
 enum RowEntry : int {
   E_GBB = 0,  // Gamma v_b^2, Gamma v_b v_a, Gamma v_a^2
   E_GBA,

@@ -784,7 +784,7 @@ __device__ __forceinline__ void tile_body_tma(const StageArgs<float>& a, const V
   phase3_pair<L, CH, F0>(a, vc.nc, box, co, sm, own, u0_hi, u0_lo, lr, lc, q0 + lr, s0 + lc);
 }
 
-// One CTA per 16 x 32 tile, on packed node pairs.
+// One CTA per TQR x 32 tile, on packed node pairs.
 // F0: the stage combines with U^n (stages 2 and 3); the first stage writes U_in + dt L(U_in).
 // TMA: interior tiles are staged by tensor-map copies (tmb: the box of fin, tmu: the tile of f0);
 // tiles whose box wraps around the grid take the per-thread copies.
