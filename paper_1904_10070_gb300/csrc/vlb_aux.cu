@@ -213,8 +213,9 @@ __global__ void __launch_bounds__(TOTAL_THREADS) totals_kernel(const T* state, i
 // sums and products (Dekker 1971, Knuth), 2^-46 relative each, and FP64 takes over at the row.  What a sum over
 // many nodes averages out may stay at that; what it does not is done as exactly as in FP64: differences keep their
 // relative accuracy (diff, 1 - phi^2 as a product), phi is summed with the rounding of its low words carried, and
-// the node of the largest |u| is evaluated again in FP64.  About 560 FP32 operations a node.  A node whose values
-// leave the range in which the pairs neither overflow nor lose bits to underflow takes the FP64 path.
+// the node of the largest |u| is evaluated again in FP64.  About 560 FP32 operations a node, 100 us (86 with pairs
+// alone).  A node whose values leave the range in which the pairs neither overflow nor lose bits to underflow takes the
+// FP64 path.
 struct FF {
   float h, l;
 };

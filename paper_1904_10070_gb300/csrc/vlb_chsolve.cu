@@ -21,7 +21,7 @@
 // transform lengths, which each CTA copies from global memory (L2) into shared memory.
 // The kernels are bound by the shared-memory passes and the barriers of the transforms, so half the data is
 // half the time: per stage at 1024 x 2048 in FP32 20.5 + 41.7 + 26.9 us with complex transforms of every row,
-// 13.6 + 21.1 + 20.0 us now.
+// 13.6 + 21.2 + 24.1 us now.
 #include <math.h>
 
 #include <vector>
@@ -467,8 +467,9 @@ namespace {
 // into one), the mirrored half enters by weight 2, and one root serves the modes m and -m.  A column CTA sums
 // S and |k| S over its strip (k = (m'/r, n'/R), m' and n' the signed frequencies; the mean mode m = n = 0 is left
 // out) and writes the two sums to part[2 b], part[2 b + 1].  The twiddles are tabulated once per call instead
-// of by every CTA.  1024 x 2048: 338 + 324 us for complex transforms with per-CTA twiddles, 123 + 145 us now.  On grids
-// of at most kOwnTwiddles rows and columns a CTA forms its own: two values a thread at most, less than the launch.
+// of by every CTA.  1024 x 2048: 338 + 324 us for complex transforms with per-CTA twiddles, 123 + 145 us
+// with real ones, 18 us less for both with butterflies of multiply-adds.  On grids
+// of at most kOwnTwiddles rows and columns a CTA forms its own: a value a thread at most, less than the launch.
 
 constexpr int kOwnTwiddles = 64;
 
